@@ -7,7 +7,7 @@
  * linearised system (sec. 2.1). A radial difference scheme couples a zone only to its neighbours,
  * so for the zones k = 0 .. n-1 of one ray, with m unknowns per zone, that linear system reads
  *
- *     A_k x_{k-1} + B_k x_k + C_k x_{k+1} = d_k        (A_0 and C_{n-1} are not read).
+ *     A_k x_{k-1} + B_k x_k + C_k x_{k+1} = d_k        (A_0 and C_{n-1} are not used).
  *
  * The pair-process source derivatives of vx_rates_spectral (blocks d(j0, chi0)/dJ and
  * d(j1, chi1)/dH of the partner spectrum) are part of B_k in such a system; the radial flux terms
@@ -15,12 +15,11 @@
  *
  * Method (GB300: FP32 arithmetic, FP64 only where accuracy needs it). Block LU along the ray
  * without pivoting across zones: D_0 = B_0, D_k = B_k - A_k G_{k-1} with G_k = D_k^{-1} C_k,
- * each D_k factored with partial pivoting inside the block. The factorisation is done in FP32 from
- * FP32 copies of the blocks, one CTA per ray: the product A_k G_{k-1} on the tensor cores (TF32
- * with each operand split into two parts, three products: about FP32 accuracy), then Gauss-Jordan
- * elimination of [D_k | C_k] with partial pivoting, whose right-hand block ends as G_k and whose
- * multipliers are kept. Then the ray is solved by replaying those eliminations on the right-hand
- * side, and
+ * each D_k inverted with partial pivoting inside the block. The factorisation is done in FP32 from
+ * FP32 copies of the blocks, one CTA per ray, its matrix products on the tensor cores (TF32 with each
+ * operand split into two parts, three products: about FP32 accuracy); D_k^{-1} and G_k are kept. Then
+ * the ray is solved by matrix-vector products with those, y_k = D_k^{-1} (d_k - A_k y_{k-1}) forward and
+ * x_k = y_k - G_k x_{k+1} backward, and
  * n_refine sweeps of iterative refinement follow, each from the FP64 residual d - M x of the
  * caller's FP64 blocks. For a ray whose Schur complements are well conditioned (e.g. block rows
  * diagonally dominant) every sweep gains a factor of about cond x 1e-7, so two sweeps reach FP64
@@ -49,7 +48,7 @@ typedef struct vx_btd vx_btd;
 
 /* Creates a solver for m unknowns per zone (1 .. VX_BTD_MAX_M) and batches of at most max_zones
  * zones (>= 0), with n_refine FP64 refinement sweeps (0 .. VX_BTD_MAX_REFINE; 0 leaves the FP32
- * solution). Allocates the device workspace: (12 m^2 + 16 m + 4) bytes per zone. *out is set to
+ * solution). Allocates the device workspace: 12 m (m + 7) + 4 (m + 7) + 12 m + 4 bytes per zone at most. *out is set to
  * NULL on failure. Errors: VX_ERR_INVALID_ARG, VX_ERR_OOM, VX_ERR_CUDA. */
 vx_status vx_btd_create(int m, long long max_zones, int n_refine, vx_btd **out);
 

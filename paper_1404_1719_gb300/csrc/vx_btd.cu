@@ -1,23 +1,25 @@
 // vx_btd.cu -- batched block-tridiagonal solve of the per-ray Newton systems (include/vx_btd.h).
 //
-// One ray per CTA (or per warp), since a ray's zones are a sequential chain; k_btd_validate first
-// checks that the ray offsets partition the zones (else every kernel returns at once):
-//  * k_btd_factor: block elimination along the ray in FP32, one CTA per ray. Per zone: stage B_k
-//    and A_k, form D_k = B_k - A_k G_{k-1} on the tensor cores (G_{k-1} is still in shared memory
-//    from the previous zone), then Gauss-Jordan elimination with partial pivoting (row indirection)
-//    on [D_k | C_k] held in registers, which leaves G_k = D_k^{-1} C_k. Each step's multiplier
-//    column, G_k and an FP32 copy of A_k are written column-major, the pivot order as an index
-//    vector.
-//  * k_btd_sweep: one warp per ray solves M delta = rhs with those: forward
-//    y_k = D_k^{-1} (rhs_k - A_k y_{k-1}) by replaying the zone's elimination on the vector,
-//    backward delta_k = y_k - G_k delta_{k+1}; a lane holds rows lane + 32 t of a zone's vector and
-//    the element being eliminated is broadcast by shuffle. The first sweep writes x = delta, later
-//    ones add delta to x in FP64.
+// A ray's zones are a sequential chain, so a ray belongs to one CTA; k_btd_validate first checks that the
+// ray offsets partition the zones (else every kernel returns at once):
+//  * k_btd_convert: the caller's FP64 blocks to FP32, with the zero patterns of the couplings' rows.
+//  * k_btd_factor: block elimination along the ray in FP32, one CTA per ray. Per zone:
+//    D_k = B_k - A_k G_{k-1} on the tensor cores, D_k inverted in place by Gauss-Jordan elimination with
+//    partial pivoting in panels of eight columns (one warp eliminates within a panel, the others apply its
+//    rank-8 transform on the tensor cores), G_k = D_k^{-1} C_k on the tensor cores. D_k^{-1} and G_k
+//    replace B_k and C_k in the workspace.
+//  * k_btd_sweep: one CTA per ray solves M delta = rhs with those: forward
+//    y_k = D_k^{-1} (rhs_k - A_k y_{k-1}), backward delta_k = y_k - G_k delta_{k+1}, a chain of
+//    matrix-vector products. The first sweep writes x = delta, later ones add delta to x in FP64.
 //  * k_btd_resid: the FP64 residual r = d - M x from the caller's FP64 blocks, a warp per zone,
 //    four lanes per row and eight rows per pass (coalesced), FMA accumulation and a fixed two-step
 //    shuffle reduction per row.
-// The host runs validate, factor, sweep, then n_refine times (resid, sweep), all on the caller's
+// The host runs validate, convert, factor, sweep, then n_refine times (resid, sweep), all on the caller's
 // stream.
+// With the inverse instead of the elimination's multipliers (which the sweeps replayed, a shuffle per
+// unknown), GB300, m = 84, 400 zones a ray: one ray factor 24.3 -> 10.0 ms, a sweep 3.0 -> 1.3 ms; 304 rays
+// 29.7 -> 14.9 ms (conversion included in the former, 8.0 ms apart in the latter) and 3.1 -> 1.8 ms (10.3 GB, 5.7 TB/s).
+// The solution's error without refinement and with one sweep is 0.2 to 0.8 of what it was (m = 34 to 128).
 #include "../../include/vx_btd.h"
 
 #include <cuda_runtime.h>
@@ -71,13 +73,14 @@ vx_status device_array(const void *p, size_t align, const char *name) {
     } while (0)
 
 struct BtdArgs {
-    int m, ld, n_rays;
+    int m, ld, mp, nbuf, nring, n_rays;  // ld: row stride of the FP32 blocks; mp: m rounded up to 8
     long long n_zones;
     const int *off;
     const double *A, *B, *C, *d, *rhs;
     double *x, *r;
-    float *Mt, *Gt, *At, *y;  // Mt: the Gauss-Jordan multipliers of D_k, column j at j m, pivot value at (j, perm[j])
-    int *perm, *zbad, *flag;
+    float *Di, *Gt, *At, *y;  // per zone B_k, then D_k^{-1}; C_k, then G_k; A_k in FP32, row-major [m][ld]; y_k [m]
+    unsigned short *nz;       // [Z][C, A][mp] zero patterns of the rows
+    int *zbad, *flag;
     const int *inval;  // set by k_btd_validate when the offsets are not a partition of the zones
 };
 
@@ -103,595 +106,801 @@ __global__ void k_btd_validate(const int *off, int n_rays, long long n_zones, in
     }
 }
 
-// Schur update on the tensor cores (1) or on the FP32 pipe (0). T = A_k G_{k-1} as m16n8k8 TF32
-// MMA tiles with three-term splitting (high x high + high x low + low x high, each operand split
-// into its nearest TF32 value and the remainder: relative error about 2^-22, near FP32's, so each
-// FP64 refinement sweep still gains about cond x 1e-7).
-#ifndef VX_BTD_MMA
-#define VX_BTD_MMA 1
-#endif
-
-__device__ __forceinline__ void btd_mma(float (&d)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3,
-                                        unsigned b0, unsigned b1) {
+__device__ __forceinline__ void btd_mma(float (&d)[4], const unsigned (&a)[4], const unsigned (&b)[2]) {
     asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
-// v = hi + lo, hi the nearest TF32 value, lo the exact remainder rounded to TF32 (error 2^-22 |v|):
-// adding half an ulp of TF32 to the magnitude bits and clearing the last 13 rounds to nearest.
+// v = hi + lo, hi the nearest TF32 value (half an ulp of TF32 added to the magnitude bits, the last 13
+// cleared), lo the exact remainder cut to TF32 (error 2^-21 |v|).
 __device__ __forceinline__ void btd_split(float v, unsigned &hi, unsigned &lo) {
     hi = (__float_as_uint(v) + 0x1000u) & 0xffffe000u;
-    lo = (__float_as_uint(__fsub_rn(v, __uint_as_float(hi))) + 0x1000u) & 0xffffe000u;
+    lo = __float_as_uint(__fsub_rn(v, __uint_as_float(hi))) & 0xffffe000u;
 }
+// A product at FP32 accuracy takes three of them: low x high, high x low, high x high (the dropped low x low is
+// 2^-22 of a product, near FP32's rounding).
 
-// D[i][j] (+/-)= sum_{k < K} X[i][xo + k] Y[yo + k][j] for rows r0 <= i < r1 and columns j < n (all
-// three with row stride ld) on the tensor cores: 16 x 16 output blocks dealt to the warps round
-// robin, each two m16n8k8 tiles that share the A fragment (split once for both), 8-deep steps
-// (zero beyond K). ACC: D is the accumulator (else overwritten); NEG: the product is subtracted.
-// Fragment layout of m16n8k8: lane = 4 g + q holds A rows g and g + 8 at columns q and q + 4 of
-// the step, B rows q and q + 4 at column g, and C rows g, g + 8 at columns 2q, 2q + 1. The rows of Y
-// that are read lie outside [r0, r1) whenever Y and D are the same array, so no block reads what
-// another writes.
-template <bool ACC, bool NEG>
-__device__ void mma_rows(const float *X, int xo, const float *Y, int yo, float *D, int ld, int r0, int r1, int n,
-                         int K) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+// Products of two m x m matrices U V in shared memory (row stride ld): eight warps (wm, wn) = 2 x 4 compute
+// NT x NT tiles of 16 x 8 each, rows 16 (wm NT + x), columns 8 (wn NT + y). Fragment layout of m16n8k8:
+// lane = 4 g + q holds U's rows g and g + 8 at columns q and q + 4 of a step of eight, V's rows q and q + 4
+// at column g, and the result's rows g, g + 8 at columns 2q, 2q + 1. The radial couplings A_k and C_k
+// are mostly zeros, so a row tile of A (a column tile of C) takes only the steps that nz marks: those whose
+// 16 x 8 (8 x 8) block holds anything else.
+//
+// One row tile: d[y] = rows r0, r1 of U (offsets) times the NT column tiles of V.
+template <int NT>
+__device__ __forceinline__ void product_row(const float *U, int r0, int r1, const float *V, int ld, int m, int wn,
+                                            int lane, unsigned nz, float (&d)[NT][4]) {
     const int g = lane >> 2, q = lane & 3;
-    const int nrb = (r1 - r0 + 15) >> 4, ncb = (n + 15) >> 4, ks = (K + 7) >> 3;
-    for (int blk = warp; blk < nrb * ncb; blk += nw) {
-        const int i0 = r0 + (blk / ncb) * 16, c0 = (blk % ncb) * 16;
-        const int ra = i0 + g, rb = ra + 8;
-        const bool va = ra < r1, vb = rb < r1;
-        float d[2][4];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int cc = c0 + 8 * h + 2 * q;
-            d[h][0] = ACC && va && cc < n ? D[ra * ld + cc] : 0.f;
-            d[h][1] = ACC && va && cc + 1 < n ? D[ra * ld + cc + 1] : 0.f;
-            d[h][2] = ACC && vb && cc < n ? D[rb * ld + cc] : 0.f;
-            d[h][3] = ACC && vb && cc + 1 < n ? D[rb * ld + cc + 1] : 0.f;
+    for (int y = 0; y < NT; ++y) d[y][0] = d[y][1] = d[y][2] = d[y][3] = 0.f;
+#pragma unroll 1
+    for (; nz; nz &= nz - 1) {
+        const int k0 = 8 * (__ffs(nz) - 1);
+        const bool ia = k0 + q < m, ib = k0 + q + 4 < m;
+        const int ka = ia ? k0 + q : 0, kb = ib ? k0 + q + 4 : 0;
+        float u[4], v[NT][2];
+        u[0] = U[r0 + ka]; u[1] = U[r1 + ka]; u[2] = U[r0 + kb]; u[3] = U[r1 + kb];
+#pragma unroll
+        for (int y = 0; y < NT; ++y) {
+            const int c = 8 * (wn * NT + y) + g;
+            v[y][0] = c < m ? V[ka * ld + c] : 0.f;
+            v[y][1] = c < m ? V[kb * ld + c] : 0.f;
         }
-        for (int k = 0; k < ks; ++k) {
-            const int ka = 8 * k + q, kb = ka + 4;
-            const bool ia = ka < K, ib = kb < K;
-            float a0 = va && ia ? X[ra * ld + xo + ka] : 0.f, a1 = vb && ia ? X[rb * ld + xo + ka] : 0.f;
-            float a2 = va && ib ? X[ra * ld + xo + kb] : 0.f, a3 = vb && ib ? X[rb * ld + xo + kb] : 0.f;
-            if (NEG) {
-                a0 = -a0; a1 = -a1; a2 = -a2; a3 = -a3;
-            }
-            unsigned ah[4], al[4];
-            btd_split(a0, ah[0], al[0]); btd_split(a1, ah[1], al[1]);
-            btd_split(a2, ah[2], al[2]); btd_split(a3, ah[3], al[3]);
+        unsigned ah[4], al[4], bh[NT][2], bl[NT][2];
+        btd_split(ia ? u[0] : 0.f, ah[0], al[0]);
+        btd_split(ia ? u[1] : 0.f, ah[1], al[1]);
+        btd_split(ib ? u[2] : 0.f, ah[2], al[2]);
+        btd_split(ib ? u[3] : 0.f, ah[3], al[3]);
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int col = c0 + 8 * h + g;
-                const float b0 = ia && col < n ? Y[(yo + ka) * ld + col] : 0.f;
-                const float b1 = ib && col < n ? Y[(yo + kb) * ld + col] : 0.f;
-                unsigned bh[2], bl[2];
-                btd_split(b0, bh[0], bl[0]); btd_split(b1, bh[1], bl[1]);
-                btd_mma(d[h], al[0], al[1], al[2], al[3], bh[0], bh[1]);
-                btd_mma(d[h], ah[0], ah[1], ah[2], ah[3], bl[0], bl[1]);
-                btd_mma(d[h], ah[0], ah[1], ah[2], ah[3], bh[0], bh[1]);
-            }
+        for (int y = 0; y < NT; ++y) {
+            btd_split(ia ? v[y][0] : 0.f, bh[y][0], bl[y][0]);
+            btd_split(ib ? v[y][1] : 0.f, bh[y][1], bl[y][1]);
         }
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int cc = c0 + 8 * h + 2 * q;
-            if (va && cc < n) D[ra * ld + cc] = d[h][0];
-            if (va && cc + 1 < n) D[ra * ld + cc + 1] = d[h][1];
-            if (vb && cc < n) D[rb * ld + cc] = d[h][2];
-            if (vb && cc + 1 < n) D[rb * ld + cc + 1] = d[h][3];
+        for (int y = 0; y < NT; ++y) btd_mma(d[y], al, bh[y]);
+#pragma unroll
+        for (int y = 0; y < NT; ++y) btd_mma(d[y], ah, bl[y]);
+#pragma unroll
+        for (int y = 0; y < NT; ++y) btd_mma(d[y], ah, bh[y]);
+    }
+}
+// One column tile: d[x] = the NT row tiles of U (row offsets ur) times column tile c0 / 8 of V, whose rows are
+// taken in the order vrow.
+template <int NT>
+__device__ __forceinline__ void product_col(const float *U, const int (&ur)[NT][2], const float *V, const int *vrow,
+                                            int ld, int m, int c0, int lane, unsigned nz, float (&d)[NT][4]) {
+    const int g = lane >> 2, q = lane & 3;
+    const bool ic = c0 + g < m;
+#pragma unroll
+    for (int x = 0; x < NT; ++x) d[x][0] = d[x][1] = d[x][2] = d[x][3] = 0.f;
+#pragma unroll 1
+    for (; nz; nz &= nz - 1) {
+        const int k0 = 8 * (__ffs(nz) - 1);
+        const bool ia = k0 + q < m, ib = k0 + q + 4 < m;
+        const int ka = ia ? k0 + q : 0, kb = ib ? k0 + q + 4 : 0;
+        float u[NT][4];
+#pragma unroll
+        for (int x = 0; x < NT; ++x) {
+            u[x][0] = U[ur[x][0] + ka]; u[x][1] = U[ur[x][1] + ka];
+            u[x][2] = U[ur[x][0] + kb]; u[x][3] = U[ur[x][1] + kb];
+        }
+        const float v0 = ic ? V[vrow[ka] * ld + c0 + g] : 0.f, v1 = ic ? V[vrow[kb] * ld + c0 + g] : 0.f;
+        unsigned ah[NT][4], al[NT][4], bh[2], bl[2];
+        btd_split(ia ? v0 : 0.f, bh[0], bl[0]);
+        btd_split(ib ? v1 : 0.f, bh[1], bl[1]);
+#pragma unroll
+        for (int x = 0; x < NT; ++x) {
+            btd_split(ia ? u[x][0] : 0.f, ah[x][0], al[x][0]);
+            btd_split(ia ? u[x][1] : 0.f, ah[x][1], al[x][1]);
+            btd_split(ib ? u[x][2] : 0.f, ah[x][2], al[x][2]);
+            btd_split(ib ? u[x][3] : 0.f, ah[x][3], al[x][3]);
+        }
+#pragma unroll
+        for (int x = 0; x < NT; ++x) btd_mma(d[x], al[x], bh);
+#pragma unroll
+        for (int x = 0; x < NT; ++x) btd_mma(d[x], ah[x], bl);
+#pragma unroll
+        for (int x = 0; x < NT; ++x) btd_mma(d[x], ah[x], bh);
+    }
+}
+
+// Shared-memory stores under a predicate (no branch around them).
+__device__ __forceinline__ void st4_if(bool p, unsigned a, float x, float y, float z, float w) {
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %0, 0;\n @p st.shared.v4.f32 [%1], {%2, %3, %4, %5};\n}" ::"r"((unsigned)p),
+                 "r"(a), "f"(x), "f"(y), "f"(z), "f"(w)
+                 : "memory");
+}
+__device__ __forceinline__ void st2_if(bool p, unsigned a, float x, float y) {
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %0, 0;\n @p st.shared.v2.f32 [%1], {%2, %3};\n}" ::"r"((unsigned)p), "r"(a),
+                 "f"(x), "f"(y)
+                 : "memory");
+}
+// The lane whose key won publishes its row (eight values at a) and the row's number (at b).
+__device__ __forceinline__ void st_row_if(unsigned key, unsigned best, unsigned a, const float (&v)[8], unsigned b, int row) {
+    asm volatile("{\n .reg .pred p;\n setp.eq.u32 p, %0, %1;\n @p st.shared.v4.f32 [%2], {%3, %4, %5, %6};\n"
+                 " @p st.shared.v4.f32 [%2 + 16], {%7, %8, %9, %10};\n @p st.shared.u32 [%11], %12;\n}" ::"r"(key), "r"(best),
+                 "r"(a), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "r"(b), "r"(row)
+                 : "memory");
+}
+__device__ __forceinline__ void st1_if(bool p, unsigned a, unsigned x) {
+    asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %0, 0;\n @p st.shared.u32 [%1], %2;\n}" ::"r"((unsigned)p), "r"(a), "r"(x)
+                 : "memory");
+}
+
+// FP64 to FP32 in integer operations, rounded to nearest (ties away): the conversion instruction runs on the
+// FP64 pipe, at 2 per clock and SM on GB300 (measured); this form is eight integer operations. Half an ulp
+// is added, the exponent rebiased by 896 and clamped: magnitudes below the normal FP32 range become (nearly)
+// 0, those above it and NaN become infinite or NaN, which fails the pivot test.
+__device__ __forceinline__ float btd_f32(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x) + 0x10000000ull;
+    const unsigned hi = (unsigned)(b >> 32);
+    const int e = min(max((int)(hi & 0x7fffffffu) - (896 << 20), 0), 0x0ff00000);
+    return __uint_as_float(__funnelshift_l((unsigned)b, (unsigned)e, 3) | (hi & 0x80000000u));
+}
+
+// The blocks in FP32, row-major with row stride ld, for the factor kernel and the sweeps: A_k to At, B_k to Di
+// and C_k to Gt (the factor kernel puts D_k^{-1} and G_k in the places of B_k and C_k, which it has read by
+// then), and per row of C and A a bit per eight columns that hold anything but zeros (nz[k][C, A][mp]). A warp
+// takes kConvRows rows at a time, all their loads in flight together. Bound by HBM (12 m^2 bytes read and
+// written per block for 8 m^2 read); apart from the factor kernel because the loads' registers, and the
+// conversions' instructions, cost that kernel more than the extra pass.
+constexpr int kConvThreads = 256, kConvRows = 4, kConvGrid = 152 * 16;
+template <int NT>
+__global__ void __launch_bounds__(kConvThreads) k_btd_convert(const BtdArgs a) {
+    if (*a.inval) return;
+    const int m = a.m, ld = a.ld, lane = threadIdx.x & 31;
+    const long long rows = 3 * a.n_zones * m, step = (long long)gridDim.x * (kConvThreads / 32) * kConvRows;
+    for (long long r0 = ((long long)blockIdx.x * (kConvThreads / 32) + (threadIdx.x >> 5)) * kConvRows; r0 < rows; r0 += step) {
+        const long long zm = r0 / m;  // (zone, matrix) of the first row: 3 k + (0 A, 1 B, 2 C)
+        double v[kConvRows][NT];
+        float *dst[kConvRows];
+        int mat[kConvRows], row[kConvRows];
+        long long zone[kConvRows];
+#pragma unroll
+        for (int r = 0; r < kConvRows; ++r) {
+            long long q = zm;
+            int i = (int)(r0 + r - zm * m);
+            while (i >= m) { i -= m; ++q; }
+            const long long k = q / 3;
+            const int w = (int)(q - 3 * k);
+            const bool in = r0 + r < rows;
+            const double *src = (w == 0 ? a.A : w == 1 ? a.B : a.C) + ((size_t)k * m + i) * m + lane;
+            dst[r] = in ? (w == 0 ? a.At : w == 1 ? a.Di : a.Gt) + ((size_t)k * m + i) * ld + lane : nullptr;
+            mat[r] = w;
+            row[r] = i;
+            zone[r] = k;
+#pragma unroll
+            for (int t = 0; t < NT; ++t) v[r][t] = in && (t < NT - 1 || lane + 32 * t < m) ? __ldg(src + 32 * t) : 0.0;
+        }
+#pragma unroll
+        for (int r = 0; r < kConvRows; ++r) {
+            if (!dst[r]) continue;
+            unsigned bits = 0u;
+#pragma unroll
+            for (int t = 0; t < NT; ++t) {
+                const float f = btd_f32(v[r][t]);
+                if (t < NT - 1 || lane + 32 * t < m) dst[r][32 * t] = f;
+                bits |= f != 0.f ? 1u << (4 * t) : 0u;
+            }
+            if (mat[r] == 1) continue;
+            bits = __reduce_or_sync(0xffffffffu, bits << (lane >> 3));
+            if (lane == 0) a.nz[((size_t)zone[r] * 2 + (mat[r] == 0)) * a.mp + row[r]] = (unsigned short)bits;
         }
     }
 }
 
-// dst[i][c] = (float) M[row(i)][c] for i, c < m, row(i) = rowmap[i] (rowmap NULL: i), thread (warp,
-// lane) taking rows warp + 8 s and columns lane + 32 t: each of NCH chunks of its rows has all its
-// loads in flight before the first conversion (one DRAM round trip per chunk, not one per element).
-template <int RS, int CS, int NCH>
-__device__ __forceinline__ void stage_rows(const double *__restrict__ M, const int *rowmap, float *dst, int m, int ld,
-                                           int warp, int lane) {
-    static_assert(RS % NCH == 0, "rows per thread in equal chunks");
-    constexpr int H = RS / NCH;
+// Asynchronous 16-byte copies of n floats (a multiple of 4) by the whole CTA.
+__device__ __forceinline__ void copy_async(float *dst, const float *src, int n, int tid, int nthreads) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst) + 16u * (unsigned)tid;
+#pragma unroll 4
+    for (int e = 4 * tid, i = 0; e < n; e += 4 * nthreads, ++i)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + 16u * (unsigned)(i * nthreads)), "l"(src + e) : "memory");
+}
+__device__ __forceinline__ void copy_wait() {
+    asm volatile("cp.async.commit_group;\n cp.async.wait_group 0;" ::: "memory");
+}
+
+__device__ __forceinline__ float btd_rcp(float p) {  // p and 1/p normal numbers
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(p));
+    return fmaf(y, fmaf(-p, y, 1.f), y);  // a Newton step: the approximation's ulp would stay in the pivot row
+}
+
+// The panel warp's state: lane x holds rows x + 32 t of the panel's eight columns.
+template <int NT>
+struct Panel {
+    float v[NT][8];
+    unsigned cand[NT];  // magnitude mask of a row that can still be a pivot, 0 once it has been one
+    unsigned piv;       // bit t: the row is one of this panel's pivots
+    unsigned kmin, kmax;
+
+    __device__ __forceinline__ void start(int m, int lane) {
 #pragma unroll
-    for (int h = 0; h < NCH; ++h) {
-        double x[H][CS];
+        for (int t = 0; t < NT; ++t) cand[t] = lane + 32 * t < m ? 0x7fffff80u : 0u;
+        kmin = 0xffffffffu;
+        kmax = 0u;
+    }
+    // Rows lane + 32 t of columns c0 .. c0 + 7 of X.
+    __device__ __forceinline__ static void fetch(float (&u)[NT][8], const float *X, int ld, int m, int c0, int lane) {
 #pragma unroll
-        for (int s = 0; s < H; ++s) {
-            const int i = warp + 8 * (h * H + s);
-            const int r = i < m ? (rowmap ? rowmap[i] : i) : 0;
-#pragma unroll
-            for (int t = 0; t < CS; ++t) {
-                const int c = lane + 32 * t;
-                x[s][t] = (i < m && c < m) ? __ldg(M + (size_t)r * m + c) : 0.0;
-            }
+        for (int t = 0; t < NT; ++t) {
+            const int i = lane + 32 * t;
+            const float4 *s = reinterpret_cast<const float4 *>(X + (i < m ? i : 0) * ld + c0);
+            const float4 a = s[0], b = s[1];
+            u[t][0] = a.x; u[t][1] = a.y; u[t][2] = a.z; u[t][3] = a.w;
+            u[t][4] = b.x; u[t][5] = b.y; u[t][6] = b.z; u[t][7] = b.w;
         }
+    }
+    // Zeros past the m-th row and column.
+    __device__ __forceinline__ void trim(int m, int c0, int lane) {
+        if (lane + 32 * (NT - 1) >= m) {
 #pragma unroll
-        for (int s = 0; s < H; ++s) {
-            const int i = warp + 8 * (h * H + s);
+            for (int c = 0; c < 8; ++c) v[NT - 1][c] = 0.f;
+        }
+        if (c0 + 8 > m) {
 #pragma unroll
-            for (int t = 0; t < CS; ++t) {
-                const int c = lane + 32 * t;
-                if (i < m && c < m) dst[i * ld + c] = (float)x[s][t];
+            for (int t = 0; t < NT; ++t)
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    if (c0 + c >= m) v[t][c] = 0.f;
+        }
+    }
+    __device__ __forceinline__ void store(float *X, int ld, int m, int c0, int lane) const {
+#pragma unroll
+        for (int t = 0; t < NT; ++t) {
+            const int i = lane + 32 * t;
+            const unsigned d = (unsigned)__cvta_generic_to_shared(X + (i < m ? i : 0) * ld + c0);
+            if (c0 + 8 <= m) {
+                st4_if(i < m, d, v[t][0], v[t][1], v[t][2], v[t][3]);
+                st4_if(i < m, d + 16, v[t][4], v[t][5], v[t][6], v[t][7]);
+            } else {
+#pragma unroll
+                for (int c = 0; c < 8; ++c) st1_if(i < m && c0 + c < m, d + 4 * c, __float_as_uint(v[t][c]));
             }
         }
     }
-}
+    // Goes on to the panel of columns c0 .. c0 + 7: they take the transform W this warp has just found (its
+    // registers; pivot rows pr[0..7]): new = (X with the pivot rows zeroed) + W X_R.
+    __device__ __forceinline__ void advance(const float *X, int ld, int m, int c0, const int *pr, int lane) {
+        const int4 p0 = reinterpret_cast<const int4 *>(pr)[0], p1 = reinterpret_cast<const int4 *>(pr)[1];
+        const int pk[8] = {p0.x, p0.y, p0.z, p0.w, p1.x, p1.y, p1.z, p1.w};
+        float u[NT][8];
+        fetch(u, X, ld, m, c0, lane);
+        float2 w[NT][4];
+#pragma unroll
+        for (int t = 0; t < NT; ++t)
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                w[t][c] = (piv >> t) & 1u ? make_float2(0.f, 0.f) : make_float2(u[t][2 * c], u[t][2 * c + 1]);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const float4 *s = reinterpret_cast<const float4 *>(X + pk[k] * ld + c0);
+            const float4 a = s[0], b = s[1];
+            const float2 y[4] = {make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(b.x, b.y), make_float2(b.z, b.w)};
+#pragma unroll
+            for (int t = 0; t < NT; ++t)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) w[t][c] = __ffma2_rn(make_float2(v[t][k], v[t][k]), y[c], w[t][c]);
+        }
+#pragma unroll
+        for (int t = 0; t < NT; ++t)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                v[t][2 * c] = w[t][c].x;
+                v[t][2 * c + 1] = w[t][c].y;
+            }
+        trim(m, c0, lane);
+    }
+    // Gauss-Jordan steps of columns c0 .. c0 + nv - 1 within the panel, in place: after step j the column
+    // holds what the elimination so far makes of the unit vector of its pivot row. The columns shift by one
+    // register per step (free: each update writes the register before), so that the loop is not unrolled
+    // and its instructions stay in the nearest cache. One warp reduction finds a pivot: the key holds the
+    // magnitude's leading bits and, below them, 127 - row, so that keys differ and the lowest row wins among
+    // magnitudes equal to 2^-16 (partial pivoting up to that factor). A second one broadcasts its value
+    // while the pivot row goes through shared memory (rowbuf, two buffers of eight). The next column is
+    // updated first and its pivot search started before the rest. The pivot rows are scaled by their
+    // reciprocal pivots at the end.
+    __device__ __forceinline__ void factor(int m, int c0, int nv, int *cur, float *rowbuf, int lane) {
+        const unsigned rb = (unsigned)__cvta_generic_to_shared(rowbuf), cb = (unsigned)__cvta_generic_to_shared(cur + c0);
+        float sc[NT];
+        unsigned kt[NT], best = 0u;
+        piv = 0u;
+#pragma unroll
+        for (int t = 0; t < NT; ++t) {
+            sc[t] = 1.f;
+            kt[t] = (__float_as_uint(v[t][0]) & cand[t]) | (unsigned)(127 - lane - 32 * t);
+            best = max(best, kt[t]);
+        }
+#pragma unroll 1
+        for (int j = 0; j < nv; ++j) {
+            best = __reduce_max_sync(0xffffffffu, best);
+            kmin = min(kmin, best);
+            kmax = max(kmax, best);
+            const unsigned rj = rb + 32u * (unsigned)(j & 1);
+            unsigned mine = 0u;
+            bool own[NT];
+#pragma unroll
+            for (int t = 0; t < NT; ++t) {
+                own[t] = kt[t] == best;
+                mine |= own[t] ? __float_as_uint(v[t][0]) : 0u;
+            }
+            const float p = __uint_as_float(__reduce_or_sync(0xffffffffu, mine));
+#pragma unroll
+            for (int t = 0; t < NT; ++t)  // a row past m - 1 wins only where no pivot is left
+                st_row_if(kt[t], best, rj, v[t], cb + 4u * (unsigned)j, min(lane + 32 * t, m - 1));
+            const float rp = best - 0x00800000u < 0x7d800000u ? btd_rcp(p) : 1.f / p;  // |p| in [2^-126, 2^125)
+            __syncwarp();
+            const float4 *rr = reinterpret_cast<const float4 *>(rowbuf + 8 * (j & 1));
+            const float4 ya = rr[0], yb = rr[1];
+            const float y[8] = {ya.x, ya.y, ya.z, ya.w, yb.x, yb.y, yb.z, yb.w};
+            float l[NT];
+            best = 0u;
+#pragma unroll
+            for (int t = 0; t < NT; ++t) {
+                l[t] = own[t] ? 0.f : -v[t][0] * rp;
+                cand[t] = own[t] ? 0u : cand[t];
+                sc[t] = own[t] ? rp : sc[t];
+                piv |= own[t] ? 1u << t : 0u;
+                v[t][0] = fmaf(l[t], y[1], v[t][1]);
+                kt[t] = (__float_as_uint(v[t][0]) & cand[t]) | (unsigned)(127 - lane - 32 * t);
+                best = max(best, kt[t]);
+            }
+#pragma unroll
+            for (int t = 0; t < NT; ++t) {
+#pragma unroll
+                for (int c = 2; c < 8; ++c) v[t][c - 1] = fmaf(l[t], y[c], v[t][c]);
+                v[t][7] = own[t] ? 1.f : l[t];
+            }
+        }
+#pragma unroll 1
+        for (int j = nv; j < 8; ++j) {  // a panel of fewer columns: zeros, shifted back into place
+            st1_if(lane == 0, cb + 4u * (unsigned)j, 0u);
+#pragma unroll
+            for (int t = 0; t < NT; ++t) {
+#pragma unroll
+                for (int c = 1; c < 8; ++c) v[t][c - 1] = v[t][c];
+                v[t][7] = 0.f;
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < NT; ++t)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) v[t][c] *= sc[t];
+        __syncwarp();
+    }
+    // A column had no pivot (all candidates zero) or one that is not finite.
+    __device__ __forceinline__ bool failed() const { return kmin < 128u || kmax >= 0x7f800000u; }
+};
 
-// stage_rows for two matrices at once (M1 may be NULL): each half of a thread's rows of both has its
-// loads in flight together.
-template <int RS, int CS>
-__device__ __forceinline__ void stage_two(const double *__restrict__ M1, float *d1, const double *__restrict__ M2,
-                                          float *d2, int m, int ld, int warp, int lane) {
-    static_assert(RS % 2 == 0, "rows per thread in two halves");
-    constexpr int H = RS / 2;
+// Applies panel p's transform to one or two other 8-column tiles of X (t1 < 0: one), on the tensor cores:
+// X = (X with the panel's pivot rows zeroed) + W X_R, a rank-8 product: one m16n8k8 step per 16 x 8 tile.
+// A warp owns all rows of its tiles, so the pivot rows X_R are read, and zeroed, before it goes through the
+// rows, NT tiles of 16 at a time so that their chains overlap. Rows past the m-th are computed from
+// whatever follows in shared memory and not stored.
+template <int NT>
+__device__ __forceinline__ void tile_update(float *X, int ld, int m, int p, int t0, int t1, const int *cur, int lane) {
+    const int g = lane >> 2, q = lane & 3;
+    const bool ia = 8 * p + q < m, ib = 8 * p + q + 4 < m;  // the last panel may hold fewer than 8 columns
+    const int ra = cur[8 * p + q] * ld, rb = cur[8 * p + q + 4] * ld;
+    unsigned bh[2][2], bl[2][2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        double x1[H][CS], x2[H][CS];
+        const int t = h ? t1 : t0;
+        if (t >= 0) {
+            const int c = 8 * t + g;
+            btd_split(ia && c < m ? X[ra + c] : 0.f, bh[h][0], bl[h][0]);
+            btd_split(ib && c < m ? X[rb + c] : 0.f, bh[h][1], bl[h][1]);
+        }
+    }
+    __syncwarp();
+    const unsigned xs = (unsigned)__cvta_generic_to_shared(X);
 #pragma unroll
-        for (int s = 0; s < H; ++s) {
-            const int i = warp + 8 * (h * H + s);
+    for (int h = 0; h < 2; ++h) {
+        const int t = h ? t1 : t0;
+        if (t >= 0) {
+            const int c = 8 * t + g;
+            st1_if(ia && c < m, xs + 4u * (unsigned)(ra + c), 0u);
+            st1_if(ib && c < m, xs + 4u * (unsigned)(rb + c), 0u);
+        }
+    }
+    __syncwarp();
+    const float *W = X + g * ld + 8 * p + q;
+    const int c0 = g * ld + 8 * t0 + 2 * q, c1 = g * ld + 8 * (t1 < 0 ? t0 : t1) + 2 * q;
+#pragma unroll 1
+    for (int i0 = 0; i0 < m; i0 += 16 * NT) {
+        unsigned ah[NT][4], al[NT][4];
 #pragma unroll
-            for (int t = 0; t < CS; ++t) {
-                const int c = lane + 32 * t;
-                const bool in = i < m && c < m;
-                x1[s][t] = in && M1 ? __ldg(M1 + (size_t)i * m + c) : 0.0;
-                x2[s][t] = in ? __ldg(M2 + (size_t)i * m + c) : 0.0;
-            }
+        for (int x = 0; x < NT; ++x) {
+            const float *w = W + (i0 + 16 * x) * ld;
+            btd_split(w[0], ah[x][0], al[x][0]);
+            btd_split(w[8 * ld], ah[x][1], al[x][1]);
+            btd_split(w[4], ah[x][2], al[x][2]);
+            btd_split(w[8 * ld + 4], ah[x][3], al[x][3]);
         }
 #pragma unroll
-        for (int s = 0; s < H; ++s) {
-            const int i = warp + 8 * (h * H + s);
+        for (int h = 0; h < 2; ++h) {
+            const int t = h ? t1 : t0;
+            if (t < 0) break;
+            float *y = X + i0 * ld + (h ? c1 : c0);
+            float d[NT][4];
+            float2 e[NT][2];
 #pragma unroll
-            for (int t = 0; t < CS; ++t) {
-                const int c = lane + 32 * t;
-                if (i < m && c < m) {
-                    if (M1) d1[i * ld + c] = (float)x1[s][t];
-                    d2[i * ld + c] = (float)x2[s][t];
+            for (int x = 0; x < NT; ++x) {
+                d[x][0] = d[x][1] = d[x][2] = d[x][3] = 0.f;
+                e[x][0] = *reinterpret_cast<const float2 *>(y + 16 * x * ld);
+                e[x][1] = *reinterpret_cast<const float2 *>(y + (16 * x + 8) * ld);
+            }
+#pragma unroll
+            for (int x = 0; x < NT; ++x) btd_mma(d[x], al[x], bh[h]);
+#pragma unroll
+            for (int x = 0; x < NT; ++x) btd_mma(d[x], ah[x], bl[h]);
+#pragma unroll
+            for (int x = 0; x < NT; ++x) btd_mma(d[x], ah[x], bh[h]);
+            // added in FP32, rounded to nearest: the tensor core's own accumulation cuts the sum's last bits
+#pragma unroll
+            for (int x = 0; x < NT; ++x) {
+                d[x][0] += e[x][0].x; d[x][1] += e[x][0].y;
+                d[x][2] += e[x][1].x; d[x][3] += e[x][1].y;
+            }
+            if (8 * t + 8 <= m) {
+#pragma unroll
+                for (int x = 0; x < NT; ++x) {
+                    const unsigned ys = xs + 4u * (unsigned)(y - X) + 64u * (unsigned)(x * ld);
+                    st2_if(i0 + 16 * x + g < m, ys, d[x][0], d[x][1]);
+                    st2_if(i0 + 16 * x + g + 8 < m, ys + 32u * (unsigned)ld, d[x][2], d[x][3]);
+                }
+            } else {
+                const bool j0 = 8 * t + 2 * q < m, j1 = 8 * t + 2 * q + 1 < m;
+#pragma unroll
+                for (int x = 0; x < NT; ++x) {
+                    const bool r0 = i0 + 16 * x + g < m, r1 = i0 + 16 * x + g + 8 < m;
+                    const unsigned ys = xs + 4u * (unsigned)(y - X) + 64u * (unsigned)(x * ld);
+                    st1_if(r0 && j0, ys, __float_as_uint(d[x][0]));
+                    st1_if(r0 && j1, ys + 4u, __float_as_uint(d[x][1]));
+                    st1_if(r1 && j0, ys + 32u * (unsigned)ld, __float_as_uint(d[x][2]));
+                    st1_if(r1 && j1, ys + 32u * (unsigned)ld + 4u, __float_as_uint(d[x][3]));
                 }
             }
         }
     }
 }
 
-// Named barriers of the column steps: the warp that publishes column j arrives, the others wait.
-// Steps alternate between barriers 1 and 2: the publishing warp arrives early and goes on to wait
-// at the next step, which on a single barrier could count towards the step still open. With two,
-// every warp reaches the barrier of step j only after waiting at step j - 1 (no warp publishes two
-// steps in a row), so the barrier's previous use, step j - 2, has completed.
-__device__ __forceinline__ void step_arrive(int j) {
-    asm volatile("bar.arrive %0, %1;" ::"r"(1 + (j & 1)), "n"(kFactorThreads) : "memory");
-}
-__device__ __forceinline__ void step_wait(int j) {
-    asm volatile("bar.sync %0, %1;" ::"r"(1 + (j & 1)), "n"(kFactorThreads) : "memory");
+// Shared memory of the factor kernel: nbuf buffers of m x ld floats (16 floats of slack each: the last
+// tiles read past the end of a row), the zero patterns of C_k's and A_{k+1}'s rows, two rows
+// of a panel, the pivot rows and their inverse.
+__host__ __device__ constexpr int factor_buf(int m, int ld) { return (m * ld + 16 + 3) & ~3; }
+__host__ __device__ constexpr size_t factor_smem(int m, int ld, int nbuf) {
+    return (size_t)nbuf * factor_buf(m, ld) * sizeof(float) + (size_t)(16 + 3 * ((m + 7) & ~7)) * sizeof(int) +
+           (size_t)m * sizeof(int);
 }
 
-// Element (slot s, row slot t) of a register tile stored as pairs of slots (s even: .x, odd: .y),
-// so that two slots update with one packed FP32 FMA.
-#define VX_SLOT(tile, s, t) (((s) & 1) ? (tile)[(s) >> 1][t].y : (tile)[(s) >> 1][t].x)
-
-// Column j of D_k, in slot S of the calling warp (column warp + 8 S): the pivot row (the largest
-// magnitude among the rows not yet pivots, the lowest row on ties, by two warp reductions) and the
-// multipliers of every other row, published to buffer j mod 2 and stored as column j of the zone's
-// multiplier matrix Mz (the pivot value in the pivot row's place), with 1 / pivot in s_rp[j]. Ends
-// with the warp's arrival at the step barrier.
-template <int RS, int CS>
-__device__ __forceinline__ void gj_publish(const float2 (&v)[RS / 2][CS], const int S, unsigned done, int j, int m,
-                                           int lane, float *sL, int *s_r, int *cur, float *s_rp, float *Mz,
-                                           int *s_bad) {
-    unsigned key = 0u;  // |x| bits + 1 (NaN: 1) for a candidate row, 0 for none
-    unsigned brow = 0xffffffffu;
-#pragma unroll
-    for (int t = 0; t < CS; ++t) {
-        const int i = lane + 32 * t;
-        if ((t < CS - 1 || i < m) && !((done >> t) & 1u)) {  // CS = ceil(m / 32): only the last slot can fall past m
-            const float x = fabsf(VX_SLOT(v, S, t));
-            const unsigned kx = x == x ? __float_as_uint(x) + 1u : 1u;
-            if (kx > key) {
-                key = kx;
-                brow = (unsigned)i;
-            }
-        }
-    }
-    const unsigned kmax = __reduce_max_sync(0xffffffffu, key);
-    const int r = (int)__reduce_min_sync(0xffffffffu, key == kmax ? brow : 0xffffffffu);
-    const int tr = r >> 5;
-    float mine = VX_SLOT(v, S, 0);
-#pragma unroll
-    for (int t = 1; t < CS; ++t)
-        if (tr == t) mine = VX_SLOT(v, S, t);
-    const float piv = __shfl_sync(0xffffffffu, mine, r & 31), rp = 1.f / piv;
-    const int buf = j & 1;
-    if (lane == 0) {
-        s_r[buf] = r;
-        cur[j] = r;
-        s_rp[j] = rp;
-        if (!(fabsf(piv) > 0.f && fabsf(piv) < INFINITY)) *s_bad = 1;
-    }
-    float *mcol = Mz + (size_t)j * m;
-#pragma unroll
-    for (int t = 0; t < CS; ++t) {
-        const int i = lane + 32 * t;
-        if (t < CS - 1 || i < m) {
-            const float lv = i != r ? VX_SLOT(v, S, t) * rp : 0.f;
-            sL[buf * m + i] = lv;
-            mcol[i] = i != r ? lv : piv;
-        }
-    }
-    step_arrive(j);
-}
-
-// The elimination of column j (slot sj of warp wj) from the calling warp's part of [D_k | C_k],
-// the pivot row's slot TR known at compile time (the pivot row's values come by shuffle from lane
-// rl): D's columns past j and all of C's updated with the multipliers lt. If the warp holds column
-// j + 1 (np), that column is updated first and published before the rest (look-ahead).
-template <int RS, int CS, int TR>
-__device__ __forceinline__ void gj_eliminate(float2 (&v)[RS / 2][CS], float2 (&w)[RS / 2][CS], const float (&lt)[CS],
-                                             int rl, const int sj, int wj, int warp, int lane, int j, int m, bool np,
-                                             unsigned done, float *sL, int *s_r, int *cur, float *s_rp, float *Mz,
-                                             int *s_bad) {
-    float pd[RS];
-#pragma unroll
-    for (int s = 0; s < RS; ++s) pd[s] = __shfl_sync(0xffffffffu, VX_SLOT(v, s, TR), rl);
-    const bool wrap = wj == 7;  // column j + 1 is in slot sj + 1 (else in slot sj)
-    if (np) {
-        if (wrap) {
-            if (sj + 1 < RS) {
-#pragma unroll
-                for (int t = 0; t < CS; ++t) VX_SLOT(v, sj + 1, t) = fmaf(-lt[t], pd[sj + 1], VX_SLOT(v, sj + 1, t));
-                gj_publish<RS, CS>(v, sj + 1 < RS ? sj + 1 : RS - 1, done, j + 1, m, lane, sL, s_r, cur, s_rp, Mz, s_bad);
-            }
-        } else {
-#pragma unroll
-            for (int t = 0; t < CS; ++t) VX_SLOT(v, sj, t) = fmaf(-lt[t], pd[sj], VX_SLOT(v, sj, t));
-            gj_publish<RS, CS>(v, sj, done, j + 1, m, lane, sL, s_r, cur, s_rp, Mz, s_bad);
-        }
-    }
-    float2 nlt[CS];
-#pragma unroll
-    for (int t = 0; t < CS; ++t) nlt[t] = make_float2(-lt[t], -lt[t]);
-#pragma unroll
-    for (int q = 0; q < RS / 2; ++q) {
-        bool upd[2];
-#pragma unroll
-        for (int e = 0; e < 2; ++e) {
-            const int s = 2 * q + e;
-            const bool past = s > sj || (s == sj && warp > wj);
-            const bool ahead = np && ((s == sj && !wrap) || (s == sj + 1 && wrap));  // done above
-            upd[e] = past && !ahead;
-        }
-        if (upd[0] && upd[1]) {
-            const float2 p2 = make_float2(pd[2 * q], pd[2 * q + 1]);
-#pragma unroll
-            for (int t = 0; t < CS; ++t) v[q][t] = __ffma2_rn(nlt[t], p2, v[q][t]);
-        } else {
-            if (upd[0]) {
-#pragma unroll
-                for (int t = 0; t < CS; ++t) v[q][t].x = fmaf(-lt[t], pd[2 * q], v[q][t].x);
-            }
-            if (upd[1]) {
-#pragma unroll
-                for (int t = 0; t < CS; ++t) v[q][t].y = fmaf(-lt[t], pd[2 * q + 1], v[q][t].y);
-            }
-        }
-        const float2 c2 = make_float2(__shfl_sync(0xffffffffu, w[q][TR].x, rl), __shfl_sync(0xffffffffu, w[q][TR].y, rl));
-#pragma unroll
-        for (int t = 0; t < CS; ++t) w[q][t] = __ffma2_rn(nlt[t], c2, w[q][t]);
-    }
-}
-
-// The factor kernel, one CTA of eight warps per ray, its zones in order. B_k and A_k are staged
-// in shared memory and D_k = B_k - A_k G_{k-1} is formed there (tensor cores). Then thread (warp w,
-// lane x) takes into registers the elements of D_k and of C_k in rows x + 32 t (t < CS) and columns
-// w + 8 s (s < RS), so that column j lies in warp j mod 8 alone, and Gauss-Jordan elimination with
-// partial pivoting runs on [D_k | C_k] one column at a time:
-//  - the warp that holds column j finds the pivot row and publishes it with the multipliers of
-//    every other row (gj_publish), then arrives at the step barrier, at which the other warps wait;
-//  - every warp takes the pivot row's values in its columns by shuffle and subtracts the multiples
-//    from the other rows, in the columns of D past j and in all of C (gj_eliminate); the warp that
-//    holds column j + 1 updates and publishes it first.
-// The rows already pivots are eliminated as well, so at the end the C part of pivot row j is
-// U_jj G_k[j] and no substitution is left. Rows are never moved: cur maps pivot positions to
-// physical rows. What the solve sweeps need of D_k is the elimination itself: the multiplier
-// columns (with the pivot values), stored as they are published, and cur.
-template <int RS, int CS>
-__global__ void __launch_bounds__(kFactorThreads, RS > 12 ? 1 : 2) k_btd_factor(const BtdArgs a) {  // m > 96: one CTA per SM (shared memory)
+// The factor kernel, one CTA of eight warps per ray, its zones in order. Per zone k:
+//  - D_k = B_k - A_k G_{k-1} on the tensor cores (all three in shared memory);
+//  - D_k is inverted in place by Gauss-Jordan elimination with partial pivoting, eight columns (a panel) at
+//    a time: warp 0 eliminates within a panel in registers, with no barrier between its eight pivots;
+//    the other warps apply the panel's rank-8 transform to the remaining column tiles on the tensor
+//    cores while warp 0 brings the next panel up to date and eliminates in it. One CTA barrier per
+//    panel. Rows are never moved: pivot j's row is cur[j], and D_k^{-1}[j][cur[q]] = X[cur[j]][q];
+//  - meanwhile C_k, A_{k+1} and (with a fourth buffer) B_{k+1} arrive in shared memory (cp.async);
+//  - G_k = D_k^{-1} C_k on the tensor cores.
+// D_k^{-1}, G_k and the FP32 copy of A_k go to the workspace for the sweeps. The chain of pivots (a warp
+// reduction, a shuffle and a reciprocal each) bounds a zone; the warps beside it do everything else.
+template <int NT>
+__global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(const BtdArgs a) {
     extern __shared__ __align__(16) float sm[];
     __shared__ int s_bad;
-    __shared__ int s_r[2];
     const int m = a.m, ld = a.ld, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    float *sA = sm;           // A_k
-    float *sW = sA + m * ld;  // G_{k-1}, then C_k, then G_k
-    float *sT = sW + m * ld;  // B_k, then D_k
-    float *sL = sT + m * ld;  // [2][m] the multipliers of the current column (two buffers)
-    float *s_rp = sL + 2 * m;  // [m] 1 / the pivot of each column
-    int *cur = reinterpret_cast<int *>(s_rp + m), *pos = cur + m;
+    const int nw = kFactorThreads / 32, bs = factor_buf(m, ld), P = (m + 7) >> 3;
+    const bool four = a.nbuf == 4;
+    // D_k and the next zone's B come first: tile_update reads up to 15 rows past the end of D_k
+    // (offsets, not pointers, are exchanged from zone to zone: the compiler then knows the address space)
+    int xo = 0, bo = four ? bs : 0;
+    float *const sG = sm + bo + bs, *const sA = sG + bs;
+    unsigned short *nzr = reinterpret_cast<unsigned short *>(sm + a.nbuf * bs);  // [C, A][mp]
+    float *rowbuf = sm + a.nbuf * bs + a.mp;  // [2][8]
+    int *cur = reinterpret_cast<int *>(rowbuf + 16);
+    int *pos = cur + 8 * P;
     long long z0, z1;
     if (!ray_range(a, blockIdx.x, z0, z1) || z1 == z0) return;
     if (tid == 0) s_bad = 0;
-    const size_t mm = (size_t)m * m;
+    if (tid < m) pos[tid] = tid;  // in range also where a failed pivot leaves an entry unset
+    const int mw = m * ld;
+    const int g = lane >> 2, q = lane & 3, wm = warp & 1, wn = warp >> 1;
+    // zeros behind every buffer: the last panel's transform, if it has fewer than eight columns, is read that far
+    // (and multiplied by zeros, so it must be finite)
+    for (int i = tid; i < a.nbuf * (bs - mw); i += kFactorThreads) sm[i / (bs - mw) * bs + mw + i % (bs - mw)] = 0.f;
+    copy_async(sm, a.Di + (size_t)z0 * mw, mw, tid, kFactorThreads);  // B_{z0}
+    copy_wait();
+    __syncthreads();
     for (long long k = z0; k < z1; ++k) {
-        const bool prev = k > z0, next = k + 1 < z1;
-        stage_two<RS, CS>(prev ? a.A + k * mm : nullptr, sA, a.B + k * mm, sT, m, ld, warp, lane);
-        __syncthreads();
-        if (prev) {
-#if VX_BTD_MMA
-            mma_rows<true, true>(sA, 0, sW, 0, sT, ld, 0, m, m, m);  // sT = B_k - A_k G_{k-1}
-#else
-            for (int e = tid; e < m * m; e += kFactorThreads) {
-                const int i = e / m, c = e % m;
-                float acc = sT[i * ld + c];
-                for (int q = 0; q < m; ++q) acc = fmaf(-sA[i * ld + q], sW[q * ld + c], acc);
-                sT[i * ld + c] = acc;
-            }
-#endif
-            float *At = a.At + k * mm;  // FP32 column-major copy for the solve sweeps
-            for (int c = warp; c < m; c += 8)
-                for (int i = lane; i < m; i += 32) At[(size_t)c * m + i] = sA[i * ld + c];
-        }
-        __syncthreads();
-        if (next) stage_rows<RS, CS, 2>(a.C + k * mm, nullptr, sW, m, ld, warp, lane);
-        float2 v[RS / 2][CS], w[RS / 2][CS];  // D_k and C_k: rows lane + 32 t, columns warp + 8 s (VX_SLOT)
+        const bool next = k + 1 < z1;
+        float *const X = sm + xo, *const sB = sm + bo;
+        if (k > z0) {  // D_k = B_k - A_k G_{k-1}
+#pragma unroll 1
+            for (int x = 0; x < NT; ++x) {
+                const int i0 = 16 * (wm * NT + x), i = i0 + (lane & 15);
+                const unsigned nz = __reduce_or_sync(0xffffffffu, i < m ? (unsigned)nzr[a.mp + i] : 0u);
+                float d[NT][4];
+                const int r0 = i0 + g < m ? i0 + g : m - 1, r1 = i0 + g + 8 < m ? i0 + g + 8 : m - 1;
+                product_row<NT>(sA, r0 * ld, r1 * ld, sG, ld, m, wn, lane, nz, d);
+                const bool i0m = i0 + g < m, i1m = i0 + g + 8 < m;
 #pragma unroll
-        for (int s = 0; s < RS; ++s)
-#pragma unroll
-            for (int t = 0; t < CS; ++t) {
-                const int i = lane + 32 * t, c = warp + 8 * s;
-                VX_SLOT(v, s, t) = i < m && c < m ? sT[i * ld + c] : 0.f;
-            }
-        __syncthreads();
-#pragma unroll
-        for (int s = 0; s < RS; ++s)
-#pragma unroll
-            for (int t = 0; t < CS; ++t) {
-                const int i = lane + 32 * t, c = warp + 8 * s;
-                VX_SLOT(w, s, t) = next && i < m && c < m ? sW[i * ld + c] : 0.f;
-            }
-        float *Mz = a.Mt + k * mm;  // the zone's multiplier columns
-        unsigned done = 0u;  // bit t: my row lane + 32 t has been a pivot
-        if (warp == 0) gj_publish<RS, CS>(v, 0, done, 0, m, lane, sL, s_r, cur, s_rp, Mz, &s_bad);
-#pragma unroll
-        for (int sj = 0; sj < RS; ++sj) {
-            for (int wj = 0; wj < 8; ++wj) {
-                const int j = 8 * sj + wj;
-                if (j >= m) break;
-                if (warp != wj) step_wait(j);  // the warp of column j arrived when it published
-                const int buf = j & 1;
-                const int r = s_r[buf], rl = r & 31, tr = r >> 5;
-                float lt[CS];
-#pragma unroll
-                for (int t = 0; t < CS; ++t) {
-                    const int i = lane + 32 * t;
-                    lt[t] = t < CS - 1 || i < m ? sL[buf * m + i] : 0.f;
-                }
-                if (lane == rl) done |= 1u << tr;
-                const bool np = j + 1 < m && warp == ((j + 1) & 7);
-                if (tr == 0)
-                    gj_eliminate<RS, CS, 0>(v, w, lt, rl, sj, wj, warp, lane, j, m, np, done, sL, s_r, cur, s_rp, Mz, &s_bad);
-                else if (CS > 1 && tr == 1)
-                    gj_eliminate<RS, CS, (CS > 1 ? 1 : 0)>(v, w, lt, rl, sj, wj, warp, lane, j, m, np, done, sL, s_r, cur, s_rp, Mz, &s_bad);
-                else if (CS > 2 && tr == 2)
-                    gj_eliminate<RS, CS, (CS > 2 ? 2 : 0)>(v, w, lt, rl, sj, wj, warp, lane, j, m, np, done, sL, s_r, cur, s_rp, Mz, &s_bad);
-                else if (CS > 3)
-                    gj_eliminate<RS, CS, (CS > 3 ? 3 : 0)>(v, w, lt, rl, sj, wj, warp, lane, j, m, np, done, sL, s_r, cur, s_rp, Mz, &s_bad);
-            }
-        }
-        __syncthreads();
-        for (int q = tid; q < m; q += kFactorThreads) pos[cur[q]] = q;
-        __syncthreads();
-        if (next) {  // G_k[p] = (C part of pivot row p) / U_pp
-#pragma unroll
-            for (int t = 0; t < CS; ++t) {
-                const int i = lane + 32 * t;
-                if (i < m) {
-                    const int p = pos[i];
-                    const float ru = s_rp[p];
-#pragma unroll
-                    for (int s = 0; s < RS; ++s) {
-                        const int c = warp + 8 * s;
-                        if (c < m) sW[p * ld + c] = VX_SLOT(w, s, t) * ru;
+                for (int y = 0; y < NT; ++y) {
+                    const int c = 8 * (wn * NT + y) + 2 * q;
+                    float *x0 = X + r0 * ld + c, *x1 = X + r1 * ld + c;
+                    if (c + 1 < m) {
+                        const float2 e0 = *reinterpret_cast<float2 *>(x0), e1 = *reinterpret_cast<float2 *>(x1);
+                        if (i0m) *reinterpret_cast<float2 *>(x0) = make_float2(e0.x - d[y][0], e0.y - d[y][1]);
+                        if (i1m) *reinterpret_cast<float2 *>(x1) = make_float2(e1.x - d[y][2], e1.y - d[y][3]);
+                    } else if (c < m) {
+                        if (i0m) *x0 -= d[y][0];
+                        if (i1m) *x1 -= d[y][2];
                     }
                 }
             }
+            __syncthreads();
         }
-        __syncthreads();
-        for (int i = tid; i < m; i += kFactorThreads) a.perm[k * m + i] = cur[i];
         if (next) {
-            float *Gt = a.Gt + k * mm;
-            for (int c = warp; c < m; c += 8)
-                for (int i = lane; i < m; i += 32) Gt[(size_t)c * m + i] = sW[i * ld + c];
+            copy_async(sG, a.Gt + (size_t)k * mw, mw, tid, kFactorThreads);  // C_k
+            copy_async(sA, a.At + (size_t)(k + 1) * mw, mw, tid, kFactorThreads);
+            if (four) copy_async(sB, a.Di + (size_t)(k + 1) * mw, mw, tid, kFactorThreads);  // B_{k+1}
+            const float *nc = reinterpret_cast<const float *>(a.nz + (size_t)k * 2 * a.mp);
+            copy_async(reinterpret_cast<float *>(nzr), nc, a.mp / 2, tid, kFactorThreads);
+            copy_async(reinterpret_cast<float *>(nzr + a.mp), nc + a.mp + a.mp / 2, a.mp / 2, tid, kFactorThreads);  // A_{k+1}
         }
+        // the elimination: in step it, warp 0 factors panel it, the others apply panel it - 1
+        Panel<NT> pn;
+        if (warp == 0) pn.start(m, lane);
+        for (int it = 0; it <= P; ++it) {  // step P: the last panel's transform, by all warps
+            const int nu = it < P ? nw - 1 : nw, u = warp - (nw - nu);  // the warps that update, and this one's number
+            if (u < 0) {
+                if (it == 0) {
+                    Panel<NT>::fetch(pn.v, X, ld, m, 0, lane);
+                    pn.trim(m, 0, lane);
+                } else {
+                    pn.advance(X, ld, m, 8 * it, cur + 8 * (it - 1), lane);
+                }
+                pn.factor(m, 8 * it, m - 8 * it < 8 ? m - 8 * it : 8, cur, rowbuf, lane);
+                pn.store(X, ld, m, 8 * it, lane);
+            } else {
+                if (it > 0) {  // every tile but it - 1 (the transform itself) and it
+                    const int t0 = u, t1 = u + nu, nt = it < P ? P - 2 : P - 1;
+                    if (t0 < nt)
+                        tile_update<NT>(X, ld, m, it - 1, t0 < it - 1 ? t0 : t0 + 2,
+                                        t1 < nt ? (t1 < it - 1 ? t1 : t1 + 2) : -1, cur, lane);
+                }
+                if (it == P && tid < m) pos[cur[tid]] = tid;
+            }
+            if (it < P) __syncthreads();
+        }
+        if (warp == 0 && lane == 0 && pn.failed()) s_bad = 1;
+        copy_wait();
         __syncthreads();
+        {  // D_k^{-1} row by row, and G_k = D_k^{-1} C_k
+            float *Di = a.Di + (size_t)k * mw;
+            int pc[NT];
+#pragma unroll
+            for (int t = 0; t < NT; ++t) pc[t] = lane + 32 * t < m ? pos[lane + 32 * t] : 0;
+            for (int j = warp; j < m; j += nw) {
+                const float *row = X + cur[j] * ld;
+#pragma unroll
+                for (int t = 0; t < NT; ++t) {
+                    const int c = lane + 32 * t;
+                    if (c < m) Di[j * ld + c] = row[pc[t]];
+                }
+            }
+        }
+        if (next) {
+            float acc[NT][NT][4];  // [column tile][row tile]
+            int ur[NT][2];
+            unsigned nz[NT];
+#pragma unroll
+            for (int x = 0; x < NT; ++x) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int i = 16 * (wm * NT + x) + g + 8 * h;
+                    ur[x][h] = cur[i < m ? i : m - 1] * ld;
+                }
+                nz[x] = 0u;
+            }
+#pragma unroll
+            for (int t = 0; t < NT; ++t) {  // row lane + 32 t in pivot order belongs to step (lane >> 3) + 4 t
+                const int j = lane + 32 * t;
+                const unsigned f = j < m ? (unsigned)nzr[cur[j]] >> (wn * NT) : 0u;
+#pragma unroll
+                for (int x = 0; x < NT; ++x) nz[x] |= ((f >> x) & 1u) << ((lane >> 3) + 4 * t);
+            }
+#pragma unroll
+            for (int y = 0; y < NT; ++y) {
+                const unsigned todo = __reduce_or_sync(0xffffffffu, nz[y]);
+                product_col<NT>(X, ur, sG, cur, ld, m, 8 * (wn * NT + y), lane, todo, acc[y]);
+            }
+            __syncthreads();  // C_k and D_k^{-1} have been read
+            float *Gt = a.Gt + (size_t)k * mw;
+#pragma unroll
+            for (int x = 0; x < NT; ++x)
+#pragma unroll
+                for (int y = 0; y < NT; ++y)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int i = 16 * (wm * NT + x) + g + 8 * h, c = 8 * (wn * NT + y) + 2 * q;
+                        if (i < m && c < m) {
+                            const float e0 = acc[y][x][2 * h], e1 = acc[y][x][2 * h + 1];
+                            if (!(fabsf(e0) < INFINITY && fabsf(e1) < INFINITY)) s_bad = 1;
+                            if (c + 1 < m) {
+                                *reinterpret_cast<float2 *>(sG + i * ld + c) = make_float2(e0, e1);
+                                *reinterpret_cast<float2 *>(Gt + i * ld + c) = make_float2(e0, e1);
+                            } else {
+                                sG[i * ld + c] = e0;
+                                Gt[i * ld + c] = e0;
+                            }
+                        }
+                    }
+            if (four) {
+                const int t = xo;
+                xo = bo;
+                bo = t;
+            } else {
+                copy_async(X, a.Di + (size_t)(k + 1) * mw, mw, tid, kFactorThreads);
+                copy_wait();
+            }
+            __syncthreads();
+        }
     }
+    __syncthreads();
     if (tid == 0) {
         a.zbad[z0] = s_bad;
         if (s_bad) atomicOr(a.flag, 2);
     }
 }
 
-// Asynchronous copy of n floats from global to shared memory by one warp (16-byte cp.async where
-// both ends are 16-byte aligned and n is a multiple of 4, else plain loads), as one commit group.
-__device__ __forceinline__ void warp_stage(float *dst, const float *src, int n, int lane) {
-    const bool vec = ((reinterpret_cast<uintptr_t>(src) | reinterpret_cast<uintptr_t>(dst)) & 15) == 0 && (n & 3) == 0;
-    if (vec) {
-        const unsigned base = (unsigned)__cvta_generic_to_shared(dst);
-        for (int e = 4 * lane; e < n; e += 128)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(base + 4u * (unsigned)e), "l"(src + e)
-                         : "memory");
-    } else {
-        for (int e = lane; e < n; e += 32) dst[e] = src[e];
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-}
-template <int N>
-__device__ __forceinline__ void stage_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-    __syncwarp();
-}
-
-// One warp per ray (one warp per CTA). Each zone's FP32 matrices are staged in shared memory
-// (two buffers: the next matrix is in flight while the current one is used) and the vector being
-// eliminated is broadcast by shuffle: rows lane + 32 t (t < NT = ceil(m / 32)) of a zone's vector
-// live in lane `lane`; only the last slot can fall past m.
-template <int NT>
-__device__ __forceinline__ float slot_of(const float (&v)[NT], int t) {
-    float r = v[0];
-#pragma unroll
-    for (int q = 1; q < NT; ++q)
-        if (t == q) r = v[q];
-    return r;
-}
+// The solve sweep, one CTA of eight warps per ray: forward y_k = D_k^{-1} (rhs_k - A_k y_{k-1}), backward
+// delta_k = y_k - G_k delta_{k+1}, x += delta in FP64 (FIRST: x = delta). Every step is one
+// matrix-vector product with an m x m FP32 matrix that is used once, so the matrices of the whole
+// sweep run through a ring of nring shared-memory buffers (16-byte cp.async by all threads), and each
+// step costs one CTA barrier: eight lanes take a row (128 consecutive bytes per load; rows
+// 4 warp + lane / 8 + 32 u, u < NT = ceil(m / 32)), three shuffles finish it, and the row's first lane
+// holds its vector entries. What a step needs from the vectors in memory is loaded kAhead zones ahead.
+constexpr int kSweepThreads = 256;
+constexpr int kAhead = 2;
 template <bool FIRST, bool LAST, int NT>
-__global__ void __launch_bounds__(32) k_btd_sweep(const BtdArgs a) {
+__global__ void __launch_bounds__(kSweepThreads, 2) k_btd_sweep(const BtdArgs a) {
     extern __shared__ __align__(16) float sbuf[];
-    const int lane = threadIdx.x;
-    const int ray = blockIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gl = lane & 7;
     long long z0, z1;
-    if (!ray_range(a, ray, z0, z1) || z1 == z0) return;
-    const int m = a.m, mm = m * m;
-    float *S0 = sbuf, *S1 = sbuf + ((mm + 3) & ~3), *sv = S1 + ((mm + 3) & ~3);
+    if (!ray_range(a, blockIdx.x, z0, z1) || z1 == z0) return;
+    const int m = a.m, lw = a.ld, nb = a.nring, mw = m * lw;
+    float *vin = sbuf + nb * mw;  // [2][VX_BTD_MAX_M] the vector of a step and of the next
     if (a.zbad[z0]) {
         if (LAST)
-            for (long long e = z0 * m + lane; e < z1 * m; e += 32) a.x[e] = __longlong_as_double(0x7ff8000000000000ll);
+            for (long long e = z0 * m + tid; e < z1 * m; e += kSweepThreads) a.x[e] = __longlong_as_double(0x7ff8000000000000ll);
         return;
     }
-    float v[NT], yp[NT];
+    for (int i = tid; i < 2 * VX_BTD_MAX_M; i += kSweepThreads) vin[i] = 0.f;
+    const int n = (int)(z1 - z0), nf = 2 * n - 1, total = nf + n - 1;
+    // step s: D_{z0}^{-1}, then A_k and D_k^{-1} of the later zones, then G_k from the last but one zone back
+    const unsigned sb = (unsigned)__cvta_generic_to_shared(sbuf) + 16u * (unsigned)tid;
+    int si = 0, bi = 0;  // the next step to bring in and its buffer
+    auto issue = [&]() {
+        if (si < total) {
+            const float *src = (si < nf ? ((si & 1) ? a.At : a.Di) + (size_t)(z0 + (si + 1) / 2) * mw
+                                        : a.Gt + (size_t)(z1 - 2 - (si - nf)) * mw) + 4 * tid;
+            const unsigned dst = sb + 4u * (unsigned)(bi * mw);
 #pragma unroll
-    for (int t = 0; t < NT; ++t) yp[t] = 0.f;
-    // forward: S0 holds A_k (zones after the first), S1 the LU factors of D_k. Every zone commits
-    // two groups in the order they are needed (an empty one where nothing is copied), so
-    // wait_group 1 always completes the older of the two in flight.
-    warp_stage(S1, a.Mt + (size_t)z0 * mm, mm, lane);
-    if (z0 + 1 < z1) warp_stage(S0, a.At + (size_t)(z0 + 1) * mm, mm, lane);
-    else asm volatile("cp.async.commit_group;" ::: "memory");
-    for (long long k = z0; k < z1; ++k) {
-        // the zone's right-hand side and row permutation are loaded first and used after the
-        // product A_k y_{k-1}, which accumulates apart, so their latency hides behind it
-        const double *rhs = a.rhs + k * m;
-        const int *perm = a.perm + k * m;
-        double rv[NT];
-        int pv[NT];
-#pragma unroll
-        for (int t = 0; t < NT; ++t) {
-            const int i = lane + 32 * t;
-            rv[t] = t < NT - 1 || i < m ? rhs[i] : 0.0;
-            pv[t] = t < NT - 1 || i < m ? perm[i] : 0;
-            v[t] = 0.f;
+            for (int i = 0; i <= NT * NT; ++i)  // 1024 (NT^2 + 1) >= m lw
+                if (4 * (tid + kSweepThreads * i) < mw)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16u * (unsigned)(kSweepThreads * i)),
+                                 "l"(src + 4 * kSweepThreads * i)
+                                 : "memory");
         }
-        if (k > z0) {  // A_k y_{k-1}
-            stage_wait<1>();  // A_k (the LU factors of D_k are the newer group)
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        ++si;
+        bi = bi + 1 == nb ? 0 : bi + 1;
+    };
+    for (int s = 0; s < nb - 1; ++s) issue();
+    bool own[NT];  // this lane keeps the row's vector entries
+    int row[NT];
+    double rn[kAhead][NT];  // right-hand sides (forward) or x (backward) of the next zones
+    float yn[kAhead][NT];
 #pragma unroll
-            for (int tc = 0; tc < NT; ++tc) {
-                if (32 * tc >= m) break;
-                const int lim = m - 32 * tc < 32 ? m - 32 * tc : 32;
-                for (int l = 0; l < lim; ++l) {
-                    const int c = 32 * tc + l;
-                    const float yc = __shfl_sync(0xffffffffu, yp[tc], l);
+    for (int u = 0; u < NT; ++u) {
+        row[u] = 4 * warp + 32 * u + (lane >> 3);
+        own[u] = gl == 0 && row[u] < m;
 #pragma unroll
-                    for (int t = 0; t < NT; ++t) {
-                        const int i = lane + 32 * t;
-                        if (t < NT - 1 || i < m) v[t] = fmaf(S0[c * m + i], yc, v[t]);
-                    }
-                }
-            }
-            __syncwarp();
-            if (k + 1 < z1) warp_stage(S0, a.At + (size_t)(k + 1) * mm, mm, lane);
-            else asm volatile("cp.async.commit_group;" ::: "memory");
-        }
-        stage_wait<1>();  // the multiplier columns of zone k
-        // x = rhs_k - A_k y_{k-1}, rows in physical order
-#pragma unroll
-        for (int t = 0; t < NT; ++t) v[t] = (float)rv[t] - v[t];
-        // the factor's elimination replayed on x: at step j every row but cur[j] subtracts its
-        // multiplier times x_{cur[j]} (one chain of m steps)
-#pragma unroll
-        for (int tj = 0; tj < NT; ++tj) {
-            if (32 * tj >= m) break;
-            const int lim = m - 32 * tj < 32 ? m - 32 * tj : 32;
-            for (int l = 0; l < lim; ++l) {
-                const int j = 32 * tj + l;
-                const int rj = __shfl_sync(0xffffffffu, pv[tj], l);  // cur[j]
-                const float xr = __shfl_sync(0xffffffffu, slot_of<NT>(v, rj >> 5), rj & 31);
-                const float *col = S1 + j * m;
-#pragma unroll
-                for (int t = 0; t < NT; ++t) {
-                    const int i = lane + 32 * t;
-                    if ((t < NT - 1 || i < m) && i != rj) v[t] = fmaf(-col[i], xr, v[t]);
-                }
-            }
-        }
-        // y_j = x_{cur[j]} / pivot_j, in the order of the unknowns
-#pragma unroll
-        for (int t = 0; t < NT; ++t) {
-            const int i = lane + 32 * t;
-            if (t < NT - 1 || i < m) sv[i] = v[t];
-        }
-        __syncwarp();
-#pragma unroll
-        for (int t = 0; t < NT; ++t) {
-            const int j = lane + 32 * t;
-            if (t < NT - 1 || j < m) v[t] = sv[pv[t]] / S1[j * m + pv[t]];
-        }
-        __syncwarp();
-        if (k + 1 < z1) warp_stage(S1, a.Mt + (size_t)(k + 1) * mm, mm, lane);
-        else asm volatile("cp.async.commit_group;" ::: "memory");
-        float *yk = a.y + k * m;
-#pragma unroll
-        for (int t = 0; t < NT; ++t) {
-            const int i = lane + 32 * t;
-            if (t < NT - 1 || i < m) yk[i] = v[t];
-            yp[t] = v[t];
+        for (int h = 0; h < kAhead; ++h) {
+            rn[h][u] = own[u] && h + 1 < n ? a.rhs[(z0 + h + 1) * m + row[u]] : 0.0;
+            yn[h][u] = 0.f;
         }
     }
-    stage_wait<0>();
-    // backward: delta_k = y_k - G_k delta_{k+1}; x += delta (FP64). G of zone k in buffer k & 1.
-    float dn[NT];
+    __syncthreads();
 #pragma unroll
-    for (int t = 0; t < NT; ++t) dn[t] = 0.f;
-    if (z1 - 2 >= z0) warp_stage(((z1 - 2) & 1) ? S1 : S0, a.Gt + (size_t)(z1 - 2) * mm, mm, lane);
-    for (long long k = z1 - 1; k >= z0; --k) {
-        // y_k and x_k are loaded first and used after the product G_k delta_{k+1}
-        const float *yk = a.y + k * m;
-        double *xk = a.x + k * m;
-        float yv[NT];
-        double xv[NT];
+    for (int u = 0; u < NT; ++u)
+        if (own[u]) vin[row[u]] = (float)a.rhs[z0 * m + row[u]];
+    int bs = 0, par = 0;  // the step's buffer and vector
+    float p[NT];
+    auto step = [&]() {  // p = (the step's matrix) (its vector), in every lane of a row's group
+        // all but the newest nb - 2 groups have landed: the step's matrix is in its buffer
+        if (nb == 4) asm volatile("cp.async.wait_group 2;" ::: "memory");
+        else if (nb == 3) asm volatile("cp.async.wait_group 1;" ::: "memory");
+        else asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();  // ... for every thread; the step before is done with its buffer and its vector
+        issue();
+        const float *M = sbuf + bs * mw + 4 * gl, *v = vin + VX_BTD_MAX_M * par + 4 * gl;
+        float4 x[NT];
 #pragma unroll
-        for (int t = 0; t < NT; ++t) {
-            const int i = lane + 32 * t;
-            yv[t] = t < NT - 1 || i < m ? yk[i] : 0.f;
-            xv[t] = !FIRST && (t < NT - 1 || i < m) ? xk[i] : 0.0;
-            v[t] = 0.f;
+        for (int c = 0; c < NT; ++c) x[c] = *reinterpret_cast<const float4 *>(v + 32 * c);
+#pragma unroll
+        for (int u = 0; u < NT; ++u) {
+            const float *r = M + min(row[u], m - 1) * lw;
+            float e0 = 0.f, e1 = 0.f;
+#pragma unroll
+            for (int c = 0; c < NT; ++c) {
+                float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (c < NT - 1 || 32 * c + 4 * gl < lw) w = *reinterpret_cast<const float4 *>(r + 32 * c);
+                e0 = fmaf(w.x, x[c].x, e0);
+                e1 = fmaf(w.y, x[c].y, e1);
+                e0 = fmaf(w.z, x[c].z, e0);
+                e1 = fmaf(w.w, x[c].w, e1);
+            }
+            p[u] = e0 + e1;
         }
-        if (k + 1 < z1) {
-            const float *G = (k & 1) ? S1 : S0;
-            if (k - 1 >= z0) warp_stage(((k - 1) & 1) ? S1 : S0, a.Gt + (size_t)(k - 1) * mm, mm, lane);
-            else asm volatile("cp.async.commit_group;" ::: "memory");
-            stage_wait<1>();  // G_k (G_{k-1} is the newer group)
 #pragma unroll
-            for (int tc = 0; tc < NT; ++tc) {
-                if (32 * tc >= m) break;
-                const int lim = m - 32 * tc < 32 ? m - 32 * tc : 32;
-                for (int l = 0; l < lim; ++l) {
-                    const int c = 32 * tc + l;
-                    const float dc = __shfl_sync(0xffffffffu, dn[tc], l);
+        for (int o = 4; o > 0; o >>= 1)
 #pragma unroll
-                    for (int t = 0; t < NT; ++t) {
-                        const int i = lane + 32 * t;
-                        if (t < NT - 1 || i < m) v[t] = fmaf(G[c * m + i], dc, v[t]);
-                    }
+            for (int u = 0; u < NT; ++u) p[u] += __shfl_xor_sync(0xffffffffu, p[u], o);
+        bs = bs + 1 == nb ? 0 : bs + 1;
+        par ^= 1;
+    };
+    for (long long k = z0;; ++k) {  // forward
+        step();  // p = y_k
+        const bool last = k + 1 == z1;
+#pragma unroll
+        for (int u = 0; u < NT; ++u)
+            if (own[u]) {
+                vin[VX_BTD_MAX_M * par + row[u]] = p[u];
+                if (!last) a.y[k * m + row[u]] = p[u];
+            }
+        if (last) break;
+        step();  // p = A_{k+1} y_k
+#pragma unroll
+        for (int u = 0; u < NT; ++u)
+            if (own[u]) {
+                vin[VX_BTD_MAX_M * par + row[u]] = (float)rn[0][u] - p[u];
+                rn[0][u] = rn[1][u];
+                rn[1][u] = k + 3 < z1 ? a.rhs[(k + 3) * m + row[u]] : 0.0;
+            }
+    }
+    static_assert(kAhead == 2, "the vectors' shifts are written out");
+#pragma unroll
+    for (int u = 0; u < NT; ++u)
+        if (own[u]) {  // the last zone: delta = y
+            double *x = a.x + (z1 - 1) * m + row[u];
+            *x = FIRST ? (double)p[u] : *x + (double)p[u];
+#pragma unroll
+            for (int h = 0; h < kAhead; ++h) {
+                const long long k = z1 - 2 - h;
+                yn[h][u] = k >= z0 ? a.y[k * m + row[u]] : 0.f;
+                if (!FIRST) rn[h][u] = k >= z0 ? a.x[k * m + row[u]] : 0.0;
+            }
+        }
+    for (long long k = z1 - 2; k >= z0; --k) {  // backward
+        step();  // p = G_k delta_{k+1}
+#pragma unroll
+        for (int u = 0; u < NT; ++u)
+            if (own[u]) {
+                const float dl = yn[0][u] - p[u];
+                vin[VX_BTD_MAX_M * par + row[u]] = dl;
+                a.x[k * m + row[u]] = FIRST ? (double)dl : rn[0][u] + (double)dl;
+                yn[0][u] = yn[1][u];
+                yn[1][u] = k - 2 >= z0 ? a.y[(k - 2) * m + row[u]] : 0.f;
+                if (!FIRST) {
+                    rn[0][u] = rn[1][u];
+                    rn[1][u] = k - 2 >= z0 ? a.x[(k - 2) * m + row[u]] : 0.0;
                 }
             }
-            __syncwarp();
-        }
-#pragma unroll
-        for (int t = 0; t < NT; ++t) {
-            const int i = lane + 32 * t;
-            v[t] = yv[t] - v[t];  // delta_k = y_k - G_k delta_{k+1}
-            if (t < NT - 1 || i < m) xk[i] = FIRST ? (double)v[t] : xv[t] + (double)v[t];
-            dn[t] = v[t];
-        }
     }
-    stage_wait<0>();
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
 // Each ray's zones are split over kResidSplit CTAs (blockIdx.y), a warp per zone. The kernel is
@@ -750,53 +959,62 @@ __global__ void __launch_bounds__(kResidThreads, VX_RESID_MINB) k_btd_resid(cons
 
 }  // namespace
 
-// The factor kernel's register tile for m unknowns per zone: rows per warp x columns per lane.
+// The factor kernel for NT = ceil(m / 32) row slots per lane.
 static const void *factor_kernel(int m) {
-    if (m <= 32) return (const void *)k_btd_factor<4, 1>;
-    if (m <= 64) return (const void *)k_btd_factor<8, 2>;
-    if (m <= 96) return (const void *)k_btd_factor<12, 3>;
-    return (const void *)k_btd_factor<16, 4>;
+    if (m <= 32) return (const void *)k_btd_factor<1>;
+    if (m <= 64) return (const void *)k_btd_factor<2>;
+    if (m <= 96) return (const void *)k_btd_factor<3>;
+    return (const void *)k_btd_factor<4>;
 }
 static void launch_factor(int m, int grid, size_t smem, cudaStream_t s, const BtdArgs &a) {
-    if (m <= 32) k_btd_factor<4, 1><<<grid, kFactorThreads, smem, s>>>(a);
-    else if (m <= 64) k_btd_factor<8, 2><<<grid, kFactorThreads, smem, s>>>(a);
-    else if (m <= 96) k_btd_factor<12, 3><<<grid, kFactorThreads, smem, s>>>(a);
-    else k_btd_factor<16, 4><<<grid, kFactorThreads, smem, s>>>(a);
+    if (m <= 32) k_btd_factor<1><<<grid, kFactorThreads, smem, s>>>(a);
+    else if (m <= 64) k_btd_factor<2><<<grid, kFactorThreads, smem, s>>>(a);
+    else if (m <= 96) k_btd_factor<3><<<grid, kFactorThreads, smem, s>>>(a);
+    else k_btd_factor<4><<<grid, kFactorThreads, smem, s>>>(a);
 }
-
-// The sweep kernel for NT = ceil(m / 32) row slots per lane.
+static void launch_convert(int m, long long zones, cudaStream_t s, const BtdArgs &a) {
+    const long long warps = (3 * zones * m + kConvRows - 1) / kConvRows, ctas = (warps + kConvThreads / 32 - 1) / (kConvThreads / 32);
+    const int grid = (int)(ctas < kConvGrid ? ctas : kConvGrid);
+    if (m <= 32) k_btd_convert<1><<<grid, kConvThreads, 0, s>>>(a);
+    else if (m <= 64) k_btd_convert<2><<<grid, kConvThreads, 0, s>>>(a);
+    else if (m <= 96) k_btd_convert<3><<<grid, kConvThreads, 0, s>>>(a);
+    else k_btd_convert<4><<<grid, kConvThreads, 0, s>>>(a);
+}
 template <bool F, bool L>
-static const void *sweep_kernel(int nt) {
-    if (nt <= 1) return (const void *)k_btd_sweep<F, L, 1>;
-    if (nt == 2) return (const void *)k_btd_sweep<F, L, 2>;
-    if (nt == 3) return (const void *)k_btd_sweep<F, L, 3>;
+static const void *sweep_kernel(int m) {
+    if (m <= 32) return (const void *)k_btd_sweep<F, L, 1>;
+    if (m <= 64) return (const void *)k_btd_sweep<F, L, 2>;
+    if (m <= 96) return (const void *)k_btd_sweep<F, L, 3>;
     return (const void *)k_btd_sweep<F, L, 4>;
 }
 template <bool F, bool L>
 static void launch_sweep(int m, int grid, size_t smem, cudaStream_t s, const BtdArgs &a) {
-    const int nt = (m + 31) / 32;
-    if (nt <= 1) k_btd_sweep<F, L, 1><<<grid, 32, smem, s>>>(a);
-    else if (nt == 2) k_btd_sweep<F, L, 2><<<grid, 32, smem, s>>>(a);
-    else if (nt == 3) k_btd_sweep<F, L, 3><<<grid, 32, smem, s>>>(a);
-    else k_btd_sweep<F, L, 4><<<grid, 32, smem, s>>>(a);
+    if (m <= 32) k_btd_sweep<F, L, 1><<<grid, kSweepThreads, smem, s>>>(a);
+    else if (m <= 64) k_btd_sweep<F, L, 2><<<grid, kSweepThreads, smem, s>>>(a);
+    else if (m <= 96) k_btd_sweep<F, L, 3><<<grid, kSweepThreads, smem, s>>>(a);
+    else k_btd_sweep<F, L, 4><<<grid, kSweepThreads, smem, s>>>(a);
 }
 
+// Shared memory that lets two CTAs share an SM (228 KB, 1 KB of it reserved per CTA), and one CTA's limit.
+constexpr size_t kSmemHalf = 113 * 1024 - 64, kSmemFull = 226 * 1024;
+
 struct vx_btd {
-    int m = 0, ld = 0, n_refine = 0;
+    int m = 0, ld = 0, mp = 0, nbuf = 3, nring = 2, n_refine = 0;
     long long max_zones = 0;
     size_t smem = 0, smem_sweep = 0;
-    float *Mt = nullptr, *Gt = nullptr, *At = nullptr, *y = nullptr;
-    int *perm = nullptr, *zbad = nullptr, *flag = nullptr;  // flag[0]: numeric flag, flag[1]: offsets invalid
+    float *Di = nullptr, *Gt = nullptr, *At = nullptr, *y = nullptr;
+    unsigned short *nz = nullptr;
+    int *zbad = nullptr, *flag = nullptr;  // flag[0]: numeric flag, flag[1]: offsets invalid
     double *r = nullptr;
 };
 
 static void btd_free(vx_btd *h) {
     if (!h) return;
-    cudaFree(h->Mt);
+    cudaFree(h->Di);
+    cudaFree(h->nz);
     cudaFree(h->Gt);
     cudaFree(h->At);
     cudaFree(h->y);
-    cudaFree(h->perm);
     cudaFree(h->zbad);
     cudaFree(h->flag);
     cudaFree(h->r);
@@ -813,29 +1031,42 @@ extern "C" vx_status vx_btd_create(int m, long long max_zones, int n_refine, vx_
     vx_btd *h = new (std::nothrow) vx_btd;
     if (!h) return bfail(VX_ERR_OOM, "host allocation failed");
     h->m = m;
-    h->ld = m | 1;  // odd row stride: column walks through shared memory hit distinct banks
+    // row stride 4 mod 8 floats: the MMA fragments of the left operand (eight rows, four columns) fall in
+    // distinct banks, and a matrix is copied in whole 16-byte pieces
+    h->ld = m + ((12 - m % 8) % 8);
+    h->mp = (m + 7) & ~7;
     h->n_refine = n_refine;
     h->max_zones = max_zones;
-    h->smem = ((size_t)3 * m * h->ld + 3 * m) * sizeof(float) + (size_t)2 * m * sizeof(int);
-    h->smem_sweep = ((size_t)2 * ((m * m + 3) & ~3) + m) * sizeof(float);
-    const size_t zc = (size_t)(max_zones > 0 ? max_zones : 1), mm = (size_t)m * m;
+    // a fourth buffer (the next zone's B) where it costs no second CTA per SM: m <= 84, and from 97 on
+    // where one CTA fills an SM with three as well
+    const size_t s3 = factor_smem(m, h->ld, 3), s4 = factor_smem(m, h->ld, 4);
+    h->nbuf = s4 <= kSmemHalf || (s3 > kSmemHalf && s4 <= kSmemFull) ? 4 : 3;
+    h->smem = h->nbuf == 4 ? s4 : s3;
+    const size_t mw = (size_t)m * h->ld;
+    auto ring = [&](int nb) { return (nb * mw + 2 * VX_BTD_MAX_M) * sizeof(float); };
+    h->nring = ring(4) <= kSmemHalf ? 4 : ring(3) <= kSmemFull ? 3 : 2;
+    h->smem_sweep = ring(h->nring);
+    const size_t zc = (size_t)(max_zones > 0 ? max_zones : 1);
     cudaError_t e = cudaSuccess;
-    if (e == cudaSuccess) e = cudaMalloc(&h->Mt, zc * mm * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&h->Gt, zc * mm * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&h->At, zc * mm * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc(&h->Di, zc * mw * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc(&h->Gt, zc * mw * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc(&h->At, zc * mw * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc(&h->nz, zc * 2 * h->mp * sizeof(unsigned short));
     if (e == cudaSuccess) e = cudaMalloc(&h->y, zc * m * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&h->perm, zc * m * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&h->zbad, zc * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&h->r, zc * m * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&h->flag, 2 * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(h->flag, 0, 2 * sizeof(int));
+    if (h->ld != m)  // the columns that pad a row are read by the sweeps and never written
+        for (float *w : {h->Di, h->Gt, h->At})
+            if (e == cudaSuccess) e = cudaMemset(w, 0, zc * mw * sizeof(float));
+    // the kernels' limit, not this handle's size: handles of several m share them
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(factor_kernel(m), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->smem);
-    const int nt = (m + 31) / 32;
-    const void *sweeps[4] = {sweep_kernel<true, true>(nt), sweep_kernel<true, false>(nt), sweep_kernel<false, true>(nt),
-                             sweep_kernel<false, false>(nt)};
+        e = cudaFuncSetAttribute(factor_kernel(m), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFull);
+    const void *sweeps[4] = {sweep_kernel<true, true>(m), sweep_kernel<true, false>(m), sweep_kernel<false, true>(m),
+                             sweep_kernel<false, false>(m)};
     for (int i = 0; i < 4 && e == cudaSuccess; ++i)
-        e = cudaFuncSetAttribute(sweeps[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->smem_sweep);
+        e = cudaFuncSetAttribute(sweeps[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFull);
     if (e != cudaSuccess) {
         btd_free(h);
         return bfail(e == cudaErrorMemoryAllocation ? VX_ERR_OOM : VX_ERR_CUDA, "vx_btd_create: %s",
@@ -872,6 +1103,9 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
     BtdArgs a;
     a.m = h->m;
     a.ld = h->ld;
+    a.mp = h->mp;
+    a.nbuf = h->nbuf;
+    a.nring = h->nring;
     a.n_rays = n_rays;
     a.n_zones = n_zones;
     a.off = ray_offsets;
@@ -882,16 +1116,18 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
     a.rhs = d;
     a.x = x;
     a.r = h->r;
-    a.Mt = h->Mt;
+    a.Di = h->Di;
+    a.nz = h->nz;
     a.Gt = h->Gt;
     a.At = h->At;
     a.y = h->y;
-    a.perm = h->perm;
     a.zbad = h->zbad;
     a.flag = h->flag;
     a.inval = h->flag + 1;
     BTD_CU(cudaMemsetAsync(h->flag + 1, 0, sizeof(int), s));
     k_btd_validate<<<(unsigned)((n_rays + 256) / 256), 256, 0, s>>>(ray_offsets, n_rays, n_zones, h->flag + 1, h->flag);
+    BTD_CU(cudaGetLastError());
+    launch_convert(h->m, n_zones, s, a);
     BTD_CU(cudaGetLastError());
     launch_factor(h->m, n_rays, h->smem, s, a);
     BTD_CU(cudaGetLastError());
