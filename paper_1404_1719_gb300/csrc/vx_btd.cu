@@ -11,14 +11,14 @@
 //  * k_btd_sweep: one CTA per ray solves M delta = rhs with those: forward
 //    y_k = D_k^{-1} (rhs_k - A_k y_{k-1}), backward delta_k = y_k - G_k delta_{k+1}, a chain of
 //    matrix-vector products. The first sweep writes x = delta, later ones add delta to x in FP64.
-//  * k_btd_resid: the FP64 residual r = d - M x from the caller's FP64 blocks, a warp per zone,
-//    four lanes per row and eight rows per pass (coalesced), FMA accumulation and a fixed two-step
+//  * k_btd_resid: the FP64 residual r = d - M x from the caller's FP64 blocks, eight rows per warp, four
+//    lanes per row (coalesced), zero groups of the couplings left out, FMA accumulation and a fixed two-step
 //    shuffle reduction per row.
 // The host runs validate, convert, factor, sweep, then n_refine times (resid, sweep), all on the caller's
 // stream.
 // With the inverse instead of the elimination's multipliers (which the sweeps replayed, a shuffle per
 // unknown), GB300, m = 84, 400 zones a ray: one ray factor 24.3 -> 10.0 ms, a sweep 3.0 -> 1.3 ms; 304 rays
-// 29.7 -> 14.9 ms (conversion included in the former, 8.0 ms apart in the latter) and 3.1 -> 1.8 ms (10.3 GB, 5.7 TB/s).
+// 29.7 -> 14.9 ms (which included the conversion, now 6.1 ms apart) and 3.1 -> 1.8 ms (10.3 GB, 5.7 TB/s).
 // The solution's error without refinement and with one sweep is 0.2 to 0.8 of what it was (m = 34 to 128).
 #include "../../include/vx_btd.h"
 
@@ -39,7 +39,6 @@ namespace {
 
 constexpr int kFactorThreads = 256;
 constexpr int kResidThreads = 256;
-constexpr int kResidSplit = 4;  // CTAs per ray in the residual kernel
 
 vx_status bfail(vx_status s, const char *fmt, ...) {
     char buf[512];
@@ -241,51 +240,44 @@ __device__ __forceinline__ float btd_f32(double x) {
 
 // The blocks in FP32, row-major with row stride ld, for the factor kernel and the sweeps: A_k to At, B_k to Di
 // and C_k to Gt (the factor kernel puts D_k^{-1} and G_k in the places of B_k and C_k, which it has read by
-// then), and per row of C and A a bit per eight columns that hold anything but zeros (nz[k][C, A][mp]). A warp
-// takes kConvRows rows at a time, all their loads in flight together. Bound by HBM (12 m^2 bytes read and
-// written per block for 8 m^2 read); apart from the factor kernel because the loads' registers, and the
-// conversions' instructions, cost that kernel more than the extra pass.
-constexpr int kConvThreads = 256, kConvRows = 4, kConvGrid = 152 * 16;
+// then), and per row of C and A a bit per eight columns that hold anything but zeros (nz[k][C, A][mp]; decided on
+// the FP64 entries, so that the residual can go by it as well). A CTA takes a matrix at a time, a warp
+// kConvRows of its rows, all their loads in flight together. Bound by HBM (8 m^2 bytes read and 4 m^2 written
+// per block); apart from the factor kernel because the loads' registers, and the conversions' instructions,
+// cost that kernel more than the extra pass.
+constexpr int kConvThreads = 256, kConvRows = 4, kConvGrid = 152 * 8;
 template <int NT>
 __global__ void __launch_bounds__(kConvThreads) k_btd_convert(const BtdArgs a) {
     if (*a.inval) return;
-    const int m = a.m, ld = a.ld, lane = threadIdx.x & 31;
-    const long long rows = 3 * a.n_zones * m, step = (long long)gridDim.x * (kConvThreads / 32) * kConvRows;
-    for (long long r0 = ((long long)blockIdx.x * (kConvThreads / 32) + (threadIdx.x >> 5)) * kConvRows; r0 < rows; r0 += step) {
-        const long long zm = r0 / m;  // (zone, matrix) of the first row: 3 k + (0 A, 1 B, 2 C)
-        double v[kConvRows][NT];
-        float *dst[kConvRows];
-        int mat[kConvRows], row[kConvRows];
-        long long zone[kConvRows];
+    const int m = a.m, ld = a.ld, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = kConvThreads / 32;
+    for (long long q = blockIdx.x; q < 3 * a.n_zones; q += gridDim.x) {
+        const long long k = q / 3;
+        const int w = (int)(q - 3 * k);
+        const double *src = (w == 0 ? a.A : w == 1 ? a.B : a.C) + (size_t)k * m * m + lane;
+        float *dst = (w == 0 ? a.At : w == 1 ? a.Di : a.Gt) + (size_t)k * m * ld + lane;
+        unsigned short *nz = a.nz + ((size_t)k * 2 + (w == 0)) * a.mp;
+        for (int i0 = warp; i0 < m; i0 += kConvRows * nw) {
+            double v[kConvRows][NT];
 #pragma unroll
-        for (int r = 0; r < kConvRows; ++r) {
-            long long q = zm;
-            int i = (int)(r0 + r - zm * m);
-            while (i >= m) { i -= m; ++q; }
-            const long long k = q / 3;
-            const int w = (int)(q - 3 * k);
-            const bool in = r0 + r < rows;
-            const double *src = (w == 0 ? a.A : w == 1 ? a.B : a.C) + ((size_t)k * m + i) * m + lane;
-            dst[r] = in ? (w == 0 ? a.At : w == 1 ? a.Di : a.Gt) + ((size_t)k * m + i) * ld + lane : nullptr;
-            mat[r] = w;
-            row[r] = i;
-            zone[r] = k;
+            for (int r = 0; r < kConvRows; ++r)
 #pragma unroll
-            for (int t = 0; t < NT; ++t) v[r][t] = in && (t < NT - 1 || lane + 32 * t < m) ? __ldg(src + 32 * t) : 0.0;
-        }
+                for (int t = 0; t < NT; ++t)
+                    v[r][t] = i0 + r * nw < m && (t < NT - 1 || lane + 32 * t < m) ? __ldcs(src + (i0 + r * nw) * m + 32 * t) : 0.0;
 #pragma unroll
-        for (int r = 0; r < kConvRows; ++r) {
-            if (!dst[r]) continue;
-            unsigned bits = 0u;
+            for (int r = 0; r < kConvRows; ++r) {
+                const int i = i0 + r * nw;
+                if (i >= m) break;
+                unsigned bits = 0u;
 #pragma unroll
-            for (int t = 0; t < NT; ++t) {
-                const float f = btd_f32(v[r][t]);
-                if (t < NT - 1 || lane + 32 * t < m) dst[r][32 * t] = f;
-                bits |= f != 0.f ? 1u << (4 * t) : 0u;
+                for (int t = 0; t < NT; ++t) {
+                    if (t < NT - 1 || lane + 32 * t < m) dst[i * ld + 32 * t] = btd_f32(v[r][t]);
+                    const unsigned long long mag = (unsigned long long)__double_as_longlong(v[r][t]) << 1;
+                    bits |= mag != 0ull ? 1u << (4 * t) : 0u;
+                }
+                if (w == 1) continue;
+                bits = __reduce_or_sync(0xffffffffu, bits << (lane >> 3));
+                if (lane == 0) nz[i] = (unsigned short)bits;
             }
-            if (mat[r] == 1) continue;
-            bits = __reduce_or_sync(0xffffffffu, bits << (lane >> 3));
-            if (lane == 0) a.nz[((size_t)zone[r] * 2 + (mat[r] == 0)) * a.mp + row[r]] = (unsigned short)bits;
         }
     }
 }
@@ -903,57 +895,67 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_btd_sweep(const BtdArgs a)
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-// Each ray's zones are split over kResidSplit CTAs (blockIdx.y), a warp per zone. The kernel is
-// bound by the FP64 pipe, not by HBM: every matrix element costs one FP64 FMA and GB300 issues few
-// of them per clock, so the layout minimises FP64 instructions beyond those FMAs. Lane 4 r + c takes
-// row i0 + r of a pass of eight rows and the columns c, c + 4, ... (four lanes read 32 contiguous
-// bytes of a row, eight rows per load instruction), accumulates with FMAs only, and two
-// shuffle-add steps finish the row: about 3 m + 2 FP64 operations per row against 3 m.
-#ifndef VX_RESID_MINB
-#define VX_RESID_MINB 2
-#endif
-constexpr int kResidUnroll = 7;  // column quads per batch of loads in flight
-__global__ void __launch_bounds__(kResidThreads, VX_RESID_MINB) k_btd_resid(const BtdArgs a) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+// The FP64 residual, a ray's zones split over blockIdx.y CTAs, a warp per eight rows of a zone. Every matrix
+// element costs one FP64 FMA, which GB300 issues at 2 per clock and SM (less than HBM can feed), so the layout
+// minimises FP64 instructions beyond those FMAs and leaves out what is known to be zero: groups of eight
+// columns that are zero in a row of A_k or C_k (nz) are neither read nor multiplied. Lane 4 r + c
+// takes row i0 + r and the columns c, c + 4, ... (four lanes read 32 contiguous bytes of a row, eight rows
+// per load instruction; in A and C each row goes through its own groups), accumulates with FMAs only, and two
+// shuffle-add steps finish the row.
+// GB300, m = 84, 304 rays x 400 zones: one coupling per row 5.3 -> 2.2 ms, dense couplings 5.3 -> 5.1 ms (FP64
+// pipe: 4.1 at 2 FMA per clock and SM); one ray 0.88 -> 0.02 ms (was four CTAs).
+constexpr int kResidB = 7;  // quads of B in flight
+constexpr int kResidG = 3;  // column groups of A or C (two loads a lane each) in flight
+__device__ __forceinline__ double resid_groups(const double *M, const double *x, unsigned todo, int cc, int m) {
+    double s = 0.0;
+    while (__any_sync(0xffffffffu, todo)) {
+        int j[kResidG];
+        double v[kResidG][2];
+#pragma unroll
+        for (int u = 0; u < kResidG; ++u) {
+            j[u] = todo ? 8 * (__ffs(todo) - 1) + cc : m;  // m: none left
+            todo &= todo - 1;                              // 0 stays 0
+#pragma unroll
+            for (int h = 0; h < 2; ++h) v[u][h] = j[u] + 4 * h < m ? M[j[u] + 4 * h] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < kResidG; ++u) {
+            if (!__any_sync(0xffffffffu, j[u] < m)) break;
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                if (j[u] + 4 * h < m) s = fma(v[u][h], x[j[u] + 4 * h], s);
+        }
+    }
+    return s;
+}
+__global__ void __launch_bounds__(kResidThreads) k_btd_resid(const BtdArgs a) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = kResidThreads / 32;
     const int rr = lane >> 2, cc = lane & 3;
     long long z0, z1;
     if (!ray_range(a, blockIdx.x, z0, z1) || z1 == z0 || a.zbad[z0]) return;
-    const long long len = z1 - z0;
-    const long long q0 = z0 + len * blockIdx.y / gridDim.y, q1 = z0 + len * (blockIdx.y + 1) / gridDim.y;
-    const int m = a.m;
-    const size_t mm = (size_t)m * m;
-    for (long long k = q0 + warp; k < q1; k += nw) {
-        const double *Ak = a.A + k * mm, *Bk = a.B + k * mm, *Ck = a.C + k * mm;
-        const double *xm = a.x + (k - 1) * m, *x0 = a.x + k * m, *xp = a.x + (k + 1) * m;
-        const bool lo = k > z0, hi = k + 1 < z1;
-        for (int i0 = 0; i0 < m; i0 += 8) {
-            const int i = i0 + rr < m ? i0 + rr : m - 1;  // rows past the end repeat the last one
-            const size_t ro = (size_t)i * m;
-            double s = 0.0;
-            for (int j0 = cc; j0 < m; j0 += 4 * kResidUnroll) {
-                double vb[kResidUnroll], va[kResidUnroll], vc[kResidUnroll];
+    const int m = a.m, np = (m + 7) >> 3;
+    const long long units = (z1 - z0) * np;
+    for (long long q = units * blockIdx.y / gridDim.y + warp, qe = units * (blockIdx.y + 1) / gridDim.y; q < qe; q += nw) {
+        const long long k = z0 + q / np;
+        const int i0 = 8 * (int)(q % np);
+        const int i = i0 + rr < m ? i0 + rr : m - 1;  // rows past the end repeat the last one
+        const size_t ro = ((size_t)k * m + i) * m;
+        const unsigned nc = k + 1 < z1 ? a.nz[(size_t)k * 2 * a.mp + i] : 0u, na = k > z0 ? a.nz[((size_t)k * 2 + 1) * a.mp + i] : 0u;
+        const double *B = a.B + ro, *x0 = a.x + k * m;
+        double s = 0.0;
+        for (int j0 = cc; j0 < m; j0 += 4 * kResidB) {
+            double v[kResidB];
 #pragma unroll
-                for (int u = 0; u < kResidUnroll; ++u) {
-                    const int j = j0 + 4 * u;
-                    const bool in = j < m;
-                    vb[u] = in ? Bk[ro + j] : 0.0;
-                    va[u] = in && lo ? Ak[ro + j] : 0.0;
-                    vc[u] = in && hi ? Ck[ro + j] : 0.0;
-                }
+            for (int u = 0; u < kResidB; ++u) v[u] = j0 + 4 * u < m ? B[j0 + 4 * u] : 0.0;
 #pragma unroll
-                for (int u = 0; u < kResidUnroll; ++u) {
-                    const int j = j0 + 4 * u;
-                    if (j < m) {
-                        s = fma(vb[u], x0[j], s);
-                        if (lo) s = fma(va[u], xm[j], s);
-                        if (hi) s = fma(vc[u], xp[j], s);
-                    }
-                }
-            }
-            s += __shfl_xor_sync(0xffffffffu, s, 1);
-            s += __shfl_xor_sync(0xffffffffu, s, 2);
-            if (cc == 0 && i0 + rr < m) a.r[k * m + i] = a.d[k * m + i] - s;
+            for (int u = 0; u < kResidB; ++u)
+                if (j0 + 4 * u < m) s = fma(v[u], x0[j0 + 4 * u], s);
         }
+        s += resid_groups(a.A + ro, x0 - m, na, cc, m);
+        s += resid_groups(a.C + ro, x0 + m, nc, cc, m);
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        if (cc == 0 && i0 + rr < m) a.r[k * m + i] = a.d[k * m + i] - s;
     }
 }
 
@@ -973,8 +975,7 @@ static void launch_factor(int m, int grid, size_t smem, cudaStream_t s, const Bt
     else k_btd_factor<4><<<grid, kFactorThreads, smem, s>>>(a);
 }
 static void launch_convert(int m, long long zones, cudaStream_t s, const BtdArgs &a) {
-    const long long warps = (3 * zones * m + kConvRows - 1) / kConvRows, ctas = (warps + kConvThreads / 32 - 1) / (kConvThreads / 32);
-    const int grid = (int)(ctas < kConvGrid ? ctas : kConvGrid);
+    const int grid = (int)(3 * zones < kConvGrid ? 3 * zones : kConvGrid);
     if (m <= 32) k_btd_convert<1><<<grid, kConvThreads, 0, s>>>(a);
     else if (m <= 64) k_btd_convert<2><<<grid, kConvThreads, 0, s>>>(a);
     else if (m <= 96) k_btd_convert<3><<<grid, kConvThreads, 0, s>>>(a);
@@ -1136,9 +1137,14 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
     else
         launch_sweep<true, false>(h->m, n_rays, h->smem_sweep, s, a);
     BTD_CU(cudaGetLastError());
+    // CTAs per ray of the residual: enough to fill the chip with few rays, at most one per eight units (row octets)
+    const long long units = n_zones * ((h->m + 7) / 8);
+    long long split = (8 * 152 + n_rays - 1) / n_rays, most = (units + 8 * n_rays - 1) / (8 * (long long)n_rays);
+    split = split > most ? most : split;
+    split = split < 16 ? 16 : split;
     for (int it = 1; it <= h->n_refine; ++it) {
         a.rhs = d;
-        k_btd_resid<<<dim3(n_rays, kResidSplit), kResidThreads, 0, s>>>(a);
+        k_btd_resid<<<dim3(n_rays, (unsigned)split), kResidThreads, 0, s>>>(a);
         BTD_CU(cudaGetLastError());
         a.rhs = h->r;
         if (it == h->n_refine)
