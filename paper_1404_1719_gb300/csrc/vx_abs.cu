@@ -1,12 +1,11 @@
 // vx_abs.cu -- charged-current absorption and emission on free nucleons (include/vx_abs.h).
 //
 // A streaming kernel: every (zone, species, bin) entry is independent and costs a few dozen
-// arithmetic operations against 32 B (rates) or 128 B (rates and Jacobian) of output. A block
-// takes a contiguous range of whole zones per iteration of a grid-stride loop, so a warp's stores
-// are contiguous; the zone quantities its entries share (1/T, the nucleon densities, the state
-// check) are formed once per zone into shared memory by the block's first threads. The lepton
+// arithmetic operations against 32 B (rates) or 128 B (rates and Jacobian) of output. A warp
+// takes a contiguous range of whole zones, so its stores are contiguous; the zone quantities its
+// entries share (1/T, the nucleon densities, the state check) are formed once per zone into shared memory. The lepton
 // energy E and the prefactor (g2/pi)(1 + 3 gA^2) E^2 of every (species, bin) are formed on the
-// host in FP64 and passed by value. (A block takes whole zones, and a thread the same entry of
+// host in FP64 and passed by value. (A warp takes whole zones, and a lane the same entry of
 // each: no 64-bit integer division per entry, which would run on the FP64 unit.)
 // Forms: FP64 (library exp, true division, FP64 products) and mixed. GB300 issues FP64 about 75x
 // slower than FP32, so the mixed form runs no FP64 arithmetic per entry. The exponent argument
@@ -40,7 +39,8 @@ constexpr double kMu = 1.66053906660e-24;    // atomic mass unit, g
 constexpr double kPi = 3.14159265358979323846;
 constexpr int kAbsBlock = 256;
 constexpr int kAbsWarps = kAbsBlock / 32;
-constexpr int kZoneSlots = 32;  // zones a warp's 32 consecutive entries can span (S N >= 1)
+constexpr int kAbsFill = 24;
+constexpr int kZoneSlots = 32;  // most zones a warp takes
 
 vx_status afail(vx_status s, const char *fmt, ...) {
     char buf[512];
@@ -92,6 +92,7 @@ struct AbsLaunch {
     const double *state;
     double *j0, *chi0, *j1, *chi1, *jac;
     int *flag;
+    int zpw;  // zones per warp, at most kZoneSlots
 };
 
 __device__ __forceinline__ float ex2f(float x) {
@@ -158,7 +159,7 @@ __device__ __forceinline__ void occupation(double x, double &f, double &omf) {
 
 template <bool F64, bool ADJ>
 __global__ void __launch_bounds__(kAbsBlock) k_abs(const __grid_constant__ AbsLaunch L) {
-    // Each warp takes 32 consecutive zones at a time, with no CTA barrier: lane l forms zone l's
+    // Each warp takes zpw consecutive zones, with no CTA barrier: lane l forms zone l's
     // scalars in the warp's shared slots (the FP64 set-up with every lane busy), then the warp runs
     // through the group's entries (zone, species, bin) 32 at a time, staging their Jacobian rows in
     // its own slice of shared memory (row stride 13: banks) and storing them as one contiguous run.
@@ -178,9 +179,9 @@ __global__ void __launch_bounds__(kAbsBlock) k_abs(const __grid_constant__ AbsLa
     // entry q = lane of a group as (zone slot k0, species s0, bin i0), and the step of 32 entries
     const int k0 = lane / SN, s0 = (lane - k0 * SN) / C.N, i0 = lane - k0 * SN - s0 * C.N;
     const int dk = 32 / SN, dsi = 32 - dk * SN, ds = dsi / C.N, di = dsi - ds * C.N;
-    for (long long zg = ((long long)blockIdx.x * kAbsWarps + warp) * kZoneSlots; zg < L.Z;
-         zg += (long long)gridDim.x * kAbsWarps * kZoneSlots) {
-        const int nz = (int)min((long long)kZoneSlots, L.Z - zg);
+    for (long long zg = ((long long)blockIdx.x * kAbsWarps + warp) * L.zpw; zg < L.Z;
+         zg += (long long)gridDim.x * kAbsWarps * L.zpw) {
+        const int nz = (int)min((long long)L.zpw, L.Z - zg);
         if (lane < nz) {
             const int kk = lane;
             const double *st = L.state + 4 * (zg + kk);
@@ -320,15 +321,10 @@ __global__ void __launch_bounds__(kAbsBlock) k_abs(const __grid_constant__ AbsLa
     }
 }
 
-template <bool F64>
-const void *abs_kernel(bool adj) {
-    return adj ? (const void *)k_abs<F64, true> : (const void *)k_abs<F64, false>;
-}
-
 }  // namespace
 
 struct vx_abs {
-    int device = 0, grid = 0;
+    int device = 0, nsm = 1;
     int prec = VX_PREC_MIXED;
     AbsConst c{};
     int *d_flag = nullptr;
@@ -370,8 +366,13 @@ vx_status abs_run(vx_abs *h, const vx_batch *b, const vx_out *out, double *jac, 
     if (out) { L.j0 = out->j0; L.chi0 = out->chi0; L.j1 = out->j1; L.chi1 = out->chi1; }
     L.jac = jac;
     L.flag = h->d_flag;
-    const long long blocks = (b->n_zones + kAbsWarps * kZoneSlots - 1) / (kAbsWarps * kZoneSlots);  // 32 zones per warp
-    const int grid = (int)std::min<long long>(h->grid, blocks);
+    // One group of zones per warp, up to 32 zones, such that there are kAbsFill CTAs per SM: a grid that just
+    // fills the chip left its last third idle while the rest took a second group, and one ray ran on two CTAs.
+    // GB300, rates and Jacobian: 204,800 zones 347 us at 4 CTAs per SM, 326 at 16, 324 at 32, 360 at 64.
+    const long long fill = (long long)h->nsm * kAbsWarps * kAbsFill;
+    L.zpw = (int)std::min<long long>(kZoneSlots, std::max<long long>(1, b->n_zones / fill));
+    const long long per = (long long)kAbsWarps * L.zpw;
+    const int grid = (int)std::min<long long>(1 << 30, (b->n_zones + per - 1) / per);
     const bool f64 = h->prec == VX_PREC_FP64, adj = jac != nullptr;
     if (f64) adj ? k_abs<true, true><<<grid, kAbsBlock, 0, s>>>(L) : k_abs<true, false><<<grid, kAbsBlock, 0, s>>>(L);
     else adj ? k_abs<false, true><<<grid, kAbsBlock, 0, s>>>(L) : k_abs<false, false><<<grid, kAbsBlock, 0, s>>>(L);
@@ -428,10 +429,7 @@ vx_status vx_abs_create(const vx_config *cfg, vx_abs **out) {
         delete h;
         return afail(VX_ERR_CUDA, "no CUDA device");
     }
-    int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, abs_kernel<false>(true), kAbsBlock, 0) != cudaSuccess || occ < 1)
-        occ = 1;
-    h->grid = occ * prop.multiProcessorCount;
+    h->nsm = prop.multiProcessorCount;
     if (cudaMalloc(&h->d_flag, sizeof(int)) != cudaSuccess || cudaMemset(h->d_flag, 0, sizeof(int)) != cudaSuccess) {
         vx_abs_destroy(h);
         return afail(VX_ERR_OOM, "allocation failed");
