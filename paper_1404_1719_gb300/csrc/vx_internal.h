@@ -13,7 +13,7 @@
 #define VX_MAX_BINS 32
 #define VX_MAX_PAIRS (VX_MAX_BINS * (VX_MAX_BINS + 1) / 2)
 #define VX_MAX_SPECIES 3
-#define VX_TPB_MAX 512    // FP64 kernel: threads per CTA (bin pairs)
+#define VX_TPB_FP64 256   // FP64 kernel: threads per CTA
 #define VX_TPB_MIXED 256  // mixed kernels: largest CTA the register budgets are compiled for
 // Threads per CTA of the mixed kernels (at most VX_TPB_MIXED): the (pair, omega) units of a zone
 // are shared among them. 128 threads with 4 to 6 CTAs per SM let the other CTAs' quadrature
@@ -45,13 +45,12 @@ struct Nodes32 {
 };
 
 struct Nodes64 {
-    double u[VX_MAX_NE], v[VX_MAX_NE], cp[VX_MAX_NE], cm[VX_MAX_NE], c0[VX_MAX_NE];
+    double tau[VX_MAX_NE], cp[VX_MAX_NE], cm[VX_MAX_NE], c0[VX_MAX_NE];
 };
 
 // Per-handle constants.
 struct Common {
     int N, n_mu, n_e, npair, S;
-    int ms;                        // m-chunks per bin pair (threads per pair)
     int species[VX_MAX_SPECIES];
     int partner[VX_MAX_SPECIES];   // index (in species order) of the partner spectrum
     float bI[VX_MAX_SPECIES], bII[VX_MAX_SPECIES];
@@ -73,7 +72,7 @@ struct Launch {
     Nodes32 n32;
     const float4 *tab32;           // [npair][n_mu][2] float4 (mixed form): {|q|/2, E-} as FP32
                                    //   value + remainder; {kp, km, k0, cos(omega_m)}
-    const double *tab64;           // [n_mu][npair][5] (FP64 form)
+    const double *tab64;           // [npair][n_mu][5] (FP64 form)
     long long Z;
     const int *off;                // device ray offsets [n_rays + 1] or NULL (checked, not used)
     int n_rays;
@@ -89,7 +88,8 @@ struct Launch {
 struct Launch64 {
     Common c;
     Nodes64 n64;
-    const double *tab64;
+    const double *tab64;           // [npair][n_mu][5]: |q|/2, E-, kp, km, k0
+    const double *exptab;          // 2^{j / 4096}
     long long Z;
     const int *off;
     int n_rays;
@@ -126,6 +126,7 @@ __host__ __device__ inline size_t smem_mixed_bytes(int N, int S, bool adj, int b
     return f * 4 + 3 * (size_t)N * 8 + 64 * 8 + (size_t)block * 2 * nq * (prec ? 8 : 4) * 4;
 }
 size_t smem_fp64(const Common &c);
+#define VX_EXPTAB 4096  // entries of Launch64::exptab
 
 // Kernel launchers (return the launch error). n_e selects the unrolled instantiation, split the
 // instantiations with the split rule and prec those of the precise mode (launch_mixed reads both
@@ -134,7 +135,7 @@ size_t smem_fp64(const Common &c);
 const void *kernel_mixed(bool adj, int minb, int n_e, bool split, bool prec);
 cudaError_t launch_mixed(bool adj, int minb, const Launch &L, int grid, int block, size_t smem, cudaStream_t s);
 cudaError_t launch_fp64_fwd(const Launch64 &L, int grid, int block, size_t smem, cudaStream_t s);
-const void *kernel_fp64_fwd(int n_e);
+const void *kernel_fp64_fwd();
 
 #define VX_DECL_MIXED(sfx)                                                                            \
     const void *kernel_mixed_##sfx(int n_e, bool split);                                              \

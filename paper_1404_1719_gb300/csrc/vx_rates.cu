@@ -106,11 +106,11 @@ struct vx_rates {
     vx::Nodes32 n32{};
     vx::Nodes64 n64{};
     float4 *d_tab32 = nullptr;
-    double *d_tab64 = nullptr;
+    double *d_tab64 = nullptr, *d_exp = nullptr;
     unsigned long long *d_counter = nullptr;
     int *d_flag = nullptr;
-    // launch shapes: one thread per bin pair; mixed kernels in two register budgets
-    int ms = 1, block = 32, block_mixed = 32;
+    // launch shapes (mixed kernels in two register budgets)
+    int block = 32, block_mixed = 32;
     int grid_mixed[2][2] = {{0, 0}, {0, 0}};  // [forward, tangents][larger, smaller register budget]
     int minb[2] = {2, 3};                      // chosen budget per kind (autotuned with VX_AUTOTUNE)
     bool tuned[2] = {false, false};
@@ -267,7 +267,7 @@ vx_status vx_rates_create(const vx_config *cfg, vx_rates **out) {
     }
     for (int k = 0; k < ne; ++k) {
         double u = 1.0 + tk[k], v = 1.0 - tk[k];
-        h->n64.u[k] = u; h->n64.v[k] = v;
+        h->n64.tau[k] = tk[k];
         h->n64.cp[k] = wk[k] * u * u; h->n64.cm[k] = wk[k] * v * v; h->n64.c0[k] = wk[k] * u * v;
         h->n32.u[k] = (float)u; h->n32.v[k] = (float)v;
         h->n32.cp[k] = (float)h->n64.cp[k]; h->n32.cm[k] = (float)h->n64.cm[k]; h->n32.c0[k] = (float)h->n64.c0[k];
@@ -286,8 +286,7 @@ vx_status vx_rates_create(const vx_config *cfg, vx_rates **out) {
             h->n32.hw[k] = (float)wh[k];
         }
     }
-    // per (unordered pair p, omega node m) tables: FP32 records pair-major (a thread's consecutive
-    // units are adjacent), FP64 records omega-major
+    // per (unordered pair p, omega node m) tables, pair-major (a thread's consecutive units are adjacent)
     const int np = C.npair;
     std::vector<float4> t32((size_t)nmu * np * 2);
     std::vector<double> t64((size_t)nmu * np * 5);
@@ -311,17 +310,15 @@ vx_status vx_rates_create(const vx_config *cfg, vx_rates **out) {
             const float fh = (float)hh, fEm = (float)Em;
             r[0] = make_float4(fh, (float)(hh - fh), fEm, (float)(Em - fEm));
             r[1] = make_float4((float)kp, (float)km, (float)k0, C.t_hi[m]);
-            double *r64 = &t64[((size_t)m * np + p) * 5];
+            double *r64 = &t64[((size_t)p * nmu + m) * 5];
             r64[0] = hh; r64[1] = Em; r64[2] = kp; r64[3] = km; r64[4] = k0;
         }
     }
     C.h_max = hmax;
     C.q0h_max = q0hmax;
 
-    // launch shape: one thread per unordered bin pair
-    C.ms = 1;
-    h->ms = 1;
-    h->block = round_up(np, 32);                           // FP64 kernel (<= 496 pairs)
+    // launch shapes: the (pair, omega) units of a zone are shared among a CTA's threads
+    h->block = std::min(round_up(np * nmu, 32), VX_TPB_FP64);
     h->block_mixed = std::min(round_up(np * nmu, 32), VX_BLOCK_MIXED);  // (pair, omega) units
 
     auto cleanup = [&](vx_status s) { vx_rates_destroy(h); return s; };
@@ -348,6 +345,12 @@ vx_status vx_rates_create(const vx_config *cfg, vx_rates **out) {
     VX_CUC(cudaMemcpy(h->d_tab32, t32.data(), t32.size() * sizeof(float4), cudaMemcpyHostToDevice));
     VX_CUC(cudaMemcpy(h->d_tab64, t64.data(), t64.size() * sizeof(double), cudaMemcpyHostToDevice));
     VX_CUC(cudaMemset(h->d_flag, 0, sizeof(int)));
+    if (cfg->prec == VX_PREC_FP64) {
+        std::vector<double> ex(VX_EXPTAB);
+        for (int j = 0; j < VX_EXPTAB; ++j) ex[j] = std::exp2((double)j / VX_EXPTAB);
+        VX_CUC(cudaMalloc(&h->d_exp, ex.size() * sizeof(double)));
+        VX_CUC(cudaMemcpy(h->d_exp, ex.data(), ex.size() * sizeof(double), cudaMemcpyHostToDevice));
+    }
 
     h->smem_fwd = vx::smem_mixed_bytes(N, S, false, h->block_mixed, C.precise != 0);
     h->smem_adj = vx::smem_mixed_bytes(N, S, true, h->block_mixed, C.precise != 0);
@@ -360,7 +363,7 @@ vx_status vx_rates_create(const vx_config *cfg, vx_rates **out) {
                {vx::kernel_mixed(false, 3, ne, sp, pr), h->smem_fwd, &h->grid_mixed[0][1], h->block_mixed},
                {vx::kernel_mixed(true, 2, ne, sp, pr), h->smem_adj, &h->grid_mixed[1][0], h->block_mixed},
                {vx::kernel_mixed(true, 3, ne, sp, pr), h->smem_adj, &h->grid_mixed[1][1], h->block_mixed},
-               {vx::kernel_fp64_fwd(ne), h->smem_64, &h->grid_64, h->block}};
+               {vx::kernel_fp64_fwd(), h->smem_64, &h->grid_64, h->block}};
     for (K &k : ks) {
         // opt in to the dynamic size always: the 48 KB default bounds static + dynamic together
         VX_CUC(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem));
@@ -621,6 +624,7 @@ vx_status vx_rates_eval(vx_rates *h, const vx_batch *b, const vx_out *out, vx_st
         L.c = h->common;
         L.n64 = h->n64;
         L.tab64 = h->d_tab64;
+        L.exptab = h->d_exp;
         L.Z = b->n_zones;
         L.off = b->ray_offsets;
         L.n_rays = b->n_rays;
@@ -629,7 +633,7 @@ vx_status vx_rates_eval(vx_rates *h, const vx_batch *b, const vx_out *out, vx_st
         L.counter = h->d_counter;
         L.flag = h->d_flag;
         int grid = (int)std::min<long long>(h->grid_64, b->n_zones);
-        if (graph) return launch_graph(h, 2, vx::kernel_fp64_fwd(h->common.n_e), &L, grid, h->block, h->smem_64, s);
+        if (graph) return launch_graph(h, 2, vx::kernel_fp64_fwd(), &L, grid, h->block, h->smem_64, s);
         VX_CU(cudaMemsetAsync(h->d_counter, 0, sizeof(unsigned long long), s));
         VX_CU(vx::launch_fp64_fwd(L, grid, h->block, h->smem_64, s));
     }
@@ -891,6 +895,7 @@ void vx_rates_destroy(vx_rates *h) {
         if (g) cudaGraphExecDestroy(g);
     cudaFree(h->d_tab32);
     cudaFree(h->d_tab64);
+    cudaFree(h->d_exp);
     cudaFree(h->d_counter);
     cudaFree(h->d_flag);
     for (int k = 0; k < 2; ++k) {
@@ -968,7 +973,6 @@ static void noalloc_params(const vx_config *cfg, vx::Launch &L, NoallocTab &T) {
     memset(&T, 0, sizeof T);
     C.N = N; C.n_mu = nmu; C.n_e = ne; C.S = S;
     C.npair = N * (N + 1) / 2;
-    C.ms = 1;
     C.g2 = cfg->g2; C.norm = cfg->norm; C.eta_sw = cfg->eta_fp64 == 0.0 ? 20.0 : cfg->eta_fp64;
     const double *eps = cfg->eps;
     for (int i = 0; i < N; ++i) {
