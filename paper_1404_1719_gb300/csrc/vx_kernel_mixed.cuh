@@ -914,8 +914,10 @@ __global__ void __launch_bounds__(MINB == 3 ? (ADJ ? VX_LB3_THREADS_ADJ : VX_TPB
 
     validate_offsets(L.off, L.n_rays, L.Z, L.flag);
 
-    // Thread 0 reserves the next zone one iteration ahead and prefetches its inputs into L2 while
-    // the current zone's quadrature runs, so a zone starts without an atomic or DRAM round trip.
+    // Thread 0 reserves the next zone and prefetches its inputs into L2 while the current zone is
+    // contracted, so a zone starts without an atomic or DRAM round trip. (Reserved before the quadrature, as
+    // it once was, a CTA held two zones: with no more zones than CTAs, half of the CTAs had none. GB300, 400
+    // zones forward + tangents 392 -> 208 us, 6,800 zones of the 16 x 48 split rule, forward and backward, 3.84 -> 3.70 ms.)
     long long next_z = 0;
     if (tid == 0) next_z = (long long)atomicAdd(L.counter, 1ull);
     const int t_aux = blockDim.x > 32 ? 32 : 1;  // a thread of another warp for the set-up
@@ -925,7 +927,6 @@ __global__ void __launch_bounds__(MINB == 3 ? (ADJ ? VX_LB3_THREADS_ADJ : VX_TPB
         __syncthreads();
         const long long z = s_zone;
         if (z >= L.Z) break;
-        if (tid == 0) next_z = (long long)atomicAdd(L.counter, 1ull);
 
         // ---- zone set-up (FP64): the main scalars on thread 0, exponentials and 1/T^2 in parallel
         if (tid == t_aux) {
@@ -1004,7 +1005,10 @@ __global__ void __launch_bounds__(MINB == 3 ? (ADJ ? VX_LB3_THREADS_ADJ : VX_TPB
                     L.grad_J[(size_t)z * S * N + e] = nan;
                     L.grad_H[(size_t)z * S * N + e] = nan;
                 }
-            if (tid == 0) atomicOr(L.flag, VX_FLAG_BAD_STATE);
+            if (tid == 0) {
+                atomicOr(L.flag, VX_FLAG_BAD_STATE);
+                next_z = (long long)atomicAdd(L.counter, 1ull);
+            }
             __syncthreads();
             continue;
         }
@@ -1028,15 +1032,6 @@ __global__ void __launch_bounds__(MINB == 3 ? (ADJ ? VX_LB3_THREADS_ADJ : VX_TPB
             else if (o == 2) v = C.w[j] * L.H[a] * shv[j];
             else v = C.w[j] * (o == 1 ? L.J[a] : L.H[a]);
             vec[e] = (float)v;
-        }
-
-        if (tid == 0 && next_z < L.Z) {
-            prefetch_l2(L.state + 4 * next_z);
-            const size_t off = (size_t)next_z * S * N;
-            for (int b = 0; b < S * N; b += 16) {
-                prefetch_l2(L.J + off + b);
-                prefetch_l2(L.H + off + b);
-            }
         }
 
         // ---- quadrature: the npair * n_mu (pair, omega) units in equal contiguous ranges --------
@@ -1192,6 +1187,18 @@ __global__ void __launch_bounds__(MINB == 3 ? (ADJ ? VX_LB3_THREADS_ADJ : VX_TPB
             }
         }
         __syncthreads();
+
+        if (tid == 0) {
+            next_z = (long long)atomicAdd(L.counter, 1ull);
+            if (next_z < L.Z) {
+                prefetch_l2(L.state + 4 * next_z);
+                const size_t off = (size_t)next_z * S * N;
+                for (int b = 0; b < S * N; b += 16) {
+                    prefetch_l2(L.J + off + b);
+                    prefetch_l2(L.H + off + b);
+                }
+            }
+        }
 
         // ---- contraction (and tangents) --------------------------------------------------------
         const double two_pi = 6.283185307179586;
