@@ -40,6 +40,7 @@ namespace {
 constexpr int kNesMaxP = 32;     // nodes per panel
 constexpr int kNesMaxMu = 32;
 constexpr int kNesBlock = 128;
+
 constexpr double kTail = 30.0;   // depth of the lower panel below the lower Fermi edge, in T
 
 vx_status nfail(vx_status s, const char *fmt, ...) {
@@ -449,13 +450,15 @@ __device__ __forceinline__ void nes_unit_x2(const NesGl<float> *gl, const NesLg<
 }
 
 
-// Minimum CTAs per SM the register allocation is bounded for (1: no bound).
+// Minimum CTAs of kNesBlock threads per SM the register allocation is bounded for.
 #ifndef VX_NES_MINB
 #define VX_NES_MINB 1
 #endif
 
-template <typename R, bool ADJ, int NP>
-__global__ void __launch_bounds__(kNesBlock, VX_NES_MINB) k_nes(const __grid_constant__ NesLaunch<R> L) {
+// BLK threads: kNesBlock, or more for batches of few zones (nes_block): a zone's bin pairs are dealt to the
+// CTA's warps, and the sums of a pair stay within its group of lanes, so the results do not depend on it.
+template <typename R, bool ADJ, int NP, int BLK>
+__global__ void __launch_bounds__(BLK, std::is_same<R, float>::value && BLK == kNesBlock ? VX_NES_MINB : 1) k_nes(const __grid_constant__ NesLaunch<R> L) {
     extern __shared__ __align__(16) unsigned char smraw[];
     __shared__ NesZone zs;
     __shared__ long long s_zone;
@@ -503,12 +506,23 @@ __global__ void __launch_bounds__(kNesBlock, VX_NES_MINB) k_nes(const __grid_con
                     zr[4] = (R)zs.scale;
                     zr[5] = (R)(etas * 1.4426950408889634);
                     zs.iT2 = 1.0 / (T * T);
-                    for (int k = 0; k < C.n_p; ++k) {  // the Laguerre panel's zone factors
-                        slg[k].wT = (R)(T * C.lw[k]);
-                        slg[k].og = (R)(zs.scale * C.lg[k]);
-                    }
+                    if (BLK == kNesBlock)
+                        for (int k = 0; k < C.n_p; ++k) {  // the Laguerre panel's zone factors
+                            slg[k].wT = (R)(T * C.lw[k]);
+                            slg[k].og = (R)(zs.scale * C.lg[k]);
+                        }
                 }
             }
+        }
+        // (with few zones nothing hides that loop: the first warp's lanes share it. With five CTAs on an SM the
+        // others do, and the serial form's registers, 96, are what lets five in)
+        if (BLK > kNesBlock && warp == 0) {
+            __syncwarp();
+            if (s_zone < L.Z && !zs.bad)
+                for (int k = lane; k < C.n_p; k += 32) {
+                    slg[k].wT = (R)(zs.T * C.lw[k]);
+                    slg[k].og = (R)(zs.scale * C.lg[k]);
+                }
         }
         __syncthreads();
         const long long z = s_zone;
@@ -631,21 +645,32 @@ __global__ void __launch_bounds__(kNesBlock, VX_NES_MINB) k_nes(const __grid_con
     }
 }
 
-template <typename R, bool ADJ>
+// Threads per CTA for a batch of Z zones: four times kNesBlock up to two zones per SM, twice up to three and a
+// half, where CTAs of kNesBlock leave the SMs' issue slots idle (the slowest zone's latency sets the time).
+// GB300, 21 bins, 16 x 48, rates and Jacobian, us at 128 / 256 / 512 threads: 152 zones 70 / 50 / 44,
+// 304 zones 89 / 76 / 74, 400 zones 116 / 94 / 104, 500 zones 135 / 126 / 134, 608 zones 148 / 153 / 142,
+// 760 zones 168 / 158 / 175, 1000 zones 212 / 215 / 233. The FP64 form gains nothing (its pipe is full).
+template <typename R>
+int nes_block(long long Z, int nsm) {
+    if (!std::is_same<R, float>::value) return kNesBlock;
+    return Z <= 2ll * nsm ? 4 * kNesBlock : 2 * Z <= 7ll * nsm ? 2 * kNesBlock : kNesBlock;
+}
+
+template <typename R, bool ADJ, int BLK>
 const void *nes_kernel(int n_p) {
     switch (n_p) {
-        case 8: return (const void *)k_nes<R, ADJ, 8>;
-        case 16: return (const void *)k_nes<R, ADJ, 16>;
-        default: return (const void *)k_nes<R, ADJ, 0>;
+        case 8: return (const void *)k_nes<R, ADJ, 8, BLK>;
+        case 16: return (const void *)k_nes<R, ADJ, 16, BLK>;
+        default: return (const void *)k_nes<R, ADJ, 0, BLK>;
     }
 }
 
-template <typename R, bool ADJ>
+template <typename R, bool ADJ, int BLK>
 cudaError_t nes_launch(const NesLaunch<R> &L, int grid, size_t smem, cudaStream_t s) {
     switch (L.c.n_p) {
-        case 8: k_nes<R, ADJ, 8><<<grid, kNesBlock, smem, s>>>(L); break;
-        case 16: k_nes<R, ADJ, 16><<<grid, kNesBlock, smem, s>>>(L); break;
-        default: k_nes<R, ADJ, 0><<<grid, kNesBlock, smem, s>>>(L); break;
+        case 8: k_nes<R, ADJ, 8, BLK><<<grid, BLK, smem, s>>>(L); break;
+        case 16: k_nes<R, ADJ, 16, BLK><<<grid, BLK, smem, s>>>(L); break;
+        default: k_nes<R, ADJ, 0, BLK><<<grid, BLK, smem, s>>>(L); break;
     }
     return cudaGetLastError();
 }
@@ -856,7 +881,18 @@ vx_status nes_run(vx_nes *h, const vx_batch *b, const vx_out *out, double *jac, 
     const bool adj = jac != nullptr;
     const int grid = (int)std::min<long long>(h->grid[adj], b->n_zones);
     NES_CU(cudaMemsetAsync(L.counter, 0, sizeof(unsigned long long), s));
-    const cudaError_t e = adj ? vx::nes_launch<R, true>(L, grid, h->smem[1], s) : vx::nes_launch<R, false>(L, grid, h->smem[0], s);
+    const int blk = vx::nes_block<R>(b->n_zones, h->nsm);
+    cudaError_t e;
+    if constexpr (std::is_same<R, float>::value) {
+        if (blk == 4 * kNesBlock)
+            e = adj ? vx::nes_launch<R, true, 4 * kNesBlock>(L, grid, h->smem[1], s) : vx::nes_launch<R, false, 4 * kNesBlock>(L, grid, h->smem[0], s);
+        else if (blk == 2 * kNesBlock)
+            e = adj ? vx::nes_launch<R, true, 2 * kNesBlock>(L, grid, h->smem[1], s) : vx::nes_launch<R, false, 2 * kNesBlock>(L, grid, h->smem[0], s);
+        else
+            e = adj ? vx::nes_launch<R, true, kNesBlock>(L, grid, h->smem[1], s) : vx::nes_launch<R, false, kNesBlock>(L, grid, h->smem[0], s);
+    } else {
+        e = adj ? vx::nes_launch<R, true, kNesBlock>(L, grid, h->smem[1], s) : vx::nes_launch<R, false, kNesBlock>(L, grid, h->smem[0], s);
+    }
     NES_CU(e);
     return VX_OK;
 }
@@ -1052,10 +1088,14 @@ vx_status vx_nes_create(const vx_config *cfg, vx_nes **out) {
         return cleanup(nfail(VX_ERR_OOM, "allocation failed"));
     for (int adj = 0; adj < 2; ++adj) {
         h->smem[adj] = nes_smem(C, adj != 0, dbl);
-        const void *fn = dbl ? (adj ? vx::nes_kernel<double, true>(C.n_p) : vx::nes_kernel<double, false>(C.n_p))
-                             : (adj ? vx::nes_kernel<float, true>(C.n_p) : vx::nes_kernel<float, false>(C.n_p));
-        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->smem[adj]) != cudaSuccess)
-            return cleanup(nfail(VX_ERR_CUDA, "shared memory attribute"));
+        constexpr int B1 = kNesBlock, B2 = 2 * B1, B4 = 4 * B1;
+        const void *fn = dbl ? (adj ? vx::nes_kernel<double, true, B1>(C.n_p) : vx::nes_kernel<double, false, B1>(C.n_p))
+                             : (adj ? vx::nes_kernel<float, true, B1>(C.n_p) : vx::nes_kernel<float, false, B1>(C.n_p));
+        const void *wide[2] = {adj ? vx::nes_kernel<float, true, B2>(C.n_p) : vx::nes_kernel<float, false, B2>(C.n_p),
+                               adj ? vx::nes_kernel<float, true, B4>(C.n_p) : vx::nes_kernel<float, false, B4>(C.n_p)};
+        for (const void *f : {fn, wide[0], wide[1]})
+            if (!(dbl && f != fn) && cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)h->smem[adj]) != cudaSuccess)
+                return cleanup(nfail(VX_ERR_CUDA, "shared memory attribute"));
         int occ = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, kNesBlock, h->smem[adj]) != cudaSuccess || occ < 1)
             return cleanup(nfail(VX_ERR_UNSUPPORTED, "NES kernel does not fit on an SM"));
