@@ -233,6 +233,7 @@ __global__ void __launch_bounds__(kTpb64) k_pair_fp64(const __grid_constant__ La
             if (ta == tb) continue;
             double s[4] = {0, 0, 0, 0};
             for (int t = ta; t <= tb; ++t) {
+                if (U < TB && t * U / TB == (t + 1) * U / TB) continue;  // fewer units than threads: an empty range
                 const int sl = t == ta && ua > (long long)t * U / TB ? 1 : 0;
                 for (int c = 0; c < 4; ++c) s[c] += part[(sl * 4 + c) * TB + t];
             }

@@ -1169,6 +1169,7 @@ __global__ void __launch_bounds__(MINB == 3 ? (ADJ ? VX_LB3_THREADS_ADJ : VX_TPB
                 Proj acc;
                 acc.zero();
                 for (int t = ta; t <= tb; ++t) {
+                    if (U < TB && t * U / TB == (t + 1) * U / TB) continue;  // fewer units than threads: an empty range
                     const int sl = (t == ta && ua > t * U / TB) ? 1 : 0;
                     const Proj x = part_get<PREC>(part, TB, t, sl * nq + q);
                     if (PREC) {
