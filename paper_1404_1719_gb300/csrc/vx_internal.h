@@ -22,6 +22,7 @@
 #ifndef VX_BLOCK_MIXED
 #define VX_BLOCK_MIXED 128
 #endif
+#define VX_RED (4 * VX_MAX_BINS)  // doubles of the mixed kernels' reduction buffer
 #define VX_ETA_MAX 80.0
 
 // device numeric flag bits
@@ -100,6 +101,16 @@ struct Launch64 {
 };
 
 #ifdef __CUDACC__
+// FP32 to FP64, exactly, in integer operations for zero and normal numbers (the conversion instruction runs on the
+// FP64 pipe, at 2 per clock and SM on GB300); the rest by the conversion itself.
+static __device__ __noinline__ double widen_rest(float x) { return (double)x; }
+__device__ __forceinline__ double widen(float x) {
+    const unsigned u = __float_as_uint(x), e = u & 0x7fffffffu;
+    if (e - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)((u & 0x80000000u) | ((e >> 3) + (896u << 20))), (int)(u << 29));
+    return e == 0u ? __hiloint2double((int)u, 0) : widen_rest(x);
+}
+
 // Block 0 of a launch checks that the ray offsets partition the Z zones (off[0] = 0, no decrease,
 // off[n_rays] = Z) and raises VX_FLAG_BAD_OFFSETS if not. The rate of a zone does not depend on
 // its ray, so nothing else reads the offsets.
@@ -116,14 +127,14 @@ __device__ inline void validate_offsets(const int *off, int n_rays, long long Z,
 //   mats[q][2][N2]: per quantity q (kernel; and with tangents: T of annihilation, T of production,
 //                   eta), l = 0, 1 of Phi_I(i,j) (term II is the transpose)
 //   vec[4][S][N]  : contraction vectors per output (j0, chi0, j1, chi1) and species
-//   sc, em, shv [N] (double): per-bin FP64 factors;  red[64] (double): block reduction
+//   sc, em, shv [N] (double): per-bin FP64 factors;  red[VX_RED] (double): block reduction, spectral blocks
 //   part[2][q][4 or 8][block]: partial projections of bin pairs split between two threads (the
 //                   precise mode keeps the low parts of its double-float sums as well)
 __host__ __device__ inline size_t smem_mixed_bytes(int N, int S, bool adj, int block, bool prec = false) {
     size_t nq = adj ? 4 : 1;
     size_t f = nq * 2 * (size_t)N * N + 4 * (size_t)S * N;
     f = (f + 1) & ~(size_t)1;
-    return f * 4 + 3 * (size_t)N * 8 + 64 * 8 + (size_t)block * 2 * nq * (prec ? 8 : 4) * 4;
+    return f * 4 + 3 * (size_t)N * 8 + VX_RED * 8 + (size_t)block * 2 * nq * (prec ? 8 : 4) * 4;
 }
 size_t smem_fp64(const Common &c);
 #define VX_EXPTAB 4096  // entries of Launch64::exptab

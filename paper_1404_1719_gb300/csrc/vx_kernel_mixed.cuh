@@ -883,8 +883,8 @@ __global__ void __launch_bounds__(MINB == 3 ? (ADJ ? VX_LB3_THREADS_ADJ : VX_TPB
     double *sc = reinterpret_cast<double *>(smraw + foff * 4);
     double *em = sc + N;
     double *shv = em + N;  // exp(-(eps_j - eps_0)/T) 2^sv
-    double *red = shv + N;  // 64 doubles for block reductions
-    float *part = reinterpret_cast<float *>(red + 64);  // [2 slots][nq][4 or 8][blockDim] partial projections
+    double *red = shv + N;  // block reductions; factors of the spectral blocks
+    float *part = reinterpret_cast<float *>(red + VX_RED);  // [2 slots][nq][4 or 8][blockDim] partial projections
     const int tid = threadIdx.x;
     for (int k = tid; k < C.n_e; k += blockDim.x) {
         s_nodes[k].a = make_float4(L.n32.u[k], L.n32.v[k], L.n32.cp[k], L.n32.cm[k]);
@@ -1278,16 +1278,33 @@ __global__ void __launch_bounds__(MINB == 3 ? (ADJ ? VX_LB3_THREADS_ADJ : VX_TPB
         }
         if (!ADJ && L.blocks) {
             // d(rates)/d(partner spectrum): the coefficients of (1 - J), J, H, H in the contraction
-            // above, scaled in FP64 (production carries e^{-(eps_i + eps_j)/T} = sc[i] shv[j])
-            const int nb = 4 * N2;
-            for (int e = tid; e < S * nb; e += blockDim.x) {
-                const int s = e / nb, o = (e / N2) & 3, i = (e / N) % N, j = e % N;
-                const float *M = mats + (size_t)(o >> 1) * N2;
-                const double k = PREC ? kern2(C.bI[s], M[i * N + j], C.bII[s], M[j * N + i])
-                                      : (double)fmaf(C.bI[s], M[i * N + j], C.bII[s] * M[j * N + i]);
-                double f = ((o >> 1) ? c1 : c0) * C.w[j];
-                if ((o & 1) == 0) f *= (o == 0 ? -sc[i] : sc[i]) * shv[j];
-                L.blocks[(size_t)z * S * nb + e] = f * k;
+            // above, scaled in FP64 (production carries e^{-(eps_i + eps_j)/T} = sc[i] shv[j]). An element's two
+            // outputs per species and l share their kernel value and its conversion, and the factors
+            // that depend on j alone are formed once per zone: 1.5 FP64 operations per output instead of 4 to 5
+            // (GB300, 12,800 zones with the rates: 2.60 -> 2.36 ms).
+            double *gj = red;  // [l][annihilation, production][N]; the block reduction's slots are free here
+            __syncthreads();
+            for (int e = tid; e < 4 * N; e += blockDim.x) {
+                const int l = e / (2 * N), d = (e / N) & 1, j = e % N;
+                const double f = (l ? c1 : c0) * C.w[j];
+                gj[e] = d ? (l ? f : -f) * shv[j] : f;
+            }
+            __syncthreads();
+            double *B = L.blocks + (size_t)z * S * 4 * N2;
+            for (int ij = tid; ij < N2; ij += blockDim.x) {
+                const int i = ij / N, j = ij - i * N, ji = j * N + i;
+                const double si = sc[i];
+#pragma unroll
+                for (int l = 0; l < 2; ++l) {
+                    const float a = mats[l * N2 + ij], b = mats[l * N2 + ji];
+                    const double ga = gj[2 * l * N + j], gp = gj[(2 * l + 1) * N + j] * si;
+                    for (int s = 0; s < S; ++s) {
+                        const double k = PREC ? kern2(C.bI[s], a, C.bII[s], b) : widen(fmaf(C.bI[s], a, C.bII[s] * b));
+                        double *o = B + (size_t)(4 * s + 2 * l) * N2 + ij;
+                        __stcs(o, gp * k);
+                        __stcs(o + N2, ga * k);
+                    }
+                }
             }
         }
         if (!ADJ && L.grad_J) {
