@@ -72,14 +72,15 @@ vx_status device_array(const void *p, size_t align, const char *name) {
     } while (0)
 
 struct BtdArgs {
-    int m, ld, mp, nbuf, nring, n_rays;  // ld: row stride of the FP32 blocks; mp: m rounded up to 8
+    int m, ld, mp, nbuf, nring, halves, n_rays;  // ld: row stride of the FP32 blocks; mp: m rounded up to 8;
+                                                // halves: CTAs per ray (1 or 2)
     long long n_zones;
     const int *off;
     const double *A, *B, *C, *d, *rhs;
     double *x, *r;
     float *Di, *Gt, *At, *y;  // per zone B_k, then D_k^{-1}; C_k, then G_k; A_k in FP32, row-major [m][ld]; y_k [m]
     unsigned short *nz;       // [Z][C, A][mp] zero patterns of the rows
-    int *zbad, *flag;
+    int *zbad, *zmid, *flag;  // at a ray's first zone: a pivot failed; the zone its eliminations meet at, from there
     const int *inval;  // set by k_btd_validate when the offsets are not a partition of the zones
 };
 
@@ -91,9 +92,14 @@ __device__ __forceinline__ bool ray_range(const BtdArgs &a, int ray, long long &
     return true;
 }
 
+// The zone at which a ray's two eliminations meet: its last with one CTA per ray, or few zones.
+__device__ __forceinline__ long long ray_mid(const BtdArgs &a, long long z0, long long z1) {
+    return a.halves == 2 && z1 - z0 >= 4 ? z0 + (z1 - z0) / 2 : z1 - 1;
+}
+
 // offsets[0] = 0, offsets[n_rays] = n_zones and non-decreasing; any violation marks the whole call
 // invalid (so no two rays can share zones) and raises the numeric flag.
-__global__ void k_btd_validate(const int *off, int n_rays, long long n_zones, int *inval, int *flag) {
+__global__ void k_btd_validate(const int *off, int n_rays, long long n_zones, int *inval, int *flag, int *zbad) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i > n_rays) return;
     const long long v = off[i];
@@ -102,6 +108,8 @@ __global__ void k_btd_validate(const int *off, int n_rays, long long n_zones, in
     if (bad) {
         atomicOr(inval, 1);
         atomicOr(flag, 1);
+    } else if (v < n_zones) {
+        zbad[v] = 0;  // the factor kernel's arrival count
     }
 }
 
@@ -567,7 +575,14 @@ __host__ __device__ constexpr size_t factor_smem(int m, int ld, int nbuf) {
            (size_t)m * sizeof(int);
 }
 
-// The factor kernel, one CTA of eight warps per ray, its zones in order. Per zone k:
+// The factor kernel: CTAs of eight warps, one per ray, or two where one would leave SMs without work
+// (a.halves): then one eliminates from the ray's first zone outwards and one from its last zone inwards, D_k =
+// B_k - C_k H_{k+1} with H_k = D_k^{-1} A_k, and whichever comes second to the zone between them (mid) takes
+// that one too, D = B - A G_{mid-1} - C H_{mid+1}: the same arithmetic in half the time. Elimination from
+// the last zone needs what elimination from the first does not (a B of the last zone that can be
+// inverted, say), so if the inner-going half meets a failed pivot, or |H| above kMaxGrowth, the ray goes on from mid
+// to its last zone as if by one CTA, from blocks converted again. One CTA: mid is the last zone.
+// Per zone k, in either direction (below for the outward one):
 //  - D_k = B_k - A_k G_{k-1} on the tensor cores (all three in shared memory);
 //  - D_k is inverted in place by Gauss-Jordan elimination with partial pivoting, eight columns (a panel) at
 //    a time: warp 0 eliminates within a panel in registers, with no barrier between its eight pivots;
@@ -576,12 +591,15 @@ __host__ __device__ constexpr size_t factor_smem(int m, int ld, int nbuf) {
 //    panel. Rows are never moved: pivot j's row is cur[j], and D_k^{-1}[j][cur[q]] = X[cur[j]][q];
 //  - meanwhile C_k, A_{k+1} and (with a fourth buffer) B_{k+1} arrive in shared memory (cp.async);
 //  - G_k = D_k^{-1} C_k on the tensor cores.
-// D_k^{-1}, G_k and the FP32 copy of A_k go to the workspace for the sweeps. The chain of pivots (a warp
+// D_k^{-1} replaces B_k in the workspace and G_k replaces C_k (H_k replaces A_k); the FP32 copy of the other
+// coupling stays, for the sweeps. The chain of pivots (a warp
 // reduction, a shuffle and a reciprocal each) bounds a zone; the warps beside it do everything else.
+// GB300, m = 84, 400 zones: one ray 10.1 -> 5.1 ms with two CTAs.
+constexpr float kMaxGrowth = 64.f;
 template <int NT>
 __global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(const BtdArgs a) {
     extern __shared__ __align__(16) float sm[];
-    __shared__ int s_bad;
+    __shared__ int s_bad, s_grow, s_all;
     const int m = a.m, ld = a.ld, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nw = kFactorThreads / 32, bs = factor_buf(m, ld), P = (m + 7) >> 3;
     const bool four = a.nbuf == 4;
@@ -589,57 +607,142 @@ __global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(c
     // (offsets, not pointers, are exchanged from zone to zone: the compiler then knows the address space)
     int xo = 0, bo = four ? bs : 0;
     float *const sG = sm + bo + bs, *const sA = sG + bs;
-    unsigned short *nzr = reinterpret_cast<unsigned short *>(sm + a.nbuf * bs);  // [C, A][mp]
+    unsigned short *nzr = reinterpret_cast<unsigned short *>(sm + a.nbuf * bs);  // [next coupling, previous coupling][mp]
     float *rowbuf = sm + a.nbuf * bs + a.mp;  // [2][8]
     int *cur = reinterpret_cast<int *>(rowbuf + 16);
     int *pos = cur + 8 * P;
     long long z0, z1;
-    if (!ray_range(a, blockIdx.x, z0, z1) || z1 == z0) return;
-    if (tid == 0) s_bad = 0;
+    const int half = a.halves == 2 ? (int)(blockIdx.x & 1) : 0;
+    if (!ray_range(a, blockIdx.x / a.halves, z0, z1) || z1 == z0) return;
+    long long mid = ray_mid(a, z0, z1);
+    if (half == 1 && mid == z1 - 1) return;
+    if (tid == 0) s_bad = s_grow = 0;
     if (tid < m) pos[tid] = tid;  // in range also where a failed pivot leaves an entry unset
     const int mw = m * ld;
     const int g = lane >> 2, q = lane & 3, wm = warp & 1, wn = warp >> 1;
     // zeros behind every buffer: the last panel's transform, if it has fewer than eight columns, is read that far
     // (and multiplied by zeros, so it must be finite)
     for (int i = tid; i < a.nbuf * (bs - mw); i += kFactorThreads) sm[i / (bs - mw) * bs + mw + i % (bs - mw)] = 0.f;
-    copy_async(sm, a.Di + (size_t)z0 * mw, mw, tid, kFactorThreads);  // B_{z0}
-    copy_wait();
-    __syncthreads();
-    for (long long k = z0; k < z1; ++k) {
-        const bool next = k + 1 < z1;
-        float *const X = sm + xo, *const sB = sm + bo;
-        if (k > z0) {  // D_k = B_k - A_k G_{k-1}
+    auto load = [&](float *dst, const float *src) { copy_async(dst, src, mw, tid, kFactorThreads); };
+    auto load_nz = [&](int to, long long k, int which) {  // the zero pattern of C_k (which 0) or A_k (1)
+        copy_async(reinterpret_cast<float *>(nzr + to * a.mp), reinterpret_cast<const float *>(a.nz + ((size_t)k * 2 + which) * a.mp),
+                   a.mp / 2, tid, kFactorThreads);
+    };
+    auto at = [&](float *w, long long k) { return w + (size_t)k * mw; };
+    // X -= (coupling in sA) (matrix in sG)
+    auto schur = [&](float *X) {
 #pragma unroll 1
-            for (int x = 0; x < NT; ++x) {
-                const int i0 = 16 * (wm * NT + x), i = i0 + (lane & 15);
-                const unsigned nz = __reduce_or_sync(0xffffffffu, i < m ? (unsigned)nzr[a.mp + i] : 0u);
-                float d[NT][4];
-                const int r0 = i0 + g < m ? i0 + g : m - 1, r1 = i0 + g + 8 < m ? i0 + g + 8 : m - 1;
-                product_row<NT>(sA, r0 * ld, r1 * ld, sG, ld, m, wn, lane, nz, d);
-                const bool i0m = i0 + g < m, i1m = i0 + g + 8 < m;
+        for (int x = 0; x < NT; ++x) {
+            const int i0 = 16 * (wm * NT + x), i = i0 + (lane & 15);
+            const unsigned nz = __reduce_or_sync(0xffffffffu, i < m ? (unsigned)nzr[a.mp + i] : 0u);
+            float d[NT][4];
+            const int r0 = i0 + g < m ? i0 + g : m - 1, r1 = i0 + g + 8 < m ? i0 + g + 8 : m - 1;
+            product_row<NT>(sA, r0 * ld, r1 * ld, sG, ld, m, wn, lane, nz, d);
+            const bool i0m = i0 + g < m, i1m = i0 + g + 8 < m;
 #pragma unroll
-                for (int y = 0; y < NT; ++y) {
-                    const int c = 8 * (wn * NT + y) + 2 * q;
-                    float *x0 = X + r0 * ld + c, *x1 = X + r1 * ld + c;
-                    if (c + 1 < m) {
-                        const float2 e0 = *reinterpret_cast<float2 *>(x0), e1 = *reinterpret_cast<float2 *>(x1);
-                        if (i0m) *reinterpret_cast<float2 *>(x0) = make_float2(e0.x - d[y][0], e0.y - d[y][1]);
-                        if (i1m) *reinterpret_cast<float2 *>(x1) = make_float2(e1.x - d[y][2], e1.y - d[y][3]);
-                    } else if (c < m) {
-                        if (i0m) *x0 -= d[y][0];
-                        if (i1m) *x1 -= d[y][2];
-                    }
+            for (int y = 0; y < NT; ++y) {
+                const int c = 8 * (wn * NT + y) + 2 * q;
+                float *x0 = X + r0 * ld + c, *x1 = X + r1 * ld + c;
+                if (c + 1 < m) {
+                    const float2 e0 = *reinterpret_cast<float2 *>(x0), e1 = *reinterpret_cast<float2 *>(x1);
+                    if (i0m) *reinterpret_cast<float2 *>(x0) = make_float2(e0.x - d[y][0], e0.y - d[y][1]);
+                    if (i1m) *reinterpret_cast<float2 *>(x1) = make_float2(e1.x - d[y][2], e1.y - d[y][3]);
+                } else if (c < m) {
+                    if (i0m) *x0 -= d[y][0];
+                    if (i1m) *x1 -= d[y][2];
                 }
             }
-            __syncthreads();
         }
-        if (next) {
-            copy_async(sG, a.Gt + (size_t)k * mw, mw, tid, kFactorThreads);  // C_k
-            copy_async(sA, a.At + (size_t)(k + 1) * mw, mw, tid, kFactorThreads);
-            if (four) copy_async(sB, a.Di + (size_t)(k + 1) * mw, mw, tid, kFactorThreads);  // B_{k+1}
-            const float *nc = reinterpret_cast<const float *>(a.nz + (size_t)k * 2 * a.mp);
-            copy_async(reinterpret_cast<float *>(nzr), nc, a.mp / 2, tid, kFactorThreads);
-            copy_async(reinterpret_cast<float *>(nzr + a.mp), nc + a.mp + a.mp / 2, a.mp / 2, tid, kFactorThreads);  // A_{k+1}
+        __syncthreads();
+    };
+    // this CTA's chain: left zones from k on in direction dir, their couplings to the next zone in nx and to
+    // the one before in pv; passes: products to subtract from the zone at hand
+    int dir = half ? -1 : 1, left = (int)(half ? z1 - 1 - mid : mid - z0), passes = 0;
+    long long k = half ? z1 - 1 : z0;
+    float *nx = half ? a.At : a.Gt, *pv = half ? a.Gt : a.At;
+    bool joined = a.halves == 1 || mid == z1 - 1;  // no other half to wait for
+    if (left > 0) {
+        load(sm, at(a.Di, k));
+        copy_wait();
+        __syncthreads();
+    }
+    for (;;) {
+        const bool at_mid = left == 0;
+        float *const X = sm + xo, *const sB = sm + bo;
+        if (at_mid) {
+            __syncthreads();
+            if (!joined) {
+                // the second half to arrive goes on: + 1 each, + 16 for a failed outward half, + 256 inward
+                if (tid == 0) {
+                    const int add = 1 + (half ? ((s_bad | s_grow) ? 256 : 0) : (s_bad ? 16 : 0));
+                    __threadfence();
+                    s_all = atomicAdd(a.zbad + z0, add) + add;
+                    __threadfence();
+                }
+                __syncthreads();
+                const int all = s_all;
+                if ((all & 3) < 2) return;
+                joined = true;
+                if (tid == 0) {
+                    s_bad = (all & 16) != 0;
+                    s_grow = 0;
+                }
+                if ((all & 256) && !(all & 16)) {  // on from mid to the last zone, outwards
+                    for (long long e = (long long)mid * m * m + tid; e < z1 * m * m; e += kFactorThreads) {
+                        const long long row = e / m;
+                        const int c = (int)(e - row * m);
+                        a.At[(size_t)row * ld + c] = btd_f32(a.A[e]);
+                        a.Di[(size_t)row * ld + c] = btd_f32(a.B[e]);
+                    }
+                    __threadfence();
+                    __syncthreads();
+                    k = mid;
+                    left = (int)(z1 - 1 - mid);
+                    passes = mid > z0;
+                    mid = z1 - 1;
+                    dir = 1;
+                    nx = a.Gt;
+                    pv = a.At;
+                    load(X, at(a.Di, k));
+                    if (passes) {
+                        load(sA, at(a.At, k));
+                        load(sG, at(a.Gt, k - 1));
+                        load_nz(1, k, 1);
+                    }
+                    copy_wait();
+                    __syncthreads();
+                    if (left > 0) continue;
+                }
+            }
+            k = mid;
+            load(X, at(a.Di, k));
+            if (mid > z0) {
+                load(sA, at(a.At, k));
+                load(sG, at(a.Gt, k - 1));
+                load_nz(1, k, 1);
+                copy_wait();
+                __syncthreads();
+                schur(X);
+            }
+            if (mid < z1 - 1) {
+                load(sA, at(a.Gt, k));
+                load(sG, at(a.At, k + 1));
+                load_nz(1, k, 0);
+                copy_wait();
+                __syncthreads();
+                schur(X);
+            }
+            copy_wait();
+            __syncthreads();
+        } else {
+            if (passes) schur(X);
+            load(sG, at(nx, k));
+            load_nz(0, k, dir > 0 ? 0 : 1);
+            if (left > 1) {
+                load(sA, at(pv, k + dir));
+                load_nz(1, k + dir, dir > 0 ? 1 : 0);
+                if (four) load(sB, at(a.Di, k + dir));
+            }
         }
         // the elimination: in step it, warp 0 factors panel it, the others apply panel it - 1
         Panel<NT> pn;
@@ -683,101 +786,140 @@ __global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(c
                 }
             }
         }
-        if (next) {
-            float acc[NT][NT][4];  // [column tile][row tile]
-            int ur[NT][2];
-            unsigned nz[NT];
+        if (at_mid) break;
+        float acc[NT][NT][4];  // [column tile][row tile]
+        int ur[NT][2];
+        unsigned nz[NT];
 #pragma unroll
-            for (int x = 0; x < NT; ++x) {
+        for (int x = 0; x < NT; ++x) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int i = 16 * (wm * NT + x) + g + 8 * h;
+                ur[x][h] = cur[i < m ? i : m - 1] * ld;
+            }
+            nz[x] = 0u;
+        }
+#pragma unroll
+        for (int t = 0; t < NT; ++t) {  // row lane + 32 t in pivot order belongs to step (lane >> 3) + 4 t
+            const int j = lane + 32 * t;
+            const unsigned f = j < m ? (unsigned)nzr[cur[j]] >> (wn * NT) : 0u;
+#pragma unroll
+            for (int x = 0; x < NT; ++x) nz[x] |= ((f >> x) & 1u) << ((lane >> 3) + 4 * t);
+        }
+#pragma unroll
+        for (int y = 0; y < NT; ++y) {
+            const unsigned todo = __reduce_or_sync(0xffffffffu, nz[y]);
+            product_col<NT>(X, ur, sG, cur, ld, m, 8 * (wn * NT + y), lane, todo, acc[y]);
+        }
+        __syncthreads();  // the next coupling and D_k^{-1} have been read
+        float *Gt = at(nx, k);
+        float big = 0.f;
+#pragma unroll
+        for (int x = 0; x < NT; ++x)
+#pragma unroll
+            for (int y = 0; y < NT; ++y)
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const int i = 16 * (wm * NT + x) + g + 8 * h;
-                    ur[x][h] = cur[i < m ? i : m - 1] * ld;
-                }
-                nz[x] = 0u;
-            }
-#pragma unroll
-            for (int t = 0; t < NT; ++t) {  // row lane + 32 t in pivot order belongs to step (lane >> 3) + 4 t
-                const int j = lane + 32 * t;
-                const unsigned f = j < m ? (unsigned)nzr[cur[j]] >> (wn * NT) : 0u;
-#pragma unroll
-                for (int x = 0; x < NT; ++x) nz[x] |= ((f >> x) & 1u) << ((lane >> 3) + 4 * t);
-            }
-#pragma unroll
-            for (int y = 0; y < NT; ++y) {
-                const unsigned todo = __reduce_or_sync(0xffffffffu, nz[y]);
-                product_col<NT>(X, ur, sG, cur, ld, m, 8 * (wn * NT + y), lane, todo, acc[y]);
-            }
-            __syncthreads();  // C_k and D_k^{-1} have been read
-            float *Gt = a.Gt + (size_t)k * mw;
-#pragma unroll
-            for (int x = 0; x < NT; ++x)
-#pragma unroll
-                for (int y = 0; y < NT; ++y)
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int i = 16 * (wm * NT + x) + g + 8 * h, c = 8 * (wn * NT + y) + 2 * q;
-                        if (i < m && c < m) {
-                            const float e0 = acc[y][x][2 * h], e1 = acc[y][x][2 * h + 1];
-                            if (!(fabsf(e0) < INFINITY && fabsf(e1) < INFINITY)) s_bad = 1;
-                            if (c + 1 < m) {
-                                *reinterpret_cast<float2 *>(sG + i * ld + c) = make_float2(e0, e1);
-                                *reinterpret_cast<float2 *>(Gt + i * ld + c) = make_float2(e0, e1);
-                            } else {
-                                sG[i * ld + c] = e0;
-                                Gt[i * ld + c] = e0;
-                            }
+                    const int i = 16 * (wm * NT + x) + g + 8 * h, c = 8 * (wn * NT + y) + 2 * q;
+                    if (i < m && c < m) {
+                        const float e0 = acc[y][x][2 * h], e1 = acc[y][x][2 * h + 1];
+                        if (!(fabsf(e0) < INFINITY && fabsf(e1) < INFINITY)) s_bad = 1;
+                        big = fmaxf(big, fmaxf(fabsf(e0), fabsf(e1)));
+                        if (c + 1 < m) {
+                            *reinterpret_cast<float2 *>(sG + i * ld + c) = make_float2(e0, e1);
+                            *reinterpret_cast<float2 *>(Gt + i * ld + c) = make_float2(e0, e1);
+                        } else {
+                            sG[i * ld + c] = e0;
+                            Gt[i * ld + c] = e0;
                         }
                     }
+                }
+        if (big > kMaxGrowth) s_grow = 1;
+        --left;
+        k += dir;
+        passes = 1;
+        if (left > 0) {
             if (four) {
                 const int t = xo;
                 xo = bo;
                 bo = t;
             } else {
-                copy_async(X, a.Di + (size_t)(k + 1) * mw, mw, tid, kFactorThreads);
+                load(X, at(a.Di, k));
                 copy_wait();
             }
-            __syncthreads();
         }
+        __syncthreads();
     }
     __syncthreads();
     if (tid == 0) {
         a.zbad[z0] = s_bad;
+        a.zmid[z0] = (int)(mid - z0);
         if (s_bad) atomicOr(a.flag, 2);
     }
 }
 
-// The solve sweep, one CTA of eight warps per ray: forward y_k = D_k^{-1} (rhs_k - A_k y_{k-1}), backward
-// delta_k = y_k - G_k delta_{k+1}, x += delta in FP64 (FIRST: x = delta). Every step is one
+// The solve sweep, one CTA of eight warps per ray, or a cluster of two (a.halves) that go along with the two
+// halves of the elimination: outwards y_k = D_k^{-1} (rhs_k - A_k y_{k-1}), inwards
+// y_k = D_k^{-1} (rhs_k - C_k y_{k+1}), the zone between from both, delta = D^{-1} (rhs - A y - C y), and back
+// delta_k = y_k - G_k delta_{k+1} and y_k - H_k delta_{k-1}; x += delta in FP64 (FIRST: x = delta). The halves
+// exchange y and delta at the middle through distributed shared memory. Every step is one
 // matrix-vector product with an m x m FP32 matrix that is used once, so the matrices of the whole
 // sweep run through a ring of nring shared-memory buffers (16-byte cp.async by all threads), and each
 // step costs one CTA barrier: eight lanes take a row (128 consecutive bytes per load; rows
 // 4 warp + lane / 8 + 32 u, u < NT = ceil(m / 32)), three shuffles finish it, and the row's first lane
 // holds its vector entries. What a step needs from the vectors in memory is loaded kAhead zones ahead.
+// GB300, m = 84, 400 zones: one ray 1.25 -> 0.55 ms with two CTAs.
 constexpr int kSweepThreads = 256;
 constexpr int kAhead = 2;
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Stores to the same shared-memory variable of the cluster's CTA `rank`.
+__device__ __forceinline__ void store_remote(float *p, int rank, float v) {
+    unsigned r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(r), "f"(v) : "memory");
+}
 template <bool FIRST, bool LAST, int NT>
 __global__ void __launch_bounds__(kSweepThreads, 2) k_btd_sweep(const BtdArgs a) {
     extern __shared__ __align__(16) float sbuf[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gl = lane & 7;
     long long z0, z1;
-    if (!ray_range(a, blockIdx.x, z0, z1) || z1 == z0) return;
+    const int half = a.halves == 2 ? (int)(blockIdx.x & 1) : 0;  // the rank in the cluster
+    if (!ray_range(a, blockIdx.x / a.halves, z0, z1) || z1 == z0) return;
     const int m = a.m, lw = a.ld, nb = a.nring, mw = m * lw;
-    float *vin = sbuf + nb * mw;  // [2][VX_BTD_MAX_M] the vector of a step and of the next
+    float *vin = sbuf + nb * mw;               // [2][VX_BTD_MAX_M] the vector of a step and of the next
+    float *vx = vin + 2 * VX_BTD_MAX_M;        // [VX_BTD_MAX_M] from the other half
     if (a.zbad[z0]) {
-        if (LAST)
+        if (LAST && half == 0)
             for (long long e = z0 * m + tid; e < z1 * m; e += kSweepThreads) a.x[e] = __longlong_as_double(0x7ff8000000000000ll);
         return;
     }
-    for (int i = tid; i < 2 * VX_BTD_MAX_M; i += kSweepThreads) vin[i] = 0.f;
-    const int n = (int)(z1 - z0), nf = 2 * n - 1, total = nf + n - 1;
-    // step s: D_{z0}^{-1}, then A_k and D_k^{-1} of the later zones, then G_k from the last but one zone back
+    const long long mid = z0 + a.zmid[z0];
+    const bool both = mid < z1 - 1;  // the ray has an inward half
+    if (half == 1 && !both) return;  // (its pair does not wait for it either)
+    for (int i = tid; i < 3 * VX_BTD_MAX_M; i += kSweepThreads) vin[i] = 0.f;
+    // this half's chain: n zones from kf on in direction dir, then (outward half) the middle zone, then back
+    const int dir = half ? -1 : 1, n = (int)(half ? z1 - 1 - mid : mid - z0);
+    const long long kf = half ? z1 - 1 : z0;
+    const float *pv = half ? a.Gt : a.At, *nx = half ? a.At : a.Gt;  // couplings to the zone before; G or H
+    // steps: D^{-1} of the first zone, then coupling and D^{-1} of the later ones; at the middle zone its couplings
+    // to either side and D^{-1}; then G (H) from the last zone back
+    const int nf = n > 0 ? 2 * n - 1 : 0, nm = half ? 0 : (n > 0) + both + 1, total = nf + nm + n;
     const unsigned sb = (unsigned)__cvta_generic_to_shared(sbuf) + 16u * (unsigned)tid;
     int si = 0, bi = 0;  // the next step to bring in and its buffer
     auto issue = [&]() {
         if (si < total) {
-            const float *src = (si < nf ? ((si & 1) ? a.At : a.Di) + (size_t)(z0 + (si + 1) / 2) * mw
-                                        : a.Gt + (size_t)(z1 - 2 - (si - nf)) * mw) + 4 * tid;
+            const float *src;
+            if (si < nf) {
+                src = ((si & 1) ? pv : a.Di) + (size_t)(kf + dir * ((si + 1) / 2)) * mw;
+            } else if (si < nf + nm) {
+                const int c = si - nf + (n > 0 ? 0 : 1);  // 0: A, 1: C or D^{-1}, 2: D^{-1}
+                src = (c == 0 ? a.At : c == 1 && both ? a.Gt : a.Di) + (size_t)mid * mw;
+            } else {
+                src = nx + (size_t)(kf + dir * (n - 1 - (si - nf - nm))) * mw;
+            }
+            src += 4 * tid;
             const unsigned dst = sb + 4u * (unsigned)(bi * mw);
 #pragma unroll
             for (int i = 0; i <= NT * NT; ++i)  // 1024 (NT^2 + 1) >= m lw
@@ -793,22 +935,31 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_btd_sweep(const BtdArgs a)
     for (int s = 0; s < nb - 1; ++s) issue();
     bool own[NT];  // this lane keeps the row's vector entries
     int row[NT];
-    double rn[kAhead][NT];  // right-hand sides (forward) or x (backward) of the next zones
-    float yn[kAhead][NT];
 #pragma unroll
     for (int u = 0; u < NT; ++u) {
         row[u] = 4 * warp + 32 * u + (lane >> 3);
         own[u] = gl == 0 && row[u] < m;
+    }
+    double rn[kAhead][NT];  // right-hand sides (on the way to the middle) or x (back) of the next zones
+    float yn[kAhead][NT];
+    // right-hand side of the chain's i-th zone, the middle one (outward half) the n-th
+    const int nr = half ? n : n + 1;
+    auto rhs_at = [&](int i, int u) { return own[u] && i < nr ? a.rhs[(kf + (long long)dir * i) * m + row[u]] : 0.0; };
+    float t[NT];
+#pragma unroll
+    for (int u = 0; u < NT; ++u) {
+        t[u] = (float)rhs_at(0, u);
 #pragma unroll
         for (int h = 0; h < kAhead; ++h) {
-            rn[h][u] = own[u] && h + 1 < n ? a.rhs[(z0 + h + 1) * m + row[u]] : 0.0;
+            rn[h][u] = rhs_at(h + 1, u);
             yn[h][u] = 0.f;
         }
     }
+    if (both) cluster_sync();  // the other CTA has started and cleared its vectors
     __syncthreads();
 #pragma unroll
     for (int u = 0; u < NT; ++u)
-        if (own[u]) vin[row[u]] = (float)a.rhs[z0 * m + row[u]];
+        if (own[u]) vin[row[u]] = t[u];
     int bs = 0, par = 0;  // the step's buffer and vector
     float p[NT];
     auto step = [&]() {  // p = (the step's matrix) (its vector), in every lane of a row's group
@@ -844,40 +995,83 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_btd_sweep(const BtdArgs a)
         bs = bs + 1 == nb ? 0 : bs + 1;
         par ^= 1;
     };
-    for (long long k = z0;; ++k) {  // forward
-        step();  // p = y_k
-        const bool last = k + 1 == z1;
+    auto give = [&](const float (&v)[NT]) {  // the next step's vector
 #pragma unroll
         for (int u = 0; u < NT; ++u)
-            if (own[u]) {
-                vin[VX_BTD_MAX_M * par + row[u]] = p[u];
-                if (!last) a.y[k * m + row[u]] = p[u];
-            }
-        if (last) break;
-        step();  // p = A_{k+1} y_k
-#pragma unroll
-        for (int u = 0; u < NT; ++u)
-            if (own[u]) {
-                vin[VX_BTD_MAX_M * par + row[u]] = (float)rn[0][u] - p[u];
-                rn[0][u] = rn[1][u];
-                rn[1][u] = k + 3 < z1 ? a.rhs[(k + 3) * m + row[u]] : 0.0;
-            }
-    }
+            if (own[u]) vin[VX_BTD_MAX_M * par + row[u]] = v[u];
+    };
     static_assert(kAhead == 2, "the vectors' shifts are written out");
+    for (int i = 0; i < n; ++i) {  // to the middle
+        step();  // p = y_k
+        give(p);
+        if (i + 1 < n) {
+#pragma unroll
+            for (int u = 0; u < NT; ++u)
+                if (own[u]) a.y[(kf + (long long)dir * i) * m + row[u]] = p[u];
+            step();  // p = (coupling) y_k
+#pragma unroll
+            for (int u = 0; u < NT; ++u) {
+                t[u] = (float)rn[0][u] - p[u];
+                rn[0][u] = rn[1][u];
+                rn[1][u] = rhs_at(i + 3, u);
+            }
+            give(t);
+        }
+    }
+    float yl[NT];  // y of the chain's last zone
+#pragma unroll
+    for (int u = 0; u < NT; ++u) {
+        yl[u] = p[u];
+        if (n > 0) t[u] = (float)rn[0][u];
+    }
+    if (half == 0) {
+        if (n > 0) {
+            step();  // A y
+#pragma unroll
+            for (int u = 0; u < NT; ++u) t[u] -= p[u];
+        }
+        if (both) {
+            cluster_sync();  // the inward half's y has arrived
+#pragma unroll
+            for (int u = 0; u < NT; ++u) p[u] = own[u] ? vx[row[u]] : 0.f;
+            give(p);
+            step();  // C y
+#pragma unroll
+            for (int u = 0; u < NT; ++u) t[u] -= p[u];
+        }
+        give(t);
+        step();  // p = delta of the middle zone
+        give(p);
+#pragma unroll
+        for (int u = 0; u < NT; ++u)
+            if (own[u]) {
+                if (both) store_remote(vx + row[u], 1, p[u]);
+                double *x = a.x + mid * m + row[u];
+                *x = FIRST ? (double)p[u] : *x + (double)p[u];
+            }
+        if (both) cluster_sync();
+    } else {
+#pragma unroll
+        for (int u = 0; u < NT; ++u)
+            if (own[u]) store_remote(vx + row[u], 0, yl[u]);
+        cluster_sync();
+        cluster_sync();  // the middle zone's delta has arrived
+#pragma unroll
+        for (int u = 0; u < NT; ++u) p[u] = own[u] ? vx[row[u]] : 0.f;
+        give(p);
+    }
 #pragma unroll
     for (int u = 0; u < NT; ++u)
-        if (own[u]) {  // the last zone: delta = y
-            double *x = a.x + (z1 - 1) * m + row[u];
-            *x = FIRST ? (double)p[u] : *x + (double)p[u];
+        if (own[u]) {
+            yn[0][u] = yl[u];
+            yn[1][u] = n > 1 ? a.y[(kf + (long long)dir * (n - 2)) * m + row[u]] : 0.f;
 #pragma unroll
-            for (int h = 0; h < kAhead; ++h) {
-                const long long k = z1 - 2 - h;
-                yn[h][u] = k >= z0 ? a.y[k * m + row[u]] : 0.f;
-                if (!FIRST) rn[h][u] = k >= z0 ? a.x[k * m + row[u]] : 0.0;
-            }
+            for (int h = 0; h < kAhead; ++h)
+                if (!FIRST) rn[h][u] = n > h ? a.x[(kf + (long long)dir * (n - 1 - h)) * m + row[u]] : 0.0;
         }
-    for (long long k = z1 - 2; k >= z0; --k) {  // backward
+    for (int i = n - 1; i >= 0; --i) {  // back
         step();  // p = G_k delta_{k+1}
+        const long long k = kf + (long long)dir * i;
 #pragma unroll
         for (int u = 0; u < NT; ++u)
             if (own[u]) {
@@ -885,10 +1079,10 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_btd_sweep(const BtdArgs a)
                 vin[VX_BTD_MAX_M * par + row[u]] = dl;
                 a.x[k * m + row[u]] = FIRST ? (double)dl : rn[0][u] + (double)dl;
                 yn[0][u] = yn[1][u];
-                yn[1][u] = k - 2 >= z0 ? a.y[(k - 2) * m + row[u]] : 0.f;
+                yn[1][u] = i > 1 ? a.y[(k - 2 * dir) * m + row[u]] : 0.f;
                 if (!FIRST) {
                     rn[0][u] = rn[1][u];
-                    rn[1][u] = k - 2 >= z0 ? a.x[(k - 2) * m + row[u]] : 0.0;
+                    rn[1][u] = i > 1 ? a.x[(k - 2 * dir) * m + row[u]] : 0.0;
                 }
             }
     }
@@ -989,11 +1183,22 @@ static const void *sweep_kernel(int m) {
     return (const void *)k_btd_sweep<F, L, 4>;
 }
 template <bool F, bool L>
-static void launch_sweep(int m, int grid, size_t smem, cudaStream_t s, const BtdArgs &a) {
-    if (m <= 32) k_btd_sweep<F, L, 1><<<grid, kSweepThreads, smem, s>>>(a);
-    else if (m <= 64) k_btd_sweep<F, L, 2><<<grid, kSweepThreads, smem, s>>>(a);
-    else if (m <= 96) k_btd_sweep<F, L, 3><<<grid, kSweepThreads, smem, s>>>(a);
-    else k_btd_sweep<F, L, 4><<<grid, kSweepThreads, smem, s>>>(a);
+static cudaError_t launch_sweep(int m, int grid, size_t smem, cudaStream_t s, const BtdArgs &a) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kSweepThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)a.halves;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    if (m <= 32) return cudaLaunchKernelEx(&cfg, k_btd_sweep<F, L, 1>, a);
+    if (m <= 64) return cudaLaunchKernelEx(&cfg, k_btd_sweep<F, L, 2>, a);
+    if (m <= 96) return cudaLaunchKernelEx(&cfg, k_btd_sweep<F, L, 3>, a);
+    return cudaLaunchKernelEx(&cfg, k_btd_sweep<F, L, 4>, a);
 }
 
 // Shared memory that lets two CTAs share an SM (228 KB, 1 KB of it reserved per CTA), and one CTA's limit.
@@ -1005,7 +1210,8 @@ struct vx_btd {
     size_t smem = 0, smem_sweep = 0;
     float *Di = nullptr, *Gt = nullptr, *At = nullptr, *y = nullptr;
     unsigned short *nz = nullptr;
-    int *zbad = nullptr, *flag = nullptr;  // flag[0]: numeric flag, flag[1]: offsets invalid
+    int slots = 0;  // factor CTAs the device holds at once
+    int *zbad = nullptr, *zmid = nullptr, *flag = nullptr;  // flag[0]: numeric flag, flag[1]: offsets invalid
     double *r = nullptr;
 };
 
@@ -1017,6 +1223,7 @@ static void btd_free(vx_btd *h) {
     cudaFree(h->At);
     cudaFree(h->y);
     cudaFree(h->zbad);
+    cudaFree(h->zmid);
     cudaFree(h->flag);
     cudaFree(h->r);
     delete h;
@@ -1044,7 +1251,7 @@ extern "C" vx_status vx_btd_create(int m, long long max_zones, int n_refine, vx_
     h->nbuf = s4 <= kSmemHalf || (s3 > kSmemHalf && s4 <= kSmemFull) ? 4 : 3;
     h->smem = h->nbuf == 4 ? s4 : s3;
     const size_t mw = (size_t)m * h->ld;
-    auto ring = [&](int nb) { return (nb * mw + 2 * VX_BTD_MAX_M) * sizeof(float); };
+    auto ring = [&](int nb) { return (nb * mw + 3 * VX_BTD_MAX_M) * sizeof(float); };
     h->nring = ring(4) <= kSmemHalf ? 4 : ring(3) <= kSmemFull ? 3 : 2;
     h->smem_sweep = ring(h->nring);
     const size_t zc = (size_t)(max_zones > 0 ? max_zones : 1);
@@ -1055,6 +1262,7 @@ extern "C" vx_status vx_btd_create(int m, long long max_zones, int n_refine, vx_
     if (e == cudaSuccess) e = cudaMalloc(&h->nz, zc * 2 * h->mp * sizeof(unsigned short));
     if (e == cudaSuccess) e = cudaMalloc(&h->y, zc * m * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&h->zbad, zc * sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&h->zmid, zc * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&h->r, zc * m * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&h->flag, 2 * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(h->flag, 0, 2 * sizeof(int));
@@ -1064,6 +1272,10 @@ extern "C" vx_status vx_btd_create(int m, long long max_zones, int n_refine, vx_
     // the kernels' limit, not this handle's size: handles of several m share them
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(factor_kernel(m), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFull);
+    int dev = 0, sms = 1;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    h->slots = sms * (h->smem <= kSmemHalf && m <= 96 ? 2 : 1);
     const void *sweeps[4] = {sweep_kernel<true, true>(m), sweep_kernel<true, false>(m), sweep_kernel<false, true>(m),
                              sweep_kernel<false, false>(m)};
     for (int i = 0; i < 4 && e == cudaSuccess; ++i)
@@ -1123,20 +1335,28 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
     a.At = h->At;
     a.y = h->y;
     a.zbad = h->zbad;
+    a.zmid = h->zmid;
+    // Two CTAs per ray while they all find room at once, and with rays of 16 zones or more where the last wave of
+    // one CTA per ray would be less than 5/8 full. GB300, one -> two, 100 zones: m = 84, 20 rays 3.60 -> 1.98 ms,
+    // 152 4.76 -> 3.73, 160 5.91 -> 5.32, 330 10.58 -> 9.02, 480 13.25 -> 12.54, but 240 6.67 -> 6.70 and
+    // 304 (all slots) 7.33 -> 7.41; m = 120 (40 zones), 200 rays 8.50 -> 7.12, 110 4.40 -> 4.46; rays of
+    // 4 to 8 zones, 2000 of them, 3.04 -> 3.18.
+    const int rest = n_rays % h->slots;
+    a.halves = 2 * n_rays <= h->slots ||
+                       (n_rays < 4 * h->slots && n_zones >= 16ll * n_rays && rest > 0 && 8 * rest <= 5 * h->slots)
+                   ? 2
+                   : 1;
     a.flag = h->flag;
     a.inval = h->flag + 1;
     BTD_CU(cudaMemsetAsync(h->flag + 1, 0, sizeof(int), s));
-    k_btd_validate<<<(unsigned)((n_rays + 256) / 256), 256, 0, s>>>(ray_offsets, n_rays, n_zones, h->flag + 1, h->flag);
+    k_btd_validate<<<(unsigned)((n_rays + 256) / 256), 256, 0, s>>>(ray_offsets, n_rays, n_zones, h->flag + 1, h->flag, h->zbad);
     BTD_CU(cudaGetLastError());
     launch_convert(h->m, n_zones, s, a);
     BTD_CU(cudaGetLastError());
-    launch_factor(h->m, n_rays, h->smem, s, a);
+    const int ctas = a.halves * n_rays;
+    launch_factor(h->m, ctas, h->smem, s, a);
     BTD_CU(cudaGetLastError());
-    if (h->n_refine == 0)
-        launch_sweep<true, true>(h->m, n_rays, h->smem_sweep, s, a);
-    else
-        launch_sweep<true, false>(h->m, n_rays, h->smem_sweep, s, a);
-    BTD_CU(cudaGetLastError());
+    BTD_CU((h->n_refine == 0 ? launch_sweep<true, true> : launch_sweep<true, false>)(h->m, ctas, h->smem_sweep, s, a));
     // CTAs per ray of the residual: enough to fill the chip with few rays, at most one per eight units (row octets)
     const long long units = n_zones * ((h->m + 7) / 8);
     long long split = (8 * 152 + n_rays - 1) / n_rays, most = (units + 8 * n_rays - 1) / (8 * (long long)n_rays);
@@ -1147,11 +1367,7 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
         k_btd_resid<<<dim3(n_rays, (unsigned)split), kResidThreads, 0, s>>>(a);
         BTD_CU(cudaGetLastError());
         a.rhs = h->r;
-        if (it == h->n_refine)
-            launch_sweep<false, true>(h->m, n_rays, h->smem_sweep, s, a);
-        else
-            launch_sweep<false, false>(h->m, n_rays, h->smem_sweep, s, a);
-        BTD_CU(cudaGetLastError());
+        BTD_CU((it == h->n_refine ? launch_sweep<false, true> : launch_sweep<false, false>)(h->m, ctas, h->smem_sweep, s, a));
     }
     return VX_OK;
 }
