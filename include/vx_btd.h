@@ -17,7 +17,11 @@
  * without pivoting across zones: D_0 = B_0, D_k = B_k - A_k G_{k-1} with G_k = D_k^{-1} C_k,
  * each D_k inverted with partial pivoting inside the block. The factorisation is done in FP32 from
  * FP32 copies of the blocks, one CTA per ray, its matrix products on the tensor cores (TF32 with each
- * operand split into two parts, three products: about FP32 accuracy); D_k^{-1} and G_k are kept. Then
+ * operand split into two parts, three products: about FP32 accuracy); D_k^{-1} and G_k are kept. Where
+ * rays are few, a ray is eliminated from both ends at once by two CTAs, or in segments of its zones by a
+ * CTA each and then the system of the segments' last zones (chosen by n_rays, n_zones and m); if a
+ * pivot fails there, or entries of D^{-1} C or the like exceed 64, the ray is done again from its
+ * first zone on, so what can be solved does not depend on it. Then
  * the ray is solved by matrix-vector products with those, y_k = D_k^{-1} (d_k - A_k y_{k-1}) forward and
  * x_k = y_k - G_k x_{k+1} backward, and
  * n_refine sweeps of iterative refinement follow, each from the FP64 residual d - M x of the
@@ -48,8 +52,9 @@ typedef struct vx_btd vx_btd;
 
 /* Creates a solver for m unknowns per zone (1 .. VX_BTD_MAX_M) and batches of at most max_zones
  * zones (>= 0), with n_refine FP64 refinement sweeps (0 .. VX_BTD_MAX_REFINE; 0 leaves the FP32
- * solution). Allocates the device workspace: 12 m (m + 7) + 4 (m + 7) + 12 m + 8 bytes per zone at most. *out is set to
- * NULL on failure. Errors: VX_ERR_INVALID_ARG, VX_ERR_OOM, VX_ERR_CUDA. */
+ * solution). Allocates the device workspace: 12 m (m + 7) + 4 (m + 7) + 12 m + 8 bytes per zone at most, and for
+ * the segments (m up to about 110) 4 m (m + 7) for each of the first 16384 zones and 16 m (m + 8) per SM; without the
+ * memory for the latter, rays are not cut into segments. *out is set to NULL on failure. Errors: VX_ERR_INVALID_ARG, VX_ERR_OOM, VX_ERR_CUDA. */
 vx_status vx_btd_create(int m, long long max_zones, int n_refine, vx_btd **out);
 
 /* Solves every ray. n_rays >= 0; n_zones = the total zone count, 0 .. max_zones.

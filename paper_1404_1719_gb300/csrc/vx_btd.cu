@@ -82,13 +82,29 @@ struct BtdArgs {
     unsigned short *nz;       // [Z][C, A][mp] zero patterns of the rows
     int *zbad, *zmid, *flag;  // at a ray's first zone: a pivot failed; the zone its eliminations meet at, from there
     const int *inval;  // set by k_btd_validate when the offsets are not a partition of the zones
+    // Rays in segments (k_btd_segment): parts > 0: this is the system of the segments' last zones, ray r's from r parts
+    // on; parts = 0 and pbad: only the rays that pbad marks, whose elimination by segments failed
+    int parts;
+    int *pbad;
 };
+
+// The segments of a ray of n zones: at most `parts`, of four zones or more.
+__host__ __device__ __forceinline__ int seg_count(long long n, int parts) {
+    const long long s = n / 4 < parts ? n / 4 : parts;
+    return n < 1 ? 0 : s < 1 ? 1 : (int)s;
+}
 
 // The zone range of a ray; false (nothing to do) when the offsets failed validation.
 __device__ __forceinline__ bool ray_range(const BtdArgs &a, int ray, long long &z0, long long &z1) {
     if (*a.inval) return false;
     z0 = a.off[ray];
     z1 = a.off[ray + 1];
+    if (a.pbad && (a.parts > 0) == (a.pbad[ray] != 0)) return false;
+    if (a.parts > 0) {
+        const int s = seg_count(z1 - z0, a.parts);
+        z0 = (long long)ray * a.parts;
+        z1 = z0 + s;
+    }
     return true;
 }
 
@@ -99,9 +115,10 @@ __device__ __forceinline__ long long ray_mid(const BtdArgs &a, long long z0, lon
 
 // offsets[0] = 0, offsets[n_rays] = n_zones and non-decreasing; any violation marks the whole call
 // invalid (so no two rays can share zones) and raises the numeric flag.
-__global__ void k_btd_validate(const int *off, int n_rays, long long n_zones, int *inval, int *flag, int *zbad) {
+__global__ void k_btd_validate(const int *off, int n_rays, long long n_zones, int *inval, int *flag, int *zbad, int *pbad) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i > n_rays) return;
+    if (pbad && i < n_rays) pbad[i] = 0;
     const long long v = off[i];
     bool bad = v < 0 || v > n_zones || (i == 0 && v != 0) || (i == n_rays && v != n_zones);
     if (i < n_rays && off[i + 1] < v) bad = true;
@@ -575,6 +592,144 @@ __host__ __device__ constexpr size_t factor_smem(int m, int ld, int nbuf) {
            (size_t)m * sizeof(int);
 }
 
+// X -= U V, all in shared memory; the rows of U hold something only in the groups that nz marks.
+template <int NT>
+__device__ __forceinline__ void subtract_product(float *X, const float *U, const float *V, const unsigned short *nz, int ld,
+                                                 int m, int wm, int wn, int lane) {
+    const int g = lane >> 2, q = lane & 3;
+#pragma unroll 1
+    for (int x = 0; x < NT; ++x) {
+        const int i0 = 16 * (wm * NT + x), i = i0 + (lane & 15);
+        const unsigned todo = __reduce_or_sync(0xffffffffu, i < m ? (unsigned)nz[i] : 0u);
+        float d[NT][4];
+        const int r0 = i0 + g < m ? i0 + g : m - 1, r1 = i0 + g + 8 < m ? i0 + g + 8 : m - 1;
+        product_row<NT>(U, r0 * ld, r1 * ld, V, ld, m, wn, lane, todo, d);
+        const bool i0m = i0 + g < m, i1m = i0 + g + 8 < m;
+#pragma unroll
+        for (int y = 0; y < NT; ++y) {
+            const int c = 8 * (wn * NT + y) + 2 * q;
+            float *x0 = X + r0 * ld + c, *x1 = X + r1 * ld + c;
+            if (c + 1 < m) {
+                const float2 e0 = *reinterpret_cast<float2 *>(x0), e1 = *reinterpret_cast<float2 *>(x1);
+                if (i0m) *reinterpret_cast<float2 *>(x0) = make_float2(e0.x - d[y][0], e0.y - d[y][1]);
+                if (i1m) *reinterpret_cast<float2 *>(x1) = make_float2(e1.x - d[y][2], e1.y - d[y][3]);
+            } else if (c < m) {
+                if (i0m) *x0 -= d[y][0];
+                if (i1m) *x1 -= d[y][2];
+            }
+        }
+    }
+}
+
+// Inverts X in place up to the order of its rows and columns: eliminates panel after panel, one CTA barrier each;
+// in step it, warp 0 eliminates within panel it, the others apply panel it - 1. Pivot j's row is cur[j], pos its
+// inverse: X^{-1}[j][cur[q]] = X[cur[j]][q]. True in warp 0 if a pivot failed. No barrier at its end.
+template <int NT>
+__device__ __forceinline__ bool invert(float *X, int ld, int m, int *cur, int *pos, float *rowbuf, int tid) {
+    const int lane = tid & 31, warp = tid >> 5, nw = kFactorThreads / 32, P = (m + 7) >> 3;
+    Panel<NT> pn;
+    if (warp == 0) pn.start(m, lane);
+    for (int it = 0; it <= P; ++it) {  // step P: the last panel's transform, by all warps
+        const int nu = it < P ? nw - 1 : nw, u = warp - (nw - nu);  // the warps that update, and this one's number
+        if (u < 0) {
+            if (it == 0) {
+                Panel<NT>::fetch(pn.v, X, ld, m, 0, lane);
+                pn.trim(m, 0, lane);
+            } else {
+                pn.advance(X, ld, m, 8 * it, cur + 8 * (it - 1), lane);
+            }
+            pn.factor(m, 8 * it, m - 8 * it < 8 ? m - 8 * it : 8, cur, rowbuf, lane);
+            pn.store(X, ld, m, 8 * it, lane);
+        } else {
+            if (it > 0) {  // every tile but it - 1 (the transform itself) and it
+                const int t0 = u, t1 = u + nu, nt = it < P ? P - 2 : P - 1;
+                if (t0 < nt)
+                    tile_update<NT>(X, ld, m, it - 1, t0 < it - 1 ? t0 : t0 + 2, t1 < nt ? (t1 < it - 1 ? t1 : t1 + 2) : -1,
+                                    cur, lane);
+            }
+            if (it == P && tid < m) pos[cur[tid]] = tid;
+        }
+        if (it < P) __syncthreads();
+    }
+    return warp == 0 && pn.failed();
+}
+
+// The inverse of X (as invert leaves it), row by row, to Di.
+template <int NT>
+__device__ __forceinline__ void store_inverse(float *Di, const float *X, int ld, int m, const int *cur, const int *pos, int tid) {
+    const int lane = tid & 31, warp = tid >> 5, nw = kFactorThreads / 32;
+    int pc[NT];
+#pragma unroll
+    for (int t = 0; t < NT; ++t) pc[t] = lane + 32 * t < m ? pos[lane + 32 * t] : 0;
+    for (int j = warp; j < m; j += nw) {
+        const float *row = X + cur[j] * ld;
+#pragma unroll
+        for (int t = 0; t < NT; ++t) {
+            const int c = lane + 32 * t;
+            if (c < m) Di[j * ld + c] = row[pc[t]];
+        }
+    }
+}
+
+// acc[column tile][row tile] = X^{-1} V, X as invert leaves it; V's rows hold something only in the groups that
+// nzr marks (all: in every group).
+template <int NT>
+__device__ __forceinline__ void inverse_times(float (&acc)[NT][NT][4], const float *X, const float *V, const unsigned short *nzr,
+                                              const int *cur, int ld, int m, int wm, int wn, int lane) {
+    const int g = lane >> 2;
+    int ur[NT][2];
+    unsigned nz[NT];
+#pragma unroll
+    for (int x = 0; x < NT; ++x) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = 16 * (wm * NT + x) + g + 8 * h;
+            ur[x][h] = cur[i < m ? i : m - 1] * ld;
+        }
+        nz[x] = 0u;
+    }
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {  // row lane + 32 t in pivot order belongs to step (lane >> 3) + 4 t
+        const int j = lane + 32 * t;
+        const unsigned f = j < m ? (nzr ? (unsigned)nzr[cur[j]] : 0xffffu) >> (wn * NT) : 0u;
+#pragma unroll
+        for (int x = 0; x < NT; ++x) nz[x] |= ((f >> x) & 1u) << ((lane >> 3) + 4 * t);
+    }
+#pragma unroll
+    for (int y = 0; y < NT; ++y) {
+        const unsigned todo = __reduce_or_sync(0xffffffffu, nz[y]);
+        product_col<NT>(X, ur, V, cur, ld, m, 8 * (wn * NT + y), lane, todo, acc[y]);
+    }
+}
+
+// acc, times sign, to row-major matrices in shared (S) and global (D) memory; raises big to its largest magnitude and
+// clears finite if an entry is not.
+template <int NT>
+__device__ __forceinline__ void store_tiles(float *S, float *D, const float (&acc)[NT][NT][4], float sign, int ld, int m, int wm,
+                                            int wn, int lane, float &big, bool &finite) {
+    const int g = lane >> 2, q = lane & 3;
+#pragma unroll
+    for (int x = 0; x < NT; ++x)
+#pragma unroll
+        for (int y = 0; y < NT; ++y)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int i = 16 * (wm * NT + x) + g + 8 * h, c = 8 * (wn * NT + y) + 2 * q;
+                if (i < m && c < m) {
+                    const float e0 = sign * acc[y][x][2 * h], e1 = sign * acc[y][x][2 * h + 1];
+                    if (!(fabsf(e0) < INFINITY && fabsf(e1) < INFINITY)) finite = false;
+                    big = fmaxf(big, fmaxf(fabsf(e0), fabsf(e1)));
+                    if (c + 1 < m) {
+                        if (S) *reinterpret_cast<float2 *>(S + i * ld + c) = make_float2(e0, e1);
+                        if (D) *reinterpret_cast<float2 *>(D + i * ld + c) = make_float2(e0, e1);
+                    } else {
+                        if (S) S[i * ld + c] = e0;
+                        if (D) D[i * ld + c] = e0;
+                    }
+                }
+            }
+}
+
 // The factor kernel: CTAs of eight warps, one per ray, or two where one would leave SMs without work
 // (a.halves): then one eliminates from the ray's first zone outwards and one from its last zone inwards, D_k =
 // B_k - C_k H_{k+1} with H_k = D_k^{-1} A_k, and whichever comes second to the zone between them (mid) takes
@@ -601,7 +756,7 @@ __global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(c
     extern __shared__ __align__(16) float sm[];
     __shared__ int s_bad, s_grow, s_all;
     const int m = a.m, ld = a.ld, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nw = kFactorThreads / 32, bs = factor_buf(m, ld), P = (m + 7) >> 3;
+    const int bs = factor_buf(m, ld), P = (m + 7) >> 3;
     const bool four = a.nbuf == 4;
     // D_k and the next zone's B come first: tile_update reads up to 15 rows past the end of D_k
     // (offsets, not pointers, are exchanged from zone to zone: the compiler then knows the address space)
@@ -619,7 +774,7 @@ __global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(c
     if (tid == 0) s_bad = s_grow = 0;
     if (tid < m) pos[tid] = tid;  // in range also where a failed pivot leaves an entry unset
     const int mw = m * ld;
-    const int g = lane >> 2, q = lane & 3, wm = warp & 1, wn = warp >> 1;
+    const int wm = warp & 1, wn = warp >> 1;
     // zeros behind every buffer: the last panel's transform, if it has fewer than eight columns, is read that far
     // (and multiplied by zeros, so it must be finite)
     for (int i = tid; i < a.nbuf * (bs - mw); i += kFactorThreads) sm[i / (bs - mw) * bs + mw + i % (bs - mw)] = 0.f;
@@ -629,30 +784,8 @@ __global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(c
                    a.mp / 2, tid, kFactorThreads);
     };
     auto at = [&](float *w, long long k) { return w + (size_t)k * mw; };
-    // X -= (coupling in sA) (matrix in sG)
-    auto schur = [&](float *X) {
-#pragma unroll 1
-        for (int x = 0; x < NT; ++x) {
-            const int i0 = 16 * (wm * NT + x), i = i0 + (lane & 15);
-            const unsigned nz = __reduce_or_sync(0xffffffffu, i < m ? (unsigned)nzr[a.mp + i] : 0u);
-            float d[NT][4];
-            const int r0 = i0 + g < m ? i0 + g : m - 1, r1 = i0 + g + 8 < m ? i0 + g + 8 : m - 1;
-            product_row<NT>(sA, r0 * ld, r1 * ld, sG, ld, m, wn, lane, nz, d);
-            const bool i0m = i0 + g < m, i1m = i0 + g + 8 < m;
-#pragma unroll
-            for (int y = 0; y < NT; ++y) {
-                const int c = 8 * (wn * NT + y) + 2 * q;
-                float *x0 = X + r0 * ld + c, *x1 = X + r1 * ld + c;
-                if (c + 1 < m) {
-                    const float2 e0 = *reinterpret_cast<float2 *>(x0), e1 = *reinterpret_cast<float2 *>(x1);
-                    if (i0m) *reinterpret_cast<float2 *>(x0) = make_float2(e0.x - d[y][0], e0.y - d[y][1]);
-                    if (i1m) *reinterpret_cast<float2 *>(x1) = make_float2(e1.x - d[y][2], e1.y - d[y][3]);
-                } else if (c < m) {
-                    if (i0m) *x0 -= d[y][0];
-                    if (i1m) *x1 -= d[y][2];
-                }
-            }
-        }
+    auto schur = [&](float *X) {  // X -= (coupling in sA) (matrix in sG)
+        subtract_product<NT>(X, sA, sG, nzr + a.mp, ld, m, wm, wn, lane);
         __syncthreads();
     };
     // this CTA's chain: left zones from k on in direction dir, their couplings to the next zone in nx and to
@@ -684,10 +817,10 @@ __global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(c
                 if ((all & 3) < 2) return;
                 joined = true;
                 if (tid == 0) {
-                    s_bad = (all & 16) != 0;
+                    s_bad = (all & 16) != 0 || ((all & 256) && !a.A);
                     s_grow = 0;
                 }
-                if ((all & 256) && !(all & 16)) {  // on from mid to the last zone, outwards
+                if ((all & 256) && !(all & 16) && a.A) {  // on from mid to the last zone, outwards
                     for (long long e = (long long)mid * m * m + tid; e < z1 * m * m; e += kFactorThreads) {
                         const long long row = e / m;
                         const int c = (int)(e - row * m);
@@ -744,96 +877,17 @@ __global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(c
                 if (four) load(sB, at(a.Di, k + dir));
             }
         }
-        // the elimination: in step it, warp 0 factors panel it, the others apply panel it - 1
-        Panel<NT> pn;
-        if (warp == 0) pn.start(m, lane);
-        for (int it = 0; it <= P; ++it) {  // step P: the last panel's transform, by all warps
-            const int nu = it < P ? nw - 1 : nw, u = warp - (nw - nu);  // the warps that update, and this one's number
-            if (u < 0) {
-                if (it == 0) {
-                    Panel<NT>::fetch(pn.v, X, ld, m, 0, lane);
-                    pn.trim(m, 0, lane);
-                } else {
-                    pn.advance(X, ld, m, 8 * it, cur + 8 * (it - 1), lane);
-                }
-                pn.factor(m, 8 * it, m - 8 * it < 8 ? m - 8 * it : 8, cur, rowbuf, lane);
-                pn.store(X, ld, m, 8 * it, lane);
-            } else {
-                if (it > 0) {  // every tile but it - 1 (the transform itself) and it
-                    const int t0 = u, t1 = u + nu, nt = it < P ? P - 2 : P - 1;
-                    if (t0 < nt)
-                        tile_update<NT>(X, ld, m, it - 1, t0 < it - 1 ? t0 : t0 + 2,
-                                        t1 < nt ? (t1 < it - 1 ? t1 : t1 + 2) : -1, cur, lane);
-                }
-                if (it == P && tid < m) pos[cur[tid]] = tid;
-            }
-            if (it < P) __syncthreads();
-        }
-        if (warp == 0 && lane == 0 && pn.failed()) s_bad = 1;
+        if (invert<NT>(X, ld, m, cur, pos, rowbuf, tid) && lane == 0) s_bad = 1;
         copy_wait();
         __syncthreads();
-        {  // D_k^{-1} row by row, and G_k = D_k^{-1} C_k
-            float *Di = a.Di + (size_t)k * mw;
-            int pc[NT];
-#pragma unroll
-            for (int t = 0; t < NT; ++t) pc[t] = lane + 32 * t < m ? pos[lane + 32 * t] : 0;
-            for (int j = warp; j < m; j += nw) {
-                const float *row = X + cur[j] * ld;
-#pragma unroll
-                for (int t = 0; t < NT; ++t) {
-                    const int c = lane + 32 * t;
-                    if (c < m) Di[j * ld + c] = row[pc[t]];
-                }
-            }
-        }
+        store_inverse<NT>(at(a.Di, k), X, ld, m, cur, pos, tid);
         if (at_mid) break;
-        float acc[NT][NT][4];  // [column tile][row tile]
-        int ur[NT][2];
-        unsigned nz[NT];
-#pragma unroll
-        for (int x = 0; x < NT; ++x) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int i = 16 * (wm * NT + x) + g + 8 * h;
-                ur[x][h] = cur[i < m ? i : m - 1] * ld;
-            }
-            nz[x] = 0u;
-        }
-#pragma unroll
-        for (int t = 0; t < NT; ++t) {  // row lane + 32 t in pivot order belongs to step (lane >> 3) + 4 t
-            const int j = lane + 32 * t;
-            const unsigned f = j < m ? (unsigned)nzr[cur[j]] >> (wn * NT) : 0u;
-#pragma unroll
-            for (int x = 0; x < NT; ++x) nz[x] |= ((f >> x) & 1u) << ((lane >> 3) + 4 * t);
-        }
-#pragma unroll
-        for (int y = 0; y < NT; ++y) {
-            const unsigned todo = __reduce_or_sync(0xffffffffu, nz[y]);
-            product_col<NT>(X, ur, sG, cur, ld, m, 8 * (wn * NT + y), lane, todo, acc[y]);
-        }
+        float acc[NT][NT][4], big = 0.f;
+        bool finite = true;
+        inverse_times<NT>(acc, X, sG, nzr, cur, ld, m, wm, wn, lane);
         __syncthreads();  // the next coupling and D_k^{-1} have been read
-        float *Gt = at(nx, k);
-        float big = 0.f;
-#pragma unroll
-        for (int x = 0; x < NT; ++x)
-#pragma unroll
-            for (int y = 0; y < NT; ++y)
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int i = 16 * (wm * NT + x) + g + 8 * h, c = 8 * (wn * NT + y) + 2 * q;
-                    if (i < m && c < m) {
-                        const float e0 = acc[y][x][2 * h], e1 = acc[y][x][2 * h + 1];
-                        if (!(fabsf(e0) < INFINITY && fabsf(e1) < INFINITY)) s_bad = 1;
-                        big = fmaxf(big, fmaxf(fabsf(e0), fabsf(e1)));
-                        if (c + 1 < m) {
-                            *reinterpret_cast<float2 *>(sG + i * ld + c) = make_float2(e0, e1);
-                            *reinterpret_cast<float2 *>(Gt + i * ld + c) = make_float2(e0, e1);
-                        } else {
-                            sG[i * ld + c] = e0;
-                            Gt[i * ld + c] = e0;
-                        }
-                    }
-                }
+        store_tiles<NT>(sG, at(nx, k), acc, 1.f, ld, m, wm, wn, lane, big, finite);
+        if (!finite) s_bad = 1;
         if (big > kMaxGrowth) s_grow = 1;
         --left;
         k += dir;
@@ -854,7 +908,211 @@ __global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(c
     if (tid == 0) {
         a.zbad[z0] = s_bad;
         a.zmid[z0] = (int)(mid - z0);
-        if (s_bad) atomicOr(a.flag, 2);
+        if (s_bad) {
+            if (a.parts > 0) a.pbad[blockIdx.x / a.halves] = 1;
+            else atomicOr(a.flag, 2);
+        }
+    }
+}
+
+// Rays in segments, where there are so few that most SMs would have none: a ray of n zones is cut into S segments, all
+// eliminated at the same time by a CTA each. The segment's last zone e stays; the others, a .. e - 1, are
+// eliminated outwards, with a second right-hand side for their coupling to the zone p = a - 1 before the segment,
+//   x_k = y_k - G_k x_{k+1} - L_k x_p,  L_a = D_a^{-1} A_a,  L_k = -D_k^{-1} A_k L_{k-1},
+// and then once more inwards for the segment's first zone, x_a = y' - R x_e - L' x_p (R_k = -G_k R_{k+1},
+// L'_k = L_k - G_k L'_{k+1}). That leaves a block-tridiagonal system of the segments' last zones,
+//   Ar_e = -A_e L_{e-1},  Br_e = B_e - A_e G_{e-1} - C_e L'_{next a},  Cr_e = -C_e R_{next a},
+// for k_btd_factor. A ray in which a pivot fails, or an entry of G, L, R or L' is above kMaxGrowth, is
+// done again as a whole by k_btd_factor (pbad). The time is that of n / S + S / 2 zones, not n / 2.
+// GB300, m = 84, 400 zones, one ray: 5.11 ms by two CTAs -> 0.58 ms for 34 segments and 0.66 ms for their
+// last zones.
+struct SegArgs {
+    BtdArgs a;
+    int parts, nbuf;
+    float *Lt;                  // L_k, per zone
+    float *Dr, *Cr, *Ar, *Er;   // [n_rays][parts] Br_e without its last term, Cr_e, Ar_e, that term
+    unsigned short *nzr;        // zero patterns of Cr, Ar: none
+    int *zbadr, *pbad;
+    double *rr, *xr;            // [n_rays][parts][m] the right-hand sides and the solution of that system
+};
+
+// Segment s of ray r: its zones za .. ze (the one that stays), its row in the system of those.
+struct Seg {
+    long long za, ze, row;
+    bool first, last;
+    __device__ __forceinline__ bool find(const SegArgs &p, int block, bool good) {
+        const int ray = block / p.parts, i = block % p.parts;
+        if (*p.a.inval || (good && p.pbad[ray])) return false;
+        const long long z0 = p.a.off[ray], n = p.a.off[ray + 1] - z0;
+        const int S = seg_count(n, p.parts);
+        if (i >= S) return false;
+        za = z0 + n * i / S;
+        ze = z0 + n * (i + 1) / S - 1;
+        row = (long long)ray * p.parts + i;
+        first = i == 0;
+        last = i == S - 1;
+        return true;
+    }
+};
+
+template <int NT>
+__global__ void __launch_bounds__(kFactorThreads, 1) k_btd_segment(const SegArgs p) {
+    extern __shared__ __align__(16) float sm[];
+    __shared__ int s_bad;
+    const BtdArgs &a = p.a;
+    Seg sg;
+    if (!sg.find(p, blockIdx.x, false)) return;
+    const int m = a.m, ld = a.ld, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wm = warp & 1, wn = warp >> 1;
+    const int bs = factor_buf(m, ld), P = (m + 7) >> 3, mw = m * ld;
+    const bool five = p.nbuf == 5;  // a buffer for the next zone's B
+    int xo = 0, bo = five ? bs : 0;
+    float *const sG = sm + bo + bs, *const sA = sG + bs, *const sL = sA + bs;
+    unsigned short *nzr = reinterpret_cast<unsigned short *>(sm + p.nbuf * bs);  // [C_k, A_k][mp]
+    float *rowbuf = sm + p.nbuf * bs + a.mp;                                      // [2][8]
+    int *cur = reinterpret_cast<int *>(rowbuf + 16);
+    int *pos = cur + 8 * P;
+    if (tid == 0) s_bad = 0;
+    if (tid < m) pos[tid] = tid;
+    for (int i = tid; i < p.nbuf * (bs - mw); i += kFactorThreads) sm[i / (bs - mw) * bs + mw + i % (bs - mw)] = 0.f;
+    auto load = [&](float *dst, const float *src) { copy_async(dst, src, mw, tid, kFactorThreads); };
+    auto load_nz = [&](int to, long long k, int which) {  // the zero pattern of C_k (which 0) or A_k (1)
+        copy_async(reinterpret_cast<float *>(nzr + to * a.mp), reinterpret_cast<const float *>(a.nz + ((size_t)k * 2 + which) * a.mp),
+                   a.mp / 2, tid, kFactorThreads);
+    };
+    auto at = [&](float *w, long long k) { return w + (size_t)k * mw; };
+    // acc = U V, U's zero pattern in nz (null: none)
+    auto rows_times = [&](float (&acc)[NT][NT][4], const float *U, const float *V, const unsigned short *nz) {
+#pragma unroll
+        for (int x = 0; x < NT; ++x) {
+            const int i0 = 16 * (wm * NT + x), i = i0 + (lane & 15), g = lane >> 2;
+            const unsigned todo = nz ? __reduce_or_sync(0xffffffffu, i < m ? (unsigned)nz[i] : 0u) : (1u << P) - 1u;
+            const int r0 = i0 + g < m ? i0 + g : m - 1, r1 = i0 + g + 8 < m ? i0 + g + 8 : m - 1;
+            float d[NT][4];
+            product_row<NT>(U, r0 * ld, r1 * ld, V, ld, m, wn, lane, todo, d);
+#pragma unroll
+            for (int y = 0; y < NT; ++y)
+#pragma unroll
+                for (int h = 0; h < 4; ++h) acc[y][x][h] = d[y][h];
+        }
+    };
+    float big = 0.f, any = 0.f;  // the largest magnitude of G, L, R and L'; of products with a coupling
+    bool finite = true;
+    float acc[NT][NT][4];
+    load(sm, at(a.Di, sg.za));
+    copy_wait();
+    __syncthreads();
+    for (long long k = sg.za;; ++k) {
+        float *const X = sm + xo, *const sB = sm + bo;
+        if (k > sg.za) {
+            subtract_product<NT>(X, sA, sG, nzr + a.mp, ld, m, wm, wn, lane);
+            if (!sg.first) {
+                rows_times(acc, sA, sL, nzr + a.mp);
+                __syncthreads();
+                if (k < sg.ze) store_tiles<NT>(sL, nullptr, acc, -1.f, ld, m, wm, wn, lane, any, finite);
+                else store_tiles<NT>(nullptr, at(p.Ar, sg.row), acc, -1.f, ld, m, wm, wn, lane, any, finite);
+            }
+            __syncthreads();
+        }
+        if (k == sg.ze) {
+            for (int i = 4 * tid; i < mw; i += 4 * kFactorThreads)
+                *reinterpret_cast<float4 *>(at(p.Dr, sg.row) + i) = *reinterpret_cast<const float4 *>(X + i);
+            break;
+        }
+        load(sG, at(a.Gt, k));
+        load_nz(0, k, 0);
+        if (k == sg.za && !sg.first) load(sL, at(a.At, k));
+        load(sA, at(a.At, k + 1));
+        load_nz(1, k + 1, 1);
+        if (five) load(sB, at(a.Di, k + 1));
+        if (invert<NT>(X, ld, m, cur, pos, rowbuf, tid) && lane == 0) s_bad = 1;
+        copy_wait();
+        __syncthreads();
+        store_inverse<NT>(at(a.Di, k), X, ld, m, cur, pos, tid);
+        inverse_times<NT>(acc, X, sG, nzr, cur, ld, m, wm, wn, lane);
+        __syncthreads();
+        store_tiles<NT>(sG, at(a.Gt, k), acc, 1.f, ld, m, wm, wn, lane, big, finite);
+        if (!sg.first) {
+            inverse_times<NT>(acc, X, sL, nullptr, cur, ld, m, wm, wn, lane);
+            __syncthreads();
+            store_tiles<NT>(sL, at(p.Lt, k), acc, 1.f, ld, m, wm, wn, lane, big, finite);
+        }
+        if (five) {
+            const int t = xo;
+            xo = bo;
+            bo = t;
+        } else {
+            load(X, at(a.Di, k + 1));
+            copy_wait();
+        }
+        __syncthreads();
+    }
+    if (!sg.first) {
+        // R and L' back to the segment's first zone, in sG and sL
+        for (long long k = sg.ze - 2; k >= sg.za; --k) {
+            __syncthreads();
+            load(sA, at(a.Gt, k));
+            copy_wait();
+            __syncthreads();
+            rows_times(acc, sA, sG, nullptr);
+            __syncthreads();
+            store_tiles<NT>(sG, nullptr, acc, -1.f, ld, m, wm, wn, lane, big, finite);
+            rows_times(acc, sA, sL, nullptr);
+            const int g = lane >> 2, q = lane & 3;
+            const float *L = at(p.Lt, k);
+#pragma unroll
+            for (int x = 0; x < NT; ++x)
+#pragma unroll
+                for (int y = 0; y < NT; ++y)
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) {
+                        const int i = 16 * (wm * NT + x) + g + 8 * (h >> 1), c = 8 * (wn * NT + y) + 2 * q + (h & 1);
+                        if (i < m && c < m) acc[y][x][h] -= L[i * ld + c];
+                    }
+            __syncthreads();
+            store_tiles<NT>(sL, nullptr, acc, -1.f, ld, m, wm, wn, lane, big, finite);
+        }
+        // the terms of the zone before the segment
+        __syncthreads();
+        load(sA, at(a.Gt, sg.za - 1));
+        load_nz(0, sg.za - 1, 0);
+        copy_wait();
+        __syncthreads();
+        rows_times(acc, sA, sG, nzr);
+        store_tiles<NT>(nullptr, at(p.Cr, sg.row - 1), acc, -1.f, ld, m, wm, wn, lane, any, finite);
+        rows_times(acc, sA, sL, nzr);
+        store_tiles<NT>(nullptr, at(p.Er, sg.row - 1), acc, 1.f, ld, m, wm, wn, lane, any, finite);
+    }
+    if (!finite || big > kMaxGrowth) s_bad = 1;
+    __syncthreads();
+    if (tid == 0 && s_bad) atomicOr(p.pbad + blockIdx.x / p.parts, 1);
+}
+
+// Br_e's last term, and what k_btd_factor wants of the segments' system besides: zero patterns and arrival counts.
+__global__ void __launch_bounds__(256) k_btd_join(const SegArgs p) {
+    Seg sg;
+    if (!sg.find(p, blockIdx.x, true)) return;
+    const BtdArgs &a = p.a;
+    const int mw = a.m * a.ld;
+    if (!sg.last)
+        for (int i = 4 * (256 * blockIdx.y + threadIdx.x); i < mw; i += 4 * 256 * gridDim.y) {  // (the padding is zero in both)
+            float4 *d = reinterpret_cast<float4 *>(p.Dr + (size_t)sg.row * mw + i);
+            const float4 u = *d, v = *reinterpret_cast<const float4 *>(p.Er + (size_t)sg.row * mw + i);
+            *d = make_float4(u.x - v.x, u.y - v.y, u.z - v.z, u.w - v.w);
+        }
+    if (blockIdx.y) return;
+    for (int i = threadIdx.x; i < 2 * a.mp; i += 256) p.nzr[(size_t)sg.row * 2 * a.mp + i] = (unsigned short)((1u << (a.mp / 8)) - 1u);
+    if (threadIdx.x == 0) p.zbadr[sg.row] = 0;
+}
+
+// The blocks that k_btd_segment has overwritten, again, for the rays that it could not do.
+__global__ void __launch_bounds__(256) k_btd_again(const BtdArgs a) {
+    long long z0, z1;
+    if (!ray_range(a, blockIdx.x, z0, z1)) return;
+    const long long mm = (long long)a.m * a.m;
+    for (long long e = z0 * mm + blockIdx.y * 256 + threadIdx.x; e < z1 * mm; e += 256 * gridDim.y) {
+        const long long row = e / a.m, at = row * a.ld + (e - row * a.m);
+        a.Di[at] = btd_f32(a.B[e]);
+        a.Gt[at] = btd_f32(a.C[e]);
     }
 }
 
@@ -1089,6 +1347,191 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_btd_sweep(const BtdArgs a)
     asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
+// The sweeps of rays in segments, a CTA per segment, with the steps and the ring of k_btd_sweep.
+// BACK false: y_k outwards, and the right-hand sides of the segments' system (zero before):
+// rr_e += rhs_e - A_e y_{e-1}, rr_p -= C_p y'_a, y' = y_k - G_k y'_{k+1} (two terms: their order doesn't matter).
+// BACK true: from that system's solution, x_k = y_k - G_k x_{k+1} - L_k x_p inwards; x += (FIRST: =).
+// GB300, m = 84, 400 zones, one ray: 0.55 ms by two CTAs -> 0.029 outwards,
+// 0.049 for the segments' system and 0.028 inwards.
+template <bool BACK, bool FIRST, int NT>
+__global__ void __launch_bounds__(kSweepThreads, 1) k_btd_seg_sweep(const SegArgs pa) {
+    extern __shared__ __align__(16) float sbuf[];
+    const BtdArgs &a = pa.a;
+    Seg sg;
+    if (!sg.find(pa, blockIdx.x, true)) return;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gl = lane & 7;
+    const int m = a.m, lw = a.ld, nb = a.nring, mw = m * lw;
+    float *vin = sbuf + nb * mw;         // [2][VX_BTD_MAX_M] the vector of a step and of the next
+    float *vx = vin + 2 * VX_BTD_MAX_M;  // [VX_BTD_MAX_M] x_p
+    for (int i = tid; i < 3 * VX_BTD_MAX_M; i += kSweepThreads) vin[i] = 0.f;
+    const int n = (int)(sg.ze - sg.za), nf = 2 * n - 1, ns = sg.first ? 1 : 2;
+    const int total = n == 0 ? 0 : BACK ? ns * n : nf + 1 + (sg.first ? 0 : n);
+    const unsigned sb = (unsigned)__cvta_generic_to_shared(sbuf) + 16u * (unsigned)tid;
+    int si = 0, bi = 0;  // the next step to bring in and its buffer
+    auto issue = [&]() {
+        if (si < total) {
+            const float *src;
+            if (BACK) src = (ns == 1 || (si & 1) ? a.Gt : pa.Lt) + (size_t)(sg.ze - 1 - si / ns) * mw;
+            else if (si <= nf) src = ((si & 1) ? a.At : a.Di) + (size_t)(sg.za + (si + 1) / 2) * mw;  // si = nf: A_e
+            else src = a.Gt + (size_t)(sg.ze - 1 - (si - nf)) * mw;                                   // last: C_p
+            src += 4 * tid;
+            const unsigned dst = sb + 4u * (unsigned)(bi * mw);
+#pragma unroll
+            for (int i = 0; i <= NT * NT; ++i)  // 1024 (NT^2 + 1) >= m lw
+                if (4 * (tid + kSweepThreads * i) < mw)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16u * (unsigned)(kSweepThreads * i)),
+                                 "l"(src + 4 * kSweepThreads * i)
+                                 : "memory");
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        ++si;
+        bi = bi + 1 == nb ? 0 : bi + 1;
+    };
+    for (int s = 0; s < nb - 1; ++s) issue();
+    bool own[NT];  // this lane keeps the row's vector entries
+    int row[NT];
+#pragma unroll
+    for (int u = 0; u < NT; ++u) {
+        row[u] = 4 * warp + 32 * u + (lane >> 3);
+        own[u] = gl == 0 && row[u] < m;
+    }
+    int bs = 0, par = 0;  // the step's buffer and vector
+    float p[NT], q[NT];
+    auto step = [&](float (&p)[NT], const float *v) {  // p = (the step's matrix) v, in every lane of a row's group
+        if (nb == 4) asm volatile("cp.async.wait_group 2;" ::: "memory");
+        else if (nb == 3) asm volatile("cp.async.wait_group 1;" ::: "memory");
+        else asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();  // ... for every thread; the step before is done with its buffer and its vector
+        issue();
+        const float *M = sbuf + bs * mw + 4 * gl;
+        float4 x[NT];
+#pragma unroll
+        for (int c = 0; c < NT; ++c) x[c] = *reinterpret_cast<const float4 *>(v + 4 * gl + 32 * c);
+#pragma unroll
+        for (int u = 0; u < NT; ++u) {
+            const float *r = M + min(row[u], m - 1) * lw;
+            float e0 = 0.f, e1 = 0.f;
+#pragma unroll
+            for (int c = 0; c < NT; ++c) {
+                float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (c < NT - 1 || 32 * c + 4 * gl < lw) w = *reinterpret_cast<const float4 *>(r + 32 * c);
+                e0 = fmaf(w.x, x[c].x, e0);
+                e1 = fmaf(w.y, x[c].y, e1);
+                e0 = fmaf(w.z, x[c].z, e0);
+                e1 = fmaf(w.w, x[c].w, e1);
+            }
+            p[u] = e0 + e1;
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1)
+#pragma unroll
+            for (int u = 0; u < NT; ++u) p[u] += __shfl_xor_sync(0xffffffffu, p[u], o);
+        bs = bs + 1 == nb ? 0 : bs + 1;
+    };
+    // the vector of the next step; that step's barrier publishes it, and the one before it has read the other half
+    auto give = [&](const float (&v)[NT]) {
+        par ^= 1;
+#pragma unroll
+        for (int u = 0; u < NT; ++u)
+            if (own[u]) vin[VX_BTD_MAX_M * par + row[u]] = v[u];
+    };
+    auto given = [&]() { return (const float *)(vin + VX_BTD_MAX_M * par); };
+    double dn[kAhead][NT];  // right-hand sides (BACK: x) of the next zones
+    float yn[kAhead][NT], t[NT];
+    auto y_at = [&](long long k, int u) { return own[u] && k >= sg.za ? a.y[k * m + row[u]] : 0.f; };
+    if (!BACK) {
+        auto rhs_at = [&](long long k, int u) { return own[u] && k <= sg.ze ? a.rhs[k * m + row[u]] : 0.0; };
+#pragma unroll
+        for (int u = 0; u < NT; ++u) {
+            t[u] = (float)rhs_at(sg.za, u);
+#pragma unroll
+            for (int h = 0; h < kAhead; ++h) dn[h][u] = rhs_at(sg.za + 1 + h, u);
+        }
+        if (n == 0) {
+#pragma unroll
+            for (int u = 0; u < NT; ++u)
+                if (own[u]) atomicAdd(pa.rr + sg.row * m + row[u], (double)t[u]);
+            return;
+        }
+        __syncthreads();
+        give(t);
+        for (long long k = sg.za; k < sg.ze; ++k) {
+            step(p, given());  // y_k
+            give(p);
+#pragma unroll
+            for (int u = 0; u < NT; ++u)
+                if (own[u]) a.y[k * m + row[u]] = p[u];
+            step(q, given());  // A_{k+1} y_k
+#pragma unroll
+            for (int u = 0; u < NT; ++u) {
+                t[u] = (float)dn[0][u] - q[u];
+                dn[0][u] = dn[1][u];
+                dn[1][u] = rhs_at(k + 3, u);
+            }
+            if (k + 1 < sg.ze) give(t);
+        }
+#pragma unroll
+        for (int u = 0; u < NT; ++u)
+            if (own[u]) atomicAdd(pa.rr + sg.row * m + row[u], (double)t[u]);
+        if (sg.first) return;
+#pragma unroll
+        for (int u = 0; u < NT; ++u)
+#pragma unroll
+            for (int h = 0; h < kAhead; ++h) yn[h][u] = y_at(sg.ze - 2 - h, u);
+        give(p);
+        for (long long k = sg.ze - 2; k >= sg.za; --k) {
+            step(q, given());  // G_k y'_{k+1}
+#pragma unroll
+            for (int u = 0; u < NT; ++u) {
+                t[u] = yn[0][u] - q[u];
+                yn[0][u] = yn[1][u];
+                yn[1][u] = y_at(k - 2, u);
+            }
+            give(t);
+        }
+        step(q, given());  // C_p y'_a
+#pragma unroll
+        for (int u = 0; u < NT; ++u)
+            if (own[u]) atomicAdd(pa.rr + (sg.row - 1) * m + row[u], (double)-q[u]);
+    } else {
+        auto x_at = [&](long long k, int u) { return !FIRST && own[u] && k >= sg.za ? a.x[k * m + row[u]] : 0.0; };
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < NT; ++u) {
+            const double xe = own[u] ? pa.xr[sg.row * m + row[u]] : 0.0;
+            t[u] = (float)xe;
+            if (own[u]) {
+                if (!sg.first) vx[row[u]] = (float)pa.xr[(sg.row - 1) * m + row[u]];
+                double *x = a.x + sg.ze * m + row[u];
+                *x = FIRST ? xe : *x + xe;
+            }
+#pragma unroll
+            for (int h = 0; h < kAhead; ++h) {
+                yn[h][u] = y_at(sg.ze - 1 - h, u);
+                dn[h][u] = x_at(sg.ze - 1 - h, u);
+            }
+        }
+        give(t);
+        for (long long k = sg.ze - 1; k >= sg.za; --k) {
+#pragma unroll
+            for (int u = 0; u < NT; ++u) q[u] = 0.f;
+            if (!sg.first) step(q, vx);  // L_k x_p
+            step(p, given());            // G_k x_{k+1}
+#pragma unroll
+            for (int u = 0; u < NT; ++u) {
+                t[u] = yn[0][u] - q[u] - p[u];
+                if (own[u]) a.x[k * m + row[u]] = FIRST ? (double)t[u] : dn[0][u] + (double)t[u];
+                yn[0][u] = yn[1][u];
+                dn[0][u] = dn[1][u];
+                yn[1][u] = y_at(k - 2, u);
+                dn[1][u] = x_at(k - 2, u);
+            }
+            give(t);
+        }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
 // The FP64 residual, a ray's zones split over blockIdx.y CTAs, a warp per eight rows of a zone. Every matrix
 // element costs one FP64 FMA, which GB300 issues at 2 per clock and SM (less than HBM can feed), so the layout
 // minimises FP64 instructions beyond those FMAs and leaves out what is known to be zero: groups of eight
@@ -1201,8 +1644,29 @@ static cudaError_t launch_sweep(int m, int grid, size_t smem, cudaStream_t s, co
     return cudaLaunchKernelEx(&cfg, k_btd_sweep<F, L, 4>, a);
 }
 
+template <bool BACK, bool FIRST>
+static const void *seg_sweep_kernel(int m) {
+    if (m <= 32) return (const void *)k_btd_seg_sweep<BACK, FIRST, 1>;
+    if (m <= 64) return (const void *)k_btd_seg_sweep<BACK, FIRST, 2>;
+    if (m <= 96) return (const void *)k_btd_seg_sweep<BACK, FIRST, 3>;
+    return (const void *)k_btd_seg_sweep<BACK, FIRST, 4>;
+}
+static const void *segment_kernel(int m) {
+    if (m <= 32) return (const void *)k_btd_segment<1>;
+    if (m <= 64) return (const void *)k_btd_segment<2>;
+    if (m <= 96) return (const void *)k_btd_segment<3>;
+    return (const void *)k_btd_segment<4>;
+}
+static cudaError_t launch_seg(const void *kernel, int grid, size_t smem, cudaStream_t s, SegArgs &p) {
+    void *args[1] = {&p};
+    return cudaLaunchKernel(kernel, dim3((unsigned)grid), dim3(kFactorThreads), args, smem, s);
+}
+
 // Shared memory that lets two CTAs share an SM (228 KB, 1 KB of it reserved per CTA), and one CTA's limit.
 constexpr size_t kSmemHalf = 113 * 1024 - 64, kSmemFull = 226 * 1024;
+
+// Zones from which on segments are laid out, and for which they have room.
+constexpr long long kSegMinZones = 40, kSegMaxZones = 16384;
 
 struct vx_btd {
     int m = 0, ld = 0, mp = 0, nbuf = 3, nring = 2, n_refine = 0;
@@ -1213,6 +1677,14 @@ struct vx_btd {
     int slots = 0;  // factor CTAs the device holds at once
     int *zbad = nullptr, *zmid = nullptr, *flag = nullptr;  // flag[0]: numeric flag, flag[1]: offsets invalid
     double *r = nullptr;
+    // segments: null, or rows of the segments' system (one per SM) and zones that L has room for
+    int sms = 1, seg_nbuf = 0;
+    long long seg_zones = 0;
+    size_t smem_seg = 0;
+    float *Lt = nullptr, *Sr = nullptr;  // Sr: the system's four blocks per row, then its y
+    unsigned short *nzr = nullptr;
+    int *zr = nullptr;                   // zbad, zmid of that system, pbad
+    double *vr = nullptr;                // its right-hand sides and solution
 };
 
 static void btd_free(vx_btd *h) {
@@ -1224,6 +1696,11 @@ static void btd_free(vx_btd *h) {
     cudaFree(h->y);
     cudaFree(h->zbad);
     cudaFree(h->zmid);
+    cudaFree(h->Lt);
+    cudaFree(h->Sr);
+    cudaFree(h->nzr);
+    cudaFree(h->zr);
+    cudaFree(h->vr);
     cudaFree(h->flag);
     cudaFree(h->r);
     delete h;
@@ -1266,20 +1743,46 @@ extern "C" vx_status vx_btd_create(int m, long long max_zones, int n_refine, vx_
     if (e == cudaSuccess) e = cudaMalloc(&h->r, zc * m * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&h->flag, 2 * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(h->flag, 0, 2 * sizeof(int));
+    int dev = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev);
+    h->slots = h->sms * (h->smem <= kSmemHalf && m <= 96 ? 2 : 1);
     if (h->ld != m)  // the columns that pad a row are read by the sweeps and never written
         for (float *w : {h->Di, h->Gt, h->At})
             if (e == cudaSuccess) e = cudaMemset(w, 0, zc * mw * sizeof(float));
     // the kernels' limit, not this handle's size: handles of several m share them
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(factor_kernel(m), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFull);
-    int dev = 0, sms = 1;
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    h->slots = sms * (h->smem <= kSmemHalf && m <= 96 ? 2 : 1);
     const void *sweeps[4] = {sweep_kernel<true, true>(m), sweep_kernel<true, false>(m), sweep_kernel<false, true>(m),
                              sweep_kernel<false, false>(m)};
     for (int i = 0; i < 4 && e == cudaSuccess; ++i)
         e = cudaFuncSetAttribute(sweeps[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFull);
+    // segments where their four or five buffers fit; without the memory for them, rays go as a whole
+    h->seg_nbuf = factor_smem(m, h->ld, 5) <= kSmemFull ? 5 : factor_smem(m, h->ld, 4) <= kSmemFull ? 4 : 0;
+    if (e == cudaSuccess && h->seg_nbuf && max_zones >= kSegMinZones) {
+        const size_t rows = (size_t)h->sms;
+        h->smem_seg = factor_smem(m, h->ld, h->seg_nbuf);
+        h->seg_zones = max_zones < kSegMaxZones ? max_zones : kSegMaxZones;
+        cudaError_t q = cudaMalloc(&h->Lt, (size_t)h->seg_zones * mw * sizeof(float));
+        if (q == cudaSuccess) q = cudaMalloc(&h->Sr, rows * (4 * mw + m) * sizeof(float));
+        if (q == cudaSuccess) q = cudaMalloc(&h->nzr, rows * 2 * h->mp * sizeof(unsigned short));
+        if (q == cudaSuccess) q = cudaMalloc(&h->zr, 3 * rows * sizeof(int));
+        if (q == cudaSuccess) q = cudaMalloc(&h->vr, 2 * rows * m * sizeof(double));
+        if (q == cudaSuccess) {
+            if (h->ld != m) {
+                e = cudaMemset(h->Lt, 0, (size_t)h->seg_zones * mw * sizeof(float));
+                if (e == cudaSuccess) e = cudaMemset(h->Sr, 0, rows * 4 * mw * sizeof(float));
+            }
+            const void *ks[4] = {segment_kernel(m), seg_sweep_kernel<false, true>(m), seg_sweep_kernel<true, true>(m),
+                                 seg_sweep_kernel<true, false>(m)};
+            for (int i = 0; i < 4 && e == cudaSuccess; ++i)
+                e = cudaFuncSetAttribute(ks[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFull);
+        } else {
+            h->seg_zones = 0;
+            if (q == cudaErrorMemoryAllocation) (void)cudaGetLastError();
+            else e = q;
+        }
+    }
     if (e != cudaSuccess) {
         btd_free(h);
         return bfail(e == cudaErrorMemoryAllocation ? VX_ERR_OOM : VX_ERR_CUDA, "vx_btd_create: %s",
@@ -1348,26 +1851,90 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
                    : 1;
     a.flag = h->flag;
     a.inval = h->flag + 1;
+    a.parts = 0;
+    a.pbad = nullptr;
+    // Segments per ray: one per SM at most, and S^2 <= 3 n, about as many as make n / S zones with their extra
+    // products and S / 2 zones of the segments' system take least (S^2 = 2 n and 5 n: 4 to 12 % slower at 100
+    // zones). GB300, m = 84, by halves -> in segments: 1 ray of 400 zones 6.65 -> 1.61 ms, 8 rays 7.12 ->
+    // 2.24, 30 rays (5 segments) 8.03 -> 6.66, 38 rays (4 segments) 8.18 -> 8.12; of 100 zones, 1 ray
+    // 1.74 -> 0.82, 30 rays 2.09 -> 1.83, 38 rays 2.13 -> 2.19; of 32 zones, 8 rays 0.63 -> 0.54 but 30 rays
+    // 0.74 -> 0.76 and with m = 16 0.18 -> 0.19; of 24 zones 0.50 -> 0.49.
+    const long long mean = n_zones / n_rays;
+    int parts = n_rays < h->sms ? h->sms / n_rays : 0;
+    while (parts > 5 && (long long)parts * parts > 3 * mean) --parts;
+    const bool seg = parts >= 5 && mean >= kSegMinZones && n_zones <= h->seg_zones;
+    SegArgs p;   // the segments
+    BtdArgs b;   // their system
+    BtdArgs f = a;  // the rays whose elimination by segments failed
+    if (seg) {
+        const size_t rows = (size_t)h->sms, blk32 = rows * h->m * h->ld;
+        p.a = a;
+        p.parts = parts;
+        p.nbuf = h->seg_nbuf;
+        p.Lt = h->Lt;
+        p.Dr = h->Sr;
+        p.Cr = p.Dr + blk32;
+        p.Ar = p.Cr + blk32;
+        p.Er = p.Ar + blk32;
+        p.nzr = h->nzr;
+        p.zbadr = h->zr;
+        p.pbad = h->zr + 2 * rows;
+        p.rr = h->vr;
+        p.xr = h->vr + rows * h->m;
+        f.pbad = p.pbad;
+        b = f;
+        b.parts = parts;
+        b.halves = 2;
+        b.A = b.B = b.C = nullptr;
+        b.Di = p.Dr;
+        b.Gt = p.Cr;
+        b.At = p.Ar;
+        b.y = p.Er + blk32;
+        b.nz = p.nzr;
+        b.zbad = p.zbadr;
+        b.zmid = p.zbadr + rows;
+        b.rhs = p.rr;
+        b.x = p.xr;
+    }
     BTD_CU(cudaMemsetAsync(h->flag + 1, 0, sizeof(int), s));
-    k_btd_validate<<<(unsigned)((n_rays + 256) / 256), 256, 0, s>>>(ray_offsets, n_rays, n_zones, h->flag + 1, h->flag, h->zbad);
+    k_btd_validate<<<(unsigned)((n_rays + 256) / 256), 256, 0, s>>>(ray_offsets, n_rays, n_zones, h->flag + 1, h->flag, h->zbad,
+                                                                   f.pbad);
     BTD_CU(cudaGetLastError());
     launch_convert(h->m, n_zones, s, a);
     BTD_CU(cudaGetLastError());
+    if (seg) {
+        BTD_CU(launch_seg(segment_kernel(h->m), n_rays * parts, h->smem_seg, s, p));
+        k_btd_join<<<dim3(n_rays * parts, 4), 256, 0, s>>>(p);
+        BTD_CU(cudaGetLastError());
+        launch_factor(h->m, 2 * n_rays, h->smem, s, b);
+        BTD_CU(cudaGetLastError());
+        k_btd_again<<<dim3(n_rays, 32), 256, 0, s>>>(f);
+        BTD_CU(cudaGetLastError());
+    }
     const int ctas = a.halves * n_rays;
-    launch_factor(h->m, ctas, h->smem, s, a);
+    launch_factor(h->m, ctas, h->smem, s, f);
     BTD_CU(cudaGetLastError());
-    BTD_CU((h->n_refine == 0 ? launch_sweep<true, true> : launch_sweep<true, false>)(h->m, ctas, h->smem_sweep, s, a));
     // CTAs per ray of the residual: enough to fill the chip with few rays, at most one per eight units (row octets)
     const long long units = n_zones * ((h->m + 7) / 8);
     long long split = (8 * 152 + n_rays - 1) / n_rays, most = (units + 8 * n_rays - 1) / (8 * (long long)n_rays);
     split = split > most ? most : split;
     split = split < 16 ? 16 : split;
-    for (int it = 1; it <= h->n_refine; ++it) {
-        a.rhs = d;
-        k_btd_resid<<<dim3(n_rays, (unsigned)split), kResidThreads, 0, s>>>(a);
-        BTD_CU(cudaGetLastError());
-        a.rhs = h->r;
-        BTD_CU((it == h->n_refine ? launch_sweep<false, true> : launch_sweep<false, false>)(h->m, ctas, h->smem_sweep, s, a));
+    for (int it = 0; it <= h->n_refine; ++it) {
+        if (it > 0) {
+            k_btd_resid<<<dim3(n_rays, (unsigned)split), kResidThreads, 0, s>>>(a);
+            BTD_CU(cudaGetLastError());
+            f.rhs = p.a.rhs = h->r;
+        }
+        const bool last = it == h->n_refine;
+        if (seg) {
+            BTD_CU(cudaMemsetAsync(p.rr, 0, (size_t)n_rays * parts * h->m * sizeof(double), s));
+            BTD_CU(launch_seg(seg_sweep_kernel<false, true>(h->m), n_rays * parts, h->smem_sweep, s, p));
+            BTD_CU((launch_sweep<true, false>(h->m, 2 * n_rays, h->smem_sweep, s, b)));
+            BTD_CU(launch_seg(it == 0 ? seg_sweep_kernel<true, true>(h->m) : seg_sweep_kernel<true, false>(h->m), n_rays * parts,
+                              h->smem_sweep, s, p));
+        }
+        BTD_CU((it == 0 ? (last ? launch_sweep<true, true> : launch_sweep<true, false>)
+                        : (last ? launch_sweep<false, true> : launch_sweep<false, false>))(h->m, ctas, h->smem_sweep, s, f));
     }
     return VX_OK;
 }

@@ -1,7 +1,8 @@
-"""Few rays, each eliminated from both ends towards the middle: rays of one to nine zones and long ones, a last
-zone whose block cannot be inverted (or only with large numbers in its inverse), so that the elimination
-has to go on from the middle outwards, and a first zone for which nothing works; against the banded-LU
-oracle, and around the number of rays from which on one block of threads takes a ray."""
+"""Few rays, each eliminated from both ends towards the middle, or in segments: rays of one to nine zones and long
+ones, a zone whose block cannot be inverted (or only with large numbers in its inverse) where the
+elimination from one end can, so that the ray has to be done that way, and a first zone for which nothing
+works; against the banded-LU oracle, and around the number of rays from which on one block of threads takes a
+ray."""
 import numpy as np
 import pytest
 
@@ -68,3 +69,35 @@ def test_ray_counts(rays, zones):
     x, ok = _solve(s, m)
     assert ok
     _close(s, x, [r for r in range(rays) if s["offsets"][r] < s["offsets"][r + 1]])
+
+
+def _in_segments(m):
+    """Rays long enough to be cut into segments and, in the same call, ones that are not; with unit couplings
+    around a zone whose block is zero or small at the start, inside and at the end of a ray."""
+    zones = [1, 2, 3, 7, 8, 9, 40, 99, 100, 101, 100, 100, 100, 100]
+    s = gen.random_system(np.array(zones), m, seed=m)
+    first = [int(o) for o in s["offsets"]]
+    for r, z, f in ((10, 0, 5e-3 / np.abs(s["B"][first[10]]).max()), (11, 30, 0.0), (12, 99, 0.0), (13, 99, 1e-3)):
+        k = first[r] + z
+        if first[r] < k:
+            s["C"][k - 1] = s["A"][k] = np.eye(m)
+        if k + 1 < first[r + 1]:
+            s["A"][k + 1] = s["C"][k] = np.eye(m)
+            s["B"][k + 1] = s["B"][max(k - 1, first[r])]  # nothing cancels in the next zone's block
+        s["B"][k] *= f
+    s["A"][first[9] + 50:first[9] + 60] = 0.0  # no coupling through a whole segment
+    s["C"][first[9] + 49:first[9] + 59] = 0.0
+    return s, first
+
+
+@pytest.mark.parametrize("m", [1, 8, 13, 42, 84, 96, 113, 120])
+def test_segments(m):
+    s, first = _in_segments(m)
+    x, ok = _solve(s, m)
+    assert ok
+    _close(s, x, range(14))
+    s["B"][first[7]] = 0.0  # a ray for which nothing works
+    x, ok = _solve(s, m)
+    assert not ok
+    a, b = first[7], first[8]
+    assert np.isnan(x[a:b]).all() and np.isfinite(x[:a]).all() and np.isfinite(x[b:]).all()
