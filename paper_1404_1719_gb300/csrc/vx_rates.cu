@@ -112,7 +112,7 @@ struct vx_rates {
     // launch shapes (mixed kernels in two register budgets)
     int block = 32, block_mixed = 32;
     int grid_mixed[2][2] = {{0, 0}, {0, 0}};  // [forward, tangents][larger, smaller register budget]
-    int minb[2] = {2, 3};                      // chosen budget per kind (autotuned with VX_AUTOTUNE)
+    int minb[2] = {2, 3};                      // chosen budget per kind (autotuned with VX_AUTOTUNE; forward: mixed_budget)
     bool tuned[2] = {false, false};
     float tune_ms[2][2] = {{0, 0}, {0, 0}};
     int grid_64 = 0;
@@ -546,6 +546,18 @@ static void cache_write(const char *path, const std::string &key, const std::str
     rename(tmp.c_str(), path);
 }
 
+// The register budget of a launch: the autotuned one, else the smaller one for the tangent kernel, and for the
+// forward kernel the larger one until the batch fills its grid more than twice. Six CTAs of 128
+// threads per SM at 80 registers hide each other's MUFU and shared-memory latencies better than four at 128
+// (MUFU 55 %, FP32 pipe 50 % busy), but a zone by itself takes longer. GB300, four per SM -> six, zones at 64 nodes
+// and 21 bins: 64 74.6 -> 79.9 us, 304 115 -> 118, 1216 288 -> 273, 2400 492 -> 456, 3200 610 -> 620, 6400
+// 1196 -> 1153; at 48 nodes and eta_e to 60: 400 84 -> 86, 912 122 -> 131, 2000 234 -> 223, 9600 971 -> 942; at
+// 32 nodes and 13 bins: 400 43.7 -> 45.8, 1600 78 -> 72, 9600 293 -> 260.
+static int mixed_budget(const vx_rates *h, bool adj, long long zones) {
+    if (adj || h->tuned[0]) return h->minb[adj];
+    return zones > 2LL * h->grid_mixed[0][0] ? 3 : h->minb[0];
+}
+
 static vx_status autotune(vx_rates *h, bool adj, const vx::Launch &L, cudaStream_t s) {
     const int kind = adj ? 1 : 0;
     if (!(h->cfg.flags & VX_AUTOTUNE) || h->tuned[kind]) return VX_OK;
@@ -614,7 +626,7 @@ vx_status vx_rates_eval(vx_rates *h, const vx_batch *b, const vx_out *out, vx_st
         fill_launch(h, b, L);
         L.j0 = out->j0; L.chi0 = out->chi0; L.j1 = out->j1; L.chi1 = out->chi1; L.phi = out->phi;
         if ((st = autotune(h, false, L, s)) != VX_OK) return st;
-        const int mb = h->minb[0];
+        const int mb = mixed_budget(h, false, b->n_zones);
         int grid = (int)std::min<long long>(h->grid_mixed[0][mb - 2], b->n_zones);
         if (graph) return launch_graph(h, 0, vx::kernel_mixed(false, mb, h->common.n_e, h->common.split != 0, h->common.precise != 0), &L, grid, h->block_mixed, h->smem_fwd, s);
         VX_CU(cudaMemsetAsync(h->d_counter, 0, sizeof(unsigned long long), s));
@@ -704,7 +716,7 @@ vx_status vx_rates_spectral(vx_rates *h, const vx_batch *b, const vx_out *grad_o
     L.grad_H = grad_H;
     if (grad_J) { L.g_j0 = grad_out->j0; L.g_chi0 = grad_out->chi0; L.g_j1 = grad_out->j1; L.g_chi1 = grad_out->chi1; }
     if ((st = autotune(h, false, L, s)) != VX_OK) return st;
-    const int mb = h->minb[0];
+    const int mb = mixed_budget(h, false, b->n_zones);
     int grid = (int)std::min<long long>(h->grid_mixed[0][mb - 2], b->n_zones);
     if (h->cfg.flags & VX_USE_GRAPH)
         return launch_graph(h, 0, vx::kernel_mixed(false, mb, h->common.n_e, h->common.split != 0, h->common.precise != 0), &L, grid, h->block_mixed, h->smem_fwd, s);
@@ -826,7 +838,7 @@ static vx_status host_run(vx_rates *h, const vx_batch *b, const HostIO &io) {
         if (io.grad_J) { L.grad_J = d_gJ = take(SN * n); L.grad_H = d_gH = take(SN * n); }
         if (io.blocks) L.blocks = d_blk = take(4 * N * N * S * n);
         if ((st = autotune(h, adj, L, s)) != VX_OK) return st;
-        const int mb = h->minb[kind];
+        const int mb = mixed_budget(h, adj, n);
         const int grid = (int)std::min<long long>(h->grid_mixed[kind][mb - 2], n);
         VX_CU(cudaMemsetAsync(L.counter, 0, sizeof(unsigned long long), s));
         VX_CU(vx::launch_mixed(adj, mb, L, grid, h->block_mixed, smem, s));
