@@ -1,6 +1,6 @@
-"""The forward kernel of the mixed form, whose register budget and use of the work counter follow the number of
-zones: a zone's rates and spectral blocks have the same bits in any batch, on either side of one and of two
-zones per CTA of the larger budget's grid, replayed from a captured graph as well."""
+"""The forward kernel of the mixed form, whose register budget follows the number of zones: a zone's rates have
+the same bits in any batch, on either side of one and of two zones per CTA of the larger budget's grid,
+and replayed from a captured graph."""
 import numpy as np
 import pytest
 
