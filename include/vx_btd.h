@@ -53,7 +53,7 @@ typedef struct vx_btd vx_btd;
 /* Creates a solver for m unknowns per zone (1 .. VX_BTD_MAX_M) and batches of at most max_zones
  * zones (>= 0), with n_refine FP64 refinement sweeps (0 .. VX_BTD_MAX_REFINE; 0 leaves the FP32
  * solution). Allocates the device workspace: 12 m (m + 7) + 4 (m + 7) + 12 m + 8 bytes per zone at most, and for
- * the segments (m up to about 110) 4 m (m + 7) for each of the first 16384 zones and 16 m (m + 8) per SM; without the
+ * the segments (m up to about 110) 4 m (m + 7) for each of the first 16384 zones and 36 m (m + 8) per SM; without the
  * memory for the latter, rays are not cut into segments. *out is set to NULL on failure. Errors: VX_ERR_INVALID_ARG, VX_ERR_OOM, VX_ERR_CUDA. */
 vx_status vx_btd_create(int m, long long max_zones, int n_refine, vx_btd **out);
 

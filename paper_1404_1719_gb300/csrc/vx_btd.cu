@@ -83,8 +83,9 @@ struct BtdArgs {
     int *zbad, *zmid, *flag;  // at a ray's first zone: a pivot failed; the zone its eliminations meet at, from there
     const int *inval;  // set by k_btd_validate when the offsets are not a partition of the zones
     // Rays in segments (k_btd_segment): parts > 0: this is the system of the segments' last zones, ray r's from r parts
-    // on; parts = 0 and pbad: only the rays that pbad marks, whose elimination by segments failed
-    int parts;
+    // on (above > 0: of segments of such a system, of `above` parts a ray); parts = 0 and pbad: only the rays
+    // that pbad marks, whose elimination by segments failed
+    int parts, above;
     int *pbad;
 };
 
@@ -101,7 +102,7 @@ __device__ __forceinline__ bool ray_range(const BtdArgs &a, int ray, long long &
     z1 = a.off[ray + 1];
     if (a.pbad && (a.parts > 0) == (a.pbad[ray] != 0)) return false;
     if (a.parts > 0) {
-        const int s = seg_count(z1 - z0, a.parts);
+        const int s = seg_count(a.above > 0 ? seg_count(z1 - z0, a.above) : z1 - z0, a.parts);
         z0 = (long long)ray * a.parts;
         z1 = z0 + s;
     }
@@ -922,13 +923,13 @@ __global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(c
 // and then once more inwards for the segment's first zone, x_a = y' - R x_e - L' x_p (R_k = -G_k R_{k+1},
 // L'_k = L_k - G_k L'_{k+1}). That leaves a block-tridiagonal system of the segments' last zones,
 //   Ar_e = -A_e L_{e-1},  Br_e = B_e - A_e G_{e-1} - C_e L'_{next a},  Cr_e = -C_e R_{next a},
-// for k_btd_factor. A ray in which a pivot fails, or an entry of G, L, R or L' is above kMaxGrowth, is
+// for k_btd_factor, or of enough rows to be cut into segments once more. A ray in which a pivot fails, or an entry of G, L, R or L' is above kMaxGrowth, is
 // done again as a whole by k_btd_factor (pbad). The time is that of n / S + S / 2 zones, not n / 2.
-// GB300, m = 84, 400 zones, one ray: 5.11 ms by two CTAs -> 0.58 ms for 34 segments and 0.66 ms for their
-// last zones.
+// GB300, m = 84, 400 zones, one ray: 5.11 ms by two CTAs -> 0.27 ms for 69 segments, 0.29 for 14 of
+// their last zones and 0.29 for those segments' last zones (0.58 and 0.66 with 34 segments and one level).
 struct SegArgs {
     BtdArgs a;
-    int parts, nbuf;
+    int parts, above, nbuf;     // above: parts of the level whose last zones these segments are made of, or 0
     float *Lt;                  // L_k, per zone
     float *Dr, *Cr, *Ar, *Er;   // [n_rays][parts] Br_e without its last term, Cr_e, Ar_e, that term
     unsigned short *nzr;        // zero patterns of Cr, Ar: none
@@ -943,7 +944,11 @@ struct Seg {
     __device__ __forceinline__ bool find(const SegArgs &p, int block, bool good) {
         const int ray = block / p.parts, i = block % p.parts;
         if (*p.a.inval || (good && p.pbad[ray])) return false;
-        const long long z0 = p.a.off[ray], n = p.a.off[ray + 1] - z0;
+        long long z0 = p.a.off[ray], n = p.a.off[ray + 1] - z0;
+        if (p.above > 0) {
+            n = seg_count(n, p.above);
+            z0 = (long long)ray * p.above;
+        }
         const int S = seg_count(n, p.parts);
         if (i >= S) return false;
         za = z0 + n * i / S;
@@ -961,7 +966,7 @@ __global__ void __launch_bounds__(kFactorThreads, 1) k_btd_segment(const SegArgs
     __shared__ int s_bad;
     const BtdArgs &a = p.a;
     Seg sg;
-    if (!sg.find(p, blockIdx.x, false)) return;
+    if (!sg.find(p, blockIdx.x, p.above > 0)) return;
     const int m = a.m, ld = a.ld, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wm = warp & 1, wn = warp >> 1;
     const int bs = factor_buf(m, ld), P = (m + 7) >> 3, mw = m * ld;
     const bool five = p.nbuf == 5;  // a buffer for the next zone's B
@@ -1351,8 +1356,8 @@ __global__ void __launch_bounds__(kSweepThreads, 2) k_btd_sweep(const BtdArgs a)
 // BACK false: y_k outwards, and the right-hand sides of the segments' system (zero before):
 // rr_e += rhs_e - A_e y_{e-1}, rr_p -= C_p y'_a, y' = y_k - G_k y'_{k+1} (two terms: their order doesn't matter).
 // BACK true: from that system's solution, x_k = y_k - G_k x_{k+1} - L_k x_p inwards; x += (FIRST: =).
-// GB300, m = 84, 400 zones, one ray: 0.55 ms by two CTAs -> 0.029 outwards,
-// 0.049 for the segments' system and 0.028 inwards.
+// GB300, m = 84, 400 zones, one ray: 0.55 ms by two CTAs -> 0.016 outwards
+// and 0.016 inwards for 69 segments, 0.013 + 0.013 for 14 of their last zones, 0.025 for those' last zones.
 template <bool BACK, bool FIRST, int NT>
 __global__ void __launch_bounds__(kSweepThreads, 1) k_btd_seg_sweep(const SegArgs pa) {
     extern __shared__ __align__(16) float sbuf[];
@@ -1666,7 +1671,7 @@ static cudaError_t launch_seg(const void *kernel, int grid, size_t smem, cudaStr
 constexpr size_t kSmemHalf = 113 * 1024 - 64, kSmemFull = 226 * 1024;
 
 // Zones from which on segments are laid out, and for which they have room.
-constexpr long long kSegMinZones = 40, kSegMaxZones = 16384;
+constexpr long long kSegMinZones = 40, kSegMaxZones = 16384, kSegTwoLevels = 150;
 
 struct vx_btd {
     int m = 0, ld = 0, mp = 0, nbuf = 3, nring = 2, n_refine = 0;
@@ -1681,10 +1686,11 @@ struct vx_btd {
     int sms = 1, seg_nbuf = 0;
     long long seg_zones = 0;
     size_t smem_seg = 0;
-    float *Lt = nullptr, *Sr = nullptr;  // Sr: the system's four blocks per row, then its y
-    unsigned short *nzr = nullptr;
-    int *zr = nullptr;                   // zbad, zmid of that system, pbad
-    double *vr = nullptr;                // its right-hand sides and solution
+    float *Lt = nullptr, *Sr = nullptr;  // Lt: of the zones and of the system's rows; Sr: per level, the system's
+                                         // four blocks per row, then the levels' y
+    unsigned short *nzr = nullptr;       // per level
+    int *zr = nullptr;                   // per level zbad, zmid of that system; pbad
+    double *vr = nullptr;                // right-hand sides of both levels' systems, then the solutions
 };
 
 static void btd_free(vx_btd *h) {
@@ -1763,15 +1769,15 @@ extern "C" vx_status vx_btd_create(int m, long long max_zones, int n_refine, vx_
         const size_t rows = (size_t)h->sms;
         h->smem_seg = factor_smem(m, h->ld, h->seg_nbuf);
         h->seg_zones = max_zones < kSegMaxZones ? max_zones : kSegMaxZones;
-        cudaError_t q = cudaMalloc(&h->Lt, (size_t)h->seg_zones * mw * sizeof(float));
-        if (q == cudaSuccess) q = cudaMalloc(&h->Sr, rows * (4 * mw + m) * sizeof(float));
-        if (q == cudaSuccess) q = cudaMalloc(&h->nzr, rows * 2 * h->mp * sizeof(unsigned short));
-        if (q == cudaSuccess) q = cudaMalloc(&h->zr, 3 * rows * sizeof(int));
-        if (q == cudaSuccess) q = cudaMalloc(&h->vr, 2 * rows * m * sizeof(double));
+        cudaError_t q = cudaMalloc(&h->Lt, (h->seg_zones + rows) * mw * sizeof(float));
+        if (q == cudaSuccess) q = cudaMalloc(&h->Sr, 2 * rows * (4 * mw + m) * sizeof(float));
+        if (q == cudaSuccess) q = cudaMalloc(&h->nzr, 2 * rows * 2 * h->mp * sizeof(unsigned short));
+        if (q == cudaSuccess) q = cudaMalloc(&h->zr, 5 * rows * sizeof(int));
+        if (q == cudaSuccess) q = cudaMalloc(&h->vr, 4 * rows * m * sizeof(double));
         if (q == cudaSuccess) {
             if (h->ld != m) {
-                e = cudaMemset(h->Lt, 0, (size_t)h->seg_zones * mw * sizeof(float));
-                if (e == cudaSuccess) e = cudaMemset(h->Sr, 0, rows * 4 * mw * sizeof(float));
+                e = cudaMemset(h->Lt, 0, (h->seg_zones + rows) * mw * sizeof(float));
+                if (e == cudaSuccess) e = cudaMemset(h->Sr, 0, 2 * rows * (4 * mw + m) * sizeof(float));
             }
             const void *ks[4] = {segment_kernel(m), seg_sweep_kernel<false, true>(m), seg_sweep_kernel<true, true>(m),
                                  seg_sweep_kernel<true, false>(m)};
@@ -1851,7 +1857,7 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
                    : 1;
     a.flag = h->flag;
     a.inval = h->flag + 1;
-    a.parts = 0;
+    a.parts = a.above = 0;
     a.pbad = nullptr;
     // Segments per ray: one per SM at most, and S^2 <= 3 n, about as many as make n / S zones with their extra
     // products and S / 2 zones of the segments' system take least (S^2 = 2 n and 5 n: 4 to 12 % slower at 100
@@ -1860,41 +1866,58 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
     // 1.74 -> 0.82, 30 rays 2.09 -> 1.83, 38 rays 2.13 -> 2.19; of 32 zones, 8 rays 0.63 -> 0.54 but 30 rays
     // 0.74 -> 0.76 and with m = 16 0.18 -> 0.19; of 24 zones 0.50 -> 0.49.
     const long long mean = n_zones / n_rays;
-    int parts = n_rays < h->sms ? h->sms / n_rays : 0;
+    const int most_parts = n_rays < h->sms ? h->sms / n_rays : 0;
+    int parts = most_parts, top = 0;
     while (parts > 5 && (long long)parts * parts > 3 * mean) --parts;
     const bool seg = parts >= 5 && mean >= kSegMinZones && n_zones <= h->seg_zones;
-    SegArgs p;   // the segments
-    BtdArgs b;   // their system
+    // Two levels where there is room for more: S^1.5 <= 1.45 n segments of the ray, and 1.75 S^0.5 of their system
+    // (at 48, 58 and 38 us a zone of either level and of the last system, that takes least).
+    // GB300, m = 84, one level -> two: 1 ray of 100 zones 0.82 -> 0.82 ms, 150 1.03 -> 0.86, 400 1.61 -> 1.16, 1000
+    // 2.60 -> 1.64; 4 rays of 150 1.10 -> 0.95, 400 1.78 -> 1.52; m = 8, 100 zones 0.22 -> 0.23, 400 0.32 -> 0.28.
+    if (seg && mean >= kSegTwoLevels && most_parts >= 32) {
+        parts = most_parts;
+        while (4.0 * parts * parts * parts > 8.4 * (double)mean * (double)mean) --parts;
+        top = parts;
+        while (16ll * top * top > 49ll * parts) --top;
+    }
+    const int levels = top > 0 ? 2 : 1;
+    SegArgs p[2];   // the segments
+    BtdArgs b;      // the last level's system
     BtdArgs f = a;  // the rays whose elimination by segments failed
     if (seg) {
-        const size_t rows = (size_t)h->sms, blk32 = rows * h->m * h->ld;
-        p.a = a;
-        p.parts = parts;
-        p.nbuf = h->seg_nbuf;
-        p.Lt = h->Lt;
-        p.Dr = h->Sr;
-        p.Cr = p.Dr + blk32;
-        p.Ar = p.Cr + blk32;
-        p.Er = p.Ar + blk32;
-        p.nzr = h->nzr;
-        p.zbadr = h->zr;
-        p.pbad = h->zr + 2 * rows;
-        p.rr = h->vr;
-        p.xr = h->vr + rows * h->m;
-        f.pbad = p.pbad;
+        const size_t rows = (size_t)h->sms, mw = (size_t)h->m * h->ld, vec32 = rows * h->m;
+        f.pbad = h->zr + 4 * rows;
         b = f;
-        b.parts = parts;
-        b.halves = 2;
         b.A = b.B = b.C = nullptr;
-        b.Di = p.Dr;
-        b.Gt = p.Cr;
-        b.At = p.Ar;
-        b.y = p.Er + blk32;
-        b.nz = p.nzr;
-        b.zbad = p.zbadr;
-        b.zmid = p.zbadr + rows;
-        b.rhs = p.rr;
-        b.x = p.xr;
+        b.halves = 2;
+        for (int l = 0; l < levels; ++l) {
+            SegArgs &q = p[l];
+            q.a = l ? b : a;
+            q.parts = l ? top : parts;
+            q.above = l ? parts : 0;
+            q.nbuf = h->seg_nbuf;
+            q.Lt = h->Lt + (l ? h->seg_zones * mw : 0);
+            q.Dr = h->Sr + l * rows * 4 * mw;
+            q.Cr = q.Dr + rows * mw;
+            q.Ar = q.Cr + rows * mw;
+            q.Er = q.Ar + rows * mw;
+            q.nzr = h->nzr + l * rows * 2 * h->mp;
+            q.zbadr = h->zr + l * 2 * rows;
+            q.pbad = f.pbad;
+            q.rr = h->vr + l * vec32;
+            q.xr = h->vr + (2 + l) * vec32;
+            b.parts = q.parts;
+            b.above = q.above;
+            b.Di = q.Dr;
+            b.Gt = q.Cr;
+            b.At = q.Ar;
+            b.y = h->Sr + 2 * rows * 4 * mw + l * vec32;
+            b.nz = q.nzr;
+            b.zbad = q.zbadr;
+            b.zmid = q.zbadr + rows;
+            b.rhs = q.rr;
+            b.x = q.xr;
+        }
     }
     BTD_CU(cudaMemsetAsync(h->flag + 1, 0, sizeof(int), s));
     k_btd_validate<<<(unsigned)((n_rays + 256) / 256), 256, 0, s>>>(ray_offsets, n_rays, n_zones, h->flag + 1, h->flag, h->zbad,
@@ -1903,9 +1926,11 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
     launch_convert(h->m, n_zones, s, a);
     BTD_CU(cudaGetLastError());
     if (seg) {
-        BTD_CU(launch_seg(segment_kernel(h->m), n_rays * parts, h->smem_seg, s, p));
-        k_btd_join<<<dim3(n_rays * parts, 4), 256, 0, s>>>(p);
-        BTD_CU(cudaGetLastError());
+        for (int l = 0; l < levels; ++l) {
+            BTD_CU(launch_seg(segment_kernel(h->m), n_rays * p[l].parts, h->smem_seg, s, p[l]));
+            k_btd_join<<<dim3(n_rays * p[l].parts, 4), 256, 0, s>>>(p[l]);
+            BTD_CU(cudaGetLastError());
+        }
         launch_factor(h->m, 2 * n_rays, h->smem, s, b);
         BTD_CU(cudaGetLastError());
         k_btd_again<<<dim3(n_rays, 32), 256, 0, s>>>(f);
@@ -1923,15 +1948,17 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
         if (it > 0) {
             k_btd_resid<<<dim3(n_rays, (unsigned)split), kResidThreads, 0, s>>>(a);
             BTD_CU(cudaGetLastError());
-            f.rhs = p.a.rhs = h->r;
+            f.rhs = p[0].a.rhs = h->r;
         }
         const bool last = it == h->n_refine;
         if (seg) {
-            BTD_CU(cudaMemsetAsync(p.rr, 0, (size_t)n_rays * parts * h->m * sizeof(double), s));
-            BTD_CU(launch_seg(seg_sweep_kernel<false, true>(h->m), n_rays * parts, h->smem_sweep, s, p));
+            BTD_CU(cudaMemsetAsync(h->vr, 0, (size_t)levels * h->sms * h->m * sizeof(double), s));
+            for (int l = 0; l < levels; ++l)
+                BTD_CU(launch_seg(seg_sweep_kernel<false, true>(h->m), n_rays * p[l].parts, h->smem_sweep, s, p[l]));
             BTD_CU((launch_sweep<true, false>(h->m, 2 * n_rays, h->smem_sweep, s, b)));
-            BTD_CU(launch_seg(it == 0 ? seg_sweep_kernel<true, true>(h->m) : seg_sweep_kernel<true, false>(h->m), n_rays * parts,
-                              h->smem_sweep, s, p));
+            for (int l = levels - 1; l >= 0; --l)
+                BTD_CU(launch_seg(l || it == 0 ? seg_sweep_kernel<true, true>(h->m) : seg_sweep_kernel<true, false>(h->m),
+                                  n_rays * p[l].parts, h->smem_sweep, s, p[l]));
         }
         BTD_CU((it == 0 ? (last ? launch_sweep<true, true> : launch_sweep<true, false>)
                         : (last ? launch_sweep<false, true> : launch_sweep<false, false>))(h->m, ctas, h->smem_sweep, s, f));

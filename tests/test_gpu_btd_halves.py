@@ -101,3 +101,23 @@ def test_segments(m):
     assert not ok
     a, b = first[7], first[8]
     assert np.isnan(x[a:b]).all() and np.isfinite(x[:a]).all() and np.isfinite(x[b:]).all()
+
+
+@pytest.mark.parametrize("m", [1, 8, 42, 84, 112])
+@pytest.mark.parametrize("n_refine", [2, 3])
+def test_segments_of_segments(m, n_refine):
+    zones = [2, 9, 450, 400]
+    s = gen.random_system(np.array(zones), m, seed=m)
+    first = [int(o) for o in s["offsets"]]
+    s["A"][first[3] + 150:first[3] + 190] = 0.0  # no coupling through whole segments
+    s["C"][first[3] + 149:first[3] + 189] = 0.0
+    x, ok = _solve(s, m, n_refine)
+    assert ok
+    _close(s, x, range(4))
+    for z in (36, 37, 38, 39, 40, 41, 42, 43, 44, 45, 46, 47):  # whatever the segments: the first zone of one, and others
+        s["B"][first[2] + z] = 0.0
+        k = first[2] + z
+        s["C"][k - 1] = s["A"][k] = s["C"][k] = s["A"][k + 1] = np.eye(m)
+    x, ok = _solve(s, m, n_refine)
+    assert ok
+    _close(s, x, range(4))
