@@ -546,15 +546,24 @@ static void cache_write(const char *path, const std::string &key, const std::str
     rename(tmp.c_str(), path);
 }
 
-// The register budget of a launch: the autotuned one, else the smaller one for the tangent kernel, and for the
-// forward kernel the larger one until the batch fills its grid more than twice. Six CTAs of 128
+// The register budget of a launch: the autotuned one, else as follows. The tangent kernel takes the smaller one (five
+// CTAs per SM, not four), except with the split rule, whose two panels do not fit 96 registers, and where each
+// CTA of the larger one has at most one zone, which then ends sooner. GB300, five per SM -> four, zones at 64
+// nodes and 21 bins: 64 125 -> 117 us, 400 226 -> 223, 608 310 -> 300, 760 352 -> 364, 25,600 9690 -> 9787; at 48
+// nodes and eta_e to 60: 64 83 -> 85, 400 128 -> 124, 608 157 -> 154, 760 182 -> 193; at 32 nodes and 13 bins: 152 48.7
+// -> 50.2, 400 56.2 -> 57.4; split rule at 48 nodes: 64 156 -> 120, 400 255 -> 231, 2400 722 -> 693, 25,600
+// 6716 -> 6438. The forward kernel takes the larger one until the batch fills its grid more than twice. Six CTAs of 128
 // threads per SM at 80 registers hide each other's MUFU and shared-memory latencies better than four at 128
 // (MUFU 55 %, FP32 pipe 50 % busy), but a zone by itself takes longer. GB300, four per SM -> six, zones at 64 nodes
 // and 21 bins: 64 74.6 -> 79.9 us, 304 115 -> 118, 1216 288 -> 273, 2400 492 -> 456, 3200 610 -> 620, 6400
 // 1196 -> 1153; at 48 nodes and eta_e to 60: 400 84 -> 86, 912 122 -> 131, 2000 234 -> 223, 9600 971 -> 942; at
 // 32 nodes and 13 bins: 400 43.7 -> 45.8, 1600 78 -> 72, 9600 293 -> 260.
 static int mixed_budget(const vx_rates *h, bool adj, long long zones) {
-    if (adj || h->tuned[0]) return h->minb[adj];
+    if (h->tuned[adj]) return h->minb[adj];
+    if (adj) {
+        if (h->common.precise) return h->minb[1];
+        return h->common.split || (zones <= h->grid_mixed[1][0] && h->common.n_e >= 48) ? 2 : h->minb[1];
+    }
     return zones > 2LL * h->grid_mixed[0][0] ? 3 : h->minb[0];
 }
 
@@ -678,7 +687,7 @@ vx_status vx_rates_adjoint(vx_rates *h, const vx_batch *b, const vx_out *grad_ou
     L.grad_state = grad_state;
     if (grad_state) { L.g_j0 = grad_out->j0; L.g_chi0 = grad_out->chi0; L.g_j1 = grad_out->j1; L.g_chi1 = grad_out->chi1; }
     if ((st = autotune(h, true, L, s)) != VX_OK) return st;
-    const int mb = h->minb[1];
+    const int mb = mixed_budget(h, true, b->n_zones);
     int grid = (int)std::min<long long>(h->grid_mixed[1][mb - 2], b->n_zones);
     if (h->cfg.flags & VX_USE_GRAPH)
         return launch_graph(h, 1, vx::kernel_mixed(true, mb, h->common.n_e, h->common.split != 0, h->common.precise != 0), &L, grid, h->block_mixed, h->smem_adj, s);
