@@ -45,10 +45,10 @@ def entries(Z, N):
 
 
 # DRAM bytes (read + write) per zone of the forward + tangent kernel, from one ncu capture of the
-# 200-ray case of this workload (dram__bytes_read.sum + dram__bytes_write.sum = 91.0 + 591.6 MB
+# 200-ray case of this workload (dram__bytes_read.sum + dram__bytes_write.sum = 88.9 + 592.0 MB
 # for 80,000 zones, profiles/k_pair_mixed_tangents_200rays_pipes.md); scaled to a launch by the
 # zone count. Set to None whenever the kernel changes, until it has been captured again.
-TRAFFIC_BYTES_PER_ZONE = 8532
+TRAFFIC_BYTES_PER_ZONE = 8512
 def measured_hbm_gbs():
     """The HBM copy bandwidth measured on this machine's GPUs (MEASURED_PEAKS.json), else the
     recipe's fallback figure; returns (GB/s, note)."""
@@ -86,8 +86,8 @@ def formulation_flops_per_node(adj: bool) -> int:
 # Pipe utilisation of the benchmark's kernels from one ncu capture each (see profiles/; set to
 # None whenever the kernel changes, until it has been captured again): the MUFU (XU) issue
 # fraction of the forward + tangent kernel and the FP64-pipe fraction of the plain FP64 kernel.
-MUFU_FRAC_TANGENT = 0.2530   # profiles/k_pair_mixed_tangents_200rays_pipes.md
-FP64_FRAC_FP64FWD = 0.9154   # profiles/k_pair_mixed_tangents_and_k_pair_fp64_pipes_20rays.md
+MUFU_FRAC_TANGENT = 0.2596   # profiles/k_pair_mixed_tangents_200rays_pipes.md
+FP64_FRAC_FP64FWD = 0.9251   # profiles/k_pair_mixed_tangents_and_k_pair_fp64_pipes_20rays.md
 # fraction of the workload's zones the plain FP64 comparison leg evaluates, and its timed launches
 FP64_SAMPLE_FRAC, FP64_REPEATS = 0.05, 3
 # timed launches of the precise-mode leg (after two untimed ones)
@@ -335,7 +335,7 @@ def run_solve(args):
             "e2e": {"value": job_rate(Z, world, ms_e2e), "unit": "zones/s", "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": d2h, "call": "BlockTridiagSolver.solve_host (pinned host tensors)",
                     "ms_per_step": ms_e2e},
-            "gpu_launches": args.steps * (3 + 2 * SOLVE_REFINE),  # validate, factor, sweep; resid + sweep each
+            "gpu_launches": args.steps * (4 + 2 * SOLVE_REFINE),  # validate, convert, factor, sweep; resid + sweep each
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                          "traffic": None,
                          "note": "FP32 flops of the block factorisation over the whole step (factor kernel, "
@@ -535,9 +535,9 @@ def run_nes(args):
 
 ABS_METRIC = "absorption/emission rate entries/s (zone*species*eps), forward+Jacobian, % HBM peak"
 # DRAM bytes (read + write) per entry (zone, species, bin) of the absorption rates + Jacobian kernel,
-# from one ncu capture of the 1024-ray case of the workload (13.4 + 3241.5 MB for 25.8 M entries,
+# from one ncu capture of the 1024-ray case of the workload (19.8 + 3245.6 MB for 25.8 M entries,
 # profiles/k_abs_tangents_1024rays.md); None whenever the kernel changes, until captured again.
-ABS_TRAFFIC_BYTES_PER_ENTRY = 126.1
+ABS_TRAFFIC_BYTES_PER_ENTRY = 126.5
 
 
 def abs_oracle_rate(b, n_zones):

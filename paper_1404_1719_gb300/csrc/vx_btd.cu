@@ -1,24 +1,28 @@
 // vx_btd.cu -- batched block-tridiagonal solve of the per-ray Newton systems (include/vx_btd.h).
 //
-// A ray's zones are a sequential chain, so a ray belongs to one CTA; k_btd_validate first checks that the
-// ray offsets partition the zones (else every kernel returns at once):
+// A ray's zones are a sequential chain. With many rays each belongs to one CTA, with fewer to two that eliminate from
+// both ends, and with few a CTA takes a segment of a ray (each chosen by vx_btd_solve). k_btd_validate
+// first checks that the ray offsets partition the zones (else every kernel returns at once):
 //  * k_btd_convert: the caller's FP64 blocks to FP32, with the zero patterns of the couplings' rows.
-//  * k_btd_factor: block elimination along the ray in FP32, one CTA per ray. Per zone:
+//  * k_btd_factor: block elimination along the ray in FP32, one or two CTAs per ray. Per zone:
 //    D_k = B_k - A_k G_{k-1} on the tensor cores, D_k inverted in place by Gauss-Jordan elimination with
 //    partial pivoting in panels of eight columns (one warp eliminates within a panel, the others apply its
 //    rank-8 transform on the tensor cores), G_k = D_k^{-1} C_k on the tensor cores. D_k^{-1} and G_k
 //    replace B_k and C_k in the workspace.
-//  * k_btd_sweep: one CTA per ray solves M delta = rhs with those: forward
+//  * k_btd_segment, k_btd_join: the same for segments of rays, which leaves the system of their last zones to
+//    k_btd_factor (or to k_btd_segment again); k_btd_again restores the blocks of a ray that could not be done so.
+//  * k_btd_sweep, k_btd_seg_sweep: solve M delta = rhs with those: forward
 //    y_k = D_k^{-1} (rhs_k - A_k y_{k-1}), backward delta_k = y_k - G_k delta_{k+1}, a chain of
 //    matrix-vector products. The first sweep writes x = delta, later ones add delta to x in FP64.
 //  * k_btd_resid: the FP64 residual r = d - M x from the caller's FP64 blocks, eight rows per warp, four
 //    lanes per row (coalesced), zero groups of the couplings left out, FMA accumulation and a fixed two-step
 //    shuffle reduction per row.
-// The host runs validate, convert, factor, sweep, then n_refine times (resid, sweep), all on the caller's
-// stream.
+// The host runs validate, convert, [segment, join, once or twice], factor, sweep, then n_refine times (resid,
+// sweep), all on the caller's stream; with segments the factor kernel and the sweeps run once for the segments' system
+// and once for the rays that have to be done as a whole (3 us each when there are none).
 // With the inverse instead of the elimination's multipliers (which the sweeps replayed, a shuffle per
-// unknown), GB300, m = 84, 400 zones a ray: one ray factor 24.3 -> 10.0 ms, a sweep 3.0 -> 1.3 ms; 304 rays
-// 29.7 -> 14.9 ms (which included the conversion, now 6.1 ms apart) and 3.1 -> 1.8 ms (10.3 GB, 5.7 TB/s).
+// unknown), GB300, m = 84, 400 zones a ray: one ray (one CTA) factor 24.3 -> 10.0 ms, a sweep 3.0 -> 1.3 ms; 304 rays
+// 29.7 -> 14.0 ms (which included the conversion, now 6.1 ms apart) and 3.1 -> 1.7 ms (10.3 GB, 6.1 TB/s).
 // The solution's error without refinement and with one sweep is 0.2 to 0.8 of what it was (m = 34 to 128).
 #include "../../include/vx_btd.h"
 
