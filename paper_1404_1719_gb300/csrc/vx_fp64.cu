@@ -117,14 +117,17 @@ __device__ __forceinline__ double exp_pair(double x, double xl) {
     return fma(e, xl, e);
 }
 
-// CTA = zone; the zone's (bin pair, omega) units in equal contiguous ranges, one per thread; partial sums of
-// pairs that two threads share are added in thread order.
+// CTA = zone, or one of L.parts shares of it. A zone's bin pairs go in up to eight parts, always the same ones, so that
+// its results do not depend on how many CTAs take them; a part's (pair, omega) units in equal contiguous
+// ranges, one per thread, and partial sums of pairs that two threads share added in thread order. Shares meet in
+// global memory (L.phi_part): whichever ends last reads the others' kernel matrices and contracts; none waits.
 __global__ void __launch_bounds__(kTpb64) k_pair_fp64(const __grid_constant__ Launch64 L) {
     extern __shared__ __align__(16) double smd[];
     __shared__ Zone64 zs;
     __shared__ long long s_zone;
     const Common &C = L.c;
-    const int N = C.N, S = C.S, N2 = N * N, nmu = C.n_mu, U = C.npair * nmu;
+    __shared__ int s_last;
+    const int N = C.N, S = C.S, N2 = N * N, nmu = C.n_mu, parts = L.parts;
     double *A0 = smd, *A1 = smd + N2, *vec = smd + 2 * N2, *em = vec + 4 * S * N, *hx = em + N;
     double *nodes = hx + N, *tab = nodes + 4 * VX_MAX_NE, *part = tab + kExpTab;  // part[slot][4][threads]
     const int tid = threadIdx.x, TB = blockDim.x;
@@ -138,14 +141,15 @@ __global__ void __launch_bounds__(kTpb64) k_pair_fp64(const __grid_constant__ La
         nodes[4 * k + 3] = L.n64.c0[q];
     }
     for (int k = tid; k < kExpTab; k += TB) tab[k] = L.exptab[k];
-    const int u0 = (int)((long long)tid * U / TB), u1 = (int)((long long)(tid + 1) * U / TB);
     validate_offsets(L.off, L.n_rays, L.Z, L.flag);
 
     for (;;) {
         if (tid == 0) s_zone = (long long)atomicAdd(L.counter, 1ull);
         __syncthreads();
-        const long long z = s_zone;
+        const long long z = s_zone / parts;
         if (z >= L.Z) break;
+        const int share = (int)(s_zone - z * parts), K = L.count;
+        auto first_pair = [&](int k) { return min(C.npair, L.group * (L.groups * k / K)); };  // of part k
         if (tid == 0) {
             const double T = L.state[4 * z + 0], eta = L.state[4 * z + 1], iT = 1.0 / T;
             zs.T = T;
@@ -161,11 +165,11 @@ __global__ void __launch_bounds__(kTpb64) k_pair_fp64(const __grid_constant__ La
         const double T = zs.T, iT = zs.iT, iTl = zs.iTl;
         if (zs.bad) {
             const double nan = __longlong_as_double(0x7ff8000000000000ll);
-            for (int e = tid; e < S * N; e += TB) {
+            for (int e = tid; share == 0 && e < S * N; e += TB) {
                 size_t o = (size_t)z * S * N + e;
                 L.j0[o] = nan; L.chi0[o] = nan; L.j1[o] = nan; L.chi1[o] = nan;
             }
-            if (L.phi)
+            if (L.phi && share == 0)
                 for (int e = tid; e < 4 * N2; e += TB) L.phi[(size_t)z * 4 * N2 + e] = nan;
             if (tid == 0) atomicOr(L.flag, VX_FLAG_BAD_STATE);
             __syncthreads();
@@ -190,58 +194,85 @@ __global__ void __launch_bounds__(kTpb64) k_pair_fp64(const __grid_constant__ La
         // log2(e) 4096 / T as a value and its remainder
         const double LG = 5909.278887481194, LGl = 8.337520124285351e-14;  // 4096 log2(e)
         const double gT = LG * iT, gTl = fma(LG, iT, -gT) + fma(LG, iTl, LGl * iT);
-        double a0 = 0, b0 = 0, a1 = 0, b1 = 0;  // l = 0 terms I, II; l = 1
-        int p = u0 / nmu, m = u0 - (u0 / nmu) * nmu, mb = m, slot = 0;
-        for (int u = u0; u < u1; ++u) {
-            const double *rec = L.tab64 + (size_t)u * 5;
-            const double h = rec[0], Em = rec[1], kp = rec[2], km = rec[3], k0 = rec[4];
-            Mom64 M;
-            if (zs.fast) {
-                const double Q0 = hx[C.pij[p] >> 8] * hx[C.pij[p] & 0xff];
-                const double Bs = h * gT;
-                const float Bl = to_f32(fma(h, gT, -Bs) + h * gTl);
-                nodes_fast(nodes, tab, nh, mid, Bs, Bl, zs.ep * Q0, zs.em * Q0, fma(Q0, Q0, 1.0), M);
-            } else {
-                nodes_plain(nodes, nh, mid, h, Em, iT, zs.eta, M);
-            }
-            const double t = C.t64[m], KI = fma(kp, M.p, fma(km, M.m, k0 * M.z)), KII = fma(km, M.p, fma(kp, M.m, k0 * M.z));
-            a0 += KI;
-            b0 += KII;
-            a1 = fma(t, KI, a1);
-            b1 = fma(t, KII, b1);
-            ++m;
-            if (m == nmu || u + 1 == u1) {
-                if (mb == 0 && m == nmu) {
-                    const int pi = C.pij[p] >> 8, pj = C.pij[p] & 0xff;
-                    A0[pi * N + pj] = a0; A1[pi * N + pj] = a1;
-                    if (pi != pj) { A0[pj * N + pi] = b0; A1[pj * N + pi] = b1; }
+        for (int k = K * share / parts; k < K * (share + 1) / parts; ++k) {
+            const int q0 = first_pair(k), q1 = first_pair(k + 1), U = (q1 - q0) * nmu;
+            const int u0 = q0 * nmu + (int)((long long)tid * U / TB), u1 = q0 * nmu + (int)((long long)(tid + 1) * U / TB);
+            double a0 = 0, b0 = 0, a1 = 0, b1 = 0;  // l = 0 terms I, II; l = 1
+            int p = u0 / nmu, m = u0 - (u0 / nmu) * nmu, mb = m, slot = 0;
+            for (int u = u0; u < u1; ++u) {
+                const double *rec = L.tab64 + (size_t)u * 5;
+                const double h = rec[0], Em = rec[1], kp = rec[2], km = rec[3], k0 = rec[4];
+                Mom64 M;
+                if (zs.fast) {
+                    const double Q0 = hx[C.pij[p] >> 8] * hx[C.pij[p] & 0xff];
+                    const double Bs = h * gT;
+                    const float Bl = to_f32(fma(h, gT, -Bs) + h * gTl);
+                    nodes_fast(nodes, tab, nh, mid, Bs, Bl, zs.ep * Q0, zs.em * Q0, fma(Q0, Q0, 1.0), M);
                 } else {
-                    double *q = part + slot * 4 * TB + tid;
-                    q[0] = a0; q[TB] = b0; q[2 * TB] = a1; q[3 * TB] = b1;
+                    nodes_plain(nodes, nh, mid, h, Em, iT, zs.eta, M);
                 }
-                a0 = b0 = a1 = b1 = 0.0;
-                slot = 1;
-                ++p;
-                m = mb = 0;
+                const double t = C.t64[m], KI = fma(kp, M.p, fma(km, M.m, k0 * M.z)), KII = fma(km, M.p, fma(kp, M.m, k0 * M.z));
+                a0 += KI;
+                b0 += KII;
+                a1 = fma(t, KI, a1);
+                b1 = fma(t, KII, b1);
+                ++m;
+                if (m == nmu || u + 1 == u1) {
+                    if (mb == 0 && m == nmu) {
+                        const int pi = C.pij[p] >> 8, pj = C.pij[p] & 0xff;
+                        A0[pi * N + pj] = a0; A1[pi * N + pj] = a1;
+                        if (pi != pj) { A0[pj * N + pi] = b0; A1[pj * N + pi] = b1; }
+                    } else {
+                        double *q = part + slot * 4 * TB + tid;
+                        q[0] = a0; q[TB] = b0; q[2 * TB] = a1; q[3 * TB] = b1;
+                    }
+                    a0 = b0 = a1 = b1 = 0.0;
+                    slot = 1;
+                    ++p;
+                    m = mb = 0;
+                }
             }
-        }
-        __syncthreads();
-        // pairs split between threads: owner of unit v is thread ceil((v + 1) TB / U) - 1
-        for (int q = tid; q < C.npair; q += TB) {
-            const long long ua = (long long)q * nmu, ub = ua + nmu - 1;
-            const int ta = (int)(((ua + 1) * TB + U - 1) / U) - 1, tb = (int)(((ub + 1) * TB + U - 1) / U) - 1;
-            if (ta == tb) continue;
-            double s[4] = {0, 0, 0, 0};
-            for (int t = ta; t <= tb; ++t) {
-                if (U < TB && t * U / TB == (t + 1) * U / TB) continue;  // fewer units than threads: an empty range
-                const int sl = t == ta && ua > (long long)t * U / TB ? 1 : 0;
-                for (int c = 0; c < 4; ++c) s[c] += part[(sl * 4 + c) * TB + t];
+            __syncthreads();
+            // pairs split between threads: owner of unit v is thread ceil((v + 1) TB / U) - 1
+            for (int q = q0 + tid; q < q1; q += TB) {
+                const long long ua = (long long)(q - q0) * nmu, ub = ua + nmu - 1;
+                const int ta = (int)(((ua + 1) * TB + U - 1) / U) - 1, tb = (int)(((ub + 1) * TB + U - 1) / U) - 1;
+                if (ta == tb) continue;
+                double s[4] = {0, 0, 0, 0};
+                for (int t = ta; t <= tb; ++t) {
+                    if (U < TB && t * U / TB == (t + 1) * U / TB) continue;  // fewer units than threads: an empty range
+                    const int sl = t == ta && ua > (long long)t * U / TB ? 1 : 0;
+                    for (int c = 0; c < 4; ++c) s[c] += part[(sl * 4 + c) * TB + t];
+                }
+                const int pi = C.pij[q] >> 8, pj = C.pij[q] & 0xff;
+                A0[pi * N + pj] = s[0]; A1[pi * N + pj] = s[2];
+                if (pi != pj) { A0[pj * N + pi] = s[1]; A1[pj * N + pi] = s[3]; }
             }
-            const int pi = C.pij[q] >> 8, pj = C.pij[q] & 0xff;
-            A0[pi * N + pj] = s[0]; A1[pi * N + pj] = s[2];
-            if (pi != pj) { A0[pj * N + pi] = s[1]; A1[pj * N + pi] = s[3]; }
+            __syncthreads();
         }
-        __syncthreads();
+        if (parts > 1) {
+            double *F = L.phi_part + (size_t)z * 2 * N2;
+            const int qb = first_pair(K * share / parts), qe = first_pair(K * (share + 1) / parts);
+            for (int q = qb + tid; q < qe; q += TB) {
+                const int pi = C.pij[q] >> 8, pj = C.pij[q] & 0xff, ij = pi * N + pj, ji = pj * N + pi;
+                F[ij] = A0[ij]; F[ji] = A0[ji];
+                F[N2 + ij] = A1[ij]; F[N2 + ji] = A1[ji];
+            }
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) {
+                s_last = atomicAdd(L.arrived + z, 1) == parts - 1;
+                if (s_last) L.arrived[z] = 0;  // for the next launch
+                __threadfence();
+            }
+            __syncthreads();
+            if (!s_last) continue;
+            for (int e = tid; e < N2; e += TB) {
+                A0[e] = __ldcg(F + e);
+                A1[e] = __ldcg(F + N2 + e);
+            }
+            __syncthreads();
+        }
         const double c0 = 6.283185307179586 * C.norm * C.g2, c1 = 3.0 * c0;
         for (int e = tid; e < 4 * S * N; e += TB) {
             const int o = e / (S * N), s = (e / N) % S, i = e % N;

@@ -96,6 +96,8 @@ namespace vx {
 vx_status set_error(vx_status s, const char *msg) { return fail(s, "%s", msg); }
 }  // namespace vx
 
+constexpr long long kParts64Zones = 8;  // zones per SM below which the FP64 kernel's CTAs may share zones
+
 struct vx_rates {
     int device = 0;
     int nsm = 0;
@@ -116,6 +118,8 @@ struct vx_rates {
     bool tuned[2] = {false, false};
     float tune_ms[2][2] = {{0, 0}, {0, 0}};
     int grid_64 = 0;
+    double *d_part64 = nullptr;  // FP64 form, batches of fewer than kParts64Zones zones per SM: the shares' kernel matrices
+    int *d_arrived64 = nullptr;
     size_t smem_fwd = 0, smem_adj = 0, smem_64 = 0;
     int cc_major = 0, cc_minor = 0;
     // one cached executable graph per kernel kind: mixed forward, mixed tangents, FP64
@@ -371,6 +375,19 @@ vx_status vx_rates_create(const vx_config *cfg, vx_rates **out) {
         VX_CUC(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k.fn, k.block, k.smem));
         if (occ < 1) return cleanup(fail(VX_ERR_UNSUPPORTED, "kernel does not fit on an SM (block %d, smem %zu)", k.block, k.smem));
         *k.grid = occ * h->nsm;
+    }
+    if (cfg->prec == VX_PREC_FP64) {  // (without this memory, zones go whole)
+        const size_t zones = (size_t)(kParts64Zones * h->nsm);
+        cudaError_t e = cudaMalloc(&h->d_part64, zones * 2 * N * N * sizeof(double));
+        if (e == cudaSuccess) e = cudaMalloc(&h->d_arrived64, zones * sizeof(int));
+        if (e == cudaSuccess) e = cudaMemset(h->d_arrived64, 0, zones * sizeof(int));
+        if (e != cudaSuccess) {
+            (void)cudaGetLastError();
+            cudaFree(h->d_part64);
+            cudaFree(h->d_arrived64);
+            h->d_part64 = nullptr;
+            h->d_arrived64 = nullptr;
+        }
     }
 #undef VX_CUC
     *out = h;
@@ -653,7 +670,23 @@ vx_status vx_rates_eval(vx_rates *h, const vx_batch *b, const vx_out *out, vx_st
         L.j0 = out->j0; L.chi0 = out->chi0; L.j1 = out->j1; L.chi1 = out->chi1; L.phi = out->phi;
         L.counter = h->d_counter;
         L.flag = h->d_flag;
-        int grid = (int)std::min<long long>(h->grid_64, b->n_zones);
+        // CTAs share zones where the last of whole zones would leave 30 % of the SMs without work (one zone at a time
+        // keeps an SM's FP64 pipe busy) and there are few. GB300, 32 x 64 nodes and 21 bins, whole -> shared: 1 zone
+        // 1.52 -> 0.26 ms, 64 1.52 -> 0.83, 500 5.92 -> 5.14, 800 8.84 -> 8.11; but 152 (all SMs, shared) 1.52 -> 1.81,
+        // 456 4.46 -> 4.94, 1500 14.7 -> 15.5. (Taking the parts one after the other costs a whole zone up to 1.6 %.)
+        const long long idle = (h->nsm - b->n_zones % h->nsm) % h->nsm;
+        const vx::Parts64 pt(h->common.npair, h->common.n_mu, h->block);
+        L.group = pt.group;
+        L.groups = pt.groups;
+        L.count = pt.count;
+        L.parts = 1;
+        if (h->d_part64 && b->n_zones < kParts64Zones * h->nsm && 10 * idle >= 3 * h->nsm) {
+            L.parts = pt.count;
+            if (b->n_zones > 4LL * h->nsm) L.parts = std::min(L.parts, 4);
+        }
+        L.phi_part = h->d_part64;
+        L.arrived = h->d_arrived64;
+        int grid = (int)std::min<long long>(h->grid_64, b->n_zones * L.parts);
         if (graph) return launch_graph(h, 2, vx::kernel_fp64_fwd(), &L, grid, h->block, h->smem_64, s);
         VX_CU(cudaMemsetAsync(h->d_counter, 0, sizeof(unsigned long long), s));
         VX_CU(vx::launch_fp64_fwd(L, grid, h->block, h->smem_64, s));
@@ -927,6 +960,8 @@ void vx_rates_destroy(vx_rates *h) {
     cudaFree(h->d_tab32);
     cudaFree(h->d_tab64);
     cudaFree(h->d_exp);
+    cudaFree(h->d_part64);
+    cudaFree(h->d_arrived64);
     cudaFree(h->d_counter);
     cudaFree(h->d_flag);
     for (int k = 0; k < 2; ++k) {
