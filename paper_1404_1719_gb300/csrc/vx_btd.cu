@@ -967,10 +967,19 @@ struct Seg {
 template <int NT>
 __global__ void __launch_bounds__(kFactorThreads, 1) k_btd_segment(const SegArgs p) {
     extern __shared__ __align__(16) float sm[];
-    __shared__ int s_bad;
+    __shared__ int s_bad, s_go;
     const BtdArgs &a = p.a;
     Seg sg;
-    if (!sg.find(p, blockIdx.x, p.above > 0)) return;
+    // Whether the ray is still good is asked once for the whole CTA: another segment of the ray may mark it (pbad, at
+    // the end of this kernel) while this one starts, and threads that read the mark each for themselves
+    // would not agree on going on. Which answer a CTA gets does not matter, since a marked ray's results are not used.
+    if (threadIdx.x == 0) {
+        s_go = sg.find(p, blockIdx.x, p.above > 0);
+        s_bad = 0;
+    }
+    __syncthreads();
+    if (!s_go) return;
+    sg.find(p, blockIdx.x, false);
     const int m = a.m, ld = a.ld, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, wm = warp & 1, wn = warp >> 1;
     const int bs = factor_buf(m, ld), P = (m + 7) >> 3, mw = m * ld;
     const bool five = p.nbuf == 5;  // a buffer for the next zone's B
@@ -980,7 +989,6 @@ __global__ void __launch_bounds__(kFactorThreads, 1) k_btd_segment(const SegArgs
     float *rowbuf = sm + p.nbuf * bs + a.mp;                                      // [2][8]
     int *cur = reinterpret_cast<int *>(rowbuf + 16);
     int *pos = cur + 8 * P;
-    if (tid == 0) s_bad = 0;
     if (tid < m) pos[tid] = tid;
     for (int i = tid; i < p.nbuf * (bs - mw); i += kFactorThreads) sm[i / (bs - mw) * bs + mw + i % (bs - mw)] = 0.f;
     auto load = [&](float *dst, const float *src) { copy_async(dst, src, mw, tid, kFactorThreads); };

@@ -1,0 +1,56 @@
+"""Rays cut into segments whose elimination that way is given up late or should be: by the system of the segments' last
+zones alone, in the launch whose other segments ask whether their ray is still good."""
+import numpy as np
+import pytest
+
+from oracle import btd as obtd
+from vx_inputs import btd as gen
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+TOL = 1e-12  # normwise after two refinement sweeps, as for the other systems
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1404_1719_gb300 import _build
+    _build.build()
+
+
+def _solve(s, m, n_refine=2):
+    from paper_1404_1719_gb300 import BlockTridiagSolver
+    t = {k: torch.from_numpy(np.ascontiguousarray(s[k])).cuda() for k in ("offsets", "A", "B", "C", "d")}
+    sv = BlockTridiagSolver(m, s["d"].shape[0], n_refine=n_refine)
+    x = sv.solve(t["offsets"].to(torch.int32), t["A"], t["B"], t["C"], t["d"]).cpu().numpy()
+    ok = sv.check()
+    sv.close()
+    return x, ok
+
+
+def _segments(zones, rays):
+    """Segments per ray of the first of two levels (the rule of vx_btd_solve)."""
+    parts = torch.cuda.get_device_properties(0).multi_processor_count // rays
+    while 4 * parts ** 3 > 8.4 * zones ** 2:
+        parts -= 1
+    return parts
+
+
+@pytest.mark.parametrize("m", [1, 8, 34, 84])
+def test_second_level_alone_fails(m):
+    """Tiny blocks in the last zones of a ray's segments: the segments themselves stay small, their system does
+    not (its D^-1 C is of order 1e20), and the ray beside it goes on in segments."""
+    n = 400
+    s = gen.random_system(np.array([n, n]), m, seed=m)
+    S = _segments(n, 2)
+    tiny = [n + n * (i + 1) // S - 1 for i in range(3, S - 3, 2)]
+    for e in tiny:
+        s["A"][e], s["C"][e - 1], s["A"][e + 1] = 0.0, 0.0, 0.0
+        s["C"][e], s["B"][e] = np.eye(m), 1e-30 * np.eye(m)
+    x, ok = _solve(s, m)
+    assert ok
+    ref = obtd.solve(s["A"], s["B"], s["C"], s["d"], s["offsets"])
+    rest = np.setdiff1d(np.arange(n, 2 * n), tiny)
+    for z in (np.arange(n), rest, np.array(tiny)):  # (nothing but the tiny zones depends on their x)
+        assert np.abs(x[z] - ref[z]).max() <= TOL * np.abs(ref[z]).max()
