@@ -19,16 +19,16 @@
  * FP32 copies of the blocks, one CTA per ray, its matrix products on the tensor cores (TF32 with each
  * operand split into two parts, three products: about FP32 accuracy); D_k^{-1} and G_k are kept. Where
  * rays are few, a ray is eliminated from both ends at once by two CTAs, or in segments of its zones by a
- * CTA each and then the system of the segments' last zones (chosen by n_rays, n_zones and m); if a
- * pivot fails there, or entries of D^{-1} C or the like exceed 64, the ray is done again from its
- * first zone on, so what can be solved does not depend on it. Then
+ * CTA each and then the system of the segments' last zones (chosen by n_rays, n_zones and m, so a
+ * ray's last bits depend on the batch it is in); if a pivot fails there, or entries of D^{-1} C or the like
+ * exceed 4, the ray is done again from its first zone on. Then
  * the ray is solved by matrix-vector products with those, y_k = D_k^{-1} (d_k - A_k y_{k-1}) forward and
  * x_k = y_k - G_k x_{k+1} backward, and
  * n_refine sweeps of iterative refinement follow, each from the FP64 residual d - M x of the
  * caller's FP64 blocks. For a ray whose Schur complements are well conditioned (e.g. block rows
  * diagonally dominant) every sweep gains a factor of about cond x 1e-7, so two sweeps reach FP64
- * accuracy at moderate condition numbers. The reduction order is fixed: results are reproducible
- * run to run.
+ * accuracy at moderate condition numbers. The reduction order is fixed: the results of a batch are
+ * reproducible run to run.
  *
  * Conventions (as in vx_rates.h): arrays are dense, row-major FP64 unless stated; device pointers
  * are CUDA global memory of the current device, owned by the caller; the library never retains a

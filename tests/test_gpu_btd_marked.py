@@ -54,3 +54,29 @@ def test_second_level_alone_fails(m):
     rest = np.setdiff1d(np.arange(n, 2 * n), tiny)
     for z in (np.arange(n), rest, np.array(tiny)):  # (nothing but the tiny zones depends on their x)
         assert np.abs(x[z] - ref[z]).max() <= TOL * np.abs(ref[z]).max()
+
+
+@pytest.mark.parametrize("n_refine", [0, 1, 2])
+@pytest.mark.parametrize("m, seed, kind, scale", [(8, 99, 0, 0.3), (8, 231, 0, 0.1), (20, 10, 1, 1.0), (8, 232, 1, 0.5),
+                                                  (4, 28, 1, 1.0), (4, 106, 0, 0.3)])
+def test_growth_within_segments(m, seed, kind, scale, n_refine):
+    """Random blocks without a dominant diagonal, the entries of D^-1 C and the like between 10 and 90 in the
+    segments: alone, the ray is as accurate as among as many rays as the chip takes one block of threads each (the
+    same elimination from the first zone on, so the errors agree to a small factor)."""
+    n = 150
+    g = np.random.default_rng(seed)
+    A, B, C = (g.standard_normal((n, m, m)) for _ in range(3))
+    A, C = A * scale, C * scale
+    B = B + kind * 1.5 * np.sqrt(m) * np.eye(m)
+    A[0], C[-1] = 0.0, 0.0
+    s = dict(A=A, B=B, C=C, d=g.standard_normal((n, m)), offsets=np.array([0, n], np.int32))
+    ref = obtd.solve(A, B, C, s["d"], s["offsets"])
+    rays = 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    many = {k: np.tile(s[k], (rays,) + (1,) * (s[k].ndim - 1)) for k in ("A", "B", "C", "d")}
+    many["offsets"] = np.arange(rays + 1, dtype=np.int32) * n
+    err = []
+    for q in (s, many):
+        x, ok = _solve(q, m, n_refine)
+        assert ok
+        err.append(np.abs(x[:n] - ref).max() / np.abs(ref).max())
+    assert err[0] <= 4 * err[1] + 1e-13, err
