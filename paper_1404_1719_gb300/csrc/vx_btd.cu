@@ -257,15 +257,18 @@ __device__ __forceinline__ void st1_if(bool p, unsigned a, unsigned x) {
                  : "memory");
 }
 
-// FP64 to FP32 in integer operations, rounded to nearest (ties away): the conversion instruction runs on the
-// FP64 pipe, at 2 per clock and SM on GB300 (measured); this form is eight integer operations. Half an ulp
-// is added, the exponent rebiased by 896 and clamped: magnitudes below the normal FP32 range become (nearly)
-// 0, those above it and NaN become infinite or NaN, which fails the pivot test.
-__device__ __forceinline__ float btd_f32(double x) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x) + 0x10000000ull;
-    const unsigned hi = (unsigned)(b >> 32);
-    const int e = min(max((int)(hi & 0x7fffffffu) - (896 << 20), 0), 0x0ff00000);
-    return __uint_as_float(__funnelshift_l((unsigned)b, (unsigned)e, 3) | (hi & 0x80000000u));
+// (float)x in integer operations: the conversion instruction runs on the FP64 pipe, at 2 per clock and SM on GB300
+// (measured); this form is about ten integer operations. Nearly half an ulp is added (ties to even) and the
+// exponent rebiased by 896. For zeros and for magnitudes from 2^-126 to below 2^127, which is what
+// btd_plain says; the rest (FP32 subnormals, the last binade, infinities and NaN) goes by the instruction.
+__device__ __forceinline__ bool btd_plain(double x) {
+    const unsigned e = (unsigned)__double2hiint(x) & 0x7fffffffu;
+    return e - (897u << 20) < 253u << 20 || e == 0u;
+}
+__device__ __forceinline__ float btd_plain_f32(double x) {
+    const unsigned long long u = (unsigned long long)__double_as_longlong(x), b = u + 0x0fffffffull + ((u >> 29) & 1ull);
+    const unsigned hi = (unsigned)(b >> 32), e = hi & 0x7fffffffu;
+    return __uint_as_float((e < 1u << 20 ? 0u : __funnelshift_l((unsigned)b, e - (896u << 20), 3)) | (hi & 0x80000000u));
 }
 
 // The blocks in FP32, row-major with row stride ld, for the factor kernel and the sweeps: A_k to At, B_k to Di
@@ -298,11 +301,17 @@ __global__ void __launch_bounds__(kConvThreads) k_btd_convert(const BtdArgs a) {
                 const int i = i0 + r * nw;
                 if (i >= m) break;
                 unsigned bits = 0u;
+                bool plain = true;
 #pragma unroll
                 for (int t = 0; t < NT; ++t) {
-                    if (t < NT - 1 || lane + 32 * t < m) dst[i * ld + 32 * t] = btd_f32(v[r][t]);
+                    plain = plain && btd_plain(v[r][t]);
+                    if (t < NT - 1 || lane + 32 * t < m) dst[i * ld + 32 * t] = btd_plain_f32(v[r][t]);
                     const unsigned long long mag = (unsigned long long)__double_as_longlong(v[r][t]) << 1;
                     bits |= mag != 0ull ? 1u << (4 * t) : 0u;
+                }
+                if (!plain) {
+#pragma unroll 1
+                    for (int t = lane; t < m; t += 32) dst[i * ld + t - lane] = (float)src[i * m + t - lane];
                 }
                 if (w == 1) continue;
                 bits = __reduce_or_sync(0xffffffffu, bits << (lane >> 3));
@@ -835,8 +844,8 @@ __global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(c
                     for (long long e = (long long)mid * m * m + tid; e < z1 * m * m; e += kFactorThreads) {
                         const long long row = e / m;
                         const int c = (int)(e - row * m);
-                        a.At[(size_t)row * ld + c] = btd_f32(a.A[e]);
-                        a.Di[(size_t)row * ld + c] = btd_f32(a.B[e]);
+                        a.At[(size_t)row * ld + c] = (float)a.A[e];
+                        a.Di[(size_t)row * ld + c] = (float)a.B[e];
                     }
                     __threadfence();
                     __syncthreads();
@@ -1134,8 +1143,8 @@ __global__ void __launch_bounds__(256) k_btd_again(const BtdArgs a) {
     const long long mm = (long long)a.m * a.m;
     for (long long e = z0 * mm + blockIdx.y * 256 + threadIdx.x; e < z1 * mm; e += 256 * gridDim.y) {
         const long long row = e / a.m, at = row * a.ld + (e - row * a.m);
-        a.Di[at] = btd_f32(a.B[e]);
-        a.Gt[at] = btd_f32(a.C[e]);
+        a.Di[at] = (float)a.B[e];
+        a.Gt[at] = (float)a.C[e];
     }
 }
 

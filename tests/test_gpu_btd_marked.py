@@ -80,3 +80,40 @@ def test_growth_within_segments(m, seed, kind, scale, n_refine):
         assert ok
         err.append(np.abs(x[:n] - ref).max() / np.abs(ref).max())
     assert err[0] <= 4 * err[1] + 1e-13, err
+
+
+def _all_ones():
+    return np.array([-1], np.int64).view(np.float64)[0]  # the NaN of memory filled with 0xff
+
+
+@pytest.mark.parametrize("m, rays, zones", [(1, 3, 3), (8, 3, 5), (33, 3, 4), (20, 2, 60), (84, 1, 150)])
+@pytest.mark.parametrize("n_refine", [0, 2])
+@pytest.mark.parametrize("block", ["A", "B", "C"])
+def test_nan_of_all_ones(m, rays, zones, n_refine, block):
+    """One entry of one zone: its ray is NaN and flagged, the others are solved."""
+    s = gen.random_system(np.full(rays, zones), m, seed=m)
+    z = zones // 2
+    s[block][z, m - 1, m // 2] = _all_ones()
+    x, ok = _solve(s, m, n_refine)
+    assert not ok and np.isnan(x[:zones]).all()
+    tol = TOL if n_refine else 1e-4
+    for r in range(1, rays):
+        a = r * zones
+        ref = obtd.solve(s["A"][a:a + zones], s["B"][a:a + zones], s["C"][a:a + zones], s["d"][a:a + zones],
+                         np.array([0, zones]))
+        assert np.abs(x[a:a + zones] - ref).max() <= tol * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("zones", [3, 45])
+def test_blocks_below_the_normal_fp32_range(zones):
+    """Diagonal blocks between 2^-128 and 2^-126: subnormal FP32 numbers whose reciprocals are finite. They hold
+    21 to 23 bits, so a sweep gains about 1e-6, and three leave 1e-12."""
+    m = 8
+    s = gen.random_system(np.array([zones]), m, seed=zones)
+    s["A"][:], s["C"][:] = 0.0, 0.0
+    s["B"] *= (2.0 ** -126.1 / np.abs(s["B"]).max(axis=(1, 2)))[:, None, None]
+    s["d"] *= 1e-3
+    x, ok = _solve(s, m, 3)
+    assert ok
+    ref = np.linalg.solve(s["B"], s["d"][..., None])[..., 0]
+    assert np.abs(x - ref).max() <= TOL * np.abs(ref).max()
