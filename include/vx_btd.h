@@ -7,7 +7,7 @@
  * linearised system (sec. 2.1). A radial difference scheme couples a zone only to its neighbours,
  * so for the zones k = 0 .. n-1 of one ray, with m unknowns per zone, that linear system reads
  *
- *     A_k x_{k-1} + B_k x_k + C_k x_{k+1} = d_k        (A_0 and C_{n-1} are not used).
+ *     A_k x_{k-1} + B_k x_k + C_k x_{k+1} = d_k        (A_0 and C_{n-1} are not read).
  *
  * The pair-process source derivatives of vx_rates_spectral (blocks d(j0, chi0)/dJ and
  * d(j1, chi1)/dH of the partner spectrum) are part of B_k in such a system; the radial flux terms

@@ -84,7 +84,9 @@ struct BtdArgs {
     double *x, *r;
     float *Di, *Gt, *At, *y;  // per zone B_k, then D_k^{-1}; C_k, then G_k; A_k in FP32, row-major [m][ld]; y_k [m]
     unsigned short *nz;       // [Z][C, A][mp] zero patterns of the rows
-    int *zbad, *zmid, *flag;  // at a ray's first zone: a pivot failed; the zone its eliminations meet at, from there
+    // zbad, zmid: at a ray's first zone, whether a pivot failed, and the zone its eliminations meet at, from there;
+    // before the elimination, zmid says of every zone which ends of its ray it is (kFirst, kLast)
+    int *zbad, *zmid, *flag;
     const int *inval;  // set by k_btd_validate when the offsets are not a partition of the zones
     // Rays in segments (k_btd_segment): parts > 0: this is the system of the segments' last zones, ray r's from r parts
     // on (above > 0: of segments of such a system, of `above` parts a ray); parts = 0 and pbad: only the rays
@@ -92,6 +94,8 @@ struct BtdArgs {
     int parts, above;
     int *pbad;
 };
+
+constexpr int kFirst = 1, kLast = 2;
 
 // The segments of a ray of n zones: at most `parts`, of four zones or more.
 __host__ __device__ __forceinline__ int seg_count(long long n, int parts) {
@@ -120,18 +124,22 @@ __device__ __forceinline__ long long ray_mid(const BtdArgs &a, long long z0, lon
 
 // offsets[0] = 0, offsets[n_rays] = n_zones and non-decreasing; any violation marks the whole call
 // invalid (so no two rays can share zones) and raises the numeric flag.
-__global__ void k_btd_validate(const int *off, int n_rays, long long n_zones, int *inval, int *flag, int *zbad, int *pbad) {
+__global__ void k_btd_validate(const int *off, int n_rays, long long n_zones, int *inval, int *flag, int *zbad, int *ends,
+                               int *pbad) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i > n_rays) return;
     if (pbad && i < n_rays) pbad[i] = 0;
     const long long v = off[i];
     bool bad = v < 0 || v > n_zones || (i == 0 && v != 0) || (i == n_rays && v != n_zones);
-    if (i < n_rays && off[i + 1] < v) bad = true;
+    const long long e = i < n_rays ? off[i + 1] : v;
+    if (e < v) bad = true;
     if (bad) {
         atomicOr(inval, 1);
         atomicOr(flag, 1);
-    } else if (v < n_zones) {
-        zbad[v] = 0;  // the factor kernel's arrival count
+    } else if (v < e && e <= n_zones) {
+        zbad[v] = 0;                                 // the factor kernel's arrival count
+        ends[v] = v == e - 1 ? kFirst | kLast : kFirst;  // (zero before)
+        if (v < e - 1) ends[e - 1] = kLast;
     }
 }
 
@@ -277,15 +285,20 @@ __device__ __forceinline__ float btd_plain_f32(double x) {
 // the FP64 entries, so that the residual can go by it as well). A CTA takes a matrix at a time, a warp
 // kConvRows of its rows, all their loads in flight together. Bound by HBM (8 m^2 bytes read and 4 m^2 written
 // per block); apart from the factor kernel because the loads' registers, and the conversions' instructions,
-// cost that kernel more than the extra pass.
+// cost that kernel more than the extra pass. A of a ray's first zone and C of its last are left out: the caller's
+// blocks there are not read, and nothing later reads theirs here.
 constexpr int kConvThreads = 256, kConvRows = 4, kConvGrid = 152 * 8;
 template <int NT>
 __global__ void __launch_bounds__(kConvThreads) k_btd_convert(const BtdArgs a) {
     if (*a.inval) return;
     const int m = a.m, ld = a.ld, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = kConvThreads / 32;
+    int ends = a.zmid[blockIdx.x / 3];
     for (long long q = blockIdx.x; q < 3 * a.n_zones; q += gridDim.x) {
         const long long k = q / 3;
         const int w = (int)(q - 3 * k);
+        const bool skip = (w == 0 && (ends & kFirst)) || (w == 2 && (ends & kLast));
+        if (q + gridDim.x < 3 * a.n_zones) ends = a.zmid[(q + gridDim.x) / 3];  // on its way while this one is done
+        if (skip) continue;
         const double *src = (w == 0 ? a.A : w == 1 ? a.B : a.C) + (size_t)k * m * m + lane;
         float *dst = (w == 0 ? a.At : w == 1 ? a.Di : a.Gt) + (size_t)k * m * ld + lane;
         unsigned short *nz = a.nz + ((size_t)k * 2 + (w == 0)) * a.mp;
@@ -1144,7 +1157,7 @@ __global__ void __launch_bounds__(256) k_btd_again(const BtdArgs a) {
     for (long long e = z0 * mm + blockIdx.y * 256 + threadIdx.x; e < z1 * mm; e += 256 * gridDim.y) {
         const long long row = e / a.m, at = row * a.ld + (e - row * a.m);
         a.Di[at] = (float)a.B[e];
-        a.Gt[at] = (float)a.C[e];
+        if (e < (z1 - 1) * mm) a.Gt[at] = (float)a.C[e];
     }
 }
 
@@ -1947,8 +1960,9 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
         }
     }
     BTD_CU(cudaMemsetAsync(h->flag + 1, 0, sizeof(int), s));
+    BTD_CU(cudaMemsetAsync(h->zmid, 0, (size_t)n_zones * sizeof(int), s));
     k_btd_validate<<<(unsigned)((n_rays + 256) / 256), 256, 0, s>>>(ray_offsets, n_rays, n_zones, h->flag + 1, h->flag, h->zbad,
-                                                                   f.pbad);
+                                                                   h->zmid, f.pbad);
     BTD_CU(cudaGetLastError());
     launch_convert(h->m, n_zones, s, a);
     BTD_CU(cudaGetLastError());

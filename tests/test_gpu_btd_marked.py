@@ -117,3 +117,17 @@ def test_blocks_below_the_normal_fp32_range(zones):
     assert ok
     ref = np.linalg.solve(s["B"], s["d"][..., None])[..., 0]
     assert np.abs(x - ref).max() <= TOL * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("m, lengths", [(5, [1, 2, 0, 7, 1, 9]), (40, [3, 1, 45]), (8, [160]), (84, [44, 1]),
+                                        (13, [6] * 200)])
+def test_couplings_past_the_ends(m, lengths):
+    """A of a ray's first zone and C of its last hold anything at all."""
+    s = gen.random_system(lengths, m, seed=m)
+    want, ok = _solve(s, m)
+    assert ok
+    first = s["offsets"][:-1][np.diff(s["offsets"]) > 0]
+    last = s["offsets"][1:][np.diff(s["offsets"]) > 0] - 1
+    s["A"][first], s["C"][last] = _all_ones(), _all_ones()
+    x, ok = _solve(s, m)
+    assert ok and np.array_equal(x, want)
