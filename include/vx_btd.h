@@ -52,10 +52,16 @@ typedef struct vx_btd vx_btd;
 
 /* Creates a solver for m unknowns per zone (1 .. VX_BTD_MAX_M) and batches of at most max_zones
  * zones (>= 0), with n_refine FP64 refinement sweeps (0 .. VX_BTD_MAX_REFINE; 0 leaves the FP32
- * solution). Allocates the device workspace: 12 m (m + 7) + 4 (m + 7) + 12 m + 8 bytes per zone at most, and for
- * the segments (m up to about 110) 4 m (m + 7) for each of the first 16384 zones and 36 m (m + 8) per SM; without the
- * memory for the latter, rays are not cut into segments. *out is set to NULL on failure. Errors: VX_ERR_INVALID_ARG, VX_ERR_OOM, VX_ERR_CUDA. */
+ * solution). Allocates the device workspace: 12 m (m + 7) + 4 (m + 7) + 12 m + 8 bytes per zone at most, and, for
+ * max_zones of 40 or more and m up to 116, what rays in segments take besides: 4 m (m + 7) for each zone that
+ * 4 min(max_zones, 16384) exceeds 3 max_zones by (none from 21,846 zones on), and 36 m^2 + 300 m + 76 per SM. Without
+ * the memory for that, rays are not cut into segments. *out is set to NULL on failure. Errors: VX_ERR_INVALID_ARG,
+ * VX_ERR_OOM, VX_ERR_CUDA. */
 vx_status vx_btd_create(int m, long long max_zones, int n_refine, vx_btd **out);
+
+/* The same for calls of min_rays rays (>= 1) or more: where such calls are never cut into segments (min_rays above
+ * a fifth of the SMs), the memory for that is not taken. Calls of fewer rays are solved all the same, as a whole. */
+vx_status vx_btd_create_rays(int m, long long max_zones, int n_refine, int min_rays, vx_btd **out);
 
 /* Solves every ray. n_rays >= 0; n_zones = the total zone count, 0 .. max_zones.
  *   ray_offsets: device int32 [n_rays + 1]; ray r owns zones ray_offsets[r] .. ray_offsets[r+1]-1.

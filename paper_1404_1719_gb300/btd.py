@@ -12,11 +12,13 @@ class BlockTridiagSolver:
     """Solves, for every ray, A_k x_{k-1} + B_k x_k + C_k x_{k+1} = d_k over its zones k.
 
     m unknowns per zone (1..128); at most ``max_zones`` zones per call; ``n_refine`` FP64
-    refinement sweeps after the FP32 block factorisation (see include/vx_btd.h)."""
+    refinement sweeps after the FP32 block factorisation (see include/vx_btd.h). A program whose
+    calls hold at least ``min_rays`` rays can say so: from 31 on (GB300) the handle then does without the
+    memory for rays in segments."""
 
-    def __init__(self, m: int, max_zones: int, n_refine: int = 2):
+    def __init__(self, m: int, max_zones: int, n_refine: int = 2, min_rays: int = 1):
         self.m, self.max_zones, self.n_refine = int(m), int(max_zones), int(n_refine)
-        self.handle = capi.vx_btd_create(self.m, self.max_zones, self.n_refine)
+        self.handle = capi.vx_btd_create_rays(self.m, self.max_zones, self.n_refine, int(min_rays))
 
     def _args(self, offsets, A, B, C, d):
         m = self.m

@@ -52,7 +52,7 @@ class VxError(RuntimeError):
 SYMBOLS = ("vx_rates_create", "vx_rates_eval", "vx_rates_adjoint", "vx_rates_check",
            "vx_rates_entries_per_zone", "vx_rates_destroy", "vx_status_string", "vx_last_error",
            "vx_rates_eval_noalloc", "vx_rates_spectral", "vx_rates_eval_host", "vx_rates_adjoint_host",
-           "vx_rates_spectral_host", "vx_btd_create", "vx_btd_solve", "vx_btd_check", "vx_btd_destroy",
+           "vx_rates_spectral_host", "vx_btd_create", "vx_btd_create_rays", "vx_btd_solve", "vx_btd_check", "vx_btd_destroy",
            "vx_probe_pipes", "vx_nes_create", "vx_nes_eval", "vx_nes_adjoint", "vx_nes_check", "vx_nes_destroy",
            "vx_eos_eta", "vx_eos_chain", "vx_nes_eval_host", "vx_nes_adjoint_host", "vx_abs_create", "vx_abs_eval", "vx_abs_adjoint", "vx_abs_check",
            "vx_abs_destroy")
@@ -103,6 +103,8 @@ def lib(path: str | None = None):
     L.vx_last_error.restype = ctypes.c_char_p
     L.vx_btd_create.argtypes = [ctypes.c_int, ctypes.c_longlong, ctypes.c_int, ctypes.POINTER(ctypes.c_void_p)]
     L.vx_btd_create.restype = ctypes.c_int
+    L.vx_btd_create_rays.argtypes = [ctypes.c_int, ctypes.c_longlong, ctypes.c_int, ctypes.c_int, ctypes.POINTER(ctypes.c_void_p)]
+    L.vx_btd_create_rays.restype = ctypes.c_int
     L.vx_btd_solve.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_longlong] + [ctypes.c_void_p] * 7
     L.vx_btd_solve.restype = ctypes.c_int
     L.vx_btd_check.argtypes = [ctypes.c_void_p, ctypes.c_void_p]
@@ -236,6 +238,13 @@ VX_BTD_MAX_M, VX_BTD_MAX_REFINE = 128, 8
 def vx_btd_create(m: int, max_zones: int, n_refine: int) -> ctypes.c_void_p:
     h = ctypes.c_void_p()
     _check(lib().vx_btd_create(int(m), int(max_zones), int(n_refine), ctypes.byref(h)), "vx_btd_create")
+    return h
+
+
+def vx_btd_create_rays(m: int, max_zones: int, n_refine: int, min_rays: int) -> ctypes.c_void_p:
+    h = ctypes.c_void_p()
+    _check(lib().vx_btd_create_rays(int(m), int(max_zones), int(n_refine), int(min_rays), ctypes.byref(h)),
+           "vx_btd_create_rays")
     return h
 
 

@@ -1712,22 +1712,26 @@ constexpr size_t kSmemHalf = 113 * 1024 - 64, kSmemFull = 226 * 1024;
 
 // Zones from which on segments are laid out, and for which they have room.
 constexpr long long kSegMinZones = 40, kSegMaxZones = 16384, kSegTwoLevels = 150;
+constexpr int kSegMinParts = 5;  // fewest segments of a ray
 
 struct vx_btd {
     int m = 0, ld = 0, mp = 0, nbuf = 3, nring = 2, n_refine = 0;
     long long max_zones = 0;
     size_t smem = 0, smem_sweep = 0;
-    float *Di = nullptr, *Gt = nullptr, *At = nullptr, *y = nullptr;
+    // Room for blocks * m * ld floats: a call lays B, C and A of its zones there, one array after the other, and
+    // then L, if it cuts rays into segments and a quarter of the room holds its zones. A handle of 21,845 zones or more
+    // has that for the 16,384 zones that segments go to at most; for smaller ones the room is larger by up to a third.
+    float *blk = nullptr, *y = nullptr;
+    size_t blocks = 0;
     unsigned short *nz = nullptr;
     int slots = 0;  // factor CTAs the device holds at once
     int *zbad = nullptr, *zmid = nullptr, *flag = nullptr;  // flag[0]: numeric flag, flag[1]: offsets invalid
     double *r = nullptr;
-    // segments: null, or rows of the segments' system (one per SM) and zones that L has room for
+    // segments: most zones of a call that is cut into them (0: none), and their system's arrays (a row per SM)
     int sms = 1, seg_nbuf = 0;
     long long seg_zones = 0;
     size_t smem_seg = 0;
-    float *Lt = nullptr, *Sr = nullptr;  // Lt: of the zones and of the system's rows; Sr: per level, the system's
-                                         // four blocks per row, then the levels' y
+    float *Sr = nullptr;  // per level, the system's four blocks per row; then L of its rows, then the levels' y
     unsigned short *nzr = nullptr;       // per level
     int *zr = nullptr;                   // per level zbad, zmid of that system; pbad
     double *vr = nullptr;                // right-hand sides of both levels' systems, then the solutions
@@ -1735,14 +1739,11 @@ struct vx_btd {
 
 static void btd_free(vx_btd *h) {
     if (!h) return;
-    cudaFree(h->Di);
+    cudaFree(h->blk);
     cudaFree(h->nz);
-    cudaFree(h->Gt);
-    cudaFree(h->At);
     cudaFree(h->y);
     cudaFree(h->zbad);
     cudaFree(h->zmid);
-    cudaFree(h->Lt);
     cudaFree(h->Sr);
     cudaFree(h->nzr);
     cudaFree(h->zr);
@@ -1753,12 +1754,17 @@ static void btd_free(vx_btd *h) {
 }
 
 extern "C" vx_status vx_btd_create(int m, long long max_zones, int n_refine, vx_btd **out) {
+    return vx_btd_create_rays(m, max_zones, n_refine, 1, out);
+}
+
+extern "C" vx_status vx_btd_create_rays(int m, long long max_zones, int n_refine, int min_rays, vx_btd **out) {
     if (!out) return bfail(VX_ERR_INVALID_ARG, "out is NULL");
     *out = nullptr;
     if (m < 1 || m > VX_BTD_MAX_M) return bfail(VX_ERR_INVALID_ARG, "m = %d outside 1..%d", m, VX_BTD_MAX_M);
     if (max_zones < 0) return bfail(VX_ERR_INVALID_ARG, "max_zones = %lld < 0", max_zones);
     if (n_refine < 0 || n_refine > VX_BTD_MAX_REFINE)
         return bfail(VX_ERR_INVALID_ARG, "n_refine = %d outside 0..%d", n_refine, VX_BTD_MAX_REFINE);
+    if (min_rays < 1) return bfail(VX_ERR_INVALID_ARG, "min_rays = %d < 1", min_rays);
     vx_btd *h = new (std::nothrow) vx_btd;
     if (!h) return bfail(VX_ERR_OOM, "host allocation failed");
     h->m = m;
@@ -1778,47 +1784,25 @@ extern "C" vx_status vx_btd_create(int m, long long max_zones, int n_refine, vx_
     h->nring = ring(4) <= kSmemHalf ? 4 : ring(3) <= kSmemFull ? 3 : 2;
     h->smem_sweep = ring(h->nring);
     const size_t zc = (size_t)(max_zones > 0 ? max_zones : 1);
-    cudaError_t e = cudaSuccess;
-    if (e == cudaSuccess) e = cudaMalloc(&h->Di, zc * mw * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&h->Gt, zc * mw * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&h->At, zc * mw * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&h->nz, zc * 2 * h->mp * sizeof(unsigned short));
-    if (e == cudaSuccess) e = cudaMalloc(&h->y, zc * m * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&h->zbad, zc * sizeof(int));
-    if (e == cudaSuccess) e = cudaMalloc(&h->zmid, zc * sizeof(int));
-    if (e == cudaSuccess) e = cudaMalloc(&h->r, zc * m * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&h->flag, 2 * sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(h->flag, 0, 2 * sizeof(int));
     int dev = 0;
-    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev);
-    h->slots = h->sms * (h->smem <= kSmemHalf && m <= 96 ? 2 : 1);
-    if (h->ld != m)  // the columns that pad a row are read by the sweeps and never written
-        for (float *w : {h->Di, h->Gt, h->At})
-            if (e == cudaSuccess) e = cudaMemset(w, 0, zc * mw * sizeof(float));
-    // the kernels' limit, not this handle's size: handles of several m share them
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(factor_kernel(m), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFull);
-    const void *sweeps[4] = {sweep_kernel<true, true>(m), sweep_kernel<true, false>(m), sweep_kernel<false, true>(m),
-                             sweep_kernel<false, false>(m)};
-    for (int i = 0; i < 4 && e == cudaSuccess; ++i)
-        e = cudaFuncSetAttribute(sweeps[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFull);
     // segments where their four or five buffers fit; without the memory for them, rays go as a whole
     h->seg_nbuf = factor_smem(m, h->ld, 5) <= kSmemFull ? 5 : factor_smem(m, h->ld, 4) <= kSmemFull ? 4 : 0;
-    if (e == cudaSuccess && h->seg_nbuf && max_zones >= kSegMinZones) {
+    bool seg = h->seg_nbuf && max_zones >= kSegMinZones && min_rays <= h->sms / kSegMinParts;
+    h->blocks = 3 * zc;
+    if (e == cudaSuccess && seg) {
         const size_t rows = (size_t)h->sms;
-        h->smem_seg = factor_smem(m, h->ld, h->seg_nbuf);
         h->seg_zones = max_zones < kSegMaxZones ? max_zones : kSegMaxZones;
-        cudaError_t q = cudaMalloc(&h->Lt, (h->seg_zones + rows) * mw * sizeof(float));
-        if (q == cudaSuccess) q = cudaMalloc(&h->Sr, 2 * rows * (4 * mw + m) * sizeof(float));
+        h->smem_seg = factor_smem(m, h->ld, h->seg_nbuf);
+        if (4 * (size_t)h->seg_zones > h->blocks) h->blocks = 4 * (size_t)h->seg_zones;
+        cudaError_t q = cudaMalloc(&h->blk, h->blocks * mw * sizeof(float));
+        if (q == cudaSuccess) q = cudaMalloc(&h->Sr, rows * (9 * mw + 2 * m) * sizeof(float));
         if (q == cudaSuccess) q = cudaMalloc(&h->nzr, 2 * rows * 2 * h->mp * sizeof(unsigned short));
         if (q == cudaSuccess) q = cudaMalloc(&h->zr, 5 * rows * sizeof(int));
         if (q == cudaSuccess) q = cudaMalloc(&h->vr, 4 * rows * m * sizeof(double));
         if (q == cudaSuccess) {
-            if (h->ld != m) {
-                e = cudaMemset(h->Lt, 0, (h->seg_zones + rows) * mw * sizeof(float));
-                if (e == cudaSuccess) e = cudaMemset(h->Sr, 0, 2 * rows * (4 * mw + m) * sizeof(float));
-            }
+            if (h->ld != m) e = cudaMemset(h->Sr, 0, rows * (9 * mw + 2 * m) * sizeof(float));
             const void *ks[4] = {segment_kernel(m), seg_sweep_kernel<false, true>(m), seg_sweep_kernel<true, true>(m),
                                  seg_sweep_kernel<true, false>(m)};
             for (int i = 0; i < 4 && e == cudaSuccess; ++i)
@@ -1827,8 +1811,31 @@ extern "C" vx_status vx_btd_create(int m, long long max_zones, int n_refine, vx_
             h->seg_zones = 0;
             if (q == cudaErrorMemoryAllocation) (void)cudaGetLastError();
             else e = q;
+            if (h->blocks > 3 * zc) {
+                cudaFree(h->blk);
+                h->blk = nullptr;
+                h->blocks = 3 * zc;
+            }
         }
     }
+    if (e == cudaSuccess && !h->blk) e = cudaMalloc(&h->blk, h->blocks * mw * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc(&h->nz, zc * 2 * h->mp * sizeof(unsigned short));
+    if (e == cudaSuccess) e = cudaMalloc(&h->y, zc * m * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc(&h->zbad, zc * sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&h->zmid, zc * sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&h->r, zc * m * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc(&h->flag, 2 * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(h->flag, 0, 2 * sizeof(int));
+    h->slots = h->sms * (h->smem <= kSmemHalf && m <= 96 ? 2 : 1);
+    if (h->ld != m && e == cudaSuccess)  // the columns that pad a row are read by the sweeps and never written
+        e = cudaMemset(h->blk, 0, h->blocks * mw * sizeof(float));
+    // the kernels' limit, not this handle's size: handles of several m share them
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(factor_kernel(m), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFull);
+    const void *sweeps[4] = {sweep_kernel<true, true>(m), sweep_kernel<true, false>(m), sweep_kernel<false, true>(m),
+                             sweep_kernel<false, false>(m)};
+    for (int i = 0; i < 4 && e == cudaSuccess; ++i)
+        e = cudaFuncSetAttribute(sweeps[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFull);
     if (e != cudaSuccess) {
         btd_free(h);
         return bfail(e == cudaErrorMemoryAllocation ? VX_ERR_OOM : VX_ERR_CUDA, "vx_btd_create: %s",
@@ -1878,10 +1885,11 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
     a.rhs = d;
     a.x = x;
     a.r = h->r;
-    a.Di = h->Di;
+    const size_t arr = (size_t)n_zones * h->m * h->ld;
+    a.Di = h->blk;
+    a.Gt = a.Di + arr;
+    a.At = a.Gt + arr;
     a.nz = h->nz;
-    a.Gt = h->Gt;
-    a.At = h->At;
     a.y = h->y;
     a.zbad = h->zbad;
     a.zmid = h->zmid;
@@ -1908,8 +1916,8 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
     const long long mean = n_zones / n_rays;
     const int most_parts = n_rays < h->sms ? h->sms / n_rays : 0;
     int parts = most_parts, top = 0;
-    while (parts > 5 && (long long)parts * parts > 3 * mean) --parts;
-    const bool seg = parts >= 5 && mean >= kSegMinZones && n_zones <= h->seg_zones;
+    while (parts > kSegMinParts && (long long)parts * parts > 3 * mean) --parts;
+    const bool seg = parts >= kSegMinParts && mean >= kSegMinZones && n_zones <= h->seg_zones;
     // Two levels where there is room for more: S^1.5 <= 1.45 n segments of the ray, and 1.75 S^0.5 of their system
     // (at 48, 58 and 38 us a zone of either level and of the last system, that takes least).
     // GB300, m = 84, one level -> two: 1 ray of 100 zones 0.82 -> 0.82 ms, 150 1.03 -> 0.86, 400 1.61 -> 1.16, 1000
@@ -1936,7 +1944,7 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
             q.parts = l ? top : parts;
             q.above = l ? parts : 0;
             q.nbuf = h->seg_nbuf;
-            q.Lt = h->Lt + (l ? h->seg_zones * mw : 0);
+            q.Lt = l ? h->Sr + rows * 8 * mw : a.At + arr;
             q.Dr = h->Sr + l * rows * 4 * mw;
             q.Cr = q.Dr + rows * mw;
             q.Ar = q.Cr + rows * mw;
@@ -1951,7 +1959,7 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
             b.Di = q.Dr;
             b.Gt = q.Cr;
             b.At = q.Ar;
-            b.y = h->Sr + 2 * rows * 4 * mw + l * vec32;
+            b.y = h->Sr + rows * 9 * mw + l * vec32;
             b.nz = q.nzr;
             b.zbad = q.zbadr;
             b.zmid = q.zbadr + rows;

@@ -131,3 +131,38 @@ def test_couplings_past_the_ends(m, lengths):
     s["A"][first], s["C"][last] = _all_ones(), _all_ones()
     x, ok = _solve(s, m)
     assert ok and np.array_equal(x, want)
+
+
+@pytest.mark.parametrize("m, zones, min_rays", [(84, 30000, 1), (84, 8000, 31), (84, 8000, 1), (45, 30000, 1), (128, 4000, 1)])
+def test_workspace(m, zones, min_rays):
+    """Device memory of a handle: per zone what every call needs, and what rays in segments take besides (the header's
+    bounds; an array is rounded up to 2 MiB)."""
+    from paper_1404_1719_gb300 import BlockTridiagSolver
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    bound = (12 * m * (m + 7) + 4 * (m + 7) + 12 * m + 8) * zones
+    if m <= 116 and min_rays <= sms // 5:
+        bound += 4 * m * (m + 7) * max(0, 4 * min(zones, 16384) - 3 * zones) + (36 * m * m + 300 * m + 76) * sms
+    BlockTridiagSolver(m, 1).close()  # the kernels are loaded
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    sv = BlockTridiagSolver(m, zones, min_rays=min_rays)
+    used = before - torch.cuda.mem_get_info()[0]
+    sv.close()
+    assert used <= bound + 16 * 2 ** 21
+
+
+@pytest.mark.parametrize("m", [8, 13, 84])
+@pytest.mark.parametrize("max_zones, min_rays", [(600, 1), (600, 31), (24000, 1)])
+def test_calls_of_any_size(m, max_zones, min_rays):
+    """One handle, batches of different zone counts one after the other: whatever an earlier call left in the workspace."""
+    from paper_1404_1719_gb300 import BlockTridiagSolver
+    sv = BlockTridiagSolver(m, max_zones, min_rays=min_rays)
+    for lengths in ([600], [40, 100], [3] * 180, [150], [1], [600], [200, 200, 200]):
+        s = gen.random_system(lengths, m, seed=len(lengths) + lengths[0])
+        t = {k: torch.from_numpy(np.ascontiguousarray(s[k])).cuda() for k in ("offsets", "A", "B", "C", "d")}
+        x = sv.solve(t["offsets"].to(torch.int32), t["A"], t["B"], t["C"], t["d"]).cpu().numpy()
+        assert sv.check()
+        for a, b in zip(s["offsets"][:-1], s["offsets"][1:]):
+            ref = obtd.solve(s["A"][a:b], s["B"][a:b], s["C"][a:b], s["d"][a:b], np.array([0, b - a]))
+            assert np.abs(x[a:b] - ref).max() <= TOL * np.abs(ref).max()
+    sv.close()
