@@ -645,15 +645,31 @@ __global__ void __launch_bounds__(BLK, std::is_same<R, float>::value && BLK == k
     }
 }
 
-// Threads per CTA for a batch of Z zones: four times kNesBlock up to two zones per SM, twice up to three and a
-// half, where CTAs of kNesBlock leave the SMs' issue slots idle (the slowest zone's latency sets the time).
-// GB300, 21 bins, 16 x 48, rates and Jacobian, us at 128 / 256 / 512 threads: 152 zones 70 / 50 / 44,
-// 304 zones 89 / 76 / 74, 400 zones 116 / 94 / 104, 500 zones 135 / 126 / 134, 608 zones 148 / 153 / 142,
-// 760 zones 168 / 158 / 175, 1000 zones 212 / 215 / 233. The FP64 form gains nothing (its pipe is full).
+// Threads per CTA for a batch of Z zones: twice kNesBlock up to two zones per SM, where CTAs of kNesBlock leave the SMs'
+// issue slots idle (a zone's latency sets the time), and up to three and a half where that kernel still gains; four
+// times with at most one zone per SM (tangents: one and a half) and enough pairs for its 16 warps. Which
+// kernels gain depends on the registers: 80 let three CTAs of 256 threads share an SM (rates, any panel size but 8 and
+// 16), 89 to 104 two. The FP64 form gains nothing (its pipe is full). GB300, us at 128 / 256 / 512 threads:
+//   tangents, 21 bins, 16 angles, panels of 16 nodes: 152 zones 73 / 51 / 44, 228 92 / 77 / 75, 304 92 / 77 / 79,
+//     400 119 / 102 / 110, 500 146 / 138 / 137, 532 147 / 152 / 141, 608 148 / 160 / 146, 760 177 / 166 / 176;
+//     13 bins: 152 zones 39 / 33 / 36, 400 56 / 50 / 56, 532 67 / 63 / 71, 608 68 / 66 / 76
+//   tangents, 21 bins, 12 angles, panels of 12: 152 zones 69 / 49 / 42, 304 87 / 70 / 76, 400 106 / 118 / 106, 500 129 / 123 / 132
+//   tangents, 21 bins, 8 angles, panels of 8: 152 zones 36 / 33 / 35, 304 41 / 35 / 39, 400 49 / 48 / 52, 500 59 / 57 / 65
+//   rates, panels of 16, 21 bins: 152 zones 56 / 36 / 34 to 37, 304 60 / 44 / 48, 400 67 / 72 / 65, 500 80 / 75 / 80; 25 bins: 152
+//     74 / 46 / 36, 304 81 / 58 / 62, 400 91 / 97 / 83
+//   rates, panels of 12, 21 bins: 304 56 / 40 / 44, 500 71 / 64 / 73; 25 bins: 152 67 / 43 / 34, 400 81 / 72 / 75
+//   rates, panels of 8, 25 bins: 152 zones 36 / 31 / 34, 400 40 / 46 / 42, 500 46 / 46 / 52
+// (Two limits for all of them, as it once was, cost rates of 350 to 456 zones 8 to 15 %, and 512 threads with few pairs 10 %.)
 template <typename R>
-int nes_block(long long Z, int nsm) {
+int nes_block(const NesCommon &C, bool adj, long long Z, int nsm) {
     if (!std::is_same<R, float>::value) return kNesBlock;
-    return Z <= 2ll * nsm ? 4 * kNesBlock : 2 * Z <= 7ll * nsm ? 2 * kNesBlock : kNesBlock;
+    const bool unrolled = C.n_p == 8 || C.n_p == 16;
+    const long long work = (long long)C.npair * C.n_p, per = 16ll * C.ppw;  // of a zone; pairs that 16 warps take at once
+    if ((Z <= nsm && work >= (adj ? 50 : 85) * per) || (adj && 2 * Z <= 3ll * nsm && work >= 100 * per)) return 4 * kNesBlock;
+    if (Z <= 2ll * nsm) return 2 * kNesBlock;
+    if (Z <= 3ll * nsm) return unrolled == adj ? 2 * kNesBlock : kNesBlock;
+    if (2 * Z > 7ll * nsm || (!adj && C.n_p == 8)) return kNesBlock;
+    return adj && C.n_p == 16 && 10 * Z > 33ll * nsm && work >= 100 * per ? kNesBlock : 2 * kNesBlock;
 }
 
 template <typename R, bool ADJ, int BLK>
@@ -881,7 +897,7 @@ vx_status nes_run(vx_nes *h, const vx_batch *b, const vx_out *out, double *jac, 
     const bool adj = jac != nullptr;
     const int grid = (int)std::min<long long>(h->grid[adj], b->n_zones);
     NES_CU(cudaMemsetAsync(L.counter, 0, sizeof(unsigned long long), s));
-    const int blk = vx::nes_block<R>(b->n_zones, h->nsm);
+    const int blk = vx::nes_block<R>(L.c, adj, b->n_zones, h->nsm);
     cudaError_t e;
     if constexpr (std::is_same<R, float>::value) {
         if (blk == 4 * kNesBlock)
