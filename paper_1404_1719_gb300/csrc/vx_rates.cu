@@ -564,22 +564,32 @@ static void cache_write(const char *path, const std::string &key, const std::str
 }
 
 // The register budget of a launch: the autotuned one, else as follows. The tangent kernel takes the smaller one (five
-// CTAs per SM, not four), except with the split rule, whose two panels do not fit 96 registers, and where each
-// CTA of the larger one has at most one zone, which then ends sooner. GB300, five per SM -> four, zones at 64
+// CTAs per SM, not four), except where each CTA of the larger one has at most one zone, which then ends sooner
+// (with 48 nodes or more; with the split rule at any number of nodes, and from 48 on up to two zones), and with the split
+// rule at 32 and 48 nodes, whose two unrolled panels do not fit 96 registers. GB300, five per SM -> four, zones at 64
 // nodes and 21 bins: 64 125 -> 117 us, 400 226 -> 223, 608 310 -> 300, 760 352 -> 364, 25,600 9690 -> 9787; at 48
 // nodes and eta_e to 60: 64 83 -> 85, 400 128 -> 124, 608 157 -> 154, 760 182 -> 193; at 32 nodes and 13 bins: 152 48.7
-// -> 50.2, 400 56.2 -> 57.4; split rule at 48 nodes: 64 156 -> 120, 400 255 -> 231, 2400 722 -> 693, 25,600
-// 6716 -> 6438. The forward kernel takes the larger one until the batch fills its grid more than twice. Six CTAs of 128
+// -> 50.2, 400 56.2 -> 57.4. Split rule, 16 angles, 21 bins, eta_e to 20 | to 60: 16 nodes, 64 zones 41 -> 42 | 72 -> 63,
+// 608 65 -> 65 | 131 -> 128, 1216 109 -> 114 | 218 -> 212, 6400 485 -> 503 | 839 -> 854; 20 nodes, 608 90 -> 89 | 172 ->
+// 170, 6400 767 -> 833 | 1212 -> 1251; 32 nodes, 608 104 -> 95 | 218 -> 202, 6400 821 -> 787 | 1419 -> 1350; 48 nodes,
+// 608 133 -> 123 | 298 -> 275, 6400 1087 -> 1061 | 1948 -> 1864; 64 nodes, 608 147 -> 147 | 363 -> 346, 1216 265 -> 262 |
+// 607 -> 575, 2400 491 -> 525 | 1012 -> 983, 6400 1285 -> 1306 | 2396 -> 2364.
+// The forward kernel takes the larger one until the batch fills its grid more than twice. Six CTAs of 128
 // threads per SM at 80 registers hide each other's MUFU and shared-memory latencies better than four at 128
 // (MUFU 55 %, FP32 pipe 50 % busy), but a zone by itself takes longer. GB300, four per SM -> six, zones at 64 nodes
 // and 21 bins: 64 74.6 -> 79.9 us, 304 115 -> 118, 1216 288 -> 273, 2400 492 -> 456, 3200 610 -> 620, 6400
 // 1196 -> 1153; at 48 nodes and eta_e to 60: 400 84 -> 86, 912 122 -> 131, 2000 234 -> 223, 9600 971 -> 942; at
-// 32 nodes and 13 bins: 400 43.7 -> 45.8, 1600 78 -> 72, 9600 293 -> 260.
+// 32 nodes and 13 bins: 400 43.7 -> 45.8, 1600 78 -> 72, 9600 293 -> 260. The split rule and the precise mode follow,
+// 6400 zones, 16 angles, 21 bins: 16 nodes 319 -> 264 split, 32 nodes 395 -> 361 and 522 -> 504 precise, 48 497 -> 475 and
+// 689 -> 667, 64 624 -> 591 and 833 -> 827.
 static int mixed_budget(const vx_rates *h, bool adj, long long zones) {
     if (h->tuned[adj]) return h->minb[adj];
     if (adj) {
         if (h->common.precise) return h->minb[1];
-        return h->common.split || (zones <= h->grid_mixed[1][0] && h->common.n_e >= 48) ? 2 : h->minb[1];
+        const int n_e = h->common.n_e;
+        if (h->common.split && (n_e == 32 || n_e == 48)) return 2;
+        const long long most = n_e >= 48 ? (h->common.split ? 2 : 1) : h->common.split ? 1 : 0;  // zones per CTA
+        return zones <= most * h->grid_mixed[1][0] ? 2 : h->minb[1];
     }
     return zones > 2LL * h->grid_mixed[0][0] ? 3 : h->minb[0];
 }

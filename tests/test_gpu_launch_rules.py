@@ -38,3 +38,14 @@ def test_scattering(n_bins, n_mu, n_e):
                [n + d for n in borders for d in (0, 1)])
     assert r.check()
     r.close()
+
+
+@pytest.mark.parametrize("n_e", [16, 20, 32, 48, 64])
+def test_split_tangents(n_e):
+    from paper_1404_1719_gb300 import PairRates
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    r = PairRates(vx_inputs.energy_centres(11, 1.0, 300.0), 7, n_e, split=True)
+    _same_bits((lambda *x: r.adjoint(*x, forward=True),), 11, 12 * sms, [n + d for n in (4 * sms, 8 * sms) for d in (0, 1)],
+               eta=(0.0, 60.0))
+    assert r.check()
+    r.close()
