@@ -149,7 +149,8 @@ __device__ __forceinline__ void btd_mma(float (&d)[4], const unsigned (&a)[4], c
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 // v = hi + lo, hi the nearest TF32 value (half an ulp of TF32 added to the magnitude bits, the last 13
-// cleared), lo the exact remainder cut to TF32 (error 2^-21 |v|).
+// cleared), lo the exact remainder cut to TF32: a whole number of at most 2^12 ulps of v, of which TF32 holds all or all
+// but the last bit, so cutting and rounding are off by the same, an ulp of v at most (2^-23 |v|).
 __device__ __forceinline__ void btd_split(float v, unsigned &hi, unsigned &lo) {
     hi = (__float_as_uint(v) + 0x1000u) & 0xffffe000u;
     lo = __float_as_uint(__fsub_rn(v, __uint_as_float(hi))) & 0xffffe000u;
@@ -287,7 +288,7 @@ __device__ __forceinline__ float btd_plain_f32(double x) {
 // per block); apart from the factor kernel because the loads' registers, and the conversions' instructions,
 // cost that kernel more than the extra pass. A of a ray's first zone and C of its last are left out: the caller's
 // blocks there are not read, and nothing later reads theirs here.
-constexpr int kConvThreads = 256, kConvRows = 4, kConvGrid = 152 * 8;
+constexpr int kConvThreads = 256, kConvRows = 4, kConvGrid = 8;  // kConvGrid: CTAs per SM
 template <int NT>
 __global__ void __launch_bounds__(kConvThreads) k_btd_convert(const BtdArgs a) {
     if (*a.inval) return;
@@ -610,7 +611,7 @@ __device__ __forceinline__ void tile_update(float *X, int ld, int m, int p, int 
     }
 }
 
-// Shared memory of the factor kernel: nbuf buffers of m x ld floats (16 floats of slack each: the last
+// Shared memory of the factor and segment kernels: nbuf buffers of m x ld floats (16 floats of slack each: the last
 // tiles read past the end of a row), the zero patterns of C_k's and A_{k+1}'s rows, two rows
 // of a panel, the pivot rows and their inverse.
 __host__ __device__ constexpr int factor_buf(int m, int ld) { return (m * ld + 16 + 3) & ~3; }
@@ -618,6 +619,24 @@ __host__ __device__ constexpr size_t factor_smem(int m, int ld, int nbuf) {
     return (size_t)nbuf * factor_buf(m, ld) * sizeof(float) + (size_t)(16 + 3 * ((m + 7) & ~7)) * sizeof(int) +
            (size_t)m * sizeof(int);
 }
+
+// Row stride of the blocks: 4 mod 8 floats, so that the MMA fragments of the left operand (eight rows, four columns) fall
+// in distinct banks, and a matrix is copied in whole 16-byte pieces.
+__host__ __device__ constexpr int row_stride(int m) { return m + (12 - m % 8) % 8; }
+
+// tile_update reads whole groups of 16 NT rows, so up to 31 rows past the end of X, and eight columns of the last panel.
+// X is the first buffer, or the second of four or more: what it reads there has to be memory of the CTA.
+constexpr bool reads_stay_inside() {
+    for (int m = 1; m <= VX_BTD_MAX_M; ++m) {
+        const int nt = (m + 31) / 32, ld = row_stride(m), rows = (m + 16 * nt - 1) / (16 * nt) * 16 * nt;
+        for (int nbuf = 3; nbuf <= 5; ++nbuf) {
+            const size_t x = nbuf > 3 ? factor_buf(m, ld) : 0, end = x + (size_t)(rows - 1) * ld + 8 * ((m + 7) / 8);
+            if (end * sizeof(float) > factor_smem(m, ld, nbuf)) return false;
+        }
+    }
+    return true;
+}
+static_assert(reads_stay_inside(), "tile_update reads past the shared memory");
 
 // X -= U V, all in shared memory; the rows of U hold something only in the groups that nz marks.
 template <int NT>
@@ -791,7 +810,7 @@ __global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(c
     const int m = a.m, ld = a.ld, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int bs = factor_buf(m, ld), P = (m + 7) >> 3;
     const bool four = a.nbuf == 4;
-    // D_k and the next zone's B come first: tile_update reads up to 15 rows past the end of D_k
+    // D_k and the next zone's B come first: tile_update reads past the end of D_k (reads_stay_inside)
     // (offsets, not pointers, are exchanged from zone to zone: the compiler then knows the address space)
     int xo = 0, bo = four ? bs : 0;
     float *const sG = sm + bo + bs, *const sA = sG + bs;
@@ -1656,8 +1675,8 @@ static void launch_factor(int m, int grid, size_t smem, cudaStream_t s, const Bt
     else if (m <= 96) k_btd_factor<3><<<grid, kFactorThreads, smem, s>>>(a);
     else k_btd_factor<4><<<grid, kFactorThreads, smem, s>>>(a);
 }
-static void launch_convert(int m, long long zones, cudaStream_t s, const BtdArgs &a) {
-    const int grid = (int)(3 * zones < kConvGrid ? 3 * zones : kConvGrid);
+static void launch_convert(int m, long long zones, int sms, cudaStream_t s, const BtdArgs &a) {
+    const int grid = (int)(3 * zones < kConvGrid * sms ? 3 * zones : kConvGrid * sms);
     if (m <= 32) k_btd_convert<1><<<grid, kConvThreads, 0, s>>>(a);
     else if (m <= 64) k_btd_convert<2><<<grid, kConvThreads, 0, s>>>(a);
     else if (m <= 96) k_btd_convert<3><<<grid, kConvThreads, 0, s>>>(a);
@@ -1768,9 +1787,7 @@ extern "C" vx_status vx_btd_create_rays(int m, long long max_zones, int n_refine
     vx_btd *h = new (std::nothrow) vx_btd;
     if (!h) return bfail(VX_ERR_OOM, "host allocation failed");
     h->m = m;
-    // row stride 4 mod 8 floats: the MMA fragments of the left operand (eight rows, four columns) fall in
-    // distinct banks, and a matrix is copied in whole 16-byte pieces
-    h->ld = m + ((12 - m % 8) % 8);
+    h->ld = row_stride(m);
     h->mp = (m + 7) & ~7;
     h->n_refine = n_refine;
     h->max_zones = max_zones;
@@ -1972,7 +1989,7 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
     k_btd_validate<<<(unsigned)((n_rays + 256) / 256), 256, 0, s>>>(ray_offsets, n_rays, n_zones, h->flag + 1, h->flag, h->zbad,
                                                                    h->zmid, f.pbad);
     BTD_CU(cudaGetLastError());
-    launch_convert(h->m, n_zones, s, a);
+    launch_convert(h->m, n_zones, h->sms, s, a);
     BTD_CU(cudaGetLastError());
     if (seg) {
         for (int l = 0; l < levels; ++l) {
@@ -1990,7 +2007,7 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
     BTD_CU(cudaGetLastError());
     // CTAs per ray of the residual: enough to fill the chip with few rays, at most one per eight units (row octets)
     const long long units = n_zones * ((h->m + 7) / 8);
-    long long split = (8 * 152 + n_rays - 1) / n_rays, most = (units + 8 * n_rays - 1) / (8 * (long long)n_rays);
+    long long split = (8ll * h->sms + n_rays - 1) / n_rays, most = (units + 8 * n_rays - 1) / (8 * (long long)n_rays);
     split = split > most ? most : split;
     split = split < 16 ? 16 : split;
     for (int it = 0; it <= h->n_refine; ++it) {
