@@ -18,7 +18,7 @@
 //    lanes per row (coalesced), zero groups of the couplings left out, FMA accumulation and a fixed two-step
 //    shuffle reduction per row.
 // The host runs validate, convert, [segment, join, once or twice], factor, sweep, then n_refine times (resid,
-// sweep), all on the caller's stream; with segments the factor kernel and the sweeps run once for the segments' system
+// sweep) and once or twice more for the rays with ill-conditioned blocks, all on the caller's stream; with segments the factor kernel and the sweeps run once for the segments' system
 // and once for the rays that have to be done as a whole (3 us each when there are none).
 // With the inverse instead of the elimination's multipliers (which the sweeps replayed, a shuffle per
 // unknown), GB300, m = 84, 400 zones a ray: one ray (one CTA) factor 24.3 -> 10.0 ms, a sweep 3.0 -> 1.3 ms; 304 rays
@@ -87,6 +87,8 @@ struct BtdArgs {
     // zbad, zmid: at a ray's first zone, whether a pivot failed, and the zone its eliminations meet at, from there;
     // before the elimination, zmid says of every zone which ends of its ray it is (kFirst, kLast)
     int *zbad, *zmid, *flag;
+    int *zill;    // at a ray's first zone: how ill-conditioned its blocks are (pivot_level, the highest)
+    int min_ill;  // only the rays of that level or more
     const int *inval;  // set by k_btd_validate when the offsets are not a partition of the zones
     // Rays in segments (k_btd_segment): parts > 0: this is the system of the segments' last zones, ray r's from r parts
     // on (above > 0: of segments of such a system, of `above` parts a ray); parts = 0 and pbad: only the rays
@@ -109,6 +111,7 @@ __device__ __forceinline__ bool ray_range(const BtdArgs &a, int ray, long long &
     z0 = a.off[ray];
     z1 = a.off[ray + 1];
     if (a.pbad && (a.parts > 0) == (a.pbad[ray] != 0)) return false;
+    if (a.min_ill > 0 && (z1 == z0 || a.zill[z0] < a.min_ill)) return false;
     if (a.parts > 0) {
         const int s = seg_count(a.above > 0 ? seg_count(z1 - z0, a.above) : z1 - z0, a.parts);
         z0 = (long long)ray * a.parts;
@@ -124,8 +127,8 @@ __device__ __forceinline__ long long ray_mid(const BtdArgs &a, long long z0, lon
 
 // offsets[0] = 0, offsets[n_rays] = n_zones and non-decreasing; any violation marks the whole call
 // invalid (so no two rays can share zones) and raises the numeric flag.
-__global__ void k_btd_validate(const int *off, int n_rays, long long n_zones, int *inval, int *flag, int *zbad, int *ends,
-                               int *pbad) {
+__global__ void k_btd_validate(const int *off, int n_rays, long long n_zones, int *inval, int *flag, int *zbad, int *zill,
+                               int *ends, int *pbad) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i > n_rays) return;
     if (pbad && i < n_rays) pbad[i] = 0;
@@ -137,7 +140,8 @@ __global__ void k_btd_validate(const int *off, int n_rays, long long n_zones, in
         atomicOr(inval, 1);
         atomicOr(flag, 1);
     } else if (v < e && e <= n_zones) {
-        zbad[v] = 0;                                 // the factor kernel's arrival count
+        zbad[v] = 0;  // the factor kernel's arrival count
+        zill[v] = 0;
         ends[v] = v == e - 1 ? kFirst | kLast : kFirst;  // (zero before)
         if (v < e - 1) ends[e - 1] = kLast;
     }
@@ -352,6 +356,15 @@ __device__ __forceinline__ float btd_rcp(float p) {  // p and 1/p normal numbers
     return fmaf(y, fmaf(-p, y, 1.f), y);  // a Newton step: the approximation's ulp would stay in the pivot row
 }
 
+// D^{-1} applied to a vector, unlike the elimination done over on it, carries the inverse's own error: where the product
+// is much smaller than its terms, as with ill-conditioned blocks, the solution is further off (random blocks without a
+// dominant diagonal, coupled by 0.3 of their size: 2 to 4 times in the median, 30 times in one ray of ten). A ray
+// whose largest pivot in some zone exceeds the smallest kPivots1 or kPivots2 times is therefore refined once or twice
+// more than asked, and not cut into segments. (The pivots are at hand; max|D| max|D^{-1}| says the same, and looking
+// for it cost 2 to 4 %.) Blocks with dominant diagonals have a ratio of 1 to 2, Newton systems 10 to 13, those
+// random blocks 15 to 1e4.
+constexpr float kPivots1 = 24.f, kPivots2 = 256.f;
+
 // The panel warp's state: lane x holds rows x + 32 t of the panel's eight columns.
 template <int NT>
 struct Panel {
@@ -514,8 +527,12 @@ struct Panel {
             for (int c = 0; c < 8; ++c) v[t][c] *= sc[t];
         __syncwarp();
     }
-    // A column had no pivot (all candidates zero) or one that is not finite.
-    __device__ __forceinline__ bool failed() const { return kmin < 128u || kmax >= 0x7f800000u; }
+    // -1: a column had no pivot (all candidates zero) or one that is not finite; else how ill-conditioned the block is.
+    __device__ __forceinline__ int level() const {
+        if (kmin < 128u || kmax >= 0x7f800000u) return -1;
+        const float lo = __uint_as_float(kmin & 0x7fffff80u), hi = __uint_as_float(kmax & 0x7fffff80u);
+        return (hi > kPivots1 * lo) + (hi > kPivots2 * lo);
+    }
 };
 
 // Applies panel p's transform to one or two other 8-column tiles of X (t1 < 0: one), on the tensor cores:
@@ -669,9 +686,9 @@ __device__ __forceinline__ void subtract_product(float *X, const float *U, const
 
 // Inverts X in place up to the order of its rows and columns: eliminates panel after panel, one CTA barrier each;
 // in step it, warp 0 eliminates within panel it, the others apply panel it - 1. Pivot j's row is cur[j], pos its
-// inverse: X^{-1}[j][cur[q]] = X[cur[j]][q]. True in warp 0 if a pivot failed. No barrier at its end.
+// inverse: X^{-1}[j][cur[q]] = X[cur[j]][q]. Returns Panel::level in warp 0, else 0. No barrier at its end.
 template <int NT>
-__device__ __forceinline__ bool invert(float *X, int ld, int m, int *cur, int *pos, float *rowbuf, int tid) {
+__device__ __forceinline__ int invert(float *X, int ld, int m, int *cur, int *pos, float *rowbuf, int tid) {
     const int lane = tid & 31, warp = tid >> 5, nw = kFactorThreads / 32, P = (m + 7) >> 3;
     Panel<NT> pn;
     if (warp == 0) pn.start(m, lane);
@@ -697,7 +714,7 @@ __device__ __forceinline__ bool invert(float *X, int ld, int m, int *cur, int *p
         }
         if (it < P) __syncthreads();
     }
-    return warp == 0 && pn.failed();
+    return warp == 0 ? pn.level() : 0;
 }
 
 // The inverse of X (as invert leaves it), row by row, to Di.
@@ -806,7 +823,7 @@ constexpr float kMaxGrowth = 4.f;
 template <int NT>
 __global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(const BtdArgs a) {
     extern __shared__ __align__(16) float sm[];
-    __shared__ int s_bad, s_grow, s_all;
+    __shared__ int s_bad, s_grow, s_all, s_ill;
     const int m = a.m, ld = a.ld, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int bs = factor_buf(m, ld), P = (m + 7) >> 3;
     const bool four = a.nbuf == 4;
@@ -823,7 +840,8 @@ __global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(c
     if (!ray_range(a, blockIdx.x / a.halves, z0, z1) || z1 == z0) return;
     long long mid = ray_mid(a, z0, z1);
     if (half == 1 && mid == z1 - 1) return;
-    if (tid == 0) s_bad = s_grow = 0;
+    if (tid == 0) s_bad = s_grow = s_ill = 0;
+    int *const ill = a.zill + a.off[blockIdx.x / a.halves];
     if (tid < m) pos[tid] = tid;  // in range also where a failed pivot leaves an entry unset
     const int mw = m * ld;
     const int wm = warp & 1, wn = warp >> 1;
@@ -859,6 +877,8 @@ __global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(c
             if (!joined) {
                 // the second half to arrive goes on: + 1 each, + 16 for a failed outward half, + 256 inward
                 if (tid == 0) {
+                    if (a.parts > 0) s_bad |= s_ill;
+                    else if (s_ill) atomicMax(ill, s_ill);
                     const int add = 1 + (half ? ((s_bad | s_grow) ? 256 : 0) : (s_bad ? 16 : 0));
                     __threadfence();
                     s_all = atomicAdd(a.zbad + z0, add) + add;
@@ -929,7 +949,11 @@ __global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(c
                 if (four) load(sB, at(a.Di, k + dir));
             }
         }
-        if (invert<NT>(X, ld, m, cur, pos, rowbuf, tid) && lane == 0) s_bad = 1;
+        const int level = invert<NT>(X, ld, m, cur, pos, rowbuf, tid);
+        if (tid == 0) {
+            if (level < 0) s_bad = 1;
+            else s_ill = max(s_ill, level);
+        }
         copy_wait();
         __syncthreads();
         store_inverse<NT>(at(a.Di, k), X, ld, m, cur, pos, tid);
@@ -958,6 +982,8 @@ __global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(c
     }
     __syncthreads();
     if (tid == 0) {
+        if (a.parts > 0) s_bad |= s_ill;
+        else if (s_ill) atomicMax(ill, s_ill);
         a.zbad[z0] = s_bad;
         a.zmid[z0] = (int)(mid - z0);
         if (s_bad) {
@@ -974,8 +1000,9 @@ __global__ void __launch_bounds__(kFactorThreads, NT > 3 ? 1 : 2) k_btd_factor(c
 // and then once more inwards for the segment's first zone, x_a = y' - R x_e - L' x_p (R_k = -G_k R_{k+1},
 // L'_k = L_k - G_k L'_{k+1}). That leaves a block-tridiagonal system of the segments' last zones,
 //   Ar_e = -A_e L_{e-1},  Br_e = B_e - A_e G_{e-1} - C_e L'_{next a},  Cr_e = -C_e R_{next a},
-// for k_btd_factor, or of enough rows to be cut into segments once more. A ray in which a pivot fails, or an entry of G, L, R or L' is above kMaxGrowth, is
-// done again as a whole by k_btd_factor (pbad). The time is that of n / S + S / 2 zones, not n / 2.
+// for k_btd_factor, or of enough rows to be cut into segments once more. A ray in which a pivot fails, a block is
+// ill-conditioned (kPivots1), or an entry of G, L, R or L' is above kMaxGrowth, is done again as a whole by k_btd_factor
+// (pbad). The time is that of n / S + S / 2 zones, not n / 2.
 // GB300, m = 84, 400 zones, one ray: 5.11 ms by two CTAs -> 0.27 ms for 69 segments, 0.29 for 14 of
 // their last zones and 0.29 for those segments' last zones (0.58 and 0.66 with 34 segments and one level).
 struct SegArgs {
@@ -1088,7 +1115,7 @@ __global__ void __launch_bounds__(kFactorThreads, 1) k_btd_segment(const SegArgs
         load(sA, at(a.At, k + 1));
         load_nz(1, k + 1, 1);
         if (five) load(sB, at(a.Di, k + 1));
-        if (invert<NT>(X, ld, m, cur, pos, rowbuf, tid) && lane == 0) s_bad = 1;
+        if (invert<NT>(X, ld, m, cur, pos, rowbuf, tid) && lane == 0) s_bad = 1;  // (failed, or ill-conditioned)
         copy_wait();
         __syncthreads();
         store_inverse<NT>(at(a.Di, k), X, ld, m, cur, pos, tid);
@@ -1744,7 +1771,7 @@ struct vx_btd {
     size_t blocks = 0;
     unsigned short *nz = nullptr;
     int slots = 0;  // factor CTAs the device holds at once
-    int *zbad = nullptr, *zmid = nullptr, *flag = nullptr;  // flag[0]: numeric flag, flag[1]: offsets invalid
+    int *zbad = nullptr, *zmid = nullptr, *zill = nullptr, *flag = nullptr;  // flag[0]: numeric flag, flag[1]: offsets invalid
     double *r = nullptr;
     // segments: most zones of a call that is cut into them (0: none), and their system's arrays (a row per SM)
     int sms = 1, seg_nbuf = 0;
@@ -1763,6 +1790,7 @@ static void btd_free(vx_btd *h) {
     cudaFree(h->y);
     cudaFree(h->zbad);
     cudaFree(h->zmid);
+    cudaFree(h->zill);
     cudaFree(h->Sr);
     cudaFree(h->nzr);
     cudaFree(h->zr);
@@ -1840,6 +1868,7 @@ extern "C" vx_status vx_btd_create_rays(int m, long long max_zones, int n_refine
     if (e == cudaSuccess) e = cudaMalloc(&h->y, zc * m * sizeof(float));
     if (e == cudaSuccess) e = cudaMalloc(&h->zbad, zc * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&h->zmid, zc * sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&h->zill, zc * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&h->r, zc * m * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&h->flag, 2 * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(h->flag, 0, 2 * sizeof(int));
@@ -1910,6 +1939,8 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
     a.y = h->y;
     a.zbad = h->zbad;
     a.zmid = h->zmid;
+    a.zill = h->zill;
+    a.min_ill = 0;
     // Two CTAs per ray while they all find room at once, and with rays of 16 zones or more where the last wave of
     // one CTA per ray would be less than 5/8 full. GB300, one -> two, 100 zones: m = 84, 20 rays 3.60 -> 1.98 ms,
     // 152 4.76 -> 3.73, 160 5.91 -> 5.32, 330 10.58 -> 9.02, 480 13.25 -> 12.54, but 240 6.67 -> 6.70 and
@@ -1987,7 +2018,7 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
     BTD_CU(cudaMemsetAsync(h->flag + 1, 0, sizeof(int), s));
     BTD_CU(cudaMemsetAsync(h->zmid, 0, (size_t)n_zones * sizeof(int), s));
     k_btd_validate<<<(unsigned)((n_rays + 256) / 256), 256, 0, s>>>(ray_offsets, n_rays, n_zones, h->flag + 1, h->flag, h->zbad,
-                                                                   h->zmid, f.pbad);
+                                                                   h->zill, h->zmid, f.pbad);
     BTD_CU(cudaGetLastError());
     launch_convert(h->m, n_zones, h->sms, s, a);
     BTD_CU(cudaGetLastError());
@@ -2028,6 +2059,13 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
         }
         BTD_CU((it == 0 ? (last ? launch_sweep<true, true> : launch_sweep<true, false>)
                         : (last ? launch_sweep<false, true> : launch_sweep<false, false>))(h->m, ctas, h->smem_sweep, s, f));
+    }
+    f.rhs = h->r;
+    for (int level = 1; level <= 2; ++level) {  // rays with ill-conditioned blocks (never those in segments)
+        a.min_ill = f.min_ill = level;
+        k_btd_resid<<<dim3(n_rays, (unsigned)split), kResidThreads, 0, s>>>(a);
+        BTD_CU(cudaGetLastError());
+        BTD_CU((launch_sweep<false, false>(h->m, ctas, h->smem_sweep, s, f)));
     }
     return VX_OK;
 }

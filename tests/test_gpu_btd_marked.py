@@ -139,7 +139,7 @@ def test_workspace(m, zones, min_rays):
     bounds; an array is rounded up to 2 MiB)."""
     from paper_1404_1719_gb300 import BlockTridiagSolver
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    bound = (12 * m * (m + 7) + 4 * (m + 7) + 12 * m + 8) * zones
+    bound = (12 * m * (m + 7) + 4 * (m + 7) + 12 * m + 12) * zones
     if m <= 116 and min_rays <= sms // 5:
         bound += 4 * m * (m + 7) * max(0, 4 * min(zones, 16384) - 3 * zones) + (36 * m * m + 300 * m + 76) * sms
     BlockTridiagSolver(m, 1).close()  # the kernels are loaded
@@ -166,3 +166,48 @@ def test_calls_of_any_size(m, max_zones, min_rays):
             ref = obtd.solve(s["A"][a:b], s["B"][a:b], s["C"][a:b], s["d"][a:b], np.array([0, b - a]))
             assert np.abs(x[a:b] - ref).max() <= TOL * np.abs(ref).max()
     sv.close()
+
+
+def _fp32_elimination(A, B, C, d, n_refine):
+    """Block elimination with an LU factorisation of every block, all in FP32, and refinement from the FP64 residual."""
+    from scipy.linalg import lu_factor, lu_solve
+    f = np.float32
+    a, b, c = A.astype(f), B.astype(f), C.astype(f)
+    n, lu, G = len(B), [], []
+    for k in range(n):
+        lu.append(lu_factor(b[k] - a[k] @ G[-1] if k else b[k]))
+        G.append(lu_solve(lu[k], c[k]))
+    offsets, x = np.array([0, n]), np.zeros_like(d)
+    for _ in range(n_refine + 1):
+        r = (d - obtd.apply(A, B, C, x, offsets)).astype(f)
+        y = []
+        for k in range(n):
+            y.append(lu_solve(lu[k], r[k] - a[k] @ y[-1] if k else r[k]))
+        for k in range(n - 2, -1, -1):
+            y[k] = y[k] - G[k] @ y[k + 1]
+        x = x + np.array(y, np.float64)
+    return x
+
+
+@pytest.mark.parametrize("rays", [64, 320])
+@pytest.mark.parametrize("m, scale", [(8, 0.3), (8, 1.0), (20, 0.3), (20, 1.0)])
+def test_blocks_without_a_dominant_diagonal(m, scale, rays):
+    """Random blocks, coupled by 0.3 or all of their size: no further from the solution than block elimination in FP32
+    with LU factorisations, in nine rays of ten at least (either error is a random number; with the inverse's own
+    error in the solution the median ray was twice as far off, the tenth worst thirty times)."""
+    n, sample = 30, 64
+    g = np.random.default_rng(m + rays)
+    A, B, C = (g.standard_normal((rays * n, m, m)) for _ in range(3))
+    A, C = A * scale, C * scale
+    A[::n], C[n - 1::n] = 0.0, 0.0
+    s = dict(A=A, B=B, C=C, d=g.standard_normal((rays * n, m)), offsets=np.arange(rays + 1, dtype=np.int32) * n)
+    for n_refine in (0, 1):
+        x, ok = _solve(s, m, n_refine)
+        assert ok
+        ratio = []
+        for r in range(sample):
+            z = slice(r * n, r * n + n)
+            ref = obtd.solve(A[z], B[z], C[z], s["d"][z], np.array([0, n]))
+            e = [np.linalg.norm(q - ref) for q in (x[z], _fp32_elimination(A[z], B[z], C[z], s["d"][z], n_refine))]
+            ratio.append(e[0] / e[1])
+        assert np.quantile(ratio, 0.9) <= 1.0, (n_refine, np.quantile(ratio, [0.5, 0.9, 1.0]))
