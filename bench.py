@@ -85,10 +85,10 @@ def formulation_flops_per_node(adj: bool) -> int:
 
 # Pipe utilisation of the benchmark's kernels from one ncu capture each (see profiles/; set to
 # None whenever the kernel changes, until it has been captured again): the MUFU (XU) issue
-# fraction of the forward + tangent kernel and the FP64-pipe fraction of the plain FP64 kernel.
+# fraction of the forward + tangent kernel and the FP64-pipe fraction of the FP64 kernel.
 MUFU_FRAC_TANGENT = 0.2596   # profiles/k_pair_mixed_tangents_200rays_pipes.md
 FP64_FRAC_FP64FWD = 0.9241   # profiles/k_pair_mixed_tangents_and_k_pair_fp64_pipes_20rays.md
-# fraction of the workload's zones the plain FP64 comparison leg evaluates, and its timed launches
+# fraction of the workload's zones the FP64 comparison leg evaluates, and its timed launches
 FP64_SAMPLE_FRAC, FP64_REPEATS = 0.05, 3
 # timed launches of the precise-mode leg (after two untimed ones)
 PRECISE_REPEATS = 3
@@ -907,7 +907,7 @@ def run_ours(args):
                         "achieved_gbs": (h2d + d2h) / (ms_local / 1000) / 1e9,
                         "note": "inputs read + rates, blocks and J/H gradients written, per step"}} if spec else {}),
             "fp64_fwd": {"value": v64, "unit": UNIT, "ms_per_launch": ms64, "launches_timed": FP64_REPEATS,
-                         "sample": f"first {sub} zones ({100 * sub / Z:.1f} % of the workload), plain FP64 forward only",
+                         "sample": f"first {sub} zones ({100 * sub / Z:.1f} % of the workload), FP64 forward only",
                          "ratio_mixed_fwd_adj_over_fp64_fwd": value / world / v64,
                          "roofline": {"bound": "alu", "achieved": ach64, "peak": peak64, "unit": "TFLOP/s",
                                       "frac": ach64 / peak64,

@@ -3,7 +3,7 @@
  *
  * The pair-process quadrature does about 1e4 arithmetic operations per byte of HBM traffic, so
  * its roofline is set by the arithmetic pipes, not by memory: the FP32 FMA pipe (the mixed
- * form), the FP64 FMA pipe (the plain FP64 form) and the multi-function unit that executes the
+ * form), the FP64 FMA pipe (the FP64 form) and the multi-function unit that executes the
  * ex2 and rcp of the Fermi-Dirac blocking factors. The paper characterises its code the same way,
  * with a roofline built from measured peaks (sec. 3.2); this call measures those peaks on the
  * current device, so that a throughput can be stated as a fraction of a measured rate.

@@ -58,7 +58,7 @@ typedef enum {
 } vx_status;
 
 typedef enum {
-    VX_PREC_FP64 = 0,  /* plain FP64 quadrature (forward only): the comparison baseline        */
+    VX_PREC_FP64 = 0,  /* FP64 quadrature (forward only): the comparison baseline              */
     VX_PREC_MIXED = 1  /* FP32 quadrature; extra precision on the degeneracy-sensitive steps   */
 } vx_precision;
 
@@ -84,7 +84,7 @@ typedef enum { VX_NU_E = 0, VX_NU_EBAR = 1, VX_NU_X = 2 } vx_species;
                             contraction are carried in double-float (FP32 pairs). It bounds the
                             error of the l = 1 results and of the eta-tangents, whose sums
                             cancel, at about 1e-7 of their sums of absolute values (see the
-                            tests for the measured bounds); it costs ~15-25 % more time. Mixed
+                            tests for the measured bounds); it costs ~30-40 % more time. Mixed
                             precision only (VX_ERR_UNSUPPORTED with VX_PREC_FP64)              */
 
 typedef struct {
