@@ -1624,14 +1624,14 @@ __global__ void __launch_bounds__(kSweepThreads, 1) k_btd_seg_sweep(const SegArg
 }
 
 // The FP64 residual, a ray's zones split over blockIdx.y CTAs, a warp per eight rows of a zone. Every matrix
-// element costs one FP64 FMA, at 1.68 per clock and SM on GB300 (measured; less than HBM can feed), so the layout
+// element costs one FP64 FMA, at two per clock and SM of GB300 at most (less than HBM can feed), so the layout
 // minimises FP64 instructions beyond those FMAs and leaves out what is known to be zero: groups of eight
 // columns that are zero in a row of A_k or C_k (nz) are neither read nor multiplied. Lane 4 r + c
 // takes row i0 + r and the columns c, c + 4, ... (four lanes read 32 contiguous bytes of a row, eight rows
 // per load instruction; in A and C each row goes through its own groups), accumulates with FMAs only, and two
 // shuffle-add steps finish the row.
 // GB300, m = 84, 304 rays x 400 zones: one coupling per row 5.3 -> 2.2 ms, dense couplings 5.3 -> 5.1 ms (FP64
-// pipe: 4.9 at that rate); one ray 0.88 -> 0.02 ms (was four CTAs).
+// pipe: 4.1 at that rate); one ray 0.88 -> 0.02 ms (was four CTAs).
 constexpr int kResidB = 7;  // quads of B in flight
 constexpr int kResidG = 3;  // column groups of A or C (two loads a lane each) in flight
 __device__ __forceinline__ double resid_groups(const double *M, const double *x, unsigned todo, int cc, int m) {

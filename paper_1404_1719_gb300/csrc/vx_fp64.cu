@@ -4,8 +4,8 @@
 // element into three non-negative moments, at FP64 accuracy throughout. Production is e^{-eps_i/T} e^{-eps_j/T}
 // times annihilation, as FP64 products that underflow where the definition itself underflows.
 //
-// Bound by the FP64 pipe, two lanes wide on an SM of GB300 (1.68 FMAs per clock measured) against 128 FP32 or 64
-// integer ones, so the node loop is written for the fewest FP64 operations and leaves the rest to the
+// Bound by the FP64 pipe, two lanes wide on an SM of GB300 (a probe of FMAs gets 1.68 per clock, this kernel 1.85) against
+// 128 FP32 or 64 integer ones, so the node loop is written for the fewest FP64 operations and leaves the rest to the
 // other pipes. With d = h/T (h = |q|/2) a mirror pair of nodes tau, -tau has
 //   e1(+-tau) = c1 2^-+t,  e2(+-tau) = c2 2^+-t,  t = d tau log2 e,
 //   c1 = e^{eta - q0/2T},  c2 = e^{-eta - q0/2T},  (1 + e1)(1 + e2) = 1 + e^{-q0/T} + e1 + e2,
@@ -14,12 +14,12 @@
 // from a table of 2^{j/4096} and a polynomial in the remainder r/4096, |r| <= 1/2: its linear term in FP64, the
 // quadratic one (up to 3.6e-9) from a 32-bit integer square in units of 2^-59, the rest (up to 2e-13, so that
 // FP32's rounding of it is below 1e-20) in FP32, added in the same units. 2^t is within 2.2e-16 (the table's rounding and
-// the last one), rms 6.7e-17; with the quadratic term in FP32 it was 6.5e-16, rms 1.1e-16. About 24 FP64 operations
+// the last one), rms 6.7e-17; with the quadratic term in FP32 it was 6.5e-16, rms 1.1e-16. 23 FP64 operations
 // per mirror pair against 84 with two library exponentials and a division per node. The arguments' rounding errors
 // (of 1/T, and of d) are carried along as small corrections, so e1 and e2 are good to a few units in the last
 // place at any |t|, where a rounded argument loses |t| of them. Zones so cold that 2^+-t would leave
 // the FP64 range (q0/2T + |eta| above 690) take the plain node loop.
-// GB300, 2 rays x 400 zones, 21 bins, 32 x 64: 37.7 -> 8.5 ms. Against the same rule in 80 bits, over seven grids and
+// GB300, 2 rays x 400 zones, 21 bins, 32 x 64: 37.7 -> 8.1 ms. Against the same rule in 80 bits, over seven grids and
 // quadratures, T from 1 to 30 MeV and eta_e from -5 to 60, the mean zone's kernel and rates (2-norm) are
 // 1.4e-16 to 1.2e-15 off, 0.54 to 1.14 of what library exponentials and divisions gave (mostly below 1).
 #include "vx_internal.h"
@@ -47,6 +47,12 @@ __device__ __forceinline__ float to_f32(double x) {
     const unsigned hi = (unsigned)(b >> 32), e = hi & 0x7fffffffu;
     const float f = __uint_as_float((__funnelshift_l((unsigned)b, e - (896u << 20), 3) & 0x7fffffffu) | (hi & 0x80000000u));
     return e < (897u << 20) ? 0.f : f;
+}
+// |x| 2^32 for |x| <= 1/2, cut, by integer operations as well.
+__device__ __forceinline__ unsigned fixed32(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x) & 0x7fffffffu;
+    const unsigned w = __funnelshift_r((unsigned)__double2loint(x), (hi & 0xfffffu) | 0x100000u, 21);  // |x| = w 2^{e - 1054}
+    return __funnelshift_rc(w, 0u, 1022u - (hi >> 20));
 }
 // Moments of the blocking factor of one (pair, omega) unit over the electron-energy nodes.
 struct Mom64 {
@@ -80,9 +86,9 @@ __device__ __forceinline__ void nodes_fast(const double *__restrict__ nodes, con
         const double tau = nodes[4 * k], wp = nodes[4 * k + 1], wm = nodes[4 * k + 2], wz = nodes[4 * k + 3];
         const double u = fma(Bs, tau, magic), un = u - magic, r = fma(Bs, tau, -un);  // t 4096 = un + r, |r| <= 1/2
         const int q = __double2loint(u) - kShift, qm = -q - 2 * kShift;
-        const int ri = __double2loint(r + magic * 0x1p-32);  // r 2^32
         const float rf = to_f32(r), tf = to_f32(tau);
-        const long long ev = bBits + __umulhi(2u * (unsigned)__mulhi(ri, ri), L2u);
+        const unsigned ri = fixed32(r);
+        const long long ev = bBits + __umulhi(2u * __umulhi(ri, ri), L2u);
         const int od = __float2int_rn(fmaf(L3f * rf * rf, rf, L1f * Bl * tf));  // the cubic term, and d's remainder
         const double yp = fma(Lb, r, __longlong_as_double(ev + od)), ym = fma(-Lb, r, __longlong_as_double(ev - od));
         double tp = tab[q & (kExpTab - 1)], tm = tab[qm & (kExpTab - 1)];

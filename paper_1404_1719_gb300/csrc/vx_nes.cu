@@ -696,7 +696,7 @@ cudaError_t nes_launch(const NesLaunch<R> &L, int grid, size_t smem, cudaStream_
 // increasing and convex for eta >= 0, so Newton converges monotonically from there; either term alone gives
 // an upper bound, and the lower of the two, min(cbrt(q), q / pi^2), is within a factor 1.5 of the root),
 // then the derivatives by implicit differentiation.
-// Bound by the FP64 pipe (1.68 FMAs per clock and SM, measured). Iterating in FP64 until the step vanished took
+// Bound by the FP64 pipe (two lanes an SM). Iterating in FP64 until the step vanished took
 // about 100 iterations where the last bits alternate; now FP32 iterations come within 1e-7 of the root and two
 // or three FP64 ones, their quotient by the FP32 reciprocal, within its rounding. GB300, 204,800 zones:
 // 697 -> 50 us.
