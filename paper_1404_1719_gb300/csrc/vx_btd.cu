@@ -273,13 +273,19 @@ __device__ __forceinline__ void st1_if(bool p, unsigned a, unsigned x) {
 // (float)x in integer operations: the conversion instruction runs on the FP64 pipe, at 2 per clock and SM on GB300
 // (measured); this form is about ten integer operations. Nearly half an ulp is added (ties to even) and the
 // exponent rebiased by 896. For zeros and for magnitudes from 2^-126 to below 2^127, which is what
-// btd_plain says; the rest (FP32 subnormals, the last binade, infinities and NaN) goes by the instruction.
-__device__ __forceinline__ bool btd_plain(double x) {
-    const unsigned e = (unsigned)__double2hiint(x) & 0x7fffffffu;
+// btd_plain says; the rest (FP32 subnormals, the last binade, infinities and NaN) goes by the instruction. The
+// bits come by a move, so that the compiler does not turn the tests on them into FP64 comparisons.
+__device__ __forceinline__ unsigned long long btd_bits(double x) {
+    unsigned long long u;
+    asm("mov.b64 %0, %1;" : "=l"(u) : "d"(x));
+    return u;
+}
+__device__ __forceinline__ bool btd_plain(unsigned long long u) {
+    const unsigned e = (unsigned)(u >> 32) & 0x7fffffffu;
     return e - (897u << 20) < 253u << 20 || e == 0u;
 }
-__device__ __forceinline__ float btd_plain_f32(double x) {
-    const unsigned long long u = (unsigned long long)__double_as_longlong(x), b = u + 0x0fffffffull + ((u >> 29) & 1ull);
+__device__ __forceinline__ float btd_plain_f32(unsigned long long u) {
+    const unsigned long long b = u + 0x0fffffffull + ((u >> 29) & 1ull);
     const unsigned hi = (unsigned)(b >> 32), e = hi & 0x7fffffffu;
     return __uint_as_float((e < 1u << 20 ? 0u : __funnelshift_l((unsigned)b, e - (896u << 20), 3)) | (hi & 0x80000000u));
 }
@@ -322,10 +328,10 @@ __global__ void __launch_bounds__(kConvThreads) k_btd_convert(const BtdArgs a) {
                 bool plain = true;
 #pragma unroll
                 for (int t = 0; t < NT; ++t) {
-                    plain = plain && btd_plain(v[r][t]);
-                    if (t < NT - 1 || lane + 32 * t < m) dst[i * ld + 32 * t] = btd_plain_f32(v[r][t]);
-                    const unsigned long long mag = (unsigned long long)__double_as_longlong(v[r][t]) << 1;
-                    bits |= mag != 0ull ? 1u << (4 * t) : 0u;
+                    const unsigned long long u = btd_bits(v[r][t]);
+                    plain = plain && btd_plain(u);
+                    if (t < NT - 1 || lane + 32 * t < m) dst[i * ld + 32 * t] = btd_plain_f32(u);
+                    bits |= u << 1 != 0ull ? 1u << (4 * t) : 0u;
                 }
                 if (!plain) {
 #pragma unroll 1
