@@ -87,7 +87,9 @@ def formulation_flops_per_node(adj: bool) -> int:
 # None whenever the kernel changes, until it has been captured again): the MUFU (XU) issue
 # fraction of the forward + tangent kernel and the FP64-pipe fraction of the FP64 kernel.
 MUFU_FRAC_TANGENT = 0.2596   # profiles/k_pair_mixed_tangents_200rays_pipes.md
-FP64_FRAC_FP64FWD = 0.9241   # profiles/k_pair_mixed_tangents_and_k_pair_fp64_pipes_20rays.md
+FP64_FRAC_FP64FWD = 0.9246   # profiles/k_pair_mixed_tangents_and_k_pair_fp64_pipes_20rays.md
+# FMAs per clock and SM of the FP64 pipe (1.25 TFLOP/s nominal)
+FP64_LANES = 2
 # fraction of the workload's zones the FP64 comparison leg evaluates, and its timed launches
 FP64_SAMPLE_FRAC, FP64_REPEATS = 0.05, 3
 # timed launches of the precise-mode leg (after two untimed ones)
@@ -822,7 +824,7 @@ def run_ours(args):
         ms64 = f0.elapsed_time(f1) / FP64_REPEATS
         v64 = entries(sub, N) / (ms64 / 1000)
         nodes64 = sub * npair * b["n_mu"] * b["n_e"]
-        peak64 = pipes["dfma"] * 2 * nsm * mhz * 1e6 / 1e12
+        peak64 = FP64_LANES * 2 * nsm * mhz * 1e6 / 1e12
         ach64 = nodes64 * algorithmic_flops_per_node(False) / (ms64 / 1000) / 1e12
         r64.close()
         # the same step in the precise mode (VX_PRECISE), a few timed launches: its cost
@@ -911,8 +913,8 @@ def run_ours(args):
                          "ratio_mixed_fwd_adj_over_fp64_fwd": value / world / v64,
                          "roofline": {"bound": "alu", "achieved": ach64, "peak": peak64, "unit": "TFLOP/s",
                                       "frac": ach64 / peak64,
-                                      "peak_note": f"FP64 {nsm} SMs x {pipes['dfma']:.2f} DFMA/clk (probe) x 2 x "
-                                                   f"{mhz:.0f} MHz",
+                                      "peak_note": f"FP64 {nsm} SMs x {FP64_LANES} FMA/clk x 2 x {mhz:.0f} MHz; probe: "
+                                                   f"{pipes['dfma']:.2f} DFMA/clk/SM",
                                       "fp64_frac": FP64_FRAC_FP64FWD,
                                       "fp64_note": "ncu sm__pipe_fp64_cycles_active.avg.pct_of_peak_sustained_active "
                                                    "of k_pair_fp64 (profiles/)"}},

@@ -22,7 +22,7 @@
 // and once for the rays that have to be done as a whole (3 us each when there are none).
 // With the inverse instead of the elimination's multipliers (which the sweeps replayed, a shuffle per
 // unknown), GB300, m = 84, 400 zones a ray: one ray (one CTA) factor 24.3 -> 10.0 ms, a sweep 3.0 -> 1.3 ms; 304 rays
-// 29.7 -> 14.0 ms (which included the conversion, now 6.1 ms apart) and 3.1 -> 1.7 ms (10.3 GB, 6.1 TB/s).
+// 29.7 -> 14.0 ms (which included the conversion, now 5.9 ms apart) and 3.1 -> 1.7 ms (10.3 GB, 6.1 TB/s).
 // The solution's error without refinement and with one sweep is 0.2 to 0.8 of what it was (m = 34 to 128).
 #include "../../include/vx_btd.h"
 
