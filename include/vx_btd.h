@@ -27,9 +27,10 @@
  * n_refine sweeps of iterative refinement follow, each from the FP64 residual d - M x of the
  * caller's FP64 blocks; one or two more in a ray with an ill-conditioned block (its largest pivot more than 24 or 256
  * times the smallest), which is not cut into segments either: inverses would leave it further off than elimination
- * does. For a ray whose Schur complements are well conditioned (e.g. block rows
- * diagonally dominant) every sweep gains a factor of about cond x 1e-7, so two sweeps reach FP64
- * accuracy at moderate condition numbers. The reduction order is fixed: the results of a batch are
+ * does. If these leave a residual of more than 0.03^(n_refine + 2) of rhs (at least 1e-10), the ray is eliminated in
+ * FP64 instead, slowly: about 0.85 ms a zone at m = 84. For a ray whose Schur complements are well conditioned (e.g.
+ * block rows diagonally dominant) every sweep gains a factor of about cond x 1e-7, so two sweeps reach FP64 accuracy at
+ * moderate condition numbers. The reduction order is fixed: the results of a batch are
  * reproducible run to run.
  *
  * Conventions (as in vx_rates.h): arrays are dense, row-major FP64 unless stated; device pointers
@@ -54,8 +55,9 @@ typedef struct vx_btd vx_btd;
 
 /* Creates a solver for m unknowns per zone (1 .. VX_BTD_MAX_M) and batches of at most max_zones
  * zones (>= 0), with n_refine FP64 refinement sweeps (0 .. VX_BTD_MAX_REFINE; 0 leaves the FP32
- * solution, but in rays with ill-conditioned blocks). Allocates the device workspace: 12 m (m + 7) + 4 (m + 7) + 12 m + 12 bytes per zone at most, and, for
- * max_zones of 40 or more and m up to 116, what rays in segments take besides: 4 m (m + 7) for each zone that
+ * solution, but in rays with ill-conditioned blocks). Allocates the device workspace: 12 m (m + 7) + 4 (m + 7) + 12 m + 20
+ * bytes per zone at most, and, for max_zones of 40 or more and m up to 116, what rays in segments take besides:
+ * 4 m (m + 7) for each zone that
  * 4 min(max_zones, 16384) exceeds 3 max_zones by (none from 21,846 zones on), and 36 m^2 + 300 m + 76 per SM. Without
  * the memory for that, rays are not cut into segments. *out is set to NULL on failure. Errors: VX_ERR_INVALID_ARG,
  * VX_ERR_OOM, VX_ERR_CUDA. */

@@ -17,9 +17,11 @@
 //  * k_btd_resid: the FP64 residual r = d - M x from the caller's FP64 blocks, eight rows per warp, four
 //    lanes per row (coalesced), zero groups of the couplings left out, FMA accumulation and a fixed two-step
 //    shuffle reduction per row.
+//  * k_btd_fp64: rays with a block whose inverse in FP32 says too little, in FP64.
 // The host runs validate, convert, [segment, join, once or twice], factor, sweep, then n_refine times (resid,
-// sweep) and once or twice more for the rays with ill-conditioned blocks, all on the caller's stream; with segments the factor kernel and the sweeps run once for the segments' system
-// and once for the rays that have to be done as a whole (3 us each when there are none).
+// sweep), once or twice more for the rays with ill-conditioned blocks, and fp64, all on the caller's stream; with
+// segments the factor kernel and the sweeps run once for the segments' system and once for the rays that have to be
+// done as a whole (3 us each when there are none).
 // With the inverse instead of the elimination's multipliers (which the sweeps replayed, a shuffle per
 // unknown), GB300, m = 84, 400 zones a ray: one ray (one CTA) factor 24.3 -> 10.0 ms, a sweep 3.0 -> 1.3 ms; 304 rays
 // 29.7 -> 14.0 ms (which included the conversion, now 5.9 ms apart) and 3.1 -> 1.7 ms (10.3 GB, 6.1 TB/s).
@@ -89,6 +91,10 @@ struct BtdArgs {
     int *zbad, *zmid, *flag;
     int *zill;    // at a ray's first zone: how ill-conditioned its blocks are (pivot_level, the highest)
     int min_ill;  // only the rays of that level or more
+    // Of such rays, at 2 (the first zone): max|residual| after their last sweep and max|d|, as bits; norm: k_btd_resid
+    // raises them
+    unsigned *znorm;
+    bool norm;
     const int *inval;  // set by k_btd_validate when the offsets are not a partition of the zones
     // Rays in segments (k_btd_segment): parts > 0: this is the system of the segments' last zones, ray r's from r parts
     // on (above > 0: of segments of such a system, of `above` parts a ray); parts = 0 and pbad: only the rays
@@ -128,7 +134,7 @@ __device__ __forceinline__ long long ray_mid(const BtdArgs &a, long long z0, lon
 // offsets[0] = 0, offsets[n_rays] = n_zones and non-decreasing; any violation marks the whole call
 // invalid (so no two rays can share zones) and raises the numeric flag.
 __global__ void k_btd_validate(const int *off, int n_rays, long long n_zones, int *inval, int *flag, int *zbad, int *zill,
-                               int *ends, int *pbad) {
+                               unsigned *znorm, int *ends, int *pbad) {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i > n_rays) return;
     if (pbad && i < n_rays) pbad[i] = 0;
@@ -142,6 +148,7 @@ __global__ void k_btd_validate(const int *off, int n_rays, long long n_zones, in
     } else if (v < e && e <= n_zones) {
         zbad[v] = 0;  // the factor kernel's arrival count
         zill[v] = 0;
+        znorm[2 * v] = znorm[2 * v + 1] = 0u;
         ends[v] = v == e - 1 ? kFirst | kLast : kFirst;  // (zero before)
         if (v < e - 1) ends[e - 1] = kLast;
     }
@@ -366,10 +373,13 @@ __device__ __forceinline__ float btd_rcp(float p) {  // p and 1/p normal numbers
 // is much smaller than its terms, as with ill-conditioned blocks, the solution is further off (random blocks without a
 // dominant diagonal, coupled by 0.3 of their size: 2 to 4 times in the median, 30 times in one ray of ten). A ray
 // whose largest pivot in some zone exceeds the smallest kPivots1 or kPivots2 times is therefore refined once or twice
-// more than asked, and not cut into segments. (The pivots are at hand; max|D| max|D^{-1}| says the same, and looking
-// for it cost 2 to 4 %.) Blocks with dominant diagonals have a ratio of 1 to 2, Newton systems 10 to 13, those
-// random blocks 15 to 1e4.
-constexpr float kPivots1 = 24.f, kPivots2 = 256.f;
+// more than asked, and not cut into segments. If a residual of more than kSlowest^(n_refine + 2) of d is left then (of
+// 1e-10 of it with many sweeps, which end at the FP64 residual's rounding), a block's inverse in FP32 says too little,
+// and the ray is solved in FP64 (k_btd_fp64). (The pivots are at hand; max|D| max|D^{-1}| says the same, and looking for
+// it cost 2 to 4 %.) Blocks with dominant diagonals have a ratio of 1 to 2, Newton systems 10 to 13, those random
+// blocks 15 to 1e4. A limit on the pivots instead of the residual (4096) also took rays that converge: random blocks
+// coupled by 0.03 of their size, m = 84, 304 rays of 100 zones: 100 ms against 15.
+constexpr float kPivots1 = 24.f, kPivots2 = 256.f, kSlowest = 0.03f;
 
 // The panel warp's state: lane x holds rows x + 32 t of the panel's eight columns.
 template <int NT>
@@ -1669,6 +1679,7 @@ __global__ void __launch_bounds__(kResidThreads) k_btd_resid(const BtdArgs a) {
     if (!ray_range(a, blockIdx.x, z0, z1) || z1 == z0 || a.zbad[z0]) return;
     const int m = a.m, np = (m + 7) >> 3;
     const long long units = (z1 - z0) * np;
+    float big = 0.f, size = 0.f;  // max|r|, max|d| of this lane's rows
     for (long long q = units * blockIdx.y / gridDim.y + warp, qe = units * (blockIdx.y + 1) / gridDim.y; q < qe; q += nw) {
         const long long k = z0 + q / np;
         const int i0 = 8 * (int)(q % np);
@@ -1689,8 +1700,146 @@ __global__ void __launch_bounds__(kResidThreads) k_btd_resid(const BtdArgs a) {
         s += resid_groups(a.C + ro, x0 + m, nc, cc, m);
         s += __shfl_xor_sync(0xffffffffu, s, 1);
         s += __shfl_xor_sync(0xffffffffu, s, 2);
-        if (cc == 0 && i0 + rr < m) a.r[k * m + i] = a.d[k * m + i] - s;
+        if (cc == 0 && i0 + rr < m) {
+            const double d = a.d[k * m + i];
+            a.r[k * m + i] = d - s;
+            if (a.norm) {
+                big = fmaxf(big, fabs(d - s) <= 1e300 ? (float)fabs(d - s) : INFINITY);  // (NaN counts as infinite)
+                size = fmaxf(size, (float)fabs(d));
+            }
+        }
     }
+    if (a.norm) {
+        atomicMax(a.znorm + 2 * z0, __float_as_uint(big));
+        atomicMax(a.znorm + 2 * z0 + 1, __float_as_uint(size));
+    }
+}
+
+// Rays with ill-conditioned blocks that the sweeps do not settle (kSlowest), all in FP64: a CTA of eight warps per ray,
+// block elimination from the first zone on. D_k is eliminated in shared memory by Gauss-Jordan steps with partial
+// pivoting, its columns replaced by the multipliers; these are then done over on [C_k, d_k - A_k y_{k-1}], `cols`
+// columns at a time, which leaves G_k and y_k (an inverse would square the block's condition number in the error; so
+// would the multipliers in FP32, 0.5 ms a zone, in some rays). G_k is kept as the two words of its doubles in the places
+// of G_k and A_k, y_k in x. Bound by the FP64 pipe and the steps' barriers (2.5 m^3 FMAs a zone; 0.85 ms at m = 84):
+// for the few rays that need it.
+constexpr int kExactThreads = 256;
+constexpr size_t exact_smem(int m, int cols) {
+    return ((size_t)m * m + (size_t)m * cols + m) * sizeof(double) + (size_t)m * sizeof(int);
+}
+__global__ void __launch_bounds__(kExactThreads) k_btd_fp64(const BtdArgs a, int cols, float enough) {
+    extern __shared__ __align__(16) double W[];  // [m][m]; V: [m][cols]; t: [m]; the pivots' rows
+    __shared__ double s_best[kExactThreads / 32];
+    __shared__ int s_row[kExactThreads / 32], s_bad;
+    long long z0, z1;
+    if (!ray_range(a, blockIdx.x, z0, z1) || a.zbad[z0]) return;
+    if (__uint_as_float(a.znorm[2 * z0]) <= enough * __uint_as_float(a.znorm[2 * z0 + 1])) return;
+    const int m = a.m, ld = a.ld, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    double *V = W + m * m, *t = V + m * cols;
+    int *cur = reinterpret_cast<int *>(t + m);
+    int *const G1 = reinterpret_cast<int *>(a.Gt), *const G0 = reinterpret_cast<int *>(a.At);  // high and low words
+    auto G = [&](long long k, int i, int j) {
+        const size_t e = ((size_t)k * m + i) * ld + j;
+        return __hiloint2double(G1[e], G0[e]);
+    };
+    if (tid == 0) s_bad = 0;
+    for (long long k = z0; k < z1; ++k) {
+        const double *A = a.A + (size_t)k * m * m, *B = a.B + (size_t)k * m * m, *C = a.C + (size_t)k * m * m;
+        for (int e = tid; e < m * m; e += kExactThreads) {
+            const int i = e / m, j = e - i * m;
+            double v = B[e];
+            if (k > z0)
+                for (int q = 0; q < m; ++q) v = fma(-A[i * m + q], G(k - 1, q, j), v);
+            W[e] = v;
+        }
+        for (int i = tid; i < m; i += kExactThreads) {
+            double v = a.d[k * m + i];
+            if (k > z0)
+                for (int q = 0; q < m; ++q) v = fma(-A[i * m + q], a.x[(k - 1) * m + q], v);
+            t[i] = v;
+        }
+        bool used = false;  // row tid has been a pivot
+        for (int j = 0; j < m; ++j) {
+            __syncthreads();
+            double best = tid < m && !used ? fabs(W[tid * m + j]) : -1.0;  // (m <= kExactThreads)
+            int row = tid;
+            for (int o = 16; o > 0; o >>= 1) {
+                const double b = __shfl_down_sync(0xffffffffu, best, o);
+                const int r = __shfl_down_sync(0xffffffffu, row, o);
+                if (b > best) {
+                    best = b;
+                    row = r;
+                }
+            }
+            if (lane == 0) {
+                s_best[warp] = best;
+                s_row[warp] = row;
+            }
+            __syncthreads();
+            best = s_best[0];
+            row = s_row[0];
+            for (int w = 1; w < kExactThreads / 32; ++w)
+                if (s_best[w] > best) {
+                    best = s_best[w];
+                    row = s_row[w];
+                }
+            row = row < m ? row : m - 1;
+            const double p = W[row * m + j];
+            if (tid == 0) {
+                cur[j] = row;
+                if (!(fabs(p) > 0.0 && fabs(p) < INFINITY)) s_bad = 1;
+            }
+            if (tid == row) used = true;
+            __syncthreads();  // (everyone has the pivot)
+            if (tid < m && tid != row) W[tid * m + j] = -W[tid * m + j] / p;
+            __syncthreads();
+            const int n = m - 1 - j;
+            for (int e = tid; e < m * n; e += kExactThreads) {
+                const int i = e / n, c = j + 1 + e - i * n;
+                if (i != row) W[i * m + c] = fma(W[i * m + j], W[row * m + c], W[i * m + c]);
+            }
+        }
+        __syncthreads();
+        for (int c0 = k + 1 < z1 ? 0 : m; c0 <= m; c0 += cols) {  // columns of [C, t]
+            const int n = min(cols, m + 1 - c0);
+            for (int e = tid; e < m * n; e += kExactThreads) {
+                const int i = e / n, c = e - i * n;
+                V[e] = c0 + c < m ? C[i * m + c0 + c] : t[i];
+            }
+            for (int j = 0; j < m; ++j) {
+                __syncthreads();
+                const int row = cur[j];
+                for (int e = tid; e < m * n; e += kExactThreads) {
+                    const int i = e / n, c = e - i * n;
+                    if (i != row) V[e] = fma(W[i * m + j], V[row * n + c], V[e]);
+                }
+            }
+            __syncthreads();
+            for (int e = tid; e < m * n; e += kExactThreads) {
+                const int j = e / n, c = e - j * n;
+                const double v = V[cur[j] * n + c] / W[cur[j] * m + j];
+                if (c0 + c < m) {
+                    const size_t g = ((size_t)k * m + j) * ld + c0 + c;
+                    G1[g] = __double2hiint(v);
+                    G0[g] = __double2loint(v);
+                } else {
+                    a.x[k * m + j] = v;
+                }
+            }
+            __syncthreads();
+        }
+    }
+    for (long long k = z1 - 2; k >= z0; --k) {
+        for (int j = warp; j < m; j += kExactThreads / 32) {
+            double v = 0.0;
+            for (int q = lane; q < m; q += 32) v = fma(G(k, j, q), a.x[(k + 1) * m + q], v);
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane == 0) a.x[k * m + j] -= v;
+        }
+        __syncthreads();
+    }
+    if (!s_bad) return;
+    for (long long e = z0 * m + tid; e < z1 * m; e += kExactThreads) a.x[e] = __longlong_as_double(0x7ff8000000000000ll);
+    if (tid == 0) atomicOr(a.flag, 2);
 }
 
 }  // namespace
@@ -1777,6 +1926,7 @@ struct vx_btd {
     size_t blocks = 0;
     unsigned short *nz = nullptr;
     int slots = 0;  // factor CTAs the device holds at once
+    unsigned *znorm = nullptr;
     int *zbad = nullptr, *zmid = nullptr, *zill = nullptr, *flag = nullptr;  // flag[0]: numeric flag, flag[1]: offsets invalid
     double *r = nullptr;
     // segments: most zones of a call that is cut into them (0: none), and their system's arrays (a row per SM)
@@ -1797,6 +1947,7 @@ static void btd_free(vx_btd *h) {
     cudaFree(h->zbad);
     cudaFree(h->zmid);
     cudaFree(h->zill);
+    cudaFree(h->znorm);
     cudaFree(h->Sr);
     cudaFree(h->nzr);
     cudaFree(h->zr);
@@ -1875,6 +2026,7 @@ extern "C" vx_status vx_btd_create_rays(int m, long long max_zones, int n_refine
     if (e == cudaSuccess) e = cudaMalloc(&h->zbad, zc * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&h->zmid, zc * sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&h->zill, zc * sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&h->znorm, zc * 2 * sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMalloc(&h->r, zc * m * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&h->flag, 2 * sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(h->flag, 0, 2 * sizeof(int));
@@ -1888,6 +2040,8 @@ extern "C" vx_status vx_btd_create_rays(int m, long long max_zones, int n_refine
                              sweep_kernel<false, false>(m)};
     for (int i = 0; i < 4 && e == cudaSuccess; ++i)
         e = cudaFuncSetAttribute(sweeps[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFull);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute((const void *)k_btd_fp64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemFull);
     if (e != cudaSuccess) {
         btd_free(h);
         return bfail(e == cudaErrorMemoryAllocation ? VX_ERR_OOM : VX_ERR_CUDA, "vx_btd_create: %s",
@@ -1947,6 +2101,8 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
     a.zmid = h->zmid;
     a.zill = h->zill;
     a.min_ill = 0;
+    a.znorm = h->znorm;
+    a.norm = false;
     // Two CTAs per ray while they all find room at once, and with rays of 16 zones or more where the last wave of
     // one CTA per ray would be less than 5/8 full. GB300, one -> two, 100 zones: m = 84, 20 rays 3.60 -> 1.98 ms,
     // 152 4.76 -> 3.73, 160 5.91 -> 5.32, 330 10.58 -> 9.02, 480 13.25 -> 12.54, but 240 6.67 -> 6.70 and
@@ -2024,7 +2180,7 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
     BTD_CU(cudaMemsetAsync(h->flag + 1, 0, sizeof(int), s));
     BTD_CU(cudaMemsetAsync(h->zmid, 0, (size_t)n_zones * sizeof(int), s));
     k_btd_validate<<<(unsigned)((n_rays + 256) / 256), 256, 0, s>>>(ray_offsets, n_rays, n_zones, h->flag + 1, h->flag, h->zbad,
-                                                                   h->zill, h->zmid, f.pbad);
+                                                                   h->zill, h->znorm, h->zmid, f.pbad);
     BTD_CU(cudaGetLastError());
     launch_convert(h->m, n_zones, h->sms, s, a);
     BTD_CU(cudaGetLastError());
@@ -2073,6 +2229,15 @@ extern "C" vx_status vx_btd_solve(vx_btd *h, int n_rays, long long n_zones, cons
         BTD_CU(cudaGetLastError());
         BTD_CU((launch_sweep<false, false>(h->m, ctas, h->smem_sweep, s, f)));
     }
+    a.min_ill = 1;
+    a.norm = true;
+    k_btd_resid<<<dim3(n_rays, (unsigned)split), kResidThreads, 0, s>>>(a);
+    BTD_CU(cudaGetLastError());
+    int cols = h->m + 1;
+    while (exact_smem(h->m, cols) > kSmemFull) --cols;
+    k_btd_fp64<<<n_rays, kExactThreads, exact_smem(h->m, cols), s>>>(
+        a, cols, fmaxf(powf(kSlowest, (float)h->n_refine + 2.f), 1e-10f));
+    BTD_CU(cudaGetLastError());
     return VX_OK;
 }
 
