@@ -337,7 +337,7 @@ def run_solve(args):
             "e2e": {"value": job_rate(Z, world, ms_e2e), "unit": "zones/s", "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": d2h, "call": "BlockTridiagSolver.solve_host (pinned host tensors)",
                     "ms_per_step": ms_e2e},
-            "gpu_launches": args.steps * (4 + 2 * SOLVE_REFINE),  # validate, convert, factor, sweep; resid + sweep each
+            "gpu_launches": args.steps * (10 + 2 * SOLVE_REFINE),  # validate, convert, factor, sweep; resid + sweep each, twice more; resid, fp64
             "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                          "traffic": None,
                          "note": "FP32 flops of the block factorisation over the whole step (factor kernel, "
